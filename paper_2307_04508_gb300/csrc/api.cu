@@ -178,6 +178,210 @@ ltgw_status naf_metric_tc(ltgw_ctx *ctx, int n, int64_t n_pairs, const double *B
 ltgw_status emu_gemm(ltgw_ctx *ctx, int m, int n, int64_t K, const double *A, int64_t lda, const double *B,
                      int64_t ldb, double *C, int64_t ldc, bool sym, int s, cudaStream_t st);
 
+// ---- FP64 contractions on the tensor cores from integer digits (slice_gemm.cu)
+// The FP64 form's products: 7 digits in base 256 hold 55 bits relative to each
+// operand row's largest magnitude, and the products kept (levels i + j <= 8)
+// leave an error of about 2^-52 of the rows' scales per entry, no more than a
+// length-K FP64 sum's own rounding.
+struct SliceForm {
+  int ns, bits;
+};
+constexpr SliceForm kFp64Digits{7, 8};
+constexpr size_t kSliceOperandMax = (size_t)4 << 30;   // digits of one operand held at a time
+constexpr size_t kSlicePartialMax = (size_t)1 << 30;   // K-split partial tiles
+
+// Products this small stay on the CUDA-core kernels: a digit product costs two
+// to four launches before its first MMA (about 30 us in all; the 64 x 64 FP64
+// tiles take that long from about 2e7 multiply-adds on.  Measured at n = 264,
+// 560 pairs, 3.9e7: 0.587 ms of FP64 tiles, 0.059 ms from digits).
+bool slices_pay(int64_t m, int64_t n, int64_t k, int64_t batch) {
+  return k >= 128 && (double)m * (double)n * (double)k * (double)batch >= 2e7;
+}
+
+struct SliceOperand {
+  uint8_t *dig = nullptr;
+  int *exps = nullptr;
+  int rows_p = 0, nkb = 0;
+  int64_t dig_batch = 0;
+  void layout(Arena &A, int64_t rows, int64_t K, int batch, SliceForm f) {
+    rows_p = (int)slice_rows_padded(rows);
+    nkb = (int)((K + SL_K - 1) / SL_K);
+    dig_batch = slice_digit_bytes(rows, nkb, f.ns);
+    dig = A.take<uint8_t>((size_t)dig_batch * batch);
+    exps = A.take<int>((size_t)rows_p * batch);
+  }
+  SliceSrc source(const double *X, int64_t ld, int64_t x_batch, int rows, int64_t K, bool cols) const {
+    SliceSrc a;
+    a.X = X; a.ld = ld; a.x_batch = x_batch; a.cols = cols; a.rows = rows; a.rows_p = rows_p; a.K = K; a.nkb = nkb;
+    a.dig = dig; a.dig_batch = dig_batch; a.exps = exps; a.exp_batch = rows_p;
+    return a;
+  }
+};
+
+// Reserve `layout` in `ar`; false (and no error recorded) when the memory is
+// not there, or when growing would take more than half of what is free on the
+// device (other contexts' solves size their own workspace from it): the caller
+// then takes the CUDA-core kernels, or one K split.
+template <class Layout>
+bool slice_reserve(Arena &ar, Layout &&layout) {
+  ar.begin_sizing();
+  layout(ar);
+  if (ar.need > ar.cap) {
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
+    else if (ar.need > (free_b + ar.cap) / 2) { ar.sizing = false; return false; }
+  }
+  if (ar.commit() != cudaSuccess) return false;
+  layout(ar);
+  return true;
+}
+
+// One digit contraction: plan, K-split partials (arena a4), launch.
+ltgw_status slice_run(ltgw_ctx *ctx, SliceGemmArgs &g, SliceForm f, cudaStream_t s) {
+  g.ns = f.ns; g.bits = f.bits; g.err = ctx->flags;
+  size_t part = slice_gemm_plan(&g, ctx->n_sm, kSlicePartialMax);
+  if (part && !slice_reserve(ctx->a4, [&](Arena &A) { g.partial = A.take<double>(part / sizeof(double)); })) {
+    g.splits = 1; g.kb_per_split = g.nkb; g.partial = nullptr;   // no room for partials: one split
+  }
+  CHECK_LAUNCH(ctx, launch_slice_gemm(g, ctx->n_sm, s), g.partial || (g.sym && g.mirror) ? 2 : 1);
+  return LTGW_OK;
+}
+
+// Chunk of the contraction length so that `rows` operand rows stay within kSliceOperandMax.
+int64_t slice_k_chunk(int64_t rows, int64_t K, int batch, SliceForm f) {
+  const int64_t per_k = slice_rows_padded(rows) * 2 * f.ns * batch;
+  const int64_t most = std::max<int64_t>(2048, (int64_t)kSliceOperandMax / per_k);
+  const int64_t n = (K + most - 1) / most;
+  return std::min(K, ((K + n - 1) / n + 63) / 64 * 64);
+}
+
+// C = beta C + X X^T (full, symmetric bit for bit), X [n][ld] with K columns.
+// *done is false when the product was left to the caller (no memory).
+ltgw_status slice_syrk(ltgw_ctx *ctx, int n, int64_t K, const double *X, int64_t ld, double *C, double beta,
+                       SliceForm f, cudaStream_t s, bool *done) {
+  SliceOperand o;
+  const int64_t chunk = slice_k_chunk(n, K, 1, f);
+  *done = slice_reserve(ctx->a5, [&](Arena &A) { o.layout(A, n, chunk, 1, f); });
+  if (!*done) return LTGW_OK;
+  for (int64_t k0 = 0; k0 < K; k0 += chunk) {
+    const int64_t kc = std::min(chunk, K - k0);
+    CHECK_LAUNCH(ctx, launch_slice_operand(o.source(X + k0, ld, 0, n, kc, false), f.ns, f.bits, 1, s), 3);
+    SliceGemmArgs g;
+    g.A = g.B = o.dig; g.ea = g.eb = o.exps; g.nkb = o.nkb;
+    g.M = g.N = n; g.sym = 1; g.C = C; g.ldc = n; g.beta = k0 ? 1.0 : beta;
+    if (slice_run(ctx, g, f, s) != LTGW_OK) return ctx->status();
+  }
+  return LTGW_OK;
+}
+
+// out_b [N][ld_out] = Ut X_b for the columns of X_b [n_aux][ld] (Ut rows [N][n_aux]).
+ltgw_status slice_project(ltgw_ctx *ctx, int N, int n_aux, const double *Ut, const double *X, int64_t ld,
+                          int64_t x_batch, int64_t cols, int batch, double *out, int64_t ld_out, int64_t out_batch,
+                          SliceForm f, cudaStream_t s, bool *done) {
+  SliceOperand u, x;
+  const int64_t per_col = (int64_t)((n_aux + SL_K - 1) / SL_K) * SL_K * 2 * f.ns * batch;
+  const int64_t most = std::max<int64_t>(4096, (int64_t)kSliceOperandMax / per_col / 128 * 128);
+  const int64_t n_chunks = (cols + most - 1) / most;
+  const int64_t chunk = std::min(cols, ((cols + n_chunks - 1) / n_chunks + 127) / 128 * 128);
+  *done = slice_reserve(ctx->a5, [&](Arena &A) {
+    u.layout(A, N, n_aux, 1, f);
+    x.layout(A, chunk, n_aux, batch, f);
+  });
+  if (!*done) return LTGW_OK;
+  CHECK_LAUNCH(ctx, launch_slice_operand(u.source(Ut, n_aux, 0, N, n_aux, false), f.ns, f.bits, 1, s), 3);
+  for (int64_t c0 = 0; c0 < cols; c0 += chunk) {
+    const int cc = (int)std::min(chunk, cols - c0);
+    CHECK_LAUNCH(ctx, launch_slice_operand(x.source(X + c0, ld, x_batch, cc, n_aux, true), f.ns, f.bits, batch, s), 3);
+    SliceGemmArgs g;
+    g.A = x.dig; g.a_batch = x.dig_batch; g.ea = x.exps; g.ea_batch = x.rows_p;
+    g.B = u.dig; g.eb = u.exps; g.nkb = u.nkb; g.batch = batch;
+    g.M = cc; g.N = N; g.C = out + c0; g.ldc = ld_out; g.c_batch = out_batch;
+    if (slice_run(ctx, g, f, s) != LTGW_OK) return ctx->status();
+  }
+  return LTGW_OK;
+}
+
+// W_j[t][c] = sum_PQ Btt[t][P][c] C_j[P][Q] Btt[t][Q][c] (Eq. ScreenedCoulombOrbital)
+// with the column dot in the contraction's epilogue; frequencies in blocks.
+ltgw_status slice_wnm(ltgw_ctx *ctx, int N, int n_omega, const double *C, int T, int n_orb_act, const double *Btt,
+                      int64_t ld_btt, int64_t stride_btt, double *W, SliceForm f, cudaStream_t s, bool *done) {
+  const int cols = T * n_orb_act;
+  SliceOperand r, c;
+  double *cd = nullptr;
+  const int64_t nkb = (N + SL_K - 1) / SL_K;
+  const int blk = (int)std::min<int64_t>(
+      n_omega, std::max<int64_t>(1, (int64_t)kSliceOperandMax / slice_digit_bytes(N, nkb, f.ns)));
+  const int tiles_n = (N + 63) / 64;
+  *done = slice_reserve(ctx->a5, [&](Arena &A) {
+    r.layout(A, cols, N, 1, f);
+    c.layout(A, N, N, blk, f);
+    cd = A.take<double>((size_t)blk * 4 * tiles_n * cols);
+  });
+  if (!*done) return LTGW_OK;
+  SliceSrc rs = r.source(Btt, ld_btt, 0, cols, N, true);
+  rs.col_group = n_orb_act; rs.col_stride = stride_btt;
+  CHECK_LAUNCH(ctx, launch_slice_operand(rs, f.ns, f.bits, 1, s), 3);
+  for (int j0 = 0; j0 < n_omega; j0 += blk) {
+    const int nb = std::min(blk, n_omega - j0);
+    CHECK_LAUNCH(ctx, launch_slice_operand(c.source(C + (int64_t)j0 * N * N, N, (int64_t)N * N, N, N, false), f.ns,
+                                           f.bits, nb, s), 3);
+    SliceGemmArgs g;
+    g.A = r.dig; g.ea = r.exps;
+    g.B = c.dig; g.b_batch = c.dig_batch; g.eb = c.exps; g.eb_batch = c.rows_p;
+    g.nkb = r.nkb; g.batch = nb; g.M = cols; g.N = N;
+    g.cd_B = Btt; g.cd_ld = ld_btt; g.cd_stride = stride_btt; g.cd_cols = n_orb_act; g.cd_out = cd; g.cd_ldo = cols;
+    if (slice_run(ctx, g, f, s) != LTGW_OK) return ctx->status();
+    CHECK_LAUNCH(ctx, launch_slice_coldot_reduce(g, W + (int64_t)j0 * cols, cols, s), 1);
+  }
+  return LTGW_OK;
+}
+
+// M_t = alpha (Bt diag(f_t)) Bt^T for t < n_t (full, symmetric).  Both operands
+// are Bt diag(sqrt |f_t|), the sign of f_t with the first one: an entry's error
+// then follows the pairs that carry it, also where a factor singles out few of
+// them (a factor on one side only would weigh that side's rounding with every
+// pair of the other).
+ltgw_status slice_pi(ltgw_ctx *ctx, int N, int64_t n_pairs, const double *Bt, int64_t ldb, const double *delta,
+                     int n_t, const double *p0, const double *p1, int mode, int alpha_exp, int alpha_neg, double *M,
+                     SliceForm f, cudaStream_t s, bool *done) {
+  SliceOperand o, o2;   // o2: the unsigned operand, written and read only where some factor is negative
+  double *fac = nullptr;
+  int *neg = nullptr;
+  const int64_t per_t = 2 * slice_rows_padded(N) * 2 * f.ns;
+  // the pair range first (each chunk is another pass over M), then the points at a time
+  const int64_t chunk = slice_k_chunk(2 * N, n_pairs, 1, f);
+  const int blk = (int)std::min<int64_t>(n_t, std::max<int64_t>(1, (int64_t)kSliceOperandMax / (per_t * chunk)));
+  *done = slice_reserve(ctx->a5, [&](Arena &A) {
+    o.layout(A, N, chunk, blk, f);
+    o2.layout(A, N, chunk, blk, f);
+    fac = A.take<double>((size_t)n_t * 2 * chunk);
+    neg = A.take<int>(1);
+  });
+  if (!*done) return LTGW_OK;
+  for (int64_t k0 = 0; k0 < n_pairs; k0 += chunk) {
+    const int64_t kc = std::min(chunk, n_pairs - k0);
+    LTGW_CUDA(ctx, cudaMemsetAsync(neg, 0, sizeof(int), s));
+    CHECK_LAUNCH(ctx, launch_pi_root_factor(delta + k0, kc, n_t, p0, p1, mode, fac, fac + (int64_t)n_t * kc, neg, s), 1);
+    for (int t0 = 0; t0 < n_t; t0 += blk) {
+      const int nb = std::min(blk, n_t - t0);
+      SliceSrc a = o.source(Bt + k0, ldb, 0, N, kc, false);
+      a.colscale = fac + (int64_t)t0 * kc; a.cs_batch = kc;
+      CHECK_LAUNCH(ctx, launch_slice_operand(a, f.ns, f.bits, nb, s), 3);
+      SliceSrc b = o2.source(Bt + k0, ldb, 0, N, kc, false);
+      b.colscale = fac + (int64_t)(n_t + t0) * kc; b.cs_batch = kc; b.only_if = neg;
+      CHECK_LAUNCH(ctx, launch_slice_operand(b, f.ns, f.bits, nb, s), 3);
+      SliceGemmArgs g;
+      g.A = g.B = o.dig; g.a_batch = g.b_batch = o.dig_batch; g.ea = g.eb = o.exps; g.ea_batch = g.eb_batch = o.rows_p;
+      g.B_alt = o2.dig; g.b_sel = neg;   // |sqrt| rows have the same exponents
+      g.nkb = o.nkb; g.batch = nb; g.M = g.N = N; g.sym = 1;
+      g.C = M + (int64_t)t0 * N * N; g.ldc = N; g.c_batch = (int64_t)N * N;
+      g.beta = k0 ? 1.0 : 0.0; g.alpha_exp = alpha_exp; g.alpha_neg = alpha_neg;
+      if (slice_run(ctx, g, f, s) != LTGW_OK) return ctx->status();
+    }
+  }
+  return LTGW_OK;
+}
+
 // K builder for the streamed solve: fills w.A (n x n) itself.
 using KBuilder = std::function<ltgw_status(double *K)>;
 
@@ -226,12 +430,17 @@ ltgw_status naf_basis_dev(ltgw_ctx *ctx, Arena &ar, int n, int64_t n_pairs, cons
   } else if (emu_slices) {
     if (emu_gemm(ctx, n, n, n_pairs, B, ld, B, ld, w.A, n, true, emu_slices, s) != LTGW_OK) return ctx->status();
   } else {
-    GemmF64Args g;
-    g.M = n; g.N = n; g.K = n_pairs;
-    g.A = B; g.lda = ld; g.B = B; g.ldb = ld;
-    g.C = w.A; g.ldc = n;
-    g.syrk = 1;
-    CHECK_LAUNCH(ctx, launch_gemm_f64(g, 1, true, true, s), 1);
+    bool done = false;
+    if (slices_pay(n, n, n_pairs, 1) && slice_syrk(ctx, n, n_pairs, B, ld, w.A, 0.0, kFp64Digits, s, &done) != LTGW_OK)
+      return ctx->status();
+    if (!done) {
+      GemmF64Args g;
+      g.M = n; g.N = n; g.K = n_pairs;
+      g.A = B; g.lda = ld; g.B = B; g.ldb = ld;
+      g.C = w.A; g.ldc = n;
+      g.syrk = 1;
+      CHECK_LAUNCH(ctx, launch_gemm_f64(g, 1, true, true, s), 1);
+    }
   }
   LTGW_CUDA(ctx, cudaMemsetAsync(w.V, 0, (size_t)(n + 64) * n * sizeof(double), s));
   int nl = 0;
@@ -264,31 +473,35 @@ ltgw_status polarizability_dev(ltgw_ctx *ctx, int N, int64_t n_pairs, const doub
                                const double *delta, int n_omega, const double *d_omega,
                                int n_tau, const double *d_x, const double *d_w, const double *d_E,
                                double *M, int spin, double *Pi, cudaStream_t s, int lt_form) {
-  GemmF64Args g;
-  g.M = N; g.N = N; g.K = n_pairs;
-  g.A = Bt; g.lda = ldb; g.B = Bt; g.ldb = ldb;
-  g.ldc = N; g.strideC = (int64_t)N * N;
-  g.syrk = 1;
-  g.delta = delta;
+  const int mode = n_tau == 0 ? SCALE_DIRECT : (lt_form == 2 ? SCALE_EXPTAU : SCALE_LAPLACE);
+  const int n_t = n_tau ? n_tau : n_omega;
+  const double *p0 = n_tau ? d_x : d_omega, *p1 = mode == SCALE_LAPLACE ? d_w : nullptr;
+  double *out = n_tau ? M : Pi;
   ctx->mark(EV_PI0, s);
-  if (n_tau == 0) {
-    g.C = Pi;
-    g.alpha = -2.0 * spin;
-    g.scale_mode = SCALE_DIRECT;
-    g.batch_p0 = d_omega;
-    CHECK_LAUNCH(ctx, launch_gemm_f64(g, n_omega, true, true, s), 1);
-    ctx->mark(EV_PI1, s);
-  } else {
-    g.C = M;
-    g.alpha = 1.0;
-    g.scale_mode = lt_form == 2 ? SCALE_EXPTAU : SCALE_LAPLACE;
-    g.batch_p0 = d_x;
-    g.batch_p1 = lt_form == 2 ? nullptr : d_w;
-    CHECK_LAUNCH(ctx, launch_gemm_f64(g, n_tau, true, true, s), 1);
-    ctx->mark(EV_PI1, s);
+  bool done = false;
+  // alpha: 1 for the moments, -2 spin = -2 or -4 for Pi itself
+  if (slices_pay(N, N, n_pairs, n_t) &&
+      slice_pi(ctx, N, n_pairs, Bt, ldb, delta, n_t, p0, p1, mode, n_tau ? 0 : spin, n_tau ? 0 : 1, out, kFp64Digits,
+               s, &done) != LTGW_OK)
+    return ctx->status();
+  if (!done) {
+    GemmF64Args g;
+    g.M = N; g.N = N; g.K = n_pairs;
+    g.A = Bt; g.lda = ldb; g.B = Bt; g.ldb = ldb;
+    g.ldc = N; g.strideC = (int64_t)N * N;
+    g.syrk = 1;
+    g.delta = delta;
+    g.C = out;
+    g.alpha = n_tau ? 1.0 : -2.0 * spin;
+    g.scale_mode = mode;
+    g.batch_p0 = p0;
+    g.batch_p1 = p1;
+    CHECK_LAUNCH(ctx, launch_gemm_f64(g, n_t, true, true, s), 1);
+  }
+  ctx->mark(EV_PI1, s);
+  if (n_tau)
     CHECK_LAUNCH(ctx, launch_recombine(M, n_tau, d_E, n_omega, (int64_t)N * N, -2.0 * spin, Pi, s),
                  (n_omega + 63) / 64);
-  }
   return LTGW_OK;
 }
 
@@ -1319,11 +1532,17 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
         if (emu_prepare(ctx, n_aux, n_aux, cols, n_sl, true, 0, &ep, s, true) != LTGW_OK) return ctx->status();
         if (emu_syrk(ctx, ep, B_blk, cols, K, 1.0, s) != LTGW_OK) return ctx->status();
       } else {
-        GemmF64Args g;  // K += B_blk B_blk^T
-        g.M = n_aux; g.N = n_aux; g.K = cols;
-        g.A = B_blk; g.lda = cols; g.B = B_blk; g.ldb = cols;
-        g.C = K; g.ldc = n_aux; g.syrk = 1; g.beta = 1.0;
-        CHECK_LAUNCH(ctx, launch_gemm_f64(g, 1, true, true, s), 1);
+        bool done = false;   // K += B_blk B_blk^T
+        if (slices_pay(n_aux, n_aux, cols, 1) &&
+            slice_syrk(ctx, n_aux, cols, B_blk, cols, K, 1.0, kFp64Digits, s, &done) != LTGW_OK)
+          return ctx->status();
+        if (!done) {
+          GemmF64Args g;
+          g.M = n_aux; g.N = n_aux; g.K = cols;
+          g.A = B_blk; g.lda = cols; g.B = B_blk; g.ldb = cols;
+          g.C = K; g.ldc = n_aux; g.syrk = 1; g.beta = 1.0;
+          CHECK_LAUNCH(ctx, launch_gemm_f64(g, 1, true, true, s), 1);
+        }
       }
       if (block_done() != LTGW_OK) return ctx->status();
     }
@@ -1374,6 +1593,24 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
   if (ctx->a2.commit() != cudaSuccess) { ctx->fail(LTGW_ERR_NOMEM, "solve workspace allocation failed"); return ctx->status(); }
   layout2(ctx->a2);
 
+  // out_b = U^T X_b over `cols` columns of X_b (FP64 form)
+  auto project_f64 = [&](const double *X, int64_t ld, int64_t x_batch, int64_t cols, int batch, double *out,
+                         int64_t ld_out, int64_t out_batch) -> ltgw_status {
+    bool done = false;
+    if (slices_pay(N, cols, n_aux, batch) &&
+        slice_project(ctx, N, n_aux, d_Ut, X, ld, x_batch, cols, batch, out, ld_out, out_batch, kFp64Digits, s,
+                      &done) != LTGW_OK)
+      return ctx->status();
+    if (done) return LTGW_OK;
+    GemmF64Args g;
+    g.M = N; g.N = (int)cols; g.K = n_aux;
+    g.A = d_Ut; g.lda = n_aux;
+    g.B = X; g.ldb = ld; g.strideB = x_batch;
+    g.C = out; g.ldc = ld_out; g.strideC = out_batch;
+    CHECK_LAUNCH(ctx, launch_gemm_f64(g, batch, true, false, s), 1);
+    return LTGW_OK;
+  };
+
   const double *Bt = B_act;
   int64_t ld_bt = ld_act;
   const double *Btt = d_Btg + n_fc;
@@ -1399,12 +1636,9 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
                           n_sl, s) != LTGW_OK)
             return ctx->status();
         } else {
-          GemmF64Args g;  // R~_ov[:, block] = U^T R_blk
-          g.M = N; g.N = (int)cols; g.K = n_aux;
-          g.A = d_Ut; g.lda = n_aux;
-          g.B = B_blk; g.ldb = cols;
-          g.C = d_Bt + (int64_t)(i0 - n_fc) * n_virt; g.ldc = n_ov;
-          CHECK_LAUNCH(ctx, launch_gemm_f64(g, 1, true, false, s), 1);
+          // R~_ov[:, block] = U^T R_blk
+          if (project_f64(B_blk, cols, 0, cols, 1, d_Bt + (int64_t)(i0 - n_fc) * n_virt, n_ov, 0) != LTGW_OK)
+            return ctx->status();
         }
         if (block_done() != LTGW_OK) return ctx->status();
       }
@@ -1413,12 +1647,9 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
       if (project_emu(ctx, N, n_aux, d_Ut, B_act, ld_act, (int)n_ov, d_Bt, n_ov, n_sl, s) != LTGW_OK)
         return ctx->status();
     } else {
-      GemmF64Args g;  // R~_ov = U^T R_ov
-      g.M = N; g.N = (int)std::min<int64_t>(n_ov, INT32_MAX); g.K = n_aux;
-      g.A = d_Ut; g.lda = n_aux;
-      g.B = B_act; g.ldb = ld_act;
-      g.C = d_Bt; g.ldc = n_ov;
-      CHECK_LAUNCH(ctx, launch_gemm_f64(g, 1, true, false, s), 1);
+      // R~_ov = U^T R_ov
+      if (project_f64(B_act, ld_act, 0, std::min<int64_t>(n_ov, INT32_MAX), 1, d_Bt, n_ov, 0) != LTGW_OK)
+        return ctx->status();
     }
     if (emu) {
       for (int t = 0; t < T; ++t)   // R~_tgt[t] = U^T R_tgt[t][:, active]
@@ -1426,12 +1657,10 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
                         d_Btt + (int64_t)t * N * n_orb_act, n_orb_act, n_sl, s) != LTGW_OK)
           return ctx->status();
     } else {
-      GemmF64Args h;  // R~_tgt[t] = U^T R_tgt[t][:, active]
-      h.M = N; h.N = n_orb_act; h.K = n_aux;
-      h.A = d_Ut; h.lda = n_aux; h.strideA = 0;
-      h.B = d_Btg + n_fc; h.ldb = n_orb; h.strideB = (int64_t)n_aux * n_orb;
-      h.C = d_Btt; h.ldc = n_orb_act; h.strideC = (int64_t)N * n_orb_act;
-      CHECK_LAUNCH(ctx, launch_gemm_f64(h, T, true, false, s), 1);
+      // R~_tgt[t] = U^T R_tgt[t][:, active]
+      if (project_f64(d_Btg + n_fc, n_orb, (int64_t)n_aux * n_orb, n_orb_act, T, d_Btt, n_orb_act,
+                      (int64_t)N * n_orb_act) != LTGW_OK)
+        return ctx->status();
     }
     Bt = d_Bt; ld_bt = n_ov;
     Btt = d_Btt; ld_btt = n_orb_act; stride_btt = (int64_t)N * n_orb_act;
@@ -1490,12 +1719,18 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
       if (wnm_emu(ctx, N, n_omega, d_C, T, n_orb_act, Btt, ld_btt, stride_btt, d_W, n_sl, s) != LTGW_OK)
         return ctx->status();
     } else {
-      ColDotArgs cd;
-      cd.N = N; cd.ncols = n_orb_act; cd.n_tgt = T;
-      cd.C = d_C; cd.ldc = N; cd.strideC = (int64_t)N * N;
-      cd.Bt = Btt; cd.ldb = ld_btt; cd.strideBt = stride_btt;
-      cd.W = d_W; cd.ldw = n_orb_act;
-      CHECK_LAUNCH(ctx, launch_gemm_coldot(cd, n_omega, s), 1);
+      bool done = false;
+      if (slices_pay(N, T * n_orb_act, N, n_omega) &&
+          slice_wnm(ctx, N, n_omega, d_C, T, n_orb_act, Btt, ld_btt, stride_btt, d_W, kFp64Digits, s, &done) != LTGW_OK)
+        return ctx->status();
+      if (!done) {
+        ColDotArgs cd;
+        cd.N = N; cd.ncols = n_orb_act; cd.n_tgt = T;
+        cd.C = d_C; cd.ldc = N; cd.strideC = (int64_t)N * N;
+        cd.Bt = Btt; cd.ldb = ld_btt; cd.strideBt = stride_btt;
+        cd.W = d_W; cd.ldw = n_orb_act;
+        CHECK_LAUNCH(ctx, launch_gemm_coldot(cd, n_omega, s), 1);
+      }
     }
     ctx->mark(EV_WNM, s);
 
@@ -1605,12 +1840,12 @@ ltgw_status polarizability_dev_api(ltgw_ctx *ctx, int N, int64_t n_pairs, const 
     if (lt_form != 2) copy_in(ctx, d_w, w, n_tau * sizeof(double), s);
     copy_in(ctx, d_E, h_E.data(), h_E.size() * sizeof(double), s);
   }
+  LTGW_CUDA(ctx, cudaMemsetAsync(ctx->flags, 0, FLAG_COUNT * sizeof(int), s));
   if (ctx->status() != LTGW_OK) return ctx->status();
   if (polarizability_dev(ctx, N, n_pairs, Bt, n_pairs, delta, n_omega, d_om, n_tau, d_x, d_w, d_E, d_M,
                          spin, Pi, s, lt_form) != LTGW_OK)
     return ctx->status();
-  LTGW_CUDA(ctx, cudaStreamSynchronize(s));  // the staged grid lives in the workspace
-  return LTGW_OK;
+  return check_flags(ctx, s);   // synchronises: the staged grid lives in the workspace
 }
 
 // lt_form 1: x, w are the Laplace grid of Eq. LT; 2: x holds tau_k and gamma

@@ -171,6 +171,10 @@ cudaError_t launch_slice_rows(const double *X, int64_t ld, int rows, int64_t col
 // node (SCALE_EXPTAU, p0 = tau), no fused operations.
 cudaError_t launch_pi_factor64(const double *delta, int64_t K, int n_t, const double *p0, const double *p1,
                                int mode, double *f, cudaStream_t st);
+// Root factors of the same f for operands scaled on both sides: sgn[t][k] =
+// sign(f) sqrt|f|, mag[t][k] = sqrt|f|; *neg is set to 1 if any f < 0.
+cudaError_t launch_pi_root_factor(const double *delta, int64_t K, int n_t, const double *p0, const double *p1,
+                                  int mode, double *sgn, double *mag, int *neg, cudaStream_t st);
 // D[r][c] = beta D[r][c] + S[r][c] 2^(ea[r] + eb[c]) (rows <= 65535); lower (rows ==
 // cols, S symmetric): the entries c <= r scaled, each written to (r, c) and (c, r).
 cudaError_t launch_scale_exp2_to(const double *S, int64_t lds, double *D, int64_t ldd, int rows, int cols,
@@ -191,6 +195,73 @@ cudaError_t launch_fp8_quantize_a(const float *X, int64_t Kp, int64_t Kq, int ro
 // partial tiles as launch_tc_split_gemm (column-major).
 cudaError_t launch_tc_fp8_gemm(const TcGemmArgs &g, int n_tiles, cudaStream_t s);
 size_t tc_gemm_smem_bytes();
+
+// ---- FP64-accurate contractions from integer digits (slice_gemm.cu) ----
+// An operand's digits lie in blocks of 64 rows x 16 k: [row / 64][k / 16][digit]
+// [64 rows x 32 bytes], BF16, the 16-byte halves of a row exchanged where bit 2
+// of the row is set (the tensor core's 32-byte swizzle), zero past the rows
+// and past K.  Row r ~ 2^(exps[r]) sum_i digit_i 2^(-bits i).
+constexpr int SL_ROWS = 64, SL_K = 16;
+constexpr int SL_ZERO = -(1 << 20);        // exps of a zero row
+constexpr int SL_NONFINITE = 1 << 20;      // exps of a row with a NaN or an infinity (its products are NaN)
+inline int64_t slice_rows_padded(int64_t rows) { return (rows + 127) / 128 * 128; }
+inline int64_t slice_digit_bytes(int64_t rows, int64_t nkb, int ns) {
+  return slice_rows_padded(rows) * nkb * (int64_t)(SL_K * 2 * ns);
+}
+struct SliceSrc {
+  const double *X = nullptr;   // rows: X[r][k] (ld between rows); cols: operand row r, index k = X[k][r]
+  int64_t ld = 0, x_batch = 0;
+  int cols = 0;
+  int col_group = 0;           // cols: columns per matrix (0: all), matrix t at X + t col_stride
+  int64_t col_stride = 0;
+  const int *only_if = nullptr;   // digits are formed only where *only_if is not 0 (device)
+  int rows = 0, rows_p = 0;    // operand rows, padded to 128
+  int64_t K = 0;
+  int nkb = 0;                 // 16-k blocks held (>= ceil(K / 16))
+  const double *colscale = nullptr;   // rows only: factor of column k (one FP64 product), [batch][K] or shared
+  int64_t cs_batch = 0;
+  uint8_t *dig = nullptr;      // [batch] x dig_batch bytes
+  int64_t dig_batch = 0;
+  int *exps = nullptr;         // [batch] x exp_batch (>= rows_p) ints
+  int64_t exp_batch = 0;
+};
+// ns digits of `bits` bits: (2 .. 8, 7) or (7, 8).
+cudaError_t launch_slice_operand(const SliceSrc &a, int ns, int bits, int batch, cudaStream_t s);
+
+// C_b[n][m] = beta C_b[n][m] + (-1)^alpha_neg 2^alpha_exp sum_k A_b[m][k] B_b[n][k] from
+// digits, m < M, n < N, one rounding per output before the sum with C; sym
+// (B = A): the entries m >= n, mirrored to the others where `mirror` is set or
+// splits > 1.
+// With cd_out, instead: cd_out[b][4 tiles_n][cd_ldo] = partial sums over n of
+// D[m][n] cd_B[t][n][m - t cd_cols], t = m / cd_cols.
+struct SliceGemmArgs {
+  const uint8_t *A = nullptr, *B = nullptr;
+  int64_t a_batch = 0, b_batch = 0;      // bytes (0: shared)
+  const uint8_t *B_alt = nullptr;        // taken for B where *b_sel is not 0 (device)
+  const int *b_sel = nullptr;
+  const int *ea = nullptr, *eb = nullptr;
+  int64_t ea_batch = 0, eb_batch = 0;    // ints
+  int ns = 7, bits = 8, nkb = 0, batch = 1;
+  int M = 0, N = 0, sym = 0, mirror = 1;
+  double *C = nullptr;
+  int64_t ldc = 0, c_batch = 0;
+  double beta = 0.0;
+  int alpha_exp = 0, alpha_neg = 0;
+  const double *cd_B = nullptr;
+  int64_t cd_ld = 0, cd_stride = 0, cd_ldo = 0;
+  int cd_cols = 1;
+  double *cd_out = nullptr;
+  double *partial = nullptr;             // splits > 1: [batch][splits][n_tiles][64][128]
+  int *err = nullptr;
+  // set by slice_gemm_plan
+  int splits = 1, kb_per_split = 0, drain_kb = 0, n_tiles = 0, tiles_n = 0;
+};
+// Tiles and K splits for the shape; returns the bytes `partial` needs (0: none).
+size_t slice_gemm_plan(SliceGemmArgs *g, int n_sm, size_t max_partial);
+cudaError_t launch_slice_gemm(const SliceGemmArgs &g, int n_sm, cudaStream_t s);
+cudaError_t launch_slice_coldot_reduce(const SliceGemmArgs &g, double *W, int64_t ldw, cudaStream_t s);
+// C[m][n] = C[n][m] for m > n.
+cudaError_t launch_mirror_upper(double *C, int N, int64_t ldc, int64_t batch_stride, int batch, cudaStream_t s);
 
 // ---- mixed-precision helpers (mixed.cu) ----
 // dst[c][r] = (float)src[r][c0 + c] for r < rows, c < cols; zero up to cols_p x rows_p

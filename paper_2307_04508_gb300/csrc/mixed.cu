@@ -486,20 +486,32 @@ __global__ void __launch_bounds__(256)
 // once (no fused multiply-add): Delta / (w_t^2 + Delta^2) (direct, p0 = w),
 // (w_t Delta) exp(-Delta Delta x_t) (Laplace, p0 = x, p1 = w), exp(-Delta tau_t)
 // (imaginary time, p0 = tau).
+__device__ __forceinline__ double pi_factor64(int mode, double d, double a, double b) {
+  if (mode == SCALE_DIRECT) return __ddiv_rn(d, __dadd_rn(__dmul_rn(a, a), __dmul_rn(d, d)));
+  if (mode == SCALE_LAPLACE) return __dmul_rn(__dmul_rn(b, d), exp(__dmul_rn(__dmul_rn(-d, d), a)));
+  return exp(__dmul_rn(-d, a));   // SCALE_EXPTAU: e^{-Delta tau_t}
+}
+
 __global__ void pi_factor64_kernel(const double *__restrict__ delta, int64_t K, const double *__restrict__ p0,
                                    const double *__restrict__ p1, int mode, double *__restrict__ f) {
   const int t = blockIdx.y;
   const double a = p0[t], b = p1 ? p1[t] : 0.0;
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < K; k += (int64_t)gridDim.x * blockDim.x)
+    f[(int64_t)t * K + k] = pi_factor64(mode, delta[k], a, b);
+}
+
+// sgn = sign(f) sqrt|f|, mag = sqrt|f| of the same factors; *neg is set if any f < 0.
+__global__ void pi_root_factor_kernel(const double *__restrict__ delta, int64_t K, const double *__restrict__ p0,
+                                      const double *__restrict__ p1, int mode, double *__restrict__ sgn,
+                                      double *__restrict__ mag, int *__restrict__ neg) {
+  const int t = blockIdx.y;
+  const double a = p0[t], b = p1 ? p1[t] : 0.0;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < K; k += (int64_t)gridDim.x * blockDim.x) {
-    const double d = delta[k];
-    double v;
-    if (mode == SCALE_DIRECT)
-      v = __ddiv_rn(d, __dadd_rn(__dmul_rn(a, a), __dmul_rn(d, d)));
-    else if (mode == SCALE_LAPLACE)
-      v = __dmul_rn(__dmul_rn(b, d), exp(__dmul_rn(__dmul_rn(-d, d), a)));
-    else
-      v = exp(__dmul_rn(-d, a));   // SCALE_EXPTAU: e^{-Delta tau_t}
-    f[(int64_t)t * K + k] = v;
+    const double f = pi_factor64(mode, delta[k], a, b);
+    const double r = sqrt(fabs(f));
+    if (f < 0.0) *neg = 1;
+    sgn[(int64_t)t * K + k] = f < 0.0 ? -r : r;
+    mag[(int64_t)t * K + k] = r;
   }
 }
 
@@ -617,6 +629,15 @@ cudaError_t launch_pi_factor64(const double *delta, int64_t K, int n_t, const do
   int bx = (int)((K + 255) / 256);
   if (bx > 152) bx = 152;
   pi_factor64_kernel<<<dim3(bx, n_t), 256, 0, st>>>(delta, K, p0, p1, mode, f);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pi_root_factor(const double *delta, int64_t K, int n_t, const double *p0, const double *p1,
+                                  int mode, double *sgn, double *mag, int *neg, cudaStream_t st) {
+  if (n_t <= 0 || K <= 0) return cudaSuccess;
+  int bx = (int)((K + 255) / 256);
+  if (bx > 152) bx = 152;
+  pi_root_factor_kernel<<<dim3(bx, n_t), 256, 0, st>>>(delta, K, p0, p1, mode, sgn, mag, neg);
   return cudaGetLastError();
 }
 

@@ -36,6 +36,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "tc_ptx.cuh"
 
 namespace ltgw {
 namespace {
@@ -45,62 +46,6 @@ constexpr int MAXT = 4;                       // scales per CTA at most (TMEM: 4
 constexpr int CONV_WARPS = 16, EPI_WARPS = 4;
 constexpr uint32_t B_BYTES = TN * TK * 2;      // one bf16 tile, 16 KB
 constexpr uint32_t B_STAGE = 2 * B_BYTES;      // hi + lo
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ uint64_t globaltimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *b, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *b) {
-  asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(smem_u32(b))
-               : "memory");
-}
-
-// Bounded wait for the phase with the given parity; false on time-out (or, when
-// honor_abort, as soon as another role of the CTA has given up).
-__device__ __forceinline__ uint32_t mbar_try(uint64_t *b, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.b32 %0, 1, 0, p;\n}\n"
-      : "=r"(done)
-      : "r"(smem_u32(b)), "r"(parity)
-      : "memory");
-  return done;
-}
-
-// Bounded wait for the phase with the given parity; false on time-out (or, when
-// honor_abort, as soon as another role of the CTA has given up).  A phase that
-// has already completed costs one try_wait: the MMA issue thread waits once per
-// stage, and anything it executes between MMAs leaves the tensor pipe idle.
-__device__ __forceinline__ bool mbar_wait_slow(uint64_t *b, uint32_t parity, int *abort, int *err, bool honor_abort) {
-  const uint64_t t0 = globaltimer();
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try(b, parity)) return true;
-    if ((it & 1023) == 0) {
-      if (honor_abort && *(volatile int *)abort) return false;
-      if (globaltimer() - t0 > 2000000000ull) {
-        atomicExch(&err[FLAG_TC_TIMEOUT], 1);
-        *(volatile int *)abort = 1;
-        return false;
-      }
-    }
-  }
-}
-
-__device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity, int *abort, int *err,
-                                          bool honor_abort = true) {
-  if (mbar_try(b, parity)) return true;
-  return mbar_wait_slow(b, parity, abort, err, honor_abort);
-}
 
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
   uint64_t d = 0;
@@ -115,14 +60,6 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
 // kind::f16, D = FP32, A = B = BF16, both K-major, M = 128, N = 64.
 constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
                            ((uint32_t)(TM >> 4) << 24);
-
-
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
-}
-
 
 // Epilogue (EPI_WARPS warps): tcgen05.ld of the accumulators after each drain
 // window (set dr % nbuf), into FP64 / FP32 partial tiles or the column-dot reduction.
@@ -143,15 +80,7 @@ __device__ __forceinline__ void epilogue_drain(const TcGemmArgs &g, uint32_t tme
       for (int h = 0; h < TN / 32; ++h) {
         uint32_t r[32];
         const uint32_t a = tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)((buf * nt + t) * TN + h * 32);
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-            "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-              "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-              "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
-              "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-              "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-            : "r"(a));
+        tmem_ld32(r, a);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         if (g.ds_a) {   // FP8 form: per-row de-scales of both operands
           const float ra = g.ds_a[(int64_t)(grp * g.nt_group + t) * g.rows_a + ti * TM + row];
@@ -264,23 +193,12 @@ struct Bars3 {
   int abort;
 };
 
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *b, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
-}
-
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
           smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
       : "memory");
-}
-
-__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
 }
 
 // A operand in tensor memory: M = 128 rows on the 128 lanes, k pairs packed

@@ -1,0 +1,99 @@
+"""FP64 contractions on the tensor cores from base-256 digits (slice_gemm.cu),
+reached through the FP64 polarisability, against the exact sum in extended
+precision.
+
+Bound per entry (i, j) of M = sum_k A_ik B_jk with A = B = R~ diag(sqrt|f|)
+(the sign of f with A), K pairs and row scales 2^(e_i) > max_k |A_ik|: the
+digits hold each entry to 2^-56 2^(e_i) (two operands: 2 * 2^-56), the dropped
+levels i + j >= 9 are at most 6 * 2^14 * 2^-72 * 4 (1 + 2^-7) < 6.1 * 2^-56 per
+pair, so K 2^(e_i + e_j) 2^-53 in all; the roots, their products with R~ and the
+factor itself add 8 * 2^-53 of sum_k |A_ik B_jk|, and the final rounding and the
+sums over K splits and chunks another 8 * 2^-53 of it."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2307_04508_gb300 import ltgw
+    c = ltgw.Context(0)
+    yield c
+    c.close()
+
+
+def _pi(ctx, R, delta, omegas, **kw):
+    N, J = R.shape[0], len(omegas)
+    out = torch.full((J, N, N), float("nan"), dtype=torch.float64, device="cuda")
+    ctx.polarizability(torch.from_numpy(R).cuda(), torch.from_numpy(delta).cuda(), omegas, out, **kw)
+    return out.cpu().numpy()
+
+
+def _check(got, R, f, alpha):
+    """got ~ alpha R diag(f) R^T within the bound of the module docstring."""
+    g = np.sqrt(np.abs(f))
+    A = (R.astype(np.longdouble) * g[None, :])
+    ref = alpha * ((A * np.sign(f)[None, :]) @ A.T)
+    e = np.frexp(np.maximum(np.abs(A).max(axis=1).astype(np.float64), 1e-320))[1]
+    scale = np.exp2((e[:, None] + e[None, :]).astype(np.float64))
+    bound = abs(alpha) * (R.shape[1] * scale * U + 16 * U * (np.abs(A) @ np.abs(A).T).astype(np.float64))
+    err = np.abs((got - ref).astype(np.float64))
+    assert np.all(err <= bound), (err / np.maximum(bound, 1e-300)).max()
+    assert np.array_equal(got, got.T)
+
+
+# one tile and its edges (64 / 128 rows, 16 k), one warp-held row (512) and past
+# it, drains of 144 k, K splits, ragged tails
+@pytest.mark.parametrize("N,K", [(400, 128), (63, 5200), (64, 4880), (65, 4800), (128, 1296), (129, 1297), (257, 512),
+                                 (257, 513), (192, 2049), (321, 20000)])
+def test_pi_matches_exact_sum(ctx, N, K):
+    rng = np.random.default_rng(N * 7 + K)
+    R = rng.standard_normal((N, K)) * np.exp2(rng.integers(-40, 40, N))[:, None]
+    R[N // 2] = 0.0
+    delta = 0.3 + 3.0 * rng.random(K)
+    om = np.array([0.02, 1.7])
+    got = _pi(ctx, R, delta, om)
+    for j, w in enumerate(om):
+        f = delta / (w * w + delta * delta)
+        _check(got[j], R, f, -4.0)
+
+
+def test_pi_moments_negative_weights_and_gaps(ctx):
+    """Negative factors (the sign goes with one operand only), a factor that
+    singles out the smallest gaps, spin 1, and the recombination."""
+    rng = np.random.default_rng(3)
+    N, K = 150, 3001
+    R = rng.standard_normal((N, K))
+    delta = 0.3 + 3.0 * rng.random(K)
+    delta[::5] *= -1.0
+    x, w = np.array([0.5, 40.0]), np.array([-0.7, 2.0])
+    om = np.array([0.0])   # exp(-w^2 x) = 1: Pi = -2 (M^0 + M^1)
+    got = _pi(ctx, R, delta, om, x=x, w=w, spin=1)[0]
+    f = [w[k] * delta * np.exp(-delta * delta * x[k]) for k in range(2)]
+    ref = sum(-2.0 * ((R.astype(np.longdouble) * fk[None, :]) @ R.T) for fk in f)
+    size = sum(2.0 * ((np.abs(R) * np.abs(fk)[None, :]) @ np.abs(R).T) for fk in f)
+    scale = sum(2.0 * K * np.exp2(2.0 * np.frexp((np.abs(R) * np.sqrt(np.abs(fk))[None, :]).max())[1]) for fk in f)
+    # the factor's own exponent argument d^2 x carries a relative rounding of
+    # 2 u, an error of up to 2 u d^2 x <= 900 u in exp where it still matters
+    assert np.all(np.abs((got - ref).astype(np.float64)) <= U * scale + 1000 * U * size)
+
+
+def test_pi_nonfinite_rows_stay_in_their_rows(ctx):
+    rng = np.random.default_rng(5)
+    N, K = 140, 4000
+    R = rng.standard_normal((N, K))
+    R[7, 11], R[130, 3999] = np.nan, np.inf
+    delta = 0.3 + rng.random(K)
+    om = np.array([0.1])
+    got = _pi(ctx, R, delta, om)[0]
+    bad = np.zeros(N, dtype=bool)
+    bad[[7, 130]] = True
+    assert not np.isfinite(got[bad]).any() and not np.isfinite(got[:, bad]).any()
+    keep = np.ix_(~bad, ~bad)
+    f = delta / (om[0] ** 2 + delta * delta)
+    _check(got[keep], R[~bad], f, -4.0)
