@@ -997,6 +997,25 @@ ltgw_status wnm_emu(ltgw_ctx *ctx, int N, int n_omega, const double *C, int T, i
   return LTGW_OK;
 }
 
+// C_j = [1 - Pi_j]^-1 - 1 (Eq. ScreenedCoulombOrbital): the blocked sweep with
+// its updates from digits where N is past one pivot block of 128 by more than a
+// sliver (N = 130: 0.76 ms, FP64 tiles 0.56; N = 160: 0.59 against 0.85) and the
+// digits' memory is there, else on the FP64 tiles.
+constexpr int kScreenDigitsMinN = 144;
+
+ltgw_status screen_step(ltgw_ctx *ctx, int N, int n_omega, const double *Pi, double *work, double *C, cudaStream_t s) {
+  int nl = 0;
+  void *digits = nullptr;
+  const size_t bytes = screen_digit_bytes(N, n_omega);
+  const bool use = N >= kScreenDigitsMinN && N <= 65535 && n_omega <= 65535 &&
+                   slice_reserve(ctx->a5, [&](Arena &A) { digits = A.take<uint8_t>(bytes); });
+  const cudaError_t e = use ? launch_screen_digits(Pi, N, n_omega, work, digits, C, ctx->flags, ctx->n_sm, s, &nl)
+                            : launch_screen_blocked(Pi, N, n_omega, work, C, ctx->flags, s, &nl);
+  ctx->launches += nl;
+  if (e != cudaSuccess) ctx->fail(LTGW_ERR_DEVICE, std::string("screen: ") + cudaGetErrorString(e));
+  return ctx->status();
+}
+
 // Operands of the mixed form after the NAF step (Eq. naftrafo in split BF16):
 //   Bf       FP32 [roundup(N,128)][roundup(n_ov,64)]   R~_ov, the Pi operand
 //   BtT64    FP64 [T][n_orb_act][N]                      R~_tgt transposed (column dot)
@@ -1706,10 +1725,7 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
     ctx->mark(EV_PI, s);
 
     // ---- screening
-    int nl = 0;
-    cudaError_t e = launch_screen_blocked(d_Pi, N, n_omega, d_X0, d_C, ctx->flags, s, &nl);
-    ctx->launches += nl;
-    if (e != cudaSuccess) { ctx->fail(LTGW_ERR_DEVICE, std::string("screen: ") + cudaGetErrorString(e)); return ctx->status(); }
+    if (screen_step(ctx, N, n_omega, d_Pi, d_X0, d_C, s) != LTGW_OK) return ctx->status();
     ctx->mark(EV_SCREEN, s);
 
     // ---- W_nm(i w_j)
@@ -2094,9 +2110,7 @@ ltgw_status ltgw_screen(ltgw_ctx *ctx, int N, int n_omega, const double *Pi, dou
   if (ctx->a2.commit() != cudaSuccess) { ctx->fail(LTGW_ERR_NOMEM, "workspace allocation failed"); return ctx->status(); }
   layout(ctx->a2);
   LTGW_CUDA(ctx, cudaMemsetAsync(ctx->flags, 0, FLAG_COUNT * sizeof(int), s));
-  int nl = 0;
-  cudaError_t e = launch_screen_blocked(Pi, N, n_omega, X0, C, ctx->flags, s, &nl);
-  if (e != cudaSuccess) { ctx->fail(LTGW_ERR_DEVICE, std::string("screen: ") + cudaGetErrorString(e)); return ctx->status(); }
+  if (screen_step(ctx, N, n_omega, Pi, X0, C, s) != LTGW_OK) return ctx->status();
   LTGW_CUDA(ctx, cudaStreamSynchronize(s));
   return check_flags(ctx, s);
 }

@@ -79,6 +79,12 @@ size_t screen_blocked_scratch(int N, int n_omega);
 cudaError_t launch_screen_blocked(const double *Pi, int N, int n_omega, double *work, double *C, int *flags,
                                   cudaStream_t s, int *launches);
 
+// Pivot blocks of 128 with the updates from digits; work as above, digits:
+// screen_digit_bytes(N, n_omega) bytes, 256-byte aligned.
+size_t screen_digit_bytes(int N, int n_omega);
+cudaError_t launch_screen_digits(const double *Pi, int N, int n_omega, double *work, void *digits, double *C,
+                                 int *flags, int n_sm, cudaStream_t s, int *launches);
+
 // ---- eigensolver (eig.cu) ----
 struct EigWork {
   double *A = nullptr;      // [n][n] symmetric in, destroyed
@@ -202,7 +208,7 @@ size_t tc_gemm_smem_bytes();
 // of the row is set (the tensor core's 32-byte swizzle), zero past the rows
 // and past K.  Row r ~ 2^(exps[r]) sum_i digit_i 2^(-bits i).
 constexpr int SL_ROWS = 64, SL_K = 16;
-constexpr int SL_ZERO = -(1 << 20);        // exps of a zero row
+constexpr int SL_ZERO = -(1 << 18);        // exps of a zero row
 constexpr int SL_NONFINITE = 1 << 20;      // exps of a row with a NaN or an infinity (its products are NaN)
 inline int64_t slice_rows_padded(int64_t rows) { return (rows + 127) / 128 * 128; }
 inline int64_t slice_digit_bytes(int64_t rows, int64_t nkb, int ns) {

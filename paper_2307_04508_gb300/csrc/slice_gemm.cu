@@ -149,31 +149,47 @@ __device__ __forceinline__ SgUnit sg_unit(const SliceGemmArgs &g, int64_t u) {
   return w;
 }
 
-// FP64 value of hi 2^s + lo (|hi| < 2^62, |lo| < 2^62) times 2^E, rounded to
-// nearest once (ties away from zero).
-__device__ __forceinline__ double sg_value(long long hi, long long lo, int s, int E) {
-  const long long h0 = (long long)((unsigned long long)hi << s);
-  unsigned long long t0 = (unsigned long long)h0 + (unsigned long long)lo;
-  long long t1 = (s ? hi >> (64 - s) : (hi >> 63)) + (lo >> 63) + (t0 < (unsigned long long)lo ? 1 : 0);
-  const unsigned long long sgn = (unsigned long long)t1 & 0x8000000000000000ull;
-  unsigned long long u1 = (unsigned long long)t1;
-  if (sgn) {
-    t0 = ~t0 + 1ull;
-    u1 = ~u1 + (t0 == 0ull ? 1ull : 0ull);
+// (hi 2^S + lo) 2^E in FP64, negated with neg, rounded once (ties away from
+// zero).  |hi 2^S + lo| < 2^95.  About thirty integer instructions, where
+// three FP64 ones would take the time of a hundred.
+__device__ __noinline__ double sg_value_rare(uint32_t w2, uint32_t w1, uint32_t w0, int E, bool negative) {
+  if (E >= SL_NONFINITE / 2) return __longlong_as_double(0x7ff8000000000000ll);   // an operand row was not finite
+  double v = 0.0;
+  if (E > -SL_NONFINITE / 2)
+    v = ldexp((double)w2, E + 64) + ldexp((double)w1, E + 32) + ldexp((double)w0, E);
+  return negative ? -v : v;
+}
+
+template <int S>
+__device__ __forceinline__ double sg_value(long long hi, long long lo, int E, uint32_t neg) {
+  uint32_t w0, w1, w2;
+  if constexpr (S == 0) {
+    w0 = (uint32_t)lo; w1 = (uint32_t)((unsigned long long)lo >> 32); w2 = (uint32_t)(lo >> 63);
+  } else {
+    const unsigned long long h0 = (unsigned long long)hi << S;
+    const unsigned long long t0 = h0 + (unsigned long long)lo;
+    w2 = (uint32_t)(hi >> (64 - S)) + (uint32_t)(lo >> 63) + (t0 < h0 ? 1u : 0u);
+    w0 = (uint32_t)t0; w1 = (uint32_t)(t0 >> 32);
   }
-  int top = 128;                          // bits of the window whose upper word is u1
-  if (u1 == 0ull) { u1 = t0; t0 = 0ull; top = 64; }
-  if (u1 == 0ull) return 0.0;
-  const int lz = __clzll((long long)u1);
-  const unsigned long long m = lz ? (u1 << lz) | (t0 >> (64 - lz)) : u1;   // leading one at bit 63
-  const int be = top - lz - 1 + 1023 + E;  // biased exponent
-  if (be >= 1 && be <= 2045) {
-    // the leading one adds 1 to the exponent field; a rounding carry goes there too
-    const unsigned long long bits = ((unsigned long long)(be - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
-    return __longlong_as_double((long long)(bits | sgn));
+  const uint32_t sgn = (uint32_t)((int)w2 >> 31);   // all ones for a negative sum
+  const unsigned long long mag = ((unsigned long long)(w1 ^ sgn) << 32 | (w0 ^ sgn)) + (sgn & 1u);
+  const uint32_t a0 = (uint32_t)mag, a1 = (uint32_t)(mag >> 32), a2 = (w2 ^ sgn) + (sgn && mag == 0ull ? 1u : 0u);
+  const uint32_t sign = (sgn ^ neg) & 0x80000000u;
+  uint32_t m2 = a2, m1 = a1, m0 = a0;
+  int be = E + 1023 + 95;                           // biased exponent of a leading one at bit 95
+  if (m2 == 0u) { m2 = m1; m1 = m0; m0 = 0u; be -= 32; }
+  if (m2 == 0u) { m2 = m1; m1 = 0u; be -= 32; }
+  const int lz = __clz((int)m2);
+  m2 = __funnelshift_l(m1, m2, lz);
+  m1 = __funnelshift_l(m0, m1, lz);
+  be -= lz;
+  if (m2 == 0u || (unsigned)(be - 1) >= 2045u) {   // zero, not finite, or outside the normal range
+    if (m2 == 0u && E < SL_NONFINITE / 2) return 0.0;
+    return sg_value_rare(a2, a1, a0, E, sign != 0u);
   }
-  const double v = __longlong_as_double((long long)(((unsigned long long)1022 << 52) + (m >> 11) + ((m >> 10) & 1ull)));
-  return ldexp(sgn ? -v : v, top - lz - 1 + E);
+  // the leading one adds 1 to the exponent field; a rounding carry goes there too
+  const unsigned long long m = ((unsigned long long)(m2 >> 11) << 32 | __funnelshift_r(m1, m2, 11)) + ((m1 >> 10) & 1u);
+  return __longlong_as_double((long long)(m + ((unsigned long long)((uint32_t)(be - 1) << 20 | sign) << 32)));
 }
 
 // MMA issue of one part's levels (one thread).
@@ -215,7 +231,7 @@ __device__ __forceinline__ void sg_issue(const SliceGemmArgs &g, uint8_t *smem, 
   __syncwarp();
 }
 
-template <int NS>
+template <int NS, int BITS>
 __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(SliceGemmArgs g) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -288,8 +304,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(SliceGemmArgs
     const int ew = warp & 3;              // TMEM lane quarter this warp may read
     const int cq = (warp - SG_EPI0) >> 2;       // columns cq * 16 .. + 15 of every level
     const uint32_t tbase = tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)(cq * SG_CW);
-    const int bits = g.bits;
-    const int hs = NS > 4 ? 4 * bits : 0;   // weight of the upper sum
+    constexpr int HS = NS > 4 ? 4 * BITS : 0;   // weight of the upper sum
     uint32_t pf = 0;
     bool ok = true;
     for (int64_t u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
@@ -299,6 +314,13 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(SliceGemmArgs
       long long lo[SG_CW], hi[NS > 4 ? SG_CW : 1];
 #pragma unroll
       for (int q = 0; q < SG_CW; ++q) { lo[q] = 0; if (NS > 4) hi[NS > 4 ? q : 0] = 0; }
+      if (g.C && g.beta != 0.0 && !g.partial && (lane & 15) == 0) {
+        // the output's lines, read after the contraction: on their way to L2 meanwhile
+        const int m0 = w.I * SG_M + ew * 32 + lane, nn = w.J * SG_N + cq * SG_CW;
+        if (m0 < g.M)
+          for (int q = 0; q < SG_CW && nn + q < g.N; ++q)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(g.C + (int64_t)w.b * g.c_batch + (int64_t)(nn + q) * g.ldc + m0));
+      }
       for (int kb = kb0; kb < kb1 && ok; kb += g.drain_kb) {
 #pragma unroll
         for (int part = 1; part >= 0; --part) {   // the upper levels are complete first
@@ -308,7 +330,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(SliceGemmArgs
 #pragma unroll
           for (int l = part ? LO : 0; l < (part ? NS : LO); ++l) {
             const bool up = l < NS - 4;
-            const int wgt = 1 << (bits * ((up ? NS - 5 : NS - 1) - l));
+            const int wgt = 1 << (BITS * ((up ? NS - 5 : NS - 1) - l));
             uint32_t r[SG_CW];
             tmem_ld16(r, tbase + (uint32_t)(l * SG_N));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -328,20 +350,23 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(SliceGemmArgs
       // ---- the tile's values: A row m (contiguous in the output), B rows n0 ..
       const int m = w.I * SG_M + ew * 32 + lane, n0 = w.J * SG_N + cq * SG_CW;
       const int em = g.ea[(int64_t)w.b * g.ea_batch + m];
-      const int *ebp = g.eb + (int64_t)w.b * g.eb_batch + n0;
-      const int e0 = em + g.alpha_exp - bits * (NS + 1);
-      const bool bad_m = em >= SL_NONFINITE;
-      auto value = [&](int q) -> double {
-        const int en = __ldg(ebp + q);
-        if (bad_m || en >= SL_NONFINITE) return __longlong_as_double(0x7ff8000000000000ll);
-        const double v = sg_value(NS > 4 ? hi[NS > 4 ? q : 0] : 0ll, lo[q], hs, e0 + en);
-        return g.alpha_neg ? -v : v;
-      };
+      const int e0 = em + g.alpha_exp - BITS * (NS + 1);
+      const uint32_t neg = g.alpha_neg ? 0xffffffffu : 0u;
+      const int4 *ebp = reinterpret_cast<const int4 *>(g.eb + (int64_t)w.b * g.eb_batch + n0);   // n0 is a multiple of 16
+      double val[SG_CW];
+#pragma unroll
+      for (int q = 0; q < SG_CW; q += 4) {
+        const int4 en = __ldg(ebp + q / 4);
+        val[q] = sg_value<HS>(NS > 4 ? hi[NS > 4 ? q : 0] : 0ll, lo[q], e0 + en.x, neg);
+        val[q + 1] = sg_value<HS>(NS > 4 ? hi[NS > 4 ? q + 1 : 0] : 0ll, lo[q + 1], e0 + en.y, neg);
+        val[q + 2] = sg_value<HS>(NS > 4 ? hi[NS > 4 ? q + 2 : 0] : 0ll, lo[q + 2], e0 + en.z, neg);
+        val[q + 3] = sg_value<HS>(NS > 4 ? hi[NS > 4 ? q + 3 : 0] : 0ll, lo[q + 3], e0 + en.w, neg);
+      }
       if (g.partial) {
         double *o = g.partial + (((int64_t)w.b * g.splits + w.sp) * g.n_tiles + w.tile) * (SG_M * SG_N) +
                     (int64_t)(cq * SG_CW) * SG_M + ew * 32 + lane;
 #pragma unroll
-        for (int q = 0; q < SG_CW; ++q) o[(int64_t)q * SG_M] = value(q);
+        for (int q = 0; q < SG_CW; ++q) o[(int64_t)q * SG_M] = val[q];
       } else if (g.cd_out) {
         // column dot: sum over this tile's B rows n of D[m][n] cd_B[n][m]
         double acc = 0.0;
@@ -350,7 +375,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(SliceGemmArgs
           const double *cb = g.cd_B + (int64_t)t * g.cd_stride + (m - t * g.cd_cols) + (int64_t)n0 * g.cd_ld;
 #pragma unroll
           for (int q = 0; q < SG_CW; ++q)
-            if (n0 + q < g.N) acc = fma(value(q), cb[(int64_t)q * g.cd_ld], acc);
+            if (n0 + q < g.N) acc = fma(val[q], cb[(int64_t)q * g.cd_ld], acc);
           g.cd_out[((int64_t)w.b * (4 * g.tiles_n) + 4 * w.J + cq) * g.cd_ldo + m] = acc;
         }
       } else if (m < g.M) {
@@ -363,12 +388,12 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(SliceGemmArgs
             for (int q = 0; q < 8; ++q) c[q] = n0 + q0 + q < g.N ? o[(int64_t)(q0 + q) * g.ldc] : 0.0;
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-              if (n0 + q0 + q < g.N) o[(int64_t)(q0 + q) * g.ldc] = fma(g.beta, c[q], value(q0 + q));
+              if (n0 + q0 + q < g.N) o[(int64_t)(q0 + q) * g.ldc] = fma(g.beta, c[q], val[q0 + q]);
           }
         } else {
 #pragma unroll
           for (int q = 0; q < SG_CW; ++q)
-            if (n0 + q < g.N) o[(int64_t)q * g.ldc] = value(q);
+            if (n0 + q < g.N) o[(int64_t)q * g.ldc] = val[q];
         }
       }
     }
@@ -661,33 +686,47 @@ __global__ void __launch_bounds__(256) slice_rows_scaled_kernel(SliceSrc a, int 
   }
 }
 
-// Short rows (K <= 512): one warp per row holds it in registers, so the
-// exponent and the digits need one pass.
-template <int NS, int BITS>
-__global__ void __launch_bounds__(256) slice_rows_short_kernel(SliceSrc a) {
+// Short rows (K <= 128 W): W half-warps' worth of lanes (16 W) hold one row in
+// registers, so the exponent and the digits need one pass.  Aligned rows are
+// read 16 bytes at a time.
+template <int NS, int BITS, int W>
+__global__ void __launch_bounds__(256) slice_rows_short_kernel(SliceSrc a, int aligned) {
   if (a.only_if && !*a.only_if) return;
-  const int b = blockIdx.z, lane = threadIdx.x & 31;
-  const int r = blockIdx.y * 8 + (threadIdx.x >> 5);
+  constexpr int LANES = W >= 2 ? 32 : 16, H = W >= 2 ? W / 2 : 1;   // lanes per row, groups of eight k per lane
+  const int b = blockIdx.z, sub = threadIdx.x & (LANES - 1);
+  const int r = blockIdx.y * (256 / LANES) + threadIdx.x / LANES;
   uint8_t *dig = a.dig + (int64_t)b * a.dig_batch;
   const double *x = a.X + (int64_t)b * a.x_batch + (int64_t)r * a.ld;
   const double *f = a.colscale ? a.colscale + (int64_t)b * a.cs_batch : nullptr;
   const bool live = r < a.rows;
-  double v[2][8];
+  double v[H][8];
   unsigned long long mb = 0ull;
 #pragma unroll
-  for (int h = 0; h < 2; ++h)
+  for (int h = 0; h < H; ++h) {
+    const int64_t k0 = (int64_t)(sub + LANES * h) * 8;
+    if (aligned && live && k0 + 8 <= a.K && !f) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int64_t k = (int64_t)(lane + 32 * h) * 8 + q;
-      v[h][q] = (live && k < a.K) ? (f ? __dmul_rn(x[k], f[k]) : x[k]) : 0.0;
-      mb = max(mb, mag_bits(v[h][q]));
+      for (int q = 0; q < 8; q += 2) {
+        const double2 t = *reinterpret_cast<const double2 *>(x + k0 + q);
+        v[h][q] = t.x;
+        v[h][q + 1] = t.y;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        v[h][q] = (live && k0 + q < a.K) ? (f ? __dmul_rn(x[k0 + q], f[k0 + q]) : x[k0 + q]) : 0.0;
     }
-  mb = warp_max(mb);
-  const int e = slice_exponent(mb, BITS);
-  if (lane == 0) a.exps[(int64_t)b * a.exp_batch + r] = e;
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int g = lane + 32 * h;
+    for (int q = 0; q < 8; ++q) mb = max(mb, mag_bits(v[h][q]));
+  }
+#pragma unroll
+  for (int o = LANES / 2; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+  const int e = slice_exponent(mb, BITS);
+  if (r >= a.rows_p) return;
+  if (sub == 0) a.exps[(int64_t)b * a.exp_batch + r] = e;
+#pragma unroll
+  for (int h = 0; h < H; ++h) {
+    const int g = sub + LANES * h;
     if (g < 2 * a.nkb) store_digits<NS, BITS>(v[h], e, digit_chunk<NS>(dig, r, g, a.nkb));
   }
 }
@@ -748,8 +787,14 @@ __global__ void fill_int_kernel(int *p, int64_t n, int v) {
 
 template <int NS, int BITS>
 cudaError_t slice_operand(const SliceSrc &a, int batch, cudaStream_t s) {
-  if (!a.cols && a.K <= 512) {
-    slice_rows_short_kernel<NS, BITS><<<dim3(1, a.rows_p / 8, batch), 256, 0, s>>>(a);
+  if (!a.cols && a.nkb <= 32) {
+    const int al = a.ld % 2 == 0 && a.x_batch % 2 == 0 && ((uintptr_t)a.X & 15) == 0;
+    if (a.nkb <= 8)
+      slice_rows_short_kernel<NS, BITS, 1><<<dim3(1, a.rows_p / 16, batch), 256, 0, s>>>(a, al);
+    else if (a.nkb <= 16)
+      slice_rows_short_kernel<NS, BITS, 2><<<dim3(1, a.rows_p / 8, batch), 256, 0, s>>>(a, al);
+    else
+      slice_rows_short_kernel<NS, BITS, 4><<<dim3(1, a.rows_p / 8, batch), 256, 0, s>>>(a, al);
     return cudaGetLastError();
   }
   const int64_t n_exp = (int64_t)batch * a.exp_batch;
@@ -779,16 +824,16 @@ cudaError_t slice_operand(const SliceSrc &a, int batch, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <int NS>
+template <int NS, int BITS>
 cudaError_t launch_ns(const SliceGemmArgs &g, int blocks, cudaStream_t s) {
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
   std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(slice_gemm_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    attr_err = cudaFuncSetAttribute(slice_gemm_kernel<NS, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)sg_smem(NS));
   });
   if (attr_err != cudaSuccess) return attr_err;
-  slice_gemm_kernel<NS><<<blocks, SG_THREADS, sg_smem(NS), s>>>(g);
+  slice_gemm_kernel<NS, BITS><<<blocks, SG_THREADS, sg_smem(NS), s>>>(g);
   return cudaGetLastError();
 }
 
@@ -849,14 +894,15 @@ cudaError_t launch_slice_gemm(const SliceGemmArgs &g, int n_sm, cudaStream_t s) 
     return cudaErrorInvalidValue;
   const int blocks = (int)std::min<int64_t>(units, n_sm);
   cudaError_t e = cudaErrorInvalidValue;
-  switch (g.ns) {
-    case 2: e = launch_ns<2>(g, blocks, s); break;
-    case 3: e = launch_ns<3>(g, blocks, s); break;
-    case 4: e = launch_ns<4>(g, blocks, s); break;
-    case 5: e = launch_ns<5>(g, blocks, s); break;
-    case 6: e = launch_ns<6>(g, blocks, s); break;
-    case 7: e = launch_ns<7>(g, blocks, s); break;
-    case 8: e = launch_ns<8>(g, blocks, s); break;
+  switch (g.bits == 8 ? (g.ns == 7 ? 78 : 0) : (g.bits == 7 ? g.ns : 0)) {
+    case 2: e = launch_ns<2, 7>(g, blocks, s); break;
+    case 3: e = launch_ns<3, 7>(g, blocks, s); break;
+    case 4: e = launch_ns<4, 7>(g, blocks, s); break;
+    case 5: e = launch_ns<5, 7>(g, blocks, s); break;
+    case 6: e = launch_ns<6, 7>(g, blocks, s); break;
+    case 7: e = launch_ns<7, 7>(g, blocks, s); break;
+    case 8: e = launch_ns<8, 7>(g, blocks, s); break;
+    case 78: e = launch_ns<7, 8>(g, blocks, s); break;
   }
   if (e != cudaSuccess) return e;
   if (g.partial) {

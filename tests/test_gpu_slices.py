@@ -36,14 +36,18 @@ def _pi(ctx, R, delta, omegas, **kw):
 
 def _check(got, R, f, alpha):
     """got ~ alpha R diag(f) R^T within the bound of the module docstring."""
+    N = R.shape[0]
+    pick = np.unique(np.array([0, 1, 31, 63, 64, 65, 127, 128, N // 2, N - 2, N - 1]).clip(0, N - 1))
     g = np.sqrt(np.abs(f))
-    A = (R.astype(np.longdouble) * g[None, :])
-    ref = alpha * ((A * np.sign(f)[None, :]) @ A.T)
-    e = np.frexp(np.maximum(np.abs(A).max(axis=1).astype(np.float64), 1e-320))[1]
-    scale = np.exp2((e[:, None] + e[None, :]).astype(np.float64))
-    bound = abs(alpha) * (R.shape[1] * scale * U + 16 * U * (np.abs(A) @ np.abs(A).T).astype(np.float64))
-    err = np.abs((got - ref).astype(np.float64))
-    assert np.all(err <= bound), (err / np.maximum(bound, 1e-300)).max()
+    A = R * g[None, :]   # sizes only; the reference sums R_i f R_j in extended precision
+    Rl, fl = R.astype(np.longdouble), f.astype(np.longdouble)
+    e = np.frexp(np.maximum(np.abs(A).max(axis=1), 1e-320))[1]
+    size = np.abs(A) @ np.abs(A).T
+    for i in pick:   # whole rows, chosen at the edges of the tiles
+        ref = alpha * (Rl * (Rl[i] * fl)[None, :]).sum(axis=1)
+        bound = abs(alpha) * (R.shape[1] * np.exp2((e + e[i]).astype(np.float64)) * U + 16 * U * size[i])
+        err = np.abs((got[i] - ref).astype(np.float64))
+        assert np.all(err <= bound), (i, (err / np.maximum(bound, 1e-300)).max())
     assert np.array_equal(got, got.T)
 
 
@@ -75,7 +79,8 @@ def test_pi_moments_negative_weights_and_gaps(ctx):
     om = np.array([0.0])   # exp(-w^2 x) = 1: Pi = -2 (M^0 + M^1)
     got = _pi(ctx, R, delta, om, x=x, w=w, spin=1)[0]
     f = [w[k] * delta * np.exp(-delta * delta * x[k]) for k in range(2)]
-    ref = sum(-2.0 * ((R.astype(np.longdouble) * fk[None, :]) @ R.T) for fk in f)
+    Rl = R.astype(np.longdouble)
+    ref = sum(-2.0 * np.stack([(Rl * (Rl[i] * fk)[None, :]).sum(axis=1) for i in range(N)]) for fk in f)
     size = sum(2.0 * ((np.abs(R) * np.abs(fk)[None, :]) @ np.abs(R).T) for fk in f)
     scale = sum(2.0 * K * np.exp2(2.0 * np.frexp((np.abs(R) * np.sqrt(np.abs(fk))[None, :]).max())[1]) for fk in f)
     # the factor's own exponent argument d^2 x carries a relative rounding of
@@ -97,3 +102,32 @@ def test_pi_nonfinite_rows_stay_in_their_rows(ctx):
     keep = np.ix_(~bad, ~bad)
     f = delta / (om[0] ** 2 + delta * delta)
     _check(got[keep], R[~bad], f, -4.0)
+
+
+# one block and a remainder of 16, both sides of a block's edge, a ragged last
+# block shorter than a 16-k step; one and several frequencies
+@pytest.mark.parametrize("N,J", [(144, 3), (255, 1), (256, 2), (257, 2), (393, 2)])
+def test_screen_digits_matches_inverse(ctx, N, J):
+    """C = (1 - Pi)^-1 - 1 by the digit sweep: (1 - Pi)(C + 1) = 1 to a backward
+    error of N steps' roundings, 8 N u of |1 - Pi||C + 1| (a sweep of an SPD
+    matrix with eigenvalues >= 1 is stable; the digits' error per update is
+    below N u of the rows' scales), symmetric bit for bit, and a matrix that is
+    not positive definite is reported."""
+    from paper_2307_04508_gb300 import ltgw
+    rng = np.random.default_rng(N)
+    R = rng.standard_normal((J, N, 2 * N)) * (0.6 / np.sqrt(N)) * np.exp(-2.0 * np.arange(N) / N)[None, :, None]
+    Pi = -4.0 * R @ R.transpose(0, 2, 1)
+    Pi = 0.5 * (Pi + Pi.transpose(0, 2, 1))
+    C = torch.empty((J, N, N), dtype=torch.float64, device="cuda")
+    ctx.screen(torch.from_numpy(Pi).cuda(), C)
+    got = C.cpu().numpy()
+    eye = np.eye(N)
+    for j in range(J):
+        assert np.array_equal(got[j], got[j].T)
+        A, X = eye - Pi[j], got[j] + eye
+        res = np.abs(A @ X - eye)
+        assert res.max() <= 8 * N * U * np.linalg.norm(A, 2) * np.linalg.norm(X, 2)
+    Pi[J - 1, N - 1, N - 1] = 50.0   # the last pivot turns negative
+    with pytest.raises(ltgw.LtgwError) as e:
+        ctx.screen(torch.from_numpy(Pi).cuda(), C)
+    assert e.value.status == ltgw.LTGW_ERR_NOT_SPD
