@@ -174,19 +174,20 @@ ltgw_status check_flags(ltgw_ctx *ctx, cudaStream_t s) {
 ltgw_status naf_metric_tc(ltgw_ctx *ctx, int n, int64_t n_pairs, const double *B, int64_t ld, double *K,
                           cudaStream_t s, double beta = 0.0);
 
-// FP64-accurate C = A B^T from integer slices (defined below).
-ltgw_status emu_gemm(ltgw_ctx *ctx, int m, int n, int64_t K, const double *A, int64_t lda, const double *B,
-                     int64_t ldb, double *C, int64_t ldc, bool sym, int s, cudaStream_t st);
-
 // ---- FP64 contractions on the tensor cores from integer digits (slice_gemm.cu)
 // The FP64 form's products: 7 digits in base 256 hold 55 bits relative to each
 // operand row's largest magnitude, and the products kept (levels i + j <= 8)
 // leave an error of about 2^-52 of the rows' scales per entry, no more than a
 // length-K FP64 sum's own rounding.
+// The emulated FP64 forms: n_slices digits in base 128, one exponent per whole
+// operand row, and no CUDA-core kernel to fall back to.
 struct SliceForm {
   int ns, bits;
+  bool required;   // LTGW_ERR_NOMEM when the digits do not fit
 };
-constexpr SliceForm kFp64Digits{7, 8};
+constexpr SliceForm kFp64Digits{7, 8, false};
+constexpr int kEmuSlices = 6;   // slices per operand row in the LTGW_FP64_EMU solve
+constexpr SliceForm emu_digits(int n_slices) { return {n_slices, 7, true}; }
 constexpr size_t kSliceOperandMax = (size_t)4 << 30;   // digits of one operand held at a time
 constexpr size_t kSlicePartialMax = (size_t)1 << 30;   // K-split partial tiles
 
@@ -218,20 +219,23 @@ struct SliceOperand {
   }
 };
 
-// Reserve `layout` in `ar`; false (and no error recorded) when the memory is
-// not there, or when growing would take more than half of what is free on the
-// device (other contexts' solves size their own workspace from it): the caller
-// then takes the CUDA-core kernels, or one K split.
+// Reserve `layout` in `ar`; false when the memory is not there.  Where the form
+// has CUDA-core kernels to fall back to, also when growing would take more
+// than half of what is free on the device (other contexts' solves size their
+// own workspace from it); no error is recorded then.
 template <class Layout>
-bool slice_reserve(Arena &ar, Layout &&layout) {
+bool slice_reserve(ltgw_ctx *ctx, Arena &ar, bool required, Layout &&layout) {
   ar.begin_sizing();
   layout(ar);
-  if (ar.need > ar.cap) {
+  if (!required && ar.need > ar.cap) {
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
     else if (ar.need > (free_b + ar.cap) / 2) { ar.sizing = false; return false; }
   }
-  if (ar.commit() != cudaSuccess) return false;
+  if (ar.commit() != cudaSuccess) {
+    if (required) ctx->fail(LTGW_ERR_NOMEM, "slice operand allocation failed");
+    return false;
+  }
   layout(ar);
   return true;
 }
@@ -240,15 +244,17 @@ bool slice_reserve(Arena &ar, Layout &&layout) {
 ltgw_status slice_run(ltgw_ctx *ctx, SliceGemmArgs &g, SliceForm f, cudaStream_t s) {
   g.ns = f.ns; g.bits = f.bits; g.err = ctx->flags;
   size_t part = slice_gemm_plan(&g, ctx->n_sm, kSlicePartialMax);
-  if (part && !slice_reserve(ctx->a4, [&](Arena &A) { g.partial = A.take<double>(part / sizeof(double)); })) {
+  if (part && !slice_reserve(ctx, ctx->a4, false, [&](Arena &A) { g.partial = A.take<double>(part / sizeof(double)); })) {
     g.splits = 1; g.kb_per_split = g.nkb; g.partial = nullptr;   // no room for partials: one split
   }
   CHECK_LAUNCH(ctx, launch_slice_gemm(g, ctx->n_sm, s), g.partial || (g.sym && g.mirror) ? 2 : 1);
   return LTGW_OK;
 }
 
-// Chunk of the contraction length so that `rows` operand rows stay within kSliceOperandMax.
+// Chunk of the contraction length so that `rows` operand rows stay within
+// kSliceOperandMax (the emulated forms' exponents belong to whole rows: one chunk).
 int64_t slice_k_chunk(int64_t rows, int64_t K, int batch, SliceForm f) {
+  if (f.required) return K;
   const int64_t per_k = slice_rows_padded(rows) * 2 * f.ns * batch;
   const int64_t most = std::max<int64_t>(2048, (int64_t)kSliceOperandMax / per_k);
   const int64_t n = (K + most - 1) / most;
@@ -261,8 +267,8 @@ ltgw_status slice_syrk(ltgw_ctx *ctx, int n, int64_t K, const double *X, int64_t
                        SliceForm f, cudaStream_t s, bool *done) {
   SliceOperand o;
   const int64_t chunk = slice_k_chunk(n, K, 1, f);
-  *done = slice_reserve(ctx->a5, [&](Arena &A) { o.layout(A, n, chunk, 1, f); });
-  if (!*done) return LTGW_OK;
+  *done = slice_reserve(ctx, ctx->a5, f.required, [&](Arena &A) { o.layout(A, n, chunk, 1, f); });
+  if (!*done) return ctx->status();
   for (int64_t k0 = 0; k0 < K; k0 += chunk) {
     const int64_t kc = std::min(chunk, K - k0);
     CHECK_LAUNCH(ctx, launch_slice_operand(o.source(X + k0, ld, 0, n, kc, false), f.ns, f.bits, 1, s), 3);
@@ -283,11 +289,11 @@ ltgw_status slice_project(ltgw_ctx *ctx, int N, int n_aux, const double *Ut, con
   const int64_t most = std::max<int64_t>(4096, (int64_t)kSliceOperandMax / per_col / 128 * 128);
   const int64_t n_chunks = (cols + most - 1) / most;
   const int64_t chunk = std::min(cols, ((cols + n_chunks - 1) / n_chunks + 127) / 128 * 128);
-  *done = slice_reserve(ctx->a5, [&](Arena &A) {
+  *done = slice_reserve(ctx, ctx->a5, f.required, [&](Arena &A) {
     u.layout(A, N, n_aux, 1, f);
     x.layout(A, chunk, n_aux, batch, f);
   });
-  if (!*done) return LTGW_OK;
+  if (!*done) return ctx->status();
   CHECK_LAUNCH(ctx, launch_slice_operand(u.source(Ut, n_aux, 0, N, n_aux, false), f.ns, f.bits, 1, s), 3);
   for (int64_t c0 = 0; c0 < cols; c0 += chunk) {
     const int cc = (int)std::min(chunk, cols - c0);
@@ -312,12 +318,12 @@ ltgw_status slice_wnm(ltgw_ctx *ctx, int N, int n_omega, const double *C, int T,
   const int blk = (int)std::min<int64_t>(
       n_omega, std::max<int64_t>(1, (int64_t)kSliceOperandMax / slice_digit_bytes(N, nkb, f.ns)));
   const int tiles_n = (N + 63) / 64;
-  *done = slice_reserve(ctx->a5, [&](Arena &A) {
+  *done = slice_reserve(ctx, ctx->a5, f.required, [&](Arena &A) {
     r.layout(A, cols, N, 1, f);
     c.layout(A, N, N, blk, f);
     cd = A.take<double>((size_t)blk * 4 * tiles_n * cols);
   });
-  if (!*done) return LTGW_OK;
+  if (!*done) return ctx->status();
   SliceSrc rs = r.source(Btt, ld_btt, 0, cols, N, true);
   rs.col_group = n_orb_act; rs.col_stride = stride_btt;
   CHECK_LAUNCH(ctx, launch_slice_operand(rs, f.ns, f.bits, 1, s), 3);
@@ -351,13 +357,13 @@ ltgw_status slice_pi(ltgw_ctx *ctx, int N, int64_t n_pairs, const double *Bt, in
   // the pair range first (each chunk is another pass over M), then the points at a time
   const int64_t chunk = slice_k_chunk(2 * N, n_pairs, 1, f);
   const int blk = (int)std::min<int64_t>(n_t, std::max<int64_t>(1, (int64_t)kSliceOperandMax / (per_t * chunk)));
-  *done = slice_reserve(ctx->a5, [&](Arena &A) {
+  *done = slice_reserve(ctx, ctx->a5, f.required, [&](Arena &A) {
     o.layout(A, N, chunk, blk, f);
     o2.layout(A, N, chunk, blk, f);
     fac = A.take<double>((size_t)n_t * 2 * chunk);
     neg = A.take<int>(1);
   });
-  if (!*done) return LTGW_OK;
+  if (!*done) return ctx->status();
   for (int64_t k0 = 0; k0 < n_pairs; k0 += chunk) {
     const int64_t kc = std::min(chunk, n_pairs - k0);
     LTGW_CUDA(ctx, cudaMemsetAsync(neg, 0, sizeof(int), s));
@@ -379,6 +385,76 @@ ltgw_status slice_pi(ltgw_ctx *ctx, int N, int64_t n_pairs, const double *Bt, in
       if (slice_run(ctx, g, f, s) != LTGW_OK) return ctx->status();
     }
   }
+  return LTGW_OK;
+}
+
+// C [m][ldc] = A B^T from slices (sym: C = A A^T, whole).
+ltgw_status emu_gemm(ltgw_ctx *ctx, int m, int n, int64_t K, const double *A, int64_t lda, const double *B,
+                     int64_t ldb, double *C, int64_t ldc, bool sym, SliceForm f, cudaStream_t s) {
+  bool done = false;
+  if (sym) return slice_syrk(ctx, m, K, A, lda, C, 0.0, f, s, &done);
+  SliceOperand a, b;
+  if (!slice_reserve(ctx, ctx->a5, f.required, [&](Arena &Ar) {
+        a.layout(Ar, m, K, 1, f);
+        b.layout(Ar, n, K, 1, f);
+      }))
+    return ctx->status();
+  CHECK_LAUNCH(ctx, launch_slice_operand(a.source(A, lda, 0, m, K, false), f.ns, f.bits, 1, s), 3);
+  CHECK_LAUNCH(ctx, launch_slice_operand(b.source(B, ldb, 0, n, K, false), f.ns, f.bits, 1, s), 3);
+  SliceGemmArgs g;   // the contiguous dimension of C is B's rows
+  g.A = b.dig; g.ea = b.exps; g.B = a.dig; g.eb = a.exps; g.nkb = a.nkb;
+  g.M = n; g.N = m; g.C = C; g.ldc = ldc;
+  return slice_run(ctx, g, f, s);
+}
+
+// Pi from slices (the emulated FP64 form): per frequency (n_tau == 0, Pi_j =
+// -2 s M_j written directly) or moment t (lt_form 1: Laplace factors; 2:
+// e^{-Delta tau_t}) M_t = (Bt diag(f_t)) Bt^T, the lower triangle (rows scaled)
+// mirrored, then the recombination with d_E [n_omega][n_tau].  Pairs in equal
+// chunks of at most 131072, each with its own row exponents, their products added.
+ltgw_status polarizability_emu(ltgw_ctx *ctx, int N, int64_t n_pairs, const double *Bt, int64_t ldb,
+                               const double *delta, int n_omega, const double *d_om, int n_tau, const double *d_x,
+                               const double *d_w, const double *d_E, double *d_M, int spin, double *Pi,
+                               cudaStream_t s, int lt_form, SliceForm f) {
+  const int n_t = n_tau ? n_tau : n_omega;
+  const int64_t max_chunk = (int64_t)1 << 17;
+  const int64_t n_chunks = (n_pairs + max_chunk - 1) / max_chunk;
+  const int64_t chunk = std::min(n_pairs, ((n_pairs + n_chunks - 1) / n_chunks + 63) / 64 * 64);   // balanced
+  const int64_t per_t = slice_digit_bytes(N, (chunk + SL_K - 1) / SL_K, f.ns);
+  const int blk = (int)std::min<int64_t>(n_t, std::max<int64_t>(1, (int64_t)kSliceOperandMax / per_t));
+  SliceOperand a, b;
+  double *fac = nullptr;
+  if (!slice_reserve(ctx, ctx->a5, true, [&](Arena &A) {
+        a.layout(A, N, chunk, blk, f);
+        b.layout(A, N, chunk, 1, f);
+        fac = A.take<double>((size_t)n_t * chunk);
+      }))
+    return ctx->status();
+  ctx->mark(EV_PI0, s);
+  const int mode = n_tau ? (lt_form == 2 ? SCALE_EXPTAU : SCALE_LAPLACE) : SCALE_DIRECT;
+  double *out = n_tau ? d_M : Pi;
+  for (int64_t k0 = 0; k0 < n_pairs; k0 += chunk) {
+    const int64_t kc = std::min(chunk, n_pairs - k0);
+    CHECK_LAUNCH(ctx, launch_pi_factor64(delta + k0, kc, n_t, n_tau ? d_x : d_om,
+                                         mode == SCALE_LAPLACE ? d_w : nullptr, mode, fac, s), 1);
+    CHECK_LAUNCH(ctx, launch_slice_operand(b.source(Bt + k0, ldb, 0, N, kc, false), f.ns, f.bits, 1, s), 3);
+    for (int t0 = 0; t0 < n_t; t0 += blk) {
+      const int nb = std::min(blk, n_t - t0);
+      SliceSrc sa = a.source(Bt + k0, ldb, 0, N, kc, false);
+      sa.colscale = fac + (int64_t)t0 * kc; sa.cs_batch = kc;
+      CHECK_LAUNCH(ctx, launch_slice_operand(sa, f.ns, f.bits, nb, s), 3);
+      SliceGemmArgs g;
+      g.A = a.dig; g.a_batch = a.dig_batch; g.ea = a.exps; g.ea_batch = a.rows_p;
+      g.B = b.dig; g.eb = b.exps; g.nkb = a.nkb; g.batch = nb;
+      g.M = g.N = N; g.sym = 1; g.C = out + (int64_t)t0 * N * N; g.ldc = N; g.c_batch = (int64_t)N * N;
+      g.beta = k0 ? 1.0 : 0.0; g.alpha_exp = n_tau ? 0 : spin; g.alpha_neg = n_tau ? 0 : 1;   // -2 s: -2 or -4
+      if (slice_run(ctx, g, f, s) != LTGW_OK) return ctx->status();
+    }
+  }
+  ctx->mark(EV_PI1, s);
+  if (n_tau)
+    CHECK_LAUNCH(ctx, launch_recombine(d_M, n_tau, d_E, n_omega, (int64_t)N * N, -2.0 * spin, Pi, s),
+                 (n_omega + 63) / 64);
   return LTGW_OK;
 }
 
@@ -428,7 +504,7 @@ ltgw_status naf_basis_dev(ltgw_ctx *ctx, Arena &ar, int n, int64_t n_pairs, cons
   } else if (mixed) {
     if (naf_metric_tc(ctx, n, n_pairs, B, ld, w.A, s) != LTGW_OK) return ctx->status();
   } else if (emu_slices) {
-    if (emu_gemm(ctx, n, n, n_pairs, B, ld, B, ld, w.A, n, true, emu_slices, s) != LTGW_OK) return ctx->status();
+    if (emu_gemm(ctx, n, n, n_pairs, B, ld, B, ld, w.A, n, true, emu_digits(emu_slices), s) != LTGW_OK) return ctx->status();
   } else {
     bool done = false;
     if (slices_pay(n, n, n_pairs, 1) && slice_syrk(ctx, n, n_pairs, B, ld, w.A, 0.0, kFp64Digits, s, &done) != LTGW_OK)
@@ -596,7 +672,7 @@ ltgw_status tc_run(ltgw_ctx *ctx, Arena &ar, TcGemmArgs g, const std::vector<int
                    TcRun *run, cudaStream_t s) {
   const int n_tiles = (int)(tiles.size() / 2);
   if (g.out_mode == TC_OUT_COLDOT) g.drain_k = std::max<int64_t>(g.drain_k, (g.k_end ? g.k_end : g.Kp) - g.k_begin);
-  const int kind = g.A8 ? 2 : (g.B_hi ? (g.single ? 3 : 1) : 0);
+  const int kind = g.A8 ? 2 : (g.B_hi ? 1 : 0);
   TcPlan plan = tc_plan(ctx, g, n_tiles, g.nt_group, 0);
   std::vector<TcPlan> cands{plan};
   const ltgw_ctx::TcKey key{kind, n_tiles, g.n_t, g.out_mode, (g.k_end ? g.k_end : g.Kp) - g.k_begin, g.rows_a,
@@ -806,197 +882,6 @@ ltgw_status naf_metric_tc(ltgw_ctx *ctx, int n, int64_t n_pairs, const double *B
   return LTGW_OK;
 }
 
-// FP64-accurate products from integer slices on the tensor cores.  Each
-// operand row is cut into s balanced base-128 digits of its fixed-point form
-// (launch_slice_rows); the product sums 2^(-7(i+j)) a_i b_j^T over the digit
-// pairs with i + j <= s + 1, every pair on the split-BF16 kernel in its
-// one-product mode (A digits in FP32 convert to hi = digit exactly; B digits
-// are the hi operand), so its integer products are exact and its FP32 sums too (|sum| <=
-// 2^24: drains of 1024 pairs for the leading digits, |a_1 b_1| <= 2^14, and
-// 2048 for the others, |a_i b_j| <= 2^13); the pair results
-// are added in FP64 in the reduction, then scaled by 2^(e_A + e_B).
-constexpr int kEmuSlices = 6;   // slices per operand row in the LTGW_FP64_EMU solve
-
-struct EmuPlan {
-  int m = 0, n = 0, s = 0, nIa = 0, nIb = 0, Mpa = 0, Mpb = 0;
-  int64_t K = 0, Kp = 0, stra = 0, strb = 0;
-  bool lower = false;   // lower tiles of a square product, mirrored
-  std::vector<int> tiles, tindex;
-  float *dA = nullptr, *ones = nullptr;
-  __nv_bfloat16 *dB = nullptr;
-  int *ea = nullptr, *eb = nullptr, *d_tindex = nullptr;
-  double *factors = nullptr;   // n_factors x K FP64 column factors of A (optional)
-  double *tmp = nullptr;       // m x n FP64 (optional): the unscaled sum when C accumulates
-};
-
-ltgw_status emu_prepare(ltgw_ctx *ctx, int m, int n, int64_t K, int s, bool lower, int n_factors, EmuPlan *p,
-                        cudaStream_t st, bool need_tmp = false) {
-  p->m = m; p->n = n; p->s = s; p->K = K; p->lower = lower;
-  p->Kp = (K + 63) / 64 * 64;
-  p->nIa = (m + 127) / 128; p->nIb = (n + 127) / 128;
-  p->Mpa = p->nIa * 128; p->Mpb = p->nIb * 128;
-  p->stra = (int64_t)p->Mpa * p->Kp; p->strb = (int64_t)p->Mpb * p->Kp;
-  p->tiles = lower ? lower_tiles(p->nIa, &p->tindex) : full_tiles(p->nIa, p->nIb);
-  auto layout = [&](Arena &Ar) {
-    p->dA = Ar.take<float>((size_t)s * p->stra);
-    p->dB = Ar.take<__nv_bfloat16>((size_t)s * p->strb);
-    p->ones = Ar.take<float>((size_t)p->Kp);
-    p->ea = Ar.take<int>(p->Mpa);
-    p->eb = Ar.take<int>(p->Mpb);
-    p->d_tindex = lower ? Ar.take<int>(p->tindex.size()) : nullptr;
-    p->factors = n_factors ? Ar.take<double>((size_t)n_factors * K) : nullptr;
-    p->tmp = need_tmp ? Ar.take<double>((size_t)m * n) : nullptr;
-  };
-  ctx->a5.begin_sizing();
-  layout(ctx->a5);
-  if (ctx->a5.commit() != cudaSuccess) { ctx->fail(LTGW_ERR_NOMEM, "slice operand allocation failed"); return ctx->status(); }
-  layout(ctx->a5);
-  if (lower) copy_in(ctx, p->d_tindex, p->tindex.data(), p->tindex.size() * sizeof(int), st);
-  // padding rows (and, for column slicing, padding k) stay zero: the slicing
-  // writes rows < m (n) only; row slicing writes every k < Kp, column slicing k < K
-  LTGW_CUDA(ctx, cudaMemsetAsync(p->dA, 0, (size_t)s * p->stra * sizeof(float), st));
-  LTGW_CUDA(ctx, cudaMemsetAsync(p->dB, 0, (size_t)s * p->strb * sizeof(__nv_bfloat16), st));
-  LTGW_CUDA(ctx, cudaMemsetAsync(p->ea, 0, p->Mpa * sizeof(int), st));
-  LTGW_CUDA(ctx, cudaMemsetAsync(p->eb, 0, p->Mpb * sizeof(int), st));
-  CHECK_LAUNCH(ctx, launch_scale_table(nullptr, p->Kp, p->Kp, 1, nullptr, nullptr, SCALE_NONE, p->ones, st), 1);
-  return ctx->status();
-}
-
-// C = beta C + post * (sliced A) (sliced B)^T from the digits in p->dA / p->dB
-// and the exponents p->ea / p->eb.  C [m][ldc]; in the lower form C (ldc = n)
-// is written whole and symmetric.  post must be plus or minus a power of two:
-// it is folded into the exact 2^(-7L) factors.  beta != 0 needs p->tmp.
-ltgw_status emu_pairs(ltgw_ctx *ctx, EmuPlan &p, double post, double *C, int64_t ldc, double beta,
-                      cudaStream_t st) {
-  if (beta != 0.0 && !p.tmp) { ctx->fail(LTGW_ERR_BAD_ARG, "emulated accumulation without scratch"); return ctx->status(); }
-  double *D = beta != 0.0 ? p.tmp : C;
-  const int64_t ldd = beta != 0.0 ? p.n : (p.lower ? p.m : ldc);
-  bool first = true;
-  for (int L = 2; L <= p.s + 1; ++L) {
-    for (int i = 1; i < L; ++i) {
-      const int j = L - i;
-      if (i > p.s || j > p.s) continue;
-      TcGemmArgs g;
-      g.A = p.dA + (int64_t)(i - 1) * p.stra; g.B = nullptr; g.scale = p.ones; g.Kp = p.Kp; g.n_t = 1;
-      g.nt_group = 1;
-      g.B_hi = p.dB + (int64_t)(j - 1) * p.strb; g.B_lo = nullptr; g.rows_a = p.Mpa; g.rows_b = p.Mpb;
-      g.single = 1;   // digits are exact in BF16: one product per step
-      // FP32 sums of integers stay exact below 2^24: |a_1 b_1| <= 2^14 (1024
-      // pairs per drain), every other pair has a digit of at most 64 in
-      // magnitude, |a_i b_j| <= 2^13 (2048 pairs)
-      g.drain_k = (i == 1 && j == 1) ? 1024 : 2048;
-      g.out_colmajor = p.lower ? 1 : 0;
-      TcRun run;
-      if (tc_run(ctx, ctx->a4, g, p.tiles, 0, &run, st) != LTGW_OK) return ctx->status();
-      const double alpha = post * ldexp(1.0, -7 * L);
-      if (p.lower) {
-        CHECK_LAUNCH(ctx, launch_tc_reduce_sym(run.partial, run.partial32, run.splits, run.groups, run.n_tiles,
-                                               p.d_tindex, p.nIa, 1, p.m, alpha, D, st, first ? 0.0 : 1.0,
-                                               run.nt_group, 1),
-                     1);
-      } else {
-        CHECK_LAUNCH(ctx, launch_tc_reduce_full_acc(run.partial, run.partial32, run.splits, run.groups, run.n_tiles,
-                                                    p.nIb, p.m, p.n, alpha, D, ldd, first ? 0.0 : 1.0, st), 1);
-      }
-      first = false;
-    }
-  }
-  CHECK_LAUNCH(ctx, launch_scale_exp2_to(D, ldd, C, p.lower ? p.m : ldc, p.m, p.n, p.ea, p.eb, beta, st,
-                                         p.lower ? 1 : 0), 1);
-  return ctx->status();
-}
-
-// A (with optional column factors) sliced into p->dA, then emu_pairs.
-ltgw_status emu_product(ltgw_ctx *ctx, EmuPlan &p, const double *A, int64_t lda, const double *colscale,
-                        double post, double *C, int64_t ldc, cudaStream_t st, double beta = 0.0) {
-  CHECK_LAUNCH(ctx, launch_slice_rows(A, lda, p.m, p.K, p.Kp, p.s, p.stra, p.dA, nullptr, p.ea, st, colscale), 1);
-  return emu_pairs(ctx, p, post, C, ldc, beta, st);
-}
-
-// C = beta C + A A^T (lower form): A sliced once into both operands.
-ltgw_status emu_syrk(ltgw_ctx *ctx, EmuPlan &p, const double *A, int64_t lda, double *C, double beta,
-                     cudaStream_t st) {
-  CHECK_LAUNCH(ctx, launch_slice_rows(A, lda, p.m, p.K, p.Kp, p.s, p.stra, p.dA, p.dB, p.ea, st), 1);
-  LTGW_CUDA(ctx, cudaMemcpyAsync(p.eb, p.ea, p.Mpa * sizeof(int), cudaMemcpyDeviceToDevice, st));
-  return emu_pairs(ctx, p, 1.0, C, p.m, beta, st);
-}
-
-ltgw_status emu_gemm(ltgw_ctx *ctx, int m, int n, int64_t K, const double *A, int64_t lda, const double *B,
-                     int64_t ldb, double *C, int64_t ldc, bool sym, int s, cudaStream_t st) {
-  EmuPlan p;
-  if (emu_prepare(ctx, m, n, K, s, sym, 0, &p, st) != LTGW_OK) return ctx->status();
-  if (sym) return emu_syrk(ctx, p, A, lda, C, 0.0, st);
-  CHECK_LAUNCH(ctx, launch_slice_rows(B, ldb, n, K, p.Kp, s, p.strb, nullptr, p.dB, p.eb, st), 1);
-  return emu_product(ctx, p, A, lda, nullptr, 1.0, C, ldc, st);
-}
-
-// Pi from slices (the emulated FP64 form): per frequency (n_tau == 0, Pi_j =
-// -2 s M_j written directly) or moment t (lt_form 1: Laplace factors; 2:
-// e^{-Delta tau_t}) M_t = (Bt diag(f_t)) Bt^T, then the recombination with
-// d_E [n_omega][n_tau].
-ltgw_status polarizability_emu(ltgw_ctx *ctx, int N, int64_t n_pairs, const double *Bt, int64_t ldb,
-                               const double *delta, int n_omega, const double *d_om, int n_tau, const double *d_x,
-                               const double *d_w, const double *d_E, double *d_M, int spin, double *Pi,
-                               cudaStream_t s, int lt_form, int n_slices) {
-  const int n_t = n_tau ? n_tau : n_omega;
-  // pairs in chunks, so that the slices of one chunk are held at a time
-  // (6 slices of FP32 A and BF16 B digits: 36 bytes per value); chunks after
-  // the first are added (each chunk's product is exact to its own slices)
-  const int64_t max_chunk = (int64_t)1 << 17;
-  const int64_t n_chunks = (n_pairs + max_chunk - 1) / max_chunk;
-  const int64_t chunk = std::min(n_pairs, ((n_pairs + n_chunks - 1) / n_chunks + 63) / 64 * 64);   // balanced
-  EmuPlan p;
-  if (emu_prepare(ctx, N, N, chunk, n_slices, true, n_t, &p, s, n_pairs > chunk) != LTGW_OK) return ctx->status();
-  ctx->mark(EV_PI0, s);
-  const int mode = n_tau ? (lt_form == 2 ? SCALE_EXPTAU : SCALE_LAPLACE) : SCALE_DIRECT;
-  for (int64_t k0 = 0; k0 < n_pairs; k0 += chunk) {
-    const int64_t kc = std::min(chunk, n_pairs - k0);
-    p.K = kc;   // the row slicing writes every column < Kp: zeros past kc
-    CHECK_LAUNCH(ctx, launch_pi_factor64(delta + k0, kc, n_t, n_tau ? d_x : d_om,
-                                         mode == SCALE_LAPLACE ? d_w : nullptr, mode, p.factors, s), 1);
-    CHECK_LAUNCH(ctx, launch_slice_rows(Bt + k0, ldb, N, kc, p.Kp, n_slices, p.strb, nullptr, p.dB, p.eb, s), 1);
-    for (int t = 0; t < n_t; ++t)
-      if (emu_product(ctx, p, Bt + k0, ldb, p.factors + (int64_t)t * kc, n_tau ? 1.0 : -2.0 * spin,
-                      (n_tau ? d_M : Pi) + (int64_t)t * N * N, N, s, k0 > 0 ? 1.0 : 0.0) != LTGW_OK)
-        return ctx->status();
-  }
-  ctx->mark(EV_PI1, s);
-  if (n_tau)
-    CHECK_LAUNCH(ctx, launch_recombine(d_M, n_tau, d_E, n_omega, (int64_t)N * N, -2.0 * spin, Pi, s),
-                 (n_omega + 63) / 64);
-  return LTGW_OK;
-}
-
-// Rows of R~ = U^T R from slices: Ut [N][n_aux] (rows = kept eigenvectors),
-// R [n_aux][ld_r] with `cols` columns (pairs or orbitals); out [N][ld_out].
-ltgw_status project_emu(ltgw_ctx *ctx, int N, int n_aux, const double *Ut, const double *R, int64_t ld_r,
-                        int cols, double *out, int64_t ld_out, int n_slices, cudaStream_t s) {
-  EmuPlan p;
-  if (emu_prepare(ctx, N, cols, n_aux, n_slices, false, 0, &p, s) != LTGW_OK) return ctx->status();
-  CHECK_LAUNCH(ctx, launch_slice_cols(R, ld_r, n_aux, cols, p.Kp, n_slices, p.strb, p.dB, p.eb, s), 1);
-  return emu_product(ctx, p, Ut, n_aux, nullptr, 1.0, out, ld_out, s);
-}
-
-// W_j[t][c] = sum_PQ Btt[t][P][c] C_j[P][Q] Btt[t][Q][c] (Eq. ScreenedCoulombOrbital):
-// Y = C_j Btt (all targets side by side) from slices, then the FP64 column dot.
-ltgw_status wnm_emu(ltgw_ctx *ctx, int N, int n_omega, const double *C, int T, int n_orb_act, const double *Btt,
-                    int64_t ld_btt, int64_t stride_btt, double *W, int n_slices, cudaStream_t s) {
-  const int cols = T * n_orb_act;
-  EmuPlan p;
-  if (emu_prepare(ctx, N, cols, N, n_slices, false, 0, &p, s, true) != LTGW_OK) return ctx->status();
-  for (int t = 0; t < T; ++t)
-    CHECK_LAUNCH(ctx, launch_slice_cols(Btt + (int64_t)t * stride_btt, ld_btt, N, n_orb_act, p.Kp, n_slices,
-                                        p.strb, p.dB + (int64_t)t * n_orb_act * p.Kp, p.eb + t * n_orb_act, s),
-                 1);
-  for (int j = 0; j < n_omega; ++j) {
-    if (emu_product(ctx, p, C + (int64_t)j * N * N, N, nullptr, 1.0, p.tmp, cols, s) != LTGW_OK)
-      return ctx->status();
-    CHECK_LAUNCH(ctx, launch_coldot64(p.tmp, cols, Btt, ld_btt, stride_btt, N, n_orb_act, T,
-                                      W + (int64_t)j * T * n_orb_act, n_orb_act, s), 1);
-  }
-  return LTGW_OK;
-}
-
 // C_j = [1 - Pi_j]^-1 - 1 (Eq. ScreenedCoulombOrbital): the blocked sweep with
 // its updates from digits where N is past one pivot block of 128 by more than a
 // sliver (N = 130: 0.76 ms, FP64 tiles 0.56; N = 160: 0.59 against 0.85) and the
@@ -1008,7 +893,7 @@ ltgw_status screen_step(ltgw_ctx *ctx, int N, int n_omega, const double *Pi, dou
   void *digits = nullptr;
   const size_t bytes = screen_digit_bytes(N, n_omega);
   const bool use = N >= kScreenDigitsMinN && N <= 65535 && n_omega <= 65535 &&
-                   slice_reserve(ctx->a5, [&](Arena &A) { digits = A.take<uint8_t>(bytes); });
+                   slice_reserve(ctx, ctx->a5, false, [&](Arena &A) { digits = A.take<uint8_t>(bytes); });
   const cudaError_t e = use ? launch_screen_digits(Pi, N, n_omega, work, digits, C, ctx->flags, ctx->n_sm, s, &nl)
                             : launch_screen_blocked(Pi, N, n_omega, work, C, ctx->flags, s, &nl);
   ctx->launches += nl;
@@ -1331,7 +1216,7 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
   // emulated FP64 form: the FP64 form's data flow with K, the projections, Pi
   // and W_nm FP64-accurate from integer slices on the tensor cores
   const bool emu = p->precision == LTGW_FP64_EMU;
-  const int n_sl = kEmuSlices;
+  const SliceForm emu_f = emu_digits(kEmuSlices);
   const bool mixed = p->precision != LTGW_FP64 && !emu;   // split-BF16 / FP8 contractions
   const bool fp8 = p->precision == LTGW_FP8 || p->precision == LTGW_FP8_PI;   // Pi build in FP8 E4M3
   const bool fp8_w = p->precision == LTGW_FP8;                                // W_nm in FP8 E4M3
@@ -1547,9 +1432,8 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
                                                    1, 0, 0, s), 1);
         CHECK_LAUNCH(ctx, launch_split_bf16(d_Rt, d_Rh + off, d_Rl + off, cols * Kpa_aux, s), 1);
       } else if (emu) {
-        EmuPlan ep;   // K += B_blk B_blk^T from slices
-        if (emu_prepare(ctx, n_aux, n_aux, cols, n_sl, true, 0, &ep, s, true) != LTGW_OK) return ctx->status();
-        if (emu_syrk(ctx, ep, B_blk, cols, K, 1.0, s) != LTGW_OK) return ctx->status();
+        bool done = false;   // K += B_blk B_blk^T from slices
+        if (slice_syrk(ctx, n_aux, cols, B_blk, cols, K, 1.0, emu_f, s, &done) != LTGW_OK) return ctx->status();
       } else {
         bool done = false;   // K += B_blk B_blk^T
         if (slices_pay(n_aux, n_aux, cols, 1) &&
@@ -1576,7 +1460,7 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
   int N = n_aux, near = 0;
   if (naf) {
     if (naf_basis_dev(ctx, ctx->a3, n_aux, n_ov, B_act, ld_act, p->naf_thresh, d_Ut, d_lam, &N, &near, s,
-                      mixed, streamed ? &build_K : nullptr, emu ? n_sl : 0) != LTGW_OK)
+                      mixed, streamed ? &build_K : nullptr, emu ? kEmuSlices : 0) != LTGW_OK)
       return ctx->status();
   }
   ctx->stats.n_naf = N;
@@ -1651,8 +1535,9 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
         double *B_blk = nullptr;
         if (get_block(i0, i1, &B_blk) != LTGW_OK) return ctx->status();
         if (emu) {
-          if (project_emu(ctx, N, n_aux, d_Ut, B_blk, cols, (int)cols, d_Bt + (int64_t)(i0 - n_fc) * n_virt, n_ov,
-                          n_sl, s) != LTGW_OK)
+          bool done = false;
+          if (slice_project(ctx, N, n_aux, d_Ut, B_blk, cols, 0, cols, 1, d_Bt + (int64_t)(i0 - n_fc) * n_virt, n_ov, 0,
+                            emu_f, s, &done) != LTGW_OK)
             return ctx->status();
         } else {
           // R~_ov[:, block] = U^T R_blk
@@ -1663,7 +1548,8 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
       }
     } else if (emu) {
       REQUIRE(ctx, n_ov <= INT32_MAX, "too many pairs for one emulated projection");
-      if (project_emu(ctx, N, n_aux, d_Ut, B_act, ld_act, (int)n_ov, d_Bt, n_ov, n_sl, s) != LTGW_OK)
+      bool done = false;
+      if (slice_project(ctx, N, n_aux, d_Ut, B_act, ld_act, 0, n_ov, 1, d_Bt, n_ov, 0, emu_f, s, &done) != LTGW_OK)
         return ctx->status();
     } else {
       // R~_ov = U^T R_ov
@@ -1671,10 +1557,10 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
         return ctx->status();
     }
     if (emu) {
-      for (int t = 0; t < T; ++t)   // R~_tgt[t] = U^T R_tgt[t][:, active]
-        if (project_emu(ctx, N, n_aux, d_Ut, d_Btg + (int64_t)t * n_aux * n_orb + n_fc, n_orb, n_orb_act,
-                        d_Btt + (int64_t)t * N * n_orb_act, n_orb_act, n_sl, s) != LTGW_OK)
-          return ctx->status();
+      bool done = false;   // R~_tgt[t] = U^T R_tgt[t][:, active]
+      if (slice_project(ctx, N, n_aux, d_Ut, d_Btg + n_fc, n_orb, (int64_t)n_aux * n_orb, n_orb_act, T, d_Btt, n_orb_act,
+                        (int64_t)N * n_orb_act, emu_f, s, &done) != LTGW_OK)
+        return ctx->status();
     } else {
       // R~_tgt[t] = U^T R_tgt[t][:, active]
       if (project_f64(d_Btg + n_fc, n_orb, (int64_t)n_aux * n_orb, n_orb_act, T, d_Btt, n_orb_act,
@@ -1716,7 +1602,7 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
         return ctx->status();
     } else if (emu) {
       if (polarizability_emu(ctx, N, n_ov, Bt, ld_bt, d_delta, n_omega, d_om, n_tau, d_x, d_w, d_E, d_M, p->spin,
-                             d_Pi, s, p->use_laplace, n_sl) != LTGW_OK)
+                             d_Pi, s, p->use_laplace, emu_f) != LTGW_OK)
         return ctx->status();
     } else if (polarizability_dev(ctx, N, n_ov, Bt, ld_bt, d_delta, n_omega, d_om, n_tau, d_x, d_w, d_E, d_M,
                                   p->spin, d_Pi, s, p->use_laplace) != LTGW_OK) {
@@ -1732,7 +1618,8 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
     if (mixed) {
       if (wnm_tc(ctx, N, n_omega, d_C, T, n_orb_act, d_BtT64, d_BtT32, d_W, s, fp8_w) != LTGW_OK) return ctx->status();
     } else if (emu) {
-      if (wnm_emu(ctx, N, n_omega, d_C, T, n_orb_act, Btt, ld_btt, stride_btt, d_W, n_sl, s) != LTGW_OK)
+      bool done = false;
+      if (slice_wnm(ctx, N, n_omega, d_C, T, n_orb_act, Btt, ld_btt, stride_btt, d_W, emu_f, s, &done) != LTGW_OK)
         return ctx->status();
     } else {
       bool done = false;
@@ -2036,7 +1923,7 @@ ltgw_status ltgw_gemm_emulated(ltgw_ctx *ctx, int m, int n, int64_t k, const dou
   LTGW_CUDA(ctx, cudaMemsetAsync(ctx->flags, 0, FLAG_COUNT * sizeof(int), s));
   ctx->stats = ltgw_stats{};
   ctx->mark(EV_START, s);
-  if (emu_gemm(ctx, m, n, k, A, lda, sym ? A : B, sym ? lda : ldb, C, ldc, sym != 0, n_slices, s) != LTGW_OK)
+  if (emu_gemm(ctx, m, n, k, A, lda, sym ? A : B, sym ? lda : ldb, C, ldc, sym != 0, emu_digits(n_slices), s) != LTGW_OK)
     return ctx->status();
   ctx->mark(EV_END, s);
   LTGW_CUDA(ctx, cudaStreamSynchronize(s));
@@ -2085,7 +1972,7 @@ ltgw_status ltgw_polarizability_emulated(ltgw_ctx *ctx, int N, int64_t n_pairs, 
   }
   if (ctx->status() != LTGW_OK) return ctx->status();
   if (polarizability_emu(ctx, N, n_pairs, Bt, n_pairs, delta, n_omega, d_om, n_tau, d_x, d_w, d_E, d_M, spin, Pi, s,
-                         1, n_slices) != LTGW_OK)
+                         1, emu_digits(n_slices)) != LTGW_OK)
     return ctx->status();
   ctx->mark(EV_END, s);
   LTGW_CUDA(ctx, cudaStreamSynchronize(s));   // the staged grid lives in the workspace

@@ -142,9 +142,6 @@ struct TcGemmArgs {
   // with nt_group = 1).
   const __nv_bfloat16 *B_hi = nullptr, *B_lo = nullptr;
   int64_t rows_a = 0, rows_b = 0;   // padded row counts of A and B (tensor-map extents)
-  // single: B is exact in BF16 (B_lo not given) and so is every A value (its
-  // lo part is zero): one product per step, A_hi B_hi (integer digit operands)
-  int single = 0;
   // FP8 E4M3 form (launch_tc_fp8_gemm): codes qa [n_t][rows_a][Kp], qb [rows_b][Kp] and
   // per-row de-scales ds_a [n_t][rows_a], ds_b [rows_b], applied in the epilogue.
   const uint8_t *A8 = nullptr, *B8 = nullptr;
@@ -163,15 +160,6 @@ cudaError_t launch_split_bf16(const float *x, __nv_bfloat16 *hi, __nv_bfloat16 *
 // over the 3 Kq codes sums h_a h_b + l_a h_b + h_a l_b.
 cudaError_t launch_fp8_quantize(const float *X, int64_t Kp, int64_t Kq, const float *S, int n_t, int rows,
                                 uint8_t *qa, uint8_t *qb, float *ds_a, float *ds_b, cudaStream_t s, int split);
-// Rows of X (FP64 [rows][ld], `cols` used; with colscale, X_rk colscale_k as one
-// FP64 product) as s balanced base-128 digits of their fixed-point form
-// rint(X_r 2^(7 s - e_r)), e_r the exponent of the row's largest magnitude
-// (m < 2^e_r): digit i to dA / dB [i][r][Kp] (FP32 / BF16, either may be null; zero
-// past cols), e_r to exps[r].  The FP64-accurate product of two sliced operands sums
-// 2^(-7(i+j)) (a_i b_j^T) 2^(e_A + e_B) over i + j <= s + 1.
-cudaError_t launch_slice_rows(const double *X, int64_t ld, int rows, int64_t cols, int64_t Kp, int s,
-                              int64_t slice_stride, float *dA, __nv_bfloat16 *dB, int *exps, cudaStream_t st,
-                              const double *colscale = nullptr);
 // FP64 factors f[t][k] (k < K) of the Pi contraction per frequency (SCALE_DIRECT,
 // p0 = omega), Laplace point (SCALE_LAPLACE, p0 = x, p1 = w) or imaginary-time
 // node (SCALE_EXPTAU, p0 = tau), no fused operations.
@@ -181,18 +169,6 @@ cudaError_t launch_pi_factor64(const double *delta, int64_t K, int n_t, const do
 // sign(f) sqrt|f|, mag[t][k] = sqrt|f|; *neg is set to 1 if any f < 0.
 cudaError_t launch_pi_root_factor(const double *delta, int64_t K, int n_t, const double *p0, const double *p1,
                                   int mode, double *sgn, double *mag, int *neg, cudaStream_t st);
-// D[r][c] = beta D[r][c] + S[r][c] 2^(ea[r] + eb[c]) (rows <= 65535); lower (rows ==
-// cols, S symmetric): the entries c <= r scaled, each written to (r, c) and (c, r).
-cudaError_t launch_scale_exp2_to(const double *S, int64_t lds, double *D, int64_t ldd, int rows, int cols,
-                                 const int *ea, const int *eb, double beta, cudaStream_t st, int lower = 0);
-// The slices of X's columns 0..cols-1 as operand rows (X FP64 [rows][ld], the
-// contraction index is X's row): digit i of column c to dB[i][c][k] (BF16), its
-// exponent to exps[c]; as launch_slice_rows applied to X^T.
-cudaError_t launch_slice_cols(const double *X, int64_t ld, int rows, int cols, int64_t Kp, int s,
-                              int64_t slice_stride, __nv_bfloat16 *dB, int *exps, cudaStream_t st);
-// W[t][c] = sum_r Y[r][t ncols + c] Bt[t][r][c] in FP64 (Bt [n_tgt] x [N][ldb]).
-cudaError_t launch_coldot64(const double *Y, int64_t ldy, const double *Bt, int64_t ldb, int64_t strideB, int N,
-                            int ncols, int n_tgt, double *W, int64_t ldw, cudaStream_t st);
 // X itself quantised per row as an A operand (split: segments h | l | h).
 cudaError_t launch_fp8_quantize_a(const float *X, int64_t Kp, int64_t Kq, int rows, uint8_t *q, float *ds,
                                   cudaStream_t s, int split);
@@ -283,12 +259,7 @@ cudaError_t launch_to_f32_transposed(const double *src, int64_t lds, int64_t c0,
 cudaError_t launch_tc_reduce_full(const double *partial, const float *partial32, int splits, int groups,
                                   int n_tiles, int nJ, int rows, int cols, double alpha, double *out64,
                                   int64_t ld64, int64_t stride64, float *out32, int64_t ld32,
-                                  int rows_p32, int64_t stride32, cudaStream_t s, int64_t cols32 = -1,
-                                  double beta = 0.0);
-// out64[r][c] = alpha * (sum of the partials) + beta * out64[r][c], one group.
-cudaError_t launch_tc_reduce_full_acc(const double *partial, const float *partial32, int splits, int groups,
-                                      int n_tiles, int nJ, int rows, int cols, double alpha, double *out64,
-                                      int64_t ld64, double beta, cudaStream_t s);
+                                  int rows_p32, int64_t stride32, cudaStream_t s, int64_t cols32 = -1);
 // W[g][c] = sum over splits and tile rows of cd_out[split][g][I][c], c < cols.
 cudaError_t launch_tc_reduce_coldot(const float *cd_out, int splits, int groups, int n_tile_rows,
                                     int cols_p, int cols, double *W, int64_t ldw, cudaStream_t s);

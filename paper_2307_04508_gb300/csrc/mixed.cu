@@ -144,7 +144,7 @@ __global__ void tc_reduce_full_kernel(const double *__restrict__ partial, const 
                                       int splits, int groups, int n_tiles, int nJ, int rows, int cols,
                                       double alpha, double *__restrict__ out64, int64_t ld64, int64_t stride64,
                                       float *__restrict__ out32, int64_t ld32, int64_t cols32, int rows_p32,
-                                      int64_t stride32, double beta) {
+                                      int64_t stride32) {
   const int g = blockIdx.z;
   const int r = blockIdx.y;
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < (out32 ? cols32 : cols);
@@ -162,11 +162,7 @@ __global__ void tc_reduce_full_kernel(const double *__restrict__ partial, const 
         for (int s = 0; s < splits; ++s) acc += partial[(((int64_t)s * groups + g) * n_tiles + tile) * (128 * 128) + off];
       }
       acc *= alpha;
-      if (out64) {
-        double *o = out64 + g * stride64 + (int64_t)r * ld64 + c;
-        if (beta != 0.0) acc += beta * *o;
-        *o = acc;
-      }
+      if (out64) out64[g * stride64 + (int64_t)r * ld64 + c] = acc;
     }
     if (out32 && r < rows_p32) out32[g * stride32 + (int64_t)r * ld32 + c] = (float)acc;
   }
@@ -235,7 +231,7 @@ cudaError_t launch_to_f32_transposed(const double *src, int64_t lds, int64_t c0,
 cudaError_t launch_tc_reduce_full(const double *partial, const float *partial32, int splits, int groups,
                                   int n_tiles, int nJ, int rows, int cols, double alpha, double *out64,
                                   int64_t ld64, int64_t stride64, float *out32, int64_t ld32,
-                                  int rows_p32, int64_t stride32, cudaStream_t s, int64_t cols32, double beta) {
+                                  int rows_p32, int64_t stride32, cudaStream_t s, int64_t cols32) {
   if (cols32 < 0) cols32 = ld32;
   const int nrows = out32 ? std::max(rows, rows_p32) : rows;
   const int64_t ncols = out32 ? cols32 : cols;
@@ -244,15 +240,8 @@ cudaError_t launch_tc_reduce_full(const double *partial, const float *partial32,
   if (bx > 64) bx = 64;
   dim3 grid(bx, nrows, groups);
   tc_reduce_full_kernel<<<grid, 256, 0, s>>>(partial, partial32, splits, groups, n_tiles, nJ, rows, cols, alpha,
-                                             out64, ld64, stride64, out32, ld32, cols32, rows_p32, stride32, beta);
+                                             out64, ld64, stride64, out32, ld32, cols32, rows_p32, stride32);
   return cudaGetLastError();
-}
-
-cudaError_t launch_tc_reduce_full_acc(const double *partial, const float *partial32, int splits, int groups,
-                                      int n_tiles, int nJ, int rows, int cols, double alpha, double *out64,
-                                      int64_t ld64, double beta, cudaStream_t s) {
-  return launch_tc_reduce_full(partial, partial32, splits, groups, n_tiles, nJ, rows, cols, alpha, out64, ld64, 0,
-                               nullptr, 0, 0, 0, s, -1, beta);
 }
 
 cudaError_t launch_transpose_f64(const double *src, int64_t lds, int64_t c0, int rows, int cols, double *dst,
@@ -437,51 +426,6 @@ __global__ void __launch_bounds__(Q8_THREADS)
     write_codes(qr, k, q4, xr[k], inv, split, true);
   }
 }
-// One block per row r of X (FP64, row stride ld, `cols` columns; with
-// colscale, X_rk colscale_k, one FP64 product): e_r = the exponent of the
-// row's largest magnitude m (m = f 2^e_r, f in [0.5, 1); 0 for a zero row),
-// the fixed-point row Q = rint(X_r 2^(7 s - e_r)) (exact scaling, ties to
-// even), and Q in s balanced base-128 digits, the least significant in
-// [-64, 63], the leading one in [-128, 128]: digit i (1 = leading) goes to
-// dA[i-1][r][k] (FP32) and/or dB[i-1][r][k] (BF16), exact either way; columns
-// cols..Kp-1 are zero.  exps[r] = e_r.
-__device__ __forceinline__ double scaled_entry(const double *xr, const double *colscale, int64_t k) {
-  return colscale ? __dmul_rn(xr[k], colscale[k]) : xr[k];
-}
-
-__global__ void __launch_bounds__(256)
-    slice_rows_kernel(const double *__restrict__ X, int64_t ld, int64_t cols, int64_t Kp, int s,
-                      int64_t slice_stride, float *__restrict__ dA, __nv_bfloat16 *__restrict__ dB,
-                      int *__restrict__ exps, const double *__restrict__ colscale) {
-  __shared__ unsigned long long red[8];
-  const int r = blockIdx.x;
-  const double *xr = X + (int64_t)r * ld;
-  unsigned long long mb = 0ull;   // |x| bit patterns order like the values
-  for (int64_t k = threadIdx.x; k < cols; k += blockDim.x)
-    mb = max(mb, (unsigned long long)__double_as_longlong(scaled_entry(xr, colscale, k)) & 0x7fffffffffffffffull);
-  for (int o = 16; o > 0; o >>= 1) mb = max(mb, __shfl_down_sync(0xffffffffu, mb, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mb;
-  __syncthreads();
-  mb = 0ull;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) mb = max(mb, red[w]);
-  int e = 0;
-  if (mb != 0ull) frexp(__longlong_as_double((long long)mb), &e);   // m = f 2^e, f in [0.5, 1)
-  if (threadIdx.x == 0 && exps) exps[r] = e;
-  for (int64_t k = threadIdx.x; k < Kp; k += blockDim.x) {
-    // ldexp scales exactly without forming 2^(7 s - e), which overflows for tiny rows
-    long long Q = (k < cols && mb != 0ull) ? __double2ll_rn(ldexp(scaled_entry(xr, colscale, k), 7 * s - e)) : 0ll;
-    for (int i = s - 1; i >= 1; --i) {   // balanced digits, least significant first
-      const long long t = (Q + 64) >> 7;
-      const float d = (float)(Q - (t << 7));
-      if (dA) dA[i * slice_stride + (int64_t)r * Kp + k] = d;
-      if (dB) dB[i * slice_stride + (int64_t)r * Kp + k] = __float2bfloat16_rn(d);
-      Q = t;
-    }
-    if (dA) dA[(int64_t)r * Kp + k] = (float)Q;
-    if (dB) dB[(int64_t)r * Kp + k] = __float2bfloat16_rn((float)Q);
-  }
-}
-
 // FP64 per-pair factors f[t][k] of the Pi contraction, each operation rounded
 // once (no fused multiply-add): Delta / (w_t^2 + Delta^2) (direct, p0 = w),
 // (w_t Delta) exp(-Delta Delta x_t) (Laplace, p0 = x, p1 = w), exp(-Delta tau_t)
@@ -514,93 +458,6 @@ __global__ void pi_root_factor_kernel(const double *__restrict__ delta, int64_t 
     mag[(int64_t)t * K + k] = r;
   }
 }
-
-// D[r][c] = beta D[r][c] + S[r][c] 2^(ea[r] + eb[c]) for r < rows, c < cols
-// (the scaling is exact; S may be D with beta = 0).  lower: the product of a
-// lower-tile form (S symmetric, rows == cols) whose mirrored upper entries
-// must take the lower entry's scale 2^(ea[r] + eb[c]), r >= c: only c <= r
-// is read, and each value is written to (r, c) and (c, r).
-__global__ void scale_exp2_kernel(const double *S, int64_t lds, double *D, int64_t ldd, int rows, int cols,
-                                  const int *__restrict__ ea, const int *__restrict__ eb, double beta, int lower) {
-  const int r = blockIdx.y;
-  if (r >= rows) return;
-  const int er = ea[r];
-  const int cend = lower ? min(r + 1, cols) : cols;
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cend; c += gridDim.x * blockDim.x) {
-    const double v = ldexp(S[(int64_t)r * lds + c], er + eb[c]);
-    double *d = D + (int64_t)r * ldd + c;
-    const double o = beta != 0.0 ? beta * *d + v : v;
-    *d = o;
-    if (lower && c != r) D[(int64_t)c * ldd + r] = o;
-  }
-}
-
-// The slices of X^T's rows, i.e. of X's columns: X FP64 [rows][ld], columns
-// 0..cols-1 (each an operand row, contraction index = X's row).  Block: 32
-// columns x 8 row lanes.  Pass 1: e_c, the exponent of column c's largest
-// magnitude (as in slice_rows_kernel); pass 2: 32 x 32 tiles through shared
-// memory, the digits of column c written to dB[i][c][k] (k = X's row, BF16) so
-// that a warp's stores run along k.  exps[c] = e_c.
-__global__ void __launch_bounds__(256)
-    slice_cols_kernel(const double *__restrict__ X, int64_t ld, int rows, int cols, int64_t Kp, int s,
-                      int64_t slice_stride, __nv_bfloat16 *__restrict__ dB, int *__restrict__ exps) {
-  __shared__ unsigned long long red[8][33];
-  __shared__ double tile[32][33];
-  __shared__ int e_s[32];
-  const int c0 = blockIdx.x * 32, tx = threadIdx.x, ty = threadIdx.y;
-  const int c = c0 + tx;
-  unsigned long long mb = 0ull;
-  if (c < cols)
-    for (int r = ty; r < rows; r += 8)
-      mb = max(mb, (unsigned long long)__double_as_longlong(X[(int64_t)r * ld + c]) & 0x7fffffffffffffffull);
-  red[ty][tx] = mb;
-  __syncthreads();
-  if (ty == 0) {
-    for (int q = 1; q < 8; ++q) mb = max(mb, red[q][tx]);
-    int e = 0;
-    if (mb != 0ull) frexp(__longlong_as_double((long long)mb), &e);
-    e_s[tx] = mb != 0ull ? e : INT_MIN;   // INT_MIN: a zero column
-    if (c < cols && exps) exps[c] = e;
-  }
-  __syncthreads();
-  for (int r0 = 0; r0 < rows; r0 += 32) {
-    for (int q = ty; q < 32; q += 8) {
-      const int r = r0 + q;
-      tile[q][tx] = (r < rows && c < cols) ? X[(int64_t)r * ld + c] : 0.0;
-    }
-    __syncthreads();
-    // thread (tx, ty): row k = r0 + tx of columns c0 + ty, ty + 8, ...
-    const int k = r0 + tx;
-    for (int q = ty; q < 32; q += 8) {
-      const int cc = c0 + q;
-      if (cc >= cols || k >= rows) continue;
-      const int e = e_s[q];
-      long long Q = e != INT_MIN ? __double2ll_rn(ldexp(tile[tx][q], 7 * s - e)) : 0ll;
-      for (int i = s - 1; i >= 1; --i) {
-        const long long t = (Q + 64) >> 7;
-        dB[i * slice_stride + (int64_t)cc * Kp + k] = __float2bfloat16_rn((float)(Q - (t << 7)));
-        Q = t;
-      }
-      dB[(int64_t)cc * Kp + k] = __float2bfloat16_rn((float)Q);
-    }
-    __syncthreads();
-  }
-}
-
-// W[t][c] = sum_r Y[r][t ncols + c] Bt[t][r][c] (FP64), t < n_tgt, c < ncols:
-// the column dot of W_nm (Eq. ScreenedCoulombOrbital) on a product Y = C_j Bt.
-__global__ void coldot64_kernel(const double *__restrict__ Y, int64_t ldy, const double *__restrict__ Bt,
-                                int64_t ldb, int64_t strideB, int N, int ncols, int n_tgt, double *__restrict__ W,
-                                int64_t ldw) {
-  const int t = blockIdx.y;
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncols; c += gridDim.x * blockDim.x) {
-    double acc = 0.0;
-    const double *y = Y + (int64_t)t * ncols + c;
-    const double *b = Bt + (int64_t)t * strideB + c;
-    for (int r = 0; r < N; ++r) acc = fma(y[(int64_t)r * ldy], b[(int64_t)r * ldb], acc);
-    W[(int64_t)t * ldw + c] = acc;
-  }
-}
 }  // namespace
 
 cudaError_t launch_fp8_quantize(const float *X, int64_t Kp, int64_t Kq, const float *S, int n_t, int rows,
@@ -611,15 +468,6 @@ cudaError_t launch_fp8_quantize(const float *X, int64_t Kp, int64_t Kq, const fl
     fp8_quantize_kernel<8><<<rows, Q8_THREADS, 0, s>>>(X, Kp, Kq, S, n_t, rows, qa, qb, ds_a, ds_b, split);
   else
     fp8_quantize_kernel<32><<<rows, Q8_THREADS, 0, s>>>(X, Kp, Kq, S, n_t, rows, qa, qb, ds_a, ds_b, split);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_slice_rows(const double *X, int64_t ld, int rows, int64_t cols, int64_t Kp, int s,
-                              int64_t slice_stride, float *dA, __nv_bfloat16 *dB, int *exps, cudaStream_t st,
-                              const double *colscale) {
-  if (rows <= 0) return cudaSuccess;
-  if (s < 1 || s > 8 || Kp < cols) return cudaErrorInvalidValue;
-  slice_rows_kernel<<<rows, 256, 0, st>>>(X, ld, cols, Kp, s, slice_stride, dA, dB, exps, colscale);
   return cudaGetLastError();
 }
 
@@ -638,33 +486,6 @@ cudaError_t launch_pi_root_factor(const double *delta, int64_t K, int n_t, const
   int bx = (int)((K + 255) / 256);
   if (bx > 152) bx = 152;
   pi_root_factor_kernel<<<dim3(bx, n_t), 256, 0, st>>>(delta, K, p0, p1, mode, sgn, mag, neg);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_scale_exp2_to(const double *S, int64_t lds, double *D, int64_t ldd, int rows, int cols,
-                                 const int *ea, const int *eb, double beta, cudaStream_t st, int lower) {
-  if (rows <= 0 || cols <= 0) return cudaSuccess;
-  if (rows > 65535 || (lower && rows != cols)) return cudaErrorInvalidValue;
-  int bx = (cols + 255) / 256;
-  if (bx > 16) bx = 16;
-  scale_exp2_kernel<<<dim3(bx, rows), 256, 0, st>>>(S, lds, D, ldd, rows, cols, ea, eb, beta, lower);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_slice_cols(const double *X, int64_t ld, int rows, int cols, int64_t Kp, int s,
-                              int64_t slice_stride, __nv_bfloat16 *dB, int *exps, cudaStream_t st) {
-  if (rows <= 0 || cols <= 0) return cudaSuccess;
-  if (s < 1 || s > 8 || Kp < rows) return cudaErrorInvalidValue;
-  slice_cols_kernel<<<(cols + 31) / 32, dim3(32, 8), 0, st>>>(X, ld, rows, cols, Kp, s, slice_stride, dB, exps);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_coldot64(const double *Y, int64_t ldy, const double *Bt, int64_t ldb, int64_t strideB, int N,
-                            int ncols, int n_tgt, double *W, int64_t ldw, cudaStream_t st) {
-  if (N <= 0 || ncols <= 0 || n_tgt <= 0) return cudaSuccess;
-  int bx = (ncols + 127) / 128;
-  if (bx > 64) bx = 64;
-  coldot64_kernel<<<dim3(bx, n_tgt), 128, 0, st>>>(Y, ldy, Bt, ldb, strideB, N, ncols, n_tgt, W, ldw);
   return cudaGetLastError();
 }
 

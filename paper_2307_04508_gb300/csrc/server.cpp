@@ -237,8 +237,8 @@ size_t ltgw_request_footprint(const ltgw_params *p, int n_tgt) {
   const size_t pi_part = nN * (nN + 1) / 2 * t * std::min<size_t>(64, cdiv(n_ov, 2048)) * tile;
   const size_t partials = std::max(k_part, std::max(p_part, pi_part));
   if (p->precision == LTGW_FP64_EMU) {
-    // projected ov block; the largest slice set (6 slices: 4 bytes per A digit,
-    // 2 per B digit, of the metric's n_aux x n_ov operands) and the partials
+    // projected ov block; an upper estimate of the largest slice set (three
+    // operands of 6 slices of 2 bytes per value) and the partials
     d += N * n_ov + 9 * n_aux * n_ov / 2 + partials;
   } else if (p->precision != LTGW_FP64) {
     d += (2 * n_aux * n_ov + N * n_ov) / 2 + n_om * N * N / 2;  // FP32 copies, BF16 hi / lo of the ov block

@@ -550,15 +550,15 @@ __device__ __forceinline__ unsigned long long warp_max(unsigned long long v) {
   return v;
 }
 
-// Largest magnitude of every row over a chunk of its columns (grid: chunk,
-// row, batch), its exponent merged into exps (initialised to SL_ZERO).
+// Largest magnitude of every row over a chunk of its columns (grid: row,
+// chunk, batch), its exponent merged into exps (initialised to SL_ZERO).
 __global__ void __launch_bounds__(256) slice_max_rows_kernel(SliceSrc a, int bits, int64_t chunk) {
   __shared__ unsigned long long red[8];
   if (a.only_if && !*a.only_if) return;
-  const int r = blockIdx.y, b = blockIdx.z;
+  const int r = blockIdx.x, b = blockIdx.z;
   const double *x = a.X + (int64_t)b * a.x_batch + (int64_t)r * a.ld;
   const double *f = a.colscale ? a.colscale + (int64_t)b * a.cs_batch : nullptr;
-  const int64_t k0 = blockIdx.x * chunk, k1 = min(a.K, k0 + chunk);
+  const int64_t k0 = blockIdx.y * chunk, k1 = min(a.K, k0 + chunk);
   unsigned long long mb = 0ull;
   for (int64_t k = k0 + threadIdx.x; k < k1; k += 256)
     mb = max(mb, mag_bits(f ? __dmul_rn(x[k], f[k]) : x[k]));
@@ -577,13 +577,13 @@ template <int NS, int BITS>
 __global__ void __launch_bounds__(256) slice_rows_tiles_kernel(SliceSrc a) {
   if (a.only_if && !*a.only_if) return;
   const int b = blockIdx.z;
-  const int r = blockIdx.y * 8 + (threadIdx.x >> 5);
+  const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
   uint8_t *dig = a.dig + (int64_t)b * a.dig_batch;
   const double *x = a.X + (int64_t)b * a.x_batch + (int64_t)r * a.ld;
   const double *f = a.colscale ? a.colscale + (int64_t)b * a.cs_batch : nullptr;
   const bool live = r < a.rows;
   const int e = live ? a.exps[(int64_t)b * a.exp_batch + r] : SL_ZERO;
-  for (int g = blockIdx.x * 32 + (threadIdx.x & 31); g < 2 * a.nkb; g += gridDim.x * 32) {
+  for (int g = blockIdx.y * 32 + (threadIdx.x & 31); g < 2 * a.nkb; g += gridDim.y * 32) {
     double v[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
@@ -631,13 +631,13 @@ __device__ __forceinline__ Scaled scaled_product(double x, double f) {
 }
 
 // Exponent of the largest |X_rk f_bk| over a chunk of k, for every factor row
-// b (grid: chunk, row); X is read from memory once.
+// b (grid: row, chunk); X is read from memory once.
 __global__ void __launch_bounds__(256) slice_max_scaled_kernel(SliceSrc a, int batch, int64_t chunk) {
   __shared__ int red[8];
   if (a.only_if && !*a.only_if) return;
-  const int r = blockIdx.y;
+  const int r = blockIdx.x;
   const double *x = a.X + (int64_t)r * a.ld;
-  const int64_t k0 = blockIdx.x * chunk, k1 = min(a.K, k0 + chunk);
+  const int64_t k0 = blockIdx.y * chunk, k1 = min(a.K, k0 + chunk);
   for (int b = 0; b < batch; ++b) {
     const double *f = a.colscale + (int64_t)b * a.cs_batch;
     int m = SL_ZERO;
@@ -661,10 +661,10 @@ __global__ void __launch_bounds__(256) slice_max_scaled_kernel(SliceSrc a, int b
 __global__ void __launch_bounds__(256) slice_rows_scaled_kernel(SliceSrc a, int batch) {
   if (a.only_if && !*a.only_if) return;
   constexpr int NS = 7, BITS = 8;
-  const int r = blockIdx.y * 8 + (threadIdx.x >> 5);
+  const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
   const double *x = a.X + (int64_t)r * a.ld;
   const bool live = r < a.rows;
-  for (int g = blockIdx.x * 32 + (threadIdx.x & 31); g < 2 * a.nkb; g += gridDim.x * 32) {
+  for (int g = blockIdx.y * 32 + (threadIdx.x & 31); g < 2 * a.nkb; g += gridDim.y * 32) {
     double v[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) v[q] = (live && (int64_t)g * 8 + q < a.K) ? x[(int64_t)g * 8 + q] : 0.0;
@@ -694,7 +694,7 @@ __global__ void __launch_bounds__(256) slice_rows_short_kernel(SliceSrc a, int a
   if (a.only_if && !*a.only_if) return;
   constexpr int LANES = W >= 2 ? 32 : 16, H = W >= 2 ? W / 2 : 1;   // lanes per row, groups of eight k per lane
   const int b = blockIdx.z, sub = threadIdx.x & (LANES - 1);
-  const int r = blockIdx.y * (256 / LANES) + threadIdx.x / LANES;
+  const int r = blockIdx.x * (256 / LANES) + threadIdx.x / LANES;
   uint8_t *dig = a.dig + (int64_t)b * a.dig_batch;
   const double *x = a.X + (int64_t)b * a.x_batch + (int64_t)r * a.ld;
   const double *f = a.colscale ? a.colscale + (int64_t)b * a.cs_batch : nullptr;
@@ -790,11 +790,11 @@ cudaError_t slice_operand(const SliceSrc &a, int batch, cudaStream_t s) {
   if (!a.cols && a.nkb <= 32) {
     const int al = a.ld % 2 == 0 && a.x_batch % 2 == 0 && ((uintptr_t)a.X & 15) == 0;
     if (a.nkb <= 8)
-      slice_rows_short_kernel<NS, BITS, 1><<<dim3(1, a.rows_p / 16, batch), 256, 0, s>>>(a, al);
+      slice_rows_short_kernel<NS, BITS, 1><<<dim3(a.rows_p / 16, 1, batch), 256, 0, s>>>(a, al);
     else if (a.nkb <= 16)
-      slice_rows_short_kernel<NS, BITS, 2><<<dim3(1, a.rows_p / 8, batch), 256, 0, s>>>(a, al);
+      slice_rows_short_kernel<NS, BITS, 2><<<dim3(a.rows_p / 8, 1, batch), 256, 0, s>>>(a, al);
     else
-      slice_rows_short_kernel<NS, BITS, 4><<<dim3(1, a.rows_p / 8, batch), 256, 0, s>>>(a, al);
+      slice_rows_short_kernel<NS, BITS, 4><<<dim3(a.rows_p / 8, 1, batch), 256, 0, s>>>(a, al);
     return cudaGetLastError();
   }
   const int64_t n_exp = (int64_t)batch * a.exp_batch;
@@ -802,17 +802,17 @@ cudaError_t slice_operand(const SliceSrc &a, int batch, cudaStream_t s) {
   if (NS == 7 && BITS == 8 && a.colscale && a.x_batch == 0) {
     const int64_t want = std::max<int64_t>(1, 152 * 16 / std::max<int64_t>(1, a.rows));
     const int64_t nch = std::max<int64_t>(std::min<int64_t>(want, (a.K + 2047) / 2048), (a.K + 8191) / 8192);
-    slice_max_scaled_kernel<<<dim3((unsigned)nch, a.rows), 256, 0, s>>>(a, batch, (a.K + nch - 1) / nch);
+    slice_max_scaled_kernel<<<dim3(a.rows, (unsigned)nch), 256, 0, s>>>(a, batch, (a.K + nch - 1) / nch);
     const int gx = (int)std::min<int64_t>((2 * (int64_t)a.nkb + 31) / 32, 1024);
-    slice_rows_scaled_kernel<<<dim3(gx, a.rows_p / 8), 256, 0, s>>>(a, batch);
+    slice_rows_scaled_kernel<<<dim3(a.rows_p / 8, gx), 256, 0, s>>>(a, batch);
   } else if (!a.cols) {
     // about eight blocks per SM over rows, chunks and the batch
     const int64_t want = std::max<int64_t>(1, 152 * 8 / std::max<int64_t>(1, (int64_t)a.rows * batch));
     const int64_t nch = std::min<int64_t>(want, (a.K + 2047) / 2048);
     const int64_t chunk = (a.K + nch - 1) / nch;
-    slice_max_rows_kernel<<<dim3((unsigned)nch, a.rows, batch), 256, 0, s>>>(a, BITS, chunk);
+    slice_max_rows_kernel<<<dim3(a.rows, (unsigned)nch, batch), 256, 0, s>>>(a, BITS, chunk);
     const int gx = (int)std::min<int64_t>((2 * (int64_t)a.nkb + 31) / 32, 64);
-    slice_rows_tiles_kernel<NS, BITS><<<dim3(gx, a.rows_p / 8, batch), 256, 0, s>>>(a);
+    slice_rows_tiles_kernel<NS, BITS><<<dim3(a.rows_p / 8, gx, batch), 256, 0, s>>>(a);
   } else {
     const int64_t want = std::max<int64_t>(1, 152 * 8 / std::max<int64_t>(1, (int64_t)((a.rows + 31) / 32) * batch));
     const int64_t nch = std::min<int64_t>(want, (a.K + 63) / 64);
@@ -840,8 +840,7 @@ cudaError_t launch_ns(const SliceGemmArgs &g, int blocks, cudaStream_t s) {
 }  // namespace
 
 cudaError_t launch_slice_operand(const SliceSrc &a, int ns, int bits, int batch, cudaStream_t s) {
-  if (a.rows < 1 || a.K < 1 || batch < 1 || batch > 65535 || a.rows > a.rows_p || a.rows_p % 128 || a.rows_p > 65535 * 8 ||
-      (!a.cols && a.K > 512 && a.rows > 65535) || (int64_t)a.nkb * 16 < a.K || a.exp_batch < a.rows_p || (a.cols && (a.colscale || a.only_if)) || (!a.cols && a.col_group))
+  if (a.rows < 1 || a.K < 1 || batch < 1 || batch > 65535 || a.rows > a.rows_p || a.rows_p % 128 || (int64_t)a.nkb * 16 < a.K || a.exp_batch < a.rows_p || (a.cols && (a.colscale || a.only_if)) || (!a.cols && a.col_group))
     return cudaErrorInvalidValue;
   if (bits == 8) return ns == 7 ? slice_operand<7, 8>(a, batch, s) : cudaErrorInvalidValue;
   switch (bits == 7 ? ns : 0) {
