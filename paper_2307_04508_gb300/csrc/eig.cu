@@ -155,8 +155,8 @@ __global__ void hh_finalize_kernel(const double *A, double *d, double *e, int n)
 // Writing A^(k) for the matrix after the first k rank-2 updates, reflector k
 // comes from row k of A^(k) (= column k by symmetry), p_k = tau_k A^(k)_22 v_k,
 // w_k = p_k - (tau_k/2)(p_k.v_k) v_k and A^(k+1)_22 = A^(k)_22 - v_k w_k^T - w_k v_k^T.
-// Row r belongs to block r mod G for the whole reduction (held in shared
-// memory when the block's rows fit there, else in place in global memory).
+// Row r belongs to block r mod G for the whole reduction and stays in its
+// shared memory.
 // Step k:
 //  phase 1 (every block, identical arithmetic, so every block holds the same
 //    vectors): normalise v_{k-1}; p_{k-1}.v_{k-1} from the full p_{k-1} (so
@@ -233,7 +233,6 @@ __device__ __forceinline__ A warp_sum(A v) {
 template <typename T>
 struct HhFusedArgs {
   const double *A0;   // the input matrix (row 0 is read from here at step 0)
-  T *A;               // working rows, updated in place when they do not fit in shared memory
   T *V;               // [n][n] reflectors, row k = v_k (columns k+1..n-1 written)
   double *d, *e, *tau;
   T *P;               // [2][n] p of the step, by parity
@@ -242,6 +241,7 @@ struct HhFusedArgs {
   GridBar *gb;
   int *flags;
   int n, R;           // R = rows per block
+  int64_t ld;         // row stride of A0 and V
 };
 
 // One lane-strided pass over row[j0:j1): optional update a -= v_r w + w_r v
@@ -284,7 +284,7 @@ __device__ __forceinline__ T row_pass(T *row, int j0, int j1, const T *vp, const
 // HH_P1_FP64 threads only (the FP32 form does all of it in FP32).
 constexpr int HH_P1_FP64 = 128;
 
-template <typename T, bool SMEM>
+template <typename T>
 __global__ void __launch_bounds__(512, 1) hh_fused_kernel(HhFusedArgs<T> g) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *smem = reinterpret_cast<T *>(smem_raw);
@@ -296,13 +296,11 @@ __global__ void __launch_bounds__(512, 1) hh_fused_kernel(HhFusedArgs<T> g) {
   const int p1 = (sizeof(T) == 8) ? min(HH_P1_FP64, (int)blockDim.x) : (int)blockDim.x;  // phase-1 team
   const int p1w = p1 >> 5;
   T *wv = smem + 2 * n;
-  T *rows = smem + 3 * n;   // SMEM: [R][n], local row lr is global row lr * G + b
+  T *rows = smem + 3 * n;   // [R][n], local row lr is global row lr * G + b
   const int n_own = (b < n) ? min(R, (n - 1 - b) / G + 1) : 0;
-  if (SMEM) {
-    for (int lr = 0; lr < n_own; ++lr) {
-      const double *src = g.A0 + (int64_t)(lr * G + b) * n;
-      for (int j = threadIdx.x; j < n; j += blockDim.x) rows[(int64_t)lr * n + j] = (T)src[j];
-    }
+  for (int lr = 0; lr < n_own; ++lr) {
+    const double *src = g.A0 + (int64_t)(lr * G + b) * g.ld;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) rows[(int64_t)lr * n + j] = (T)src[j];
   }
   T *vprev = smem + n, *vcur = smem;
   T tau_prev = 0, sc_prev = 0;
@@ -345,7 +343,7 @@ __global__ void __launch_bounds__(512, 1) hh_fused_kernel(HhFusedArgs<T> g) {
         for (int j = k + threadIdx.x; j < n; j += p1) {
           const T vj = (j == k) ? (T)1 : vprev[j] * sc_prev;   // normalise v_{k-1}
           vprev[j] = vj;
-          if (b == 0) g.V[(int64_t)(k - 1) * n + j] = vj;
+          if (b == 0) g.V[(int64_t)(k - 1) * g.ld + j] = vj;
           dsum = fma(wv[j], vj, dsum);
         }
       if (warp < p1w) {
@@ -404,7 +402,7 @@ __global__ void __launch_bounds__(512, 1) hh_fused_kernel(HhFusedArgs<T> g) {
       for (int task = warp; task < nact * wpr; task += nwarp) {
         const int lr = lr0 + task / wpr, seg = task % wpr;
         const int r = lr * G + b;
-        T *row = SMEM ? rows + (int64_t)lr * n : g.A + (int64_t)r * n;
+        T *row = rows + (int64_t)lr * n;
         const int j0 = k + 1 + seg * seglen, j1 = min(n, j0 + seglen);
         T acc = 0, a1 = 0;
         if (j0 < j1) {
@@ -435,12 +433,12 @@ __global__ void __launch_bounds__(512, 1) hh_fused_kernel(HhFusedArgs<T> g) {
     // last step the owner of row n-1 also hands over that row's last two entries
     if ((k + 1) % G == b) {
       const int lr = (k + 1) / G;
-      const T *rp = SMEM ? rows + (int64_t)lr * n : g.A + (int64_t)(k + 1) * n;
+      const T *rp = rows + (int64_t)lr * n;
       T *pubp = g.pub + (size_t)((k + 1) & 1) * n;
       for (int j = k + 1 + threadIdx.x; j < n; j += blockDim.x) pubp[j] = rp[j];
     }
     if (k == n - 3 && (n - 1) % G == b && threadIdx.x == 0) {
-      const T *rp = SMEM ? rows + (int64_t)((n - 1) / G) * n : g.A + (int64_t)(n - 1) * n;
+      const T *rp = rows + (int64_t)((n - 1) / G) * n;
       g.tail[0] = rp[n - 2];
       g.tail[1] = rp[n - 1];
     }
@@ -455,8 +453,8 @@ __global__ void __launch_bounds__(512, 1) hh_fused_kernel(HhFusedArgs<T> g) {
     const T *Pk = g.P + (size_t)(kl & 1) * n;
     const T *pb = g.pub + (size_t)((kl + 1) & 1) * n;
     const T v2 = 1, v1 = vprev[n - 1] * sc_prev;
-    g.V[(int64_t)kl * n + n - 2] = v2;
-    g.V[(int64_t)kl * n + n - 1] = v1;
+    g.V[(int64_t)kl * g.ld + n - 2] = v2;
+    g.V[(int64_t)kl * g.ld + n - 1] = v1;
     const T p2 = __ldcg(Pk + n - 2), p1v = __ldcg(Pk + n - 1);
     const T gam = (T)0.5 * tau_prev * (p2 * v2 + p1v * v1);
     const T w2 = p2 - gam * v2, w1 = p1v - gam * v1;
@@ -537,6 +535,372 @@ __device__ __forceinline__ double recip_nr(double q) {
 #pragma unroll
   for (int s = 0; s < STEPS; ++s) y = y * fma(-q, y, 2.0);
   return y;
+}
+
+// ---- blocked Householder reduction (one cooperative launch per panel) ----
+// The fused reduction above spends three FP64 multiply-adds per matrix entry
+// and step, two of them on the rank-2 updates.  Here a panel of HP_NB steps
+// leaves the trailing matrix as it was at the panel's start (A) and keeps the
+// reflectors V and their w (W) beside it; each step applies
+//   A^(k) = A - sum_t (v_t w_t^T + w_t v_t^T)
+// to the one column and the one product that it needs, so the matrix pays one
+// multiply-add per entry and step, and the panel's updates reach it together,
+// as one product of length 2 HP_NB from digits on the tensor cores.
+// Row r belongs to block r mod G.  Step k = k0 + j, two grid barriers:
+//   own rows' entries of column k, x_r (known from the step before) -> barrier 1;
+//   every block: the whole x into shared memory; the own rows' products
+//     S_r = sum_c A[r][c] x_c and their share of T = x^T S; block b < 2 j also the
+//     product of x with the one earlier vector v_t (b = 2 t) or w_t (b = 2 t + 1);
+//     one warp meanwhile the reflector's scalars                   -> barrier 2;
+//   every block: with v = sc (x - beta e_{k+1}): a_t = v_t.v and b_t = w_t.v from those
+//     products, v.Av = sc^2 (T - 2 beta S_{k+1} + beta^2 A_{k+1,k+1}),
+//     p.v = tau (v.Av - 2 sum a_t b_t); the own rows' p_r = tau (y_r - sum_t (v_t[r] b_t
+//     + w_t[r] a_t)), y = sc (S - beta A e_{k+1}), their w_r and their entries of
+//     column k + 1 (w_{k+1} from S_{k+1}, which its owner published).
+// Own rows' v_t, w_t stay in shared memory.  What crosses blocks goes through
+// L2; the barriers are bounded as above.
+// On this part an FP64 instruction holds the SM's pipe for 16 clocks whether 1
+// or 32 lanes need it, and one warp's FP64 instructions follow each other at
+// about 64: so nothing between the barriers waits for the scalars (only the
+// unscaled products are published), and the sums over the panel's vectors
+// reduce four rows per warp together.
+// Bound: the step's chain, two barriers with their L2 round trips (3.5 of
+// about 10 us per step at n = 1000), beside one multiply-add per entry on the FP64
+// pipe.  Tried and slower: values in self-validating 16-byte packets that their
+// readers poll, without barriers (every block polls every packet: 4 to 6 us per
+// exchange where a barrier and the loads take 2.5).
+constexpr int HP_NB = 64;         // steps per panel: the update's length is 128
+constexpr int HP_THREADS = 512;
+constexpr int HP_MAX_ROWS = 128;  // rows per block
+constexpr int HP_SIGMA_WARPS = 4; // the last warps: sum of squares of x, then (but the last) rows
+
+struct HhPanelArgs {
+  const double *A;     // [n][n] the matrix as of step k0
+  double *V;           // [n][n] reflectors, row k = v_k
+  double *W;           // [HP_NB][n] w of the panel's steps
+  double *d, *e, *tau;
+  double *xbuf;        // [2][n] column k, by parity
+  double *part;        // [2][G] the blocks' shares of T, by parity
+  double *dots;        // [2][2 HP_NB] products of x with the earlier vectors, by parity
+  double *snext;       // [2][2] S_{k+1}, A[k+1][k+1]
+  unsigned long long *wmax;   // bits of the panel's largest |w| (zeroed)
+  GridBar *gb;
+  unsigned bar0;       // barriers passed before this launch
+  int *flags;
+  int n, k0, R;
+};
+
+__device__ __forceinline__ void grid_arrive(GridBar *gb) { red_add_release(&gb->count, 1u); }
+
+// One thread's bounded wait for barrier number j; false after a time-out anywhere.
+__device__ bool grid_wait(GridBar *gb, unsigned j, int *flags) {
+  const unsigned target = gridDim.x * (j + 1);
+  if (ld_acquire(&gb->count) >= target) return true;
+  const uint64_t t0 = gtimer();
+  unsigned it = 0;
+  while (ld_acquire(&gb->count) < target) {
+    if ((++it & 1023) == 0) {
+      if (*(volatile int *)&gb->abort) return false;
+      if (gtimer() - t0 > 2000000000ull) {
+        atomicExch(&flags[FLAG_EIG], 1);
+        atomicExch(&gb->abort, 1);
+        return false;
+      }
+    }
+  }
+  return true;
+}
+
+// Named barriers: `sync` waits, `arrive` does not.
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+__device__ __forceinline__ double warp_sum_all(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// sum over j0 <= j < j1 of row[j] x[j], lane-strided, eight loads in flight.
+template <bool L2>
+__device__ __forceinline__ double dot_pass(const double *row, int j0, int j1, const double *x) {
+  const int lane = threadIdx.x & 31;
+  double acc0 = 0.0, acc1 = 0.0;
+  int j = j0 + lane;
+  for (; j + 7 * 32 < j1; j += 8 * 32) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = L2 ? __ldcg(row + j + u * 32) : row[j + u * 32];
+#pragma unroll
+    for (int u = 0; u < 8; u += 2) {
+      acc0 = fma(v[u], x[j + u * 32], acc0);
+      acc1 = fma(v[u + 1], x[j + (u + 1) * 32], acc1);
+    }
+  }
+  double v[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u)
+    if (j + u * 32 < j1) v[u] = L2 ? __ldcg(row + j + u * 32) : row[j + u * 32];
+#pragma unroll
+  for (int u = 0; u < 8; ++u)
+    if (j + u * 32 < j1) acc0 = fma(v[u], x[j + u * 32], acc0);
+  return acc0 + acc1;
+}
+
+// Sums over the warp of four values at once: lane l returns the total of
+// value l / 8 (two exchanges halve the values held per lane, three more add up
+// the eight lanes that hold the same value).
+__device__ __forceinline__ double warp_sum4(double a0, double a1, double a2, double a3) {
+  const int lane = threadIdx.x & 31;
+  const bool hi = lane & 16, h8 = lane & 8;
+  double m0 = hi ? a2 : a0, m1 = hi ? a3 : a1;                 // kept: values 0, 1 or 2, 3
+  m0 += __shfl_xor_sync(0xffffffffu, hi ? a0 : a2, 16);
+  m1 += __shfl_xor_sync(0xffffffffu, hi ? a1 : a3, 16);
+  double m = (h8 ? m1 : m0) + __shfl_xor_sync(0xffffffffu, h8 ? m0 : m1, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+  return m;
+}
+
+// sum over t < j of o_i[t] c[t] + o_i[HP_NB + t] c[HP_NB + t] for the rows i0 .. i0 + 3
+// of `own` (below n_i), four per warp: lane l returns row i0 + l / 8's.
+__device__ __forceinline__ double own_products(const double *own, int i0, int n_i, int j, const double *c) {
+  const int lane = threadIdx.x & 31;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int t = lane; t < j; t += 32) {
+    const double c0 = c[t], c1 = c[HP_NB + t];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u < n_i) {
+        const double *o = own + (size_t)(i0 + u) * 2 * HP_NB + t;
+        acc[u] = fma(o[0], c0, fma(o[HP_NB], c1, acc[u]));
+      }
+  }
+  return warp_sum4(acc[0], acc[1], acc[2], acc[3]);
+}
+
+// tau, beta and sc of the reflector that maps (alpha, x') to (beta, 0), |x'|^2 =
+// sigma.  The square root and the reciprocal by Newton steps from the hardware's
+// estimates (each step squares the relative error; the last of each is a
+// residual correction), about a third of the IEEE routines' chain here; outside
+// the range where the squares are safe, those.
+__device__ __forceinline__ void reflector_scalars(double alpha, double sigma, double *tau, double *beta, double *sc) {
+  const double s = fma(alpha, alpha, sigma), aa = fabs(alpha);
+  if (sigma == 0.0) { *tau = 0.0; *beta = alpha; *sc = 0.0; return; }
+  double nrm, rinv, rden;
+  if (s > 1e-250 && s < 1e250) {
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(rinv) : "d"(s));
+#pragma unroll
+    for (int it = 0; it < 2; ++it) rinv = fma(0.5 * rinv, fma(-s * rinv, rinv, 1.0), rinv);
+    nrm = s * rinv;
+    nrm = fma(0.5 * rinv, fma(-nrm, nrm, s), nrm);
+    rinv = fma(rinv, fma(-nrm, rinv, 1.0), rinv);       // 1 / nrm
+    const double den = aa + nrm;
+    rden = recip_nr<2>(den);
+    rden = fma(rden, fma(-den, rden, 1.0), rden);
+  } else {
+    nrm = sqrt(s);
+    rinv = 1.0 / nrm;
+    rden = 1.0 / (aa + nrm);
+  }
+  *beta = alpha >= 0.0 ? -nrm : nrm;
+  *tau = fma(aa, rinv, 1.0);                            // (beta - alpha) / beta
+  *sc = alpha >= 0.0 ? rden : -rden;                    // 1 / (alpha - beta)
+}
+
+__global__ void __launch_bounds__(HP_THREADS, 1) hh_panel_kernel(HhPanelArgs g) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int n = g.n, G = gridDim.x, b = blockIdx.x, R = g.R;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int NW = HP_THREADS / 32, LAST = NW - 1;   // the last warp has the scalars
+  double *xs = reinterpret_cast<double *>(smem_raw);   // [n] column k
+  double *own = xs + n;                                // [R][2 HP_NB]: v_t[r], w_t[r]
+  __shared__ double ab[2 * HP_NB], rk[2 * HP_NB];      // b_t, a_t; w_t[k+1], v_t[k+1]
+  __shared__ double xo[HP_MAX_ROWS], ty[HP_MAX_ROWS], vo[HP_MAX_ROWS], qo[HP_MAX_ROWS], co[HP_MAX_ROWS];
+  __shared__ double seg_acc[HP_MAX_ROWS + NW], row_a1[HP_MAX_ROWS + 1], sig[HP_SIGMA_WARPS];
+  __shared__ double s_sc[4], s_vy, s_wk;               // tau, beta, sc, tau^2 / 2; v.Av; tau y_{k+1}
+  __shared__ int s_ok;
+  const int n_own = b < n ? (n - 1 - b) / G + 1 : 0;
+  unsigned bar = g.bar0;
+  unsigned long long wmax = 0ull;
+  if (warp == 0)
+    for (int lr = lane; lr < n_own; lr += 32) {
+      const int r = lr * G + b;
+      if (r >= g.k0) {
+        const double x = g.A[(int64_t)r * n + g.k0];
+        xo[lr] = x;
+        if (r > g.k0) g.xbuf[r] = x;
+        else g.d[r] = x;
+      }
+    }
+  for (int j = 0; j < HP_NB; ++j) {
+    const int k = g.k0 + j, par = j & 1;
+    const int lr1 = (k + 1 > b) ? (k + 1 - b + G - 1) / G : 0;   // first own row > k
+    const int nrow = n_own - lr1;
+    const double *xb = g.xbuf + (size_t)par * n;
+    double *part = g.part + (size_t)par * G, *dots = g.dots + par * 2 * HP_NB, *snext = g.snext + 2 * par;
+    // ---- barrier 1: x and the vectors of the step before are published
+    __syncthreads();
+    if (tid == 0) { grid_arrive(g.gb); s_ok = grid_wait(g.gb, bar, g.flags); }
+    ++bar;
+    __syncthreads();
+    if (!s_ok) return;
+    {
+      double t[4], rkv = 0.0;
+      // row k + 1 of the earlier vectors
+      if (tid < 2 * j) rkv = (tid & 1) ? __ldcg(g.V + (int64_t)(g.k0 + (tid >> 1)) * n + k + 1)
+                                       : __ldcg(g.W + (int64_t)(tid >> 1) * n + k + 1);
+      for (int c0 = k + 1 + tid; c0 < n; c0 += 4 * HP_THREADS) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (c0 + u * HP_THREADS < n) t[u] = __ldcg(xb + c0 + u * HP_THREADS);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (c0 + u * HP_THREADS < n) xs[c0 + u * HP_THREADS] = t[u];
+      }
+      if (tid < 2 * j) rk[(tid & 1) * HP_NB + (tid >> 1)] = rkv;
+    }
+    __syncthreads();
+    // ---- own rows' products with x, and one earlier vector's
+    const int ndot = b < 2 * j ? 1 : 0, tot = nrow + ndot;
+    const int S = max(1, LAST / tot);   // warps per row when rows are few
+    const int seglen = ((n - k - 1 + S - 1) / S + 31) & ~31;
+    if (warp >= NW - HP_SIGMA_WARPS) {   // sum of squares of x_{k+2 ..}
+      const int w4 = warp - (NW - HP_SIGMA_WARPS);
+      double s0 = 0.0;
+      for (int c = k + 2 + w4 * 32 + lane; c < n; c += 32 * HP_SIGMA_WARPS) s0 = fma(xs[c], xs[c], s0);
+      s0 = warp_sum_all(s0);
+      if (lane == 0) sig[w4] = s0;
+      if (warp != LAST) bar_arrive(1, 32 * HP_SIGMA_WARPS);
+    }
+    if (warp != LAST) {
+      for (int task = warp; task < tot * S; task += LAST) {
+        const int item = task / S, seg = task - item * S;
+        const int j0 = k + 1 + seg * seglen, j1 = min(n, j0 + seglen);
+        double acc;
+        if (item < nrow) {
+          const double *row = g.A + (int64_t)((lr1 + item) * G + b) * n;
+          acc = dot_pass<false>(row, j0, j1, xs);
+          if (seg == 0 && lane == 0) row_a1[item] = row[k + 1];
+        } else {
+          acc = dot_pass<true>((b & 1) ? g.W + (int64_t)(b >> 1) * n : g.V + (int64_t)(g.k0 + (b >> 1)) * n, j0, j1, xs);
+        }
+        acc = warp_sum_all(acc);
+        if (lane == 0) seg_acc[task] = acc;
+      }
+      bar_sync(2, 32 * LAST);
+      if (warp == 0) {
+        double T = 0.0;
+        for (int i = lane; i < nrow; i += 32) {
+          double S_r = seg_acc[i * S];
+          for (int q = 1; q < S; ++q) S_r += seg_acc[i * S + q];
+          seg_acc[i * S] = S_r;
+          T = fma(xo[lr1 + i], S_r, T);
+          if ((lr1 + i) * G + b == k + 1) { snext[0] = S_r; snext[1] = row_a1[i]; }
+        }
+        T = warp_sum_all(T);
+        if (lane == 0) part[b] = T;
+        bar_arrive(3, 64);   // the rows' sums are there
+        bar_sync(4, 64);     // warp 1's product is written
+        if (lane == 0) grid_arrive(g.gb);
+      } else if (warp == 1) {
+        if (lane == 0 && ndot) {
+          double S_t = seg_acc[nrow * S];
+          for (int q = 1; q < S; ++q) S_t += seg_acc[nrow * S + q];
+          dots[b] = S_t;
+        }
+        bar_arrive(4, 64);
+      }
+      // the own rows' column k + 1 without this step's update
+      for (int i0 = 4 * (warp - 1); warp > 0 && i0 < nrow; i0 += 4 * (LAST - 1)) {
+        const double q = own_products(own, lr1 + i0, lr1 + nrow, j, rk);
+        const int i = i0 + (lane >> 3);
+        if ((lane & 7) == 0 && i < nrow) qo[lr1 + i] = row_a1[i] - q;
+      }
+    } else {
+      bar_sync(1, 32 * HP_SIGMA_WARPS);
+      double tau, beta, sc;
+      reflector_scalars(xs[k + 1], (sig[0] + sig[1]) + (sig[2] + sig[3]), &tau, &beta, &sc);
+      if (lane == 0) {
+        s_sc[0] = tau; s_sc[1] = beta; s_sc[2] = sc; s_sc[3] = 0.5 * tau * tau;
+        if (b == 0) { g.e[k] = beta; g.tau[k] = tau; }
+      }
+      bar_sync(3, 64);
+      for (int i = lane; i < nrow; i += 32) {   // the own rows' v and tau y
+        const int lr = lr1 + i, r = lr * G + b;
+        const double v = r == k + 1 ? 1.0 : sc * xo[lr];
+        vo[lr] = v;
+        ty[lr] = tau * (sc * fma(-beta, row_a1[i], seg_acc[i * S]));
+        g.V[(int64_t)k * n + r] = v;
+      }
+    }
+    __syncthreads();
+    const double tau = s_sc[0], beta = s_sc[1], sc = s_sc[2];
+    // ---- barrier 2
+    if (tid == 0) s_ok = grid_wait(g.gb, bar, g.flags);
+    ++bar;
+    __syncthreads();
+    if (!s_ok) return;
+    if (tid < 2 * j) {   // a_t = sc (v_t.x - beta v_t[k+1]), b_t likewise: ab = (b_t | a_t)
+      const int odd = tid & 1, t = tid >> 1;
+      ab[(odd ^ 1) * HP_NB + t] = sc * fma(-beta, rk[(odd ^ 1) * HP_NB + t], __ldcg(dots + tid));
+    }
+    if (warp == LAST) {
+      double t[5], T = 0.0;
+      const double S1 = __ldcg(snext), a11 = __ldcg(snext + 1);
+      for (int q0 = lane; q0 < G; q0 += 5 * 32) {
+#pragma unroll
+        for (int u = 0; u < 5; ++u) t[u] = q0 + u * 32 < G ? __ldcg(part + q0 + u * 32) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 5; ++u) T += t[u];
+      }
+      T = warp_sum_all(T);
+      if (lane == 0) {
+        s_vy = sc * sc * fma(beta, fma(beta, a11, -2.0 * S1), T);
+        s_wk = tau * (sc * fma(-beta, a11, S1));
+      }
+    }
+    __syncthreads();
+    double abs_ = 0.0, c1 = 0.0;
+    if (warp == 0) {   // sum a_t b_t and row k + 1's correction, in warp 0
+      for (int t = lane; t < j; t += 32) {
+        abs_ = fma(ab[t], ab[HP_NB + t], abs_);
+        c1 = fma(rk[HP_NB + t], ab[t], fma(rk[t], ab[HP_NB + t], c1));   // v_t[k+1] b_t + w_t[k+1] a_t
+      }
+      const double m = warp_sum4(abs_, c1, 0.0, 0.0);
+      abs_ = __shfl_sync(0xffffffffu, m, 0);
+      c1 = __shfl_sync(0xffffffffu, m, 8);
+    } else {
+      for (int i0 = 4 * (warp - 1); i0 < nrow; i0 += 4 * (NW - 1)) {
+        const double c = own_products(own, lr1 + i0, lr1 + nrow, j, ab);
+        if ((lane & 7) == 0 && i0 + (lane >> 3) < nrow) co[lr1 + i0 + (lane >> 3)] = c;
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {   // w, and column k + 1 of the own rows
+      const double gam = s_sc[3] * fma(-2.0, abs_, s_vy);
+      const double wk1 = fma(-tau, c1, s_wk) - gam;
+      for (int i = lane; i < nrow; i += 32) {
+        const int lr = lr1 + i, r = lr * G + b;
+        const double v = vo[lr], w = fma(-gam, v, fma(-tau, co[lr], ty[lr]));
+        const double x = fma(-v, wk1, qo[lr]) - w;
+        if (r > k + 1) g.xbuf[(size_t)(par ^ 1) * n + r] = x;
+        else g.d[r] = x;
+        own[(size_t)lr * 2 * HP_NB + j] = v;
+        own[(size_t)lr * 2 * HP_NB + HP_NB + j] = w;
+        g.W[(int64_t)j * n + r] = w;
+        xo[lr] = x;
+        wmax = max(wmax, (unsigned long long)__double_as_longlong(w) & 0x7fffffffffffffffull);
+      }
+    }
+  }
+  if (warp == 0) {
+    for (int o = 16; o > 0; o >>= 1) wmax = max(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
+    if (lane == 0 && wmax) atomicMax(g.wmax, wmax);
+  }
 }
 
 // |a| < |b| on the integer pipe (finite doubles: magnitude order = bit order)
@@ -1045,11 +1409,13 @@ cudaError_t allow_max_dynamic_smem(const void *kernel, std::once_flag &flag) {
   });
   return result;
 }
-std::once_flag g_smem_hh[2], g_smem_bisect, g_smem_invit[2], g_smem_bounds, g_smem_wy, g_smem_wa;
+std::once_flag g_smem_hh, g_smem_hp, g_smem_bisect, g_smem_invit[2], g_smem_bounds, g_smem_wy, g_smem_wa;
 
-// Try the fused reduction in arithmetic T; false when it cannot be launched.
+// Try the fused reduction of the trailing block from row and column k0 on in
+// arithmetic T; false when it cannot be launched.
 template <typename T>
-bool launch_fused(EigWork &w, int n, cudaStream_t s, int *launches, cudaError_t *err) {
+bool launch_fused(EigWork &w, int n_all, int k0, cudaStream_t s, int *launches, cudaError_t *err) {
+  const int n = n_all - k0;
   int dev = 0, nsm = 0, coop = 0, optin = 0;
   *err = cudaSuccess;
   bool ok = n > 2 && w.grid_ws != nullptr && cudaGetDevice(&dev) == cudaSuccess &&
@@ -1061,25 +1427,23 @@ bool launch_fused(EigWork &w, int n, cudaStream_t s, int *launches, cudaError_t 
   const int G = std::min(nsm, std::max(1, (n + HH_MIN_ROWS - 1) / HH_MIN_ROWS));
   const int R = (n + G - 1) / G;
   const size_t reserve = 1024;   // static shared memory of the kernel
-  const size_t s_rows = (size_t)(3 + R) * n * sizeof(T), s_vec = (size_t)3 * n * sizeof(T);
-  const bool in_smem = s_rows + reserve <= (size_t)optin;
-  const size_t smem = in_smem ? s_rows : s_vec;
+  const size_t smem = (size_t)(3 + R) * n * sizeof(T);
   if (smem + reserve > (size_t)optin) return false;
-  const int fi = in_smem ? 1 : 0;
-  const void *kern = in_smem ? (const void *)hh_fused_kernel<T, true> : (const void *)hh_fused_kernel<T, false>;
+  const void *kern = (const void *)hh_fused_kernel<T>;
   int per_sm = 0;
-  ok = allow_max_dynamic_smem(kern, g_smem_hh[fi]) == cudaSuccess &&
+  ok = allow_max_dynamic_smem(kern, g_smem_hh) == cudaSuccess &&
        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 512, smem) == cudaSuccess && per_sm >= 1;
   cudaGetLastError();
   if (!ok) return false;
   HhFusedArgs<T> g;
-  g.A0 = w.A;
-  g.A = w.A;   // reduced in place when the rows do not fit in shared memory
-  g.V = reinterpret_cast<T *>(w.V);
-  g.d = w.d; g.e = w.e; g.tau = w.tau;
+  const int64_t off = (int64_t)k0 * n_all + k0;
+  g.A0 = w.A + off;
+  g.V = reinterpret_cast<T *>(w.V) + off;
+  g.d = w.d + k0; g.e = w.e + k0; g.tau = w.tau + k0;
+  g.ld = n_all;
   g.P = reinterpret_cast<T *>(w.grid_ws);
   g.pub = g.P + 2 * (size_t)n;
-  double *after = w.grid_ws + (4 * (size_t)n * sizeof(T) + sizeof(double) - 1) / sizeof(double);
+  double *after = w.grid_ws + (4 * (size_t)n_all * sizeof(T) + sizeof(double) - 1) / sizeof(double);
   g.tail = after;
   g.gb = reinterpret_cast<GridBar *>(after + 2);
   g.flags = w.flags;
@@ -1090,6 +1454,88 @@ bool launch_fused(EigWork &w, int n, cudaStream_t s, int *launches, cudaError_t 
   *err = cudaLaunchCooperativeKernel(kern, dim3(G), dim3(512), args, smem, s);
   if (*err == cudaSuccess) *launches += 1;
   return true;
+}
+
+// Panels of the blocked reduction from the front, as long as they pay; *k0 is
+// the first column left to the fused kernel (0: none, or not available here).
+// The panel's arrays and digits live in the inverse-iteration scratch.
+// Sizes: measured at n = 900 both take 8.0 ms, n = 1100 10.3 against 10.8, n = 1800
+// 20.0 against 25.4, n = 3300 58.7 against 107 ms; leaving the last 800 columns to
+// the fused kernel is 0.1 to 0.5 ms better than 500, 0.6 better than 1100.
+constexpr int HP_MIN_N = 1000, HP_TAIL = 800;
+
+cudaError_t launch_blocked(EigWork &w, int n, cudaStream_t s, int *launches, int *k0_out) {
+  *k0_out = 0;
+  int dev = 0, nsm = 0, coop = 0, optin = 0, per_sm = 0;
+  bool ok = n >= HP_MIN_N && w.grid_ws != nullptr && w.flags != nullptr && cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
+            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess;
+  cudaGetLastError();
+  if (!ok) return cudaSuccess;
+  const int G = nsm, R = (n + G - 1) / G;
+  const size_t smem = ((size_t)n + (size_t)R * 2 * HP_NB) * sizeof(double);
+  ok = G >= 2 * HP_NB && R <= HP_MAX_ROWS && smem + 12 * 1024 <= (size_t)optin &&
+       allow_max_dynamic_smem((const void *)hh_panel_kernel, g_smem_hp) == cudaSuccess &&
+       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)hh_panel_kernel, HP_THREADS, smem) ==
+           cudaSuccess && per_sm >= 1;
+  cudaGetLastError();
+  if (!ok) return cudaSuccess;
+  // scratch: 5 n^2 doubles, of which this takes about (64 + 448) n + small
+  char *base = reinterpret_cast<char *>(w.lu);
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    void *p = base + off;
+    off += (bytes + 255) / 256 * 256;
+    return p;
+  };
+  const int n_panels_max = n / HP_NB + 1, nkb = 2 * HP_NB / SL_K, np = (int)slice_rows_padded(n);
+  HhPanelArgs a;
+  a.W = (double *)take((size_t)HP_NB * n * sizeof(double));
+  a.xbuf = (double *)take((size_t)2 * n * sizeof(double));
+  a.part = (double *)take((size_t)2 * G * sizeof(double));
+  a.dots = (double *)take((size_t)4 * HP_NB * sizeof(double));
+  a.snext = (double *)take(4 * sizeof(double));
+  const size_t zero0 = off;
+  a.gb = (GridBar *)take(sizeof(GridBar));
+  unsigned long long *wmax = (unsigned long long *)take((size_t)n_panels_max * sizeof(unsigned long long));
+  const size_t zero1 = off;
+  SlicePairSrc ps;
+  const int64_t dig = slice_digit_bytes(n, nkb, 7);
+  ps.dig_p = (uint8_t *)take(dig);
+  ps.dig_q = (uint8_t *)take(dig);
+  ps.exp_p = (int *)take((size_t)np * sizeof(int));
+  ps.exp_q = (int *)take((size_t)np * sizeof(int));
+  if (off > (size_t)5 * n * n * sizeof(double)) return cudaSuccess;
+  a.A = w.A; a.V = w.V; a.d = w.d; a.e = w.e; a.tau = w.tau;
+  a.flags = w.flags; a.n = n; a.R = R; a.bar0 = 0;
+  cudaError_t e = cudaMemsetAsync(base + zero0, 0, zero1 - zero0, s);
+  if (e != cudaSuccess) return e;
+  int k0 = 0;
+  for (int q = 0; n - k0 >= HP_TAIL + HP_NB; ++q, k0 += HP_NB) {
+    a.k0 = k0;
+    a.wmax = wmax + q;
+    void *args[] = {&a};
+    e = cudaLaunchCooperativeKernel((const void *)hh_panel_kernel, dim3(G), dim3(HP_THREADS), args, smem, s);
+    if (e != cudaSuccess) return e;
+    a.bar0 += 2 * HP_NB;
+    // A22 -= V W^T + W V^T on the rows and columns past the panel
+    const int k1 = k0 + HP_NB, m = n - k1;
+    ps.X = w.V + (int64_t)k0 * n + k1; ps.Y = a.W + k1; ps.ld = n; ps.nk = HP_NB;
+    ps.rows = m; ps.rows_p = (int)slice_rows_padded(m); ps.ymax = a.wmax;
+    e = launch_slice_pair(ps, s);
+    if (e != cudaSuccess) return e;
+    SliceGemmArgs g;
+    g.A = ps.dig_p; g.ea = ps.exp_p; g.B = ps.dig_q; g.eb = ps.exp_q; g.nkb = nkb;
+    g.M = g.N = m; g.sym = 1; g.C = w.A + (int64_t)k1 * n + k1; g.ldc = n; g.beta = 1.0; g.alpha_neg = 1;
+    g.err = w.flags;
+    slice_gemm_plan(&g, nsm, 0);
+    e = launch_slice_gemm(g, nsm, s);
+    if (e != cudaSuccess) return e;
+    *launches += 4;
+  }
+  *k0_out = k0;
+  return cudaSuccess;
 }
 
 // Steps 3-6 in arithmetic T.
@@ -1292,8 +1738,12 @@ cudaError_t eig_vectors_impl(EigWork &w, int n, int k, double *Ut, int *flags, c
 
 cudaError_t launch_eig_tridiag(EigWork &w, int n, double thresh, cudaStream_t s, int *launches) {
   cudaError_t e = cudaSuccess;
-  const bool fused = launch_fused<double>(w, n, s, launches, &e);
+  int k0 = 0;
+  e = launch_blocked(w, n, s, launches, &k0);
   if (e != cudaSuccess) return e;
+  const bool fused = launch_fused<double>(w, n, k0, s, launches, &e);
+  if (e != cudaSuccess) return e;
+  if (!fused && k0 > 0) return cudaErrorNotSupported;   // not reached: the tail's rows fit in shared memory
   if (!fused) {
     for (int k = 0; k + 2 < n; ++k) {
       const int L = n - k - 1;

@@ -210,6 +210,21 @@ struct SliceSrc {
 // ns digits of `bits` bits: (2 .. 8, 7) or (7, 8).
 cudaError_t launch_slice_operand(const SliceSrc &a, int ns, int bits, int batch, cudaStream_t s);
 
+// Digits (7 in base 256) of the operands of X Y^T + Y X^T, X and Y given by
+// columns: X[k][r], Y[k][r], k < nk <= 64 (row stride ld), r < rows.  P's row r
+// is (X[.][r], 2^c Y[.][r]), Q's (2^c Y[.][r], X[.][r]) with 2^c Y's largest
+// magnitude (bits *ymax) just below 1; exp_p carries -c, so the product of P
+// and Q needs no further scale.
+struct SlicePairSrc {
+  const double *X = nullptr, *Y = nullptr;
+  int64_t ld = 0;
+  int nk = 0, rows = 0, rows_p = 0;   // nk a multiple of 16; 2 nk / 16 blocks of 16 k
+  const unsigned long long *ymax = nullptr;
+  uint8_t *dig_p = nullptr, *dig_q = nullptr;
+  int *exp_p = nullptr, *exp_q = nullptr;
+};
+cudaError_t launch_slice_pair(const SlicePairSrc &a, cudaStream_t s);
+
 // C_b[n][m] = beta C_b[n][m] + (-1)^alpha_neg 2^alpha_exp sum_k A_b[m][k] B_b[n][k] from
 // digits, m < M, n < N, one rounding per output before the sum with C; sym
 // (B = A): the entries m >= n, mirrored to the others where `mirror` is set or

@@ -781,6 +781,46 @@ __global__ void __launch_bounds__(256) slice_cols_tiles_kernel(SliceSrc a) {
     }
 }
 
+// One block per 64 rows, one thread per row and 16 k: both operands of a
+// symmetric rank-2 nk update in one pass.
+__global__ void __launch_bounds__(512) slice_pair_kernel(SlicePairSrc a) {
+  __shared__ unsigned long long red[8][SL_ROWS];
+  constexpr int NS = 7, BITS = 8;
+  const int rl = threadIdx.x & 63, kb = threadIdx.x >> 6, half = a.nk / SL_K, nkb = 2 * half;
+  const int r = blockIdx.x * SL_ROWS + rl;
+  const unsigned long long yb = *a.ymax;
+  const int c = yb ? max(-1000, min(1000, 1022 - (int)(yb >> 52))) : 0;   // |Y| 2^c < 1
+  const double f = __longlong_as_double((long long)(1023 + c) << 52);
+  double v[2][8];
+  unsigned long long mb = 0ull;
+  if (kb < nkb) {
+    const bool y = kb >= half;
+    const double *src = (y ? a.Y + (int64_t)(kb - half) * SL_K * a.ld : a.X + (int64_t)kb * SL_K * a.ld) + r;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      double t = r < a.rows ? src[(int64_t)q * a.ld] : 0.0;
+      if (y) t *= f;
+      v[q >> 3][q & 7] = t;
+      mb = max(mb, mag_bits(t));
+    }
+    red[kb][rl] = mb;
+  }
+  __syncthreads();
+  if (kb >= nkb) return;
+  for (int q = 0; q < nkb; ++q) mb = max(mb, red[q][rl]);
+  const int e = slice_exponent(mb, BITS);
+  const int kq = kb >= half ? kb - half : kb + half;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    store_digits<NS, BITS>(v[h], e, digit_chunk<NS>(a.dig_p, r, 2 * kb + h, nkb));
+    store_digits<NS, BITS>(v[h], e, digit_chunk<NS>(a.dig_q, r, 2 * kq + h, nkb));
+  }
+  if (kb == 0) {
+    a.exp_q[r] = e;
+    a.exp_p[r] = (e == SL_ZERO || e >= SL_NONFINITE) ? e : e - c;
+  }
+}
+
 __global__ void fill_int_kernel(int *p, int64_t n, int v) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = v;
 }
@@ -853,6 +893,12 @@ cudaError_t launch_slice_operand(const SliceSrc &a, int ns, int bits, int batch,
     case 8: return slice_operand<8, 7>(a, batch, s);
   }
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_slice_pair(const SlicePairSrc &a, cudaStream_t s) {
+  if (a.rows < 1 || a.rows > a.rows_p || a.rows_p % 128 || a.nk < SL_K || a.nk > 64 || a.nk % SL_K) return cudaErrorInvalidValue;
+  slice_pair_kernel<<<a.rows_p / SL_ROWS, 512, 0, s>>>(a);
+  return cudaGetLastError();
 }
 
 void slice_gemm_tiles(SliceGemmArgs *g) {

@@ -15,7 +15,7 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-U = 2.0 ** -53
+U = U_ROUND = 2.0 ** -53
 
 
 @pytest.fixture(scope="module")
@@ -131,3 +131,27 @@ def test_screen_digits_matches_inverse(ctx, N, J):
     with pytest.raises(ltgw.LtgwError) as e:
         ctx.screen(torch.from_numpy(Pi).cuda(), C)
     assert e.value.status == ltgw.LTGW_ERR_NOT_SPD
+
+
+# the blocked reduction: its smallest size, one panel and several, remainders
+# on both sides of a panel; a metric of rank 70 (reflectors of a zero column)
+@pytest.mark.parametrize("n,pairs", [(1000, 3000), (1001, 2002), (1063, 2126), (1129, 2258), (1003, 70)])
+def test_naf_blocked_reduction(ctx, n, pairs):
+    """Residual, orthonormality and eigenvalues of the kept pairs: the reduction
+    and the vectors are backward stable to n u |K| each (32 n u with the
+    constants of two-sided reflectors and the panel's sums)."""
+    rng = np.random.default_rng(n)
+    B = rng.standard_normal((n, pairs)) / np.sqrt(pairs) * np.exp(-3.0 * np.arange(n) / n)[:, None]
+    K = B @ B.T
+    ref = np.sort(np.linalg.eigvalsh(K))[::-1]
+    m = int(np.argmax(ref[20:60] - ref[21:61])) + 20
+    thr = 0.5 * (ref[m] + ref[m + 1])
+    Ut = torch.zeros((n, n), dtype=torch.float64, device="cuda")
+    lam = torch.zeros(n, dtype=torch.float64, device="cuda")
+    k = ctx.naf_basis(torch.from_numpy(B).cuda(), pairs, pairs, thr, Ut, lam)
+    assert k == m + 1
+    U, lg = Ut[:k].cpu().numpy().T, lam[:k].cpu().numpy()
+    tol = 32 * n * U_ROUND * ref[0]
+    assert np.abs(lg - ref[:k]).max() <= tol
+    assert np.linalg.norm(K @ U - U * lg[None, :], axis=0).max() <= tol
+    assert np.abs(U.T @ U - np.eye(k)).max() <= 32 * n * U_ROUND
