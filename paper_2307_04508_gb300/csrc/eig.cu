@@ -1538,6 +1538,125 @@ cudaError_t launch_blocked(EigWork &w, int n, cudaStream_t s, int *launches, int
   return cudaSuccess;
 }
 
+// ---- the eigenvectors' dense products from digits (slice_gemm.cu) ----
+// From VD_MIN_N on: the re-orthonormalisation X (3 - X^T X) / 2 and the compact-WY
+// blocks.  The vectors' columns have unit length all along, so their digits
+// take one fixed exponent (2^-56 beside the entries of a column of length 1; the
+// FP64 sums round at about that) and need no pass for the maxima.
+// V's digits are formed once; per block of 64 reflectors (last to first, rows
+// r > 64 b): the vectors' digits, W1 = V_b Y, its digits, Y -= M_b W1.
+// Measured (bisection to the transposition; a quarter of the vectors kept): n = 3300
+// 46.7 -> 22.7 ms, n = 1800 13.1 -> 9.7, n = 800 4.16 -> 3.81, n = 264 1.56 -> 1.43; the blocks
+// alone took 21.9 ms of FP64 tiles at n = 3300 and 1.5 from digits.  All eight
+// levels of digit pairs are kept: with seven the vectors' orthogonality falls
+// from 2e-15 to 2e-14 (V's rows hold a 1 beside entries of 1/sqrt(n), so their
+// scale is far above what the sums carry); with eight it is the FP64 form's.
+constexpr int VD_MIN_N = 200;
+constexpr int VD_EXP = 2;   // |x| < 2: stored exponents carry one more bit in base 256
+
+struct VecDigits {
+  int n, k, nsm;
+  int np, kp, nkb;        // padded rows, 16-k blocks of length n
+  uint8_t *dV, *dY, *dM, *dW;
+  int *eV, *eY, *eM, *eW;
+  int *flags;
+  size_t bytes;
+};
+
+// Arrays in `base` (counted only when base is null).
+VecDigits vec_digits(int n, int k, int nsm, int *flags, void *base) {
+  VecDigits d;
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    uint8_t *p = base ? (uint8_t *)base + off : nullptr;
+    off += (bytes + 255) / 256 * 256;
+    return p;
+  };
+  d.n = n; d.k = k; d.nsm = nsm; d.flags = flags;
+  d.np = (int)slice_rows_padded(n); d.kp = (int)slice_rows_padded(k);
+  d.nkb = (n + SL_K - 1) / SL_K;
+  d.dV = take(slice_digit_bytes(n, d.nkb, 7));    // V's rows; before that X's rows (K = k) and F's
+  d.dY = take(slice_digit_bytes(k, d.nkb, 7));    // the vectors' columns (K = n)
+  d.dM = take(slice_digit_bytes(n, WY_NB / SL_K, 7));
+  d.dW = take(slice_digit_bytes(k, std::max(WY_NB / SL_K, (k + SL_K - 1) / SL_K), 7));
+  d.eV = (int *)take(d.np * sizeof(int));
+  d.eY = (int *)take(d.kp * sizeof(int));
+  d.eM = (int *)take(d.np * sizeof(int));
+  d.eW = (int *)take(d.kp * sizeof(int));
+  d.bytes = off;
+  return d;
+}
+
+SliceSrc digit_rows(const double *X, int64_t ld, int rows, int64_t K, uint8_t *dig, int *exps) {
+  SliceSrc a;
+  a.X = X; a.ld = ld; a.rows = rows; a.rows_p = (int)slice_rows_padded(rows); a.K = K; a.nkb = (int)((K + SL_K - 1) / SL_K);
+  a.dig = dig; a.exps = exps; a.exp_batch = a.rows_p;
+  return a;
+}
+
+// Digits of the vectors' columns (X [n][k]) from row 16 kb_first on.
+cudaError_t slice_vectors(const VecDigits &d, const double *X, int kb_first, cudaStream_t s) {
+  SliceSrc a = digit_rows(X, d.k, d.k, d.n, d.dY, d.eY);
+  a.cols = 1; a.fixed_exp = VD_EXP; a.kb_first = kb_first;
+  return launch_slice_operand(a, 7, 8, 1, s);
+}
+
+cudaError_t run_slice(SliceGemmArgs &g, const VecDigits &d, double *partial, size_t partial_bytes, cudaStream_t s) {
+  g.err = d.flags;
+  g.levels = 8;
+  const size_t need = slice_gemm_plan(&g, d.nsm, partial_bytes);
+  g.partial = need ? partial : nullptr;
+  return launch_slice_gemm(g, d.nsm, s);
+}
+
+// X <- X (3 - X^T X) / 2 in place; G, Xn: k x k and n x k scratch.
+cudaError_t lowdin_digits(const VecDigits &d, double *X, double *G, double *Xn, double *partial, size_t partial_bytes,
+                          cudaStream_t s) {
+  const int n = d.n, k = d.k;
+  cudaError_t e = slice_vectors(d, X, 0, s);
+  if (e != cudaSuccess) return e;
+  SliceGemmArgs g;   // G = X^T X
+  g.A = g.B = d.dY; g.ea = g.eb = d.eY; g.nkb = d.nkb; g.M = g.N = k; g.sym = 1; g.C = G; g.ldc = k;
+  if ((e = run_slice(g, d, partial, partial_bytes, s)) != cudaSuccess) return e;
+  lowdin_factor_kernel<double><<<152, 256, 0, s>>>(G, k);
+  if ((e = launch_slice_operand(digit_rows(G, k, k, k, d.dW, d.eW), 7, 8, 1, s)) != cudaSuccess) return e;
+  if ((e = launch_slice_operand(digit_rows(X, k, n, k, d.dV, d.eV), 7, 8, 1, s)) != cudaSuccess) return e;
+  SliceGemmArgs h;   // Xn[r][c] = sum F[c][j] X[r][j] (F symmetric)
+  h.A = d.dW; h.ea = d.eW; h.B = d.dV; h.eb = d.eV; h.nkb = (k + SL_K - 1) / SL_K; h.M = k; h.N = n; h.C = Xn; h.ldc = k;
+  if ((e = run_slice(h, d, partial, partial_bytes, s)) != cudaSuccess) return e;
+  return cudaMemcpyAsync(X, Xn, (size_t)n * k * sizeof(double), cudaMemcpyDeviceToDevice, s);
+}
+
+// Every block Y <- Y - M_b (V_b Y), last to first; W1: 64 x k scratch.
+cudaError_t wy_digits(const VecDigits &d, const double *V, const double *Mall, int nblk, double *Y, double *W1,
+                      double *partial, size_t partial_bytes, cudaStream_t s, int *launches) {
+  const int n = d.n, k = d.k;
+  cudaError_t e = launch_slice_operand(digit_rows(V, n, n, n, d.dV, d.eV), 7, 8, 1, s);
+  if (e != cudaSuccess) return e;
+  for (int b = nblk - 1; b >= 0; --b) {
+    const int j0 = b * WY_NB, nb = std::min(WY_NB, n - 2 - j0), kb0 = j0 / SL_K;
+    if ((e = slice_vectors(d, Y, kb0, s)) != cudaSuccess) return e;
+    SliceGemmArgs g;   // W1[i][c] = sum_r V[j0 + i][r] Y[r][c]
+    g.A = d.dY; g.ea = d.eY;
+    g.B = d.dV + (int64_t)b * d.nkb * (SL_ROWS * SL_K * 2 * 7); g.eb = d.eV + j0;
+    g.nkb = d.nkb; g.kb_first = kb0; g.M = k; g.N = nb; g.C = W1; g.ldc = k;
+    if ((e = run_slice(g, d, partial, partial_bytes, s)) != cudaSuccess) return e;
+    SliceSrc w = digit_rows(W1, k, k, nb, d.dW, d.eW);
+    w.cols = 1;
+    if ((e = launch_slice_operand(w, 7, 8, 1, s)) != cudaSuccess) return e;
+    const int rows = n - 1 - j0;   // M_b's rows j0 .. n - 2 stand for Y's rows j0 + 1 ..
+    if ((e = launch_slice_operand(digit_rows(Mall + ((int64_t)b * (n - 1) + j0) * WY_NB, WY_NB, rows, nb, d.dM, d.eM), 7,
+                                  8, 1, s)) != cudaSuccess)
+      return e;
+    SliceGemmArgs u;   // Y[j0 + 1 + r][c] -= sum_i M_b[j0 + r][i] W1[i][c]
+    u.A = d.dW; u.ea = d.eW; u.B = d.dM; u.eb = d.eM; u.nkb = (nb + SL_K - 1) / SL_K;
+    u.M = k; u.N = rows; u.C = Y + (int64_t)(j0 + 1) * k; u.ldc = k; u.beta = 1.0; u.alpha_neg = 1;
+    if ((e = run_slice(u, d, nullptr, 0, s)) != cudaSuccess) return e;
+    *launches += 8;
+  }
+  return cudaSuccess;
+}
+
 // Steps 3-6 in arithmetic T.
 template <typename T>
 cudaError_t eig_vectors_impl(EigWork &w, int n, int k, double *Ut, int *flags, cudaStream_t s, int *launches) {
@@ -1600,7 +1719,28 @@ cudaError_t eig_vectors_impl(EigWork &w, int n, int k, double *Ut, int *flags, c
   // milliseconds.
   T *G = lu;                       // k*k scratch (inverse-iteration scratch is free now)
   T *Xn = lu + (int64_t)k * k;     // n*k scratch
-  {
+  // digits where the vectors are large enough and the scratch holds them: the
+  // factor F and X F first, then the digits (5 n^2 doubles in all)
+  VecDigits vd{};
+  bool digits = false;
+  double *vd_part = w.wy;
+  const size_t vd_part_bytes = (size_t)w.wy_r0 * sizeof(double);
+  if (n >= VD_MIN_N) {
+    int dev = 0, nsm = 0;
+    digits = cudaGetDevice(&dev) == cudaSuccess &&
+             cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+    cudaGetLastError();
+    const size_t head = (((size_t)k * k + (size_t)n * k) * sizeof(double) + 255) / 256 * 256;
+    vd = vec_digits(n, k, nsm, flags, (char *)w.lu + head);
+    digits = digits && head + vd.bytes <= (size_t)5 * n * n * sizeof(double);
+  }
+  if (digits) {
+    if ((e = launch_fill_int(vd.eY, vd.kp, VD_EXP, s)) != cudaSuccess) return e;
+    e = lowdin_digits(vd, reinterpret_cast<double *>(X), reinterpret_cast<double *>(G), reinterpret_cast<double *>(Xn),
+                      vd_part, vd_part_bytes, s);
+    if (e != cudaSuccess) return e;
+    *launches += 14;
+  } else {
     T *Gpart = Xn + (int64_t)n * k;
     const int64_t room = 5 * (int64_t)n * n - (int64_t)k * k - (int64_t)n * k;
     int nsp = (int)std::min<int64_t>((n + 63) / 64, std::max<int64_t>(1, room / ((int64_t)k * k)));
@@ -1667,10 +1807,17 @@ cudaError_t eig_vectors_impl(EigWork &w, int n, int k, double *Ut, int *flags, c
       if (e != cudaSuccess) return e;
     }
     *launches += 2;
-    // the blocks applied by one cooperative kernel when its CTAs fit at once
-    // and region 0 holds their partials; otherwise two GEMMs per block
+    // the blocks applied from digits; or by one cooperative kernel when its CTAs
+    // fit at once and region 0 holds their partials; otherwise two GEMMs per block
     bool applied = false;
-    if (sizeof(T) == sizeof(double)) {
+    if (digits) {
+      const size_t w1 = ((size_t)WY_NB * k + 31) / 32 * 32;   // W1 in front of the partials
+      e = wy_digits(vd, reinterpret_cast<const double *>(V), reinterpret_cast<const double *>(Mall), nblk,
+                    reinterpret_cast<double *>(X), w.wy, w.wy + w1, vd_part_bytes - w1 * sizeof(double), s, launches);
+      if (e != cudaSuccess) return e;
+      applied = true;
+    }
+    if (!applied && sizeof(T) == sizeof(double)) {
       int dev = 0, nsm = 0, coop = 0, per_sm = 0;
       const int S = (k + 63) / 64;
       if (cudaGetDevice(&dev) == cudaSuccess &&

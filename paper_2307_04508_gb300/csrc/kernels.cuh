@@ -200,6 +200,10 @@ struct SliceSrc {
   int rows = 0, rows_p = 0;    // operand rows, padded to 128
   int64_t K = 0;
   int nkb = 0;                 // 16-k blocks held (>= ceil(K / 16))
+  int kb_first = 0;            // digits are formed from this 16-k block on
+  // cols only, not 0: every column's exponent (the caller knows |x| < 2^(fixed_exp - 1)),
+  // exps filled beforehand (launch_fill_int) and no pass for the maximum
+  int fixed_exp = 0;
   const double *colscale = nullptr;   // rows only: factor of column k (one FP64 product), [batch][K] or shared
   int64_t cs_batch = 0;
   uint8_t *dig = nullptr;      // [batch] x dig_batch bytes
@@ -209,6 +213,7 @@ struct SliceSrc {
 };
 // ns digits of `bits` bits: (2 .. 8, 7) or (7, 8).
 cudaError_t launch_slice_operand(const SliceSrc &a, int ns, int bits, int batch, cudaStream_t s);
+cudaError_t launch_fill_int(int *p, int64_t n, int v, cudaStream_t s);
 
 // Digits (7 in base 256) of the operands of X Y^T + Y X^T, X and Y given by
 // columns: X[k][r], Y[k][r], k < nk <= 64 (row stride ld), r < rows.  P's row r
@@ -239,6 +244,8 @@ struct SliceGemmArgs {
   const int *ea = nullptr, *eb = nullptr;
   int64_t ea_batch = 0, eb_batch = 0;    // ints
   int ns = 7, bits = 8, nkb = 0, batch = 1;
+  int kb_first = 0;                      // contract the 16-k blocks [kb_first, nkb)
+  int levels = 0;                        // levels of digit pairs kept, ns or (base 256) ns + 1; 0: by the length
   int M = 0, N = 0, sym = 0, mirror = 1;
   double *C = nullptr;
   int64_t ldc = 0, c_batch = 0;

@@ -5,7 +5,9 @@
 // NS balanced digits a_1 .. a_NS in base 2^b (a BF16 value holds an integer of
 // up to 8 bits exactly), and
 //
-//   D = sum_{i + j <= NS + 1} 2^(-b (i + j)) (a_i b_j^T) 2^(e_A + e_B).
+//   D = sum_{i + j <= NL + 1} 2^(-b (i + j)) (a_i b_j^T) 2^(e_A + e_B),
+//
+// NL = NS levels, or (base 256, short contractions) NS + 1.
 //
 // All digit pairs of one level i + j add into ONE accumulator: the products
 // are integers, and their FP32 sums stay exact below 2^24, which bounds the
@@ -19,11 +21,11 @@
 // for one A digit i the digits 1 .. NS + 1 - i of B are ONE operand of
 // N = 64 (NS + 1 - i) rows whose products fall into consecutive level columns
 // of tensor memory: 10 MMA instructions of N = 64 .. 256 per 16 of K instead of
-// 28 of N = 64, each A tile read from shared memory at most twice (N = 64
+// 28 of N = 64 (NL = 7), each A tile read from shared memory at most twice (N = 64
 // MMAs would be bound by the A operand's shared-memory reads).
 //
-// Accumulators: NS x 64 columns of 128 lanes (448 of the 512 TMEM columns for
-// NS = 7).  Sixteen epilogue warps add each drain into two 64-bit integers per
+// Accumulators: NL x 64 columns of 128 lanes (448 or all of the 512 TMEM
+// columns for NS = 7).  Sixteen epilogue warps add each drain into two 64-bit integers per
 // output element (the four lowest levels; the others), exact over the whole
 // contraction, release the accumulators, and only then turn the sum into FP64 (one
 // rounding), while the next tile's MMAs run.  The conversion is integer code:
@@ -106,19 +108,22 @@ __device__ __forceinline__ void sg_mma(uint32_t d, uint64_t a, uint64_t b, uint3
 }
 
 // The MMAs of one 16-k block in two parts: the upper levels (0-based LO ..
-// NS - 1) and the lower ones (0 .. LO - 1).  A digit i meets the B digits
-// j0 .. j1 that land in the part; i = 0 comes first: with acc = 0 its MMAs
-// overwrite every level of the part.
-template <int NS> struct SgLevels { static constexpr int LO = NS > 4 ? (NS + 1) / 2 : NS / 2; };
+// NL - 1) and the lower ones (0 .. LO - 1).  A digit i meets the B digits
+// j0 .. j1 that land in the part.  The digit that reaches every level of the part
+// comes first: with acc = 0 its MMAs overwrite them (digit 0; with NL = NS + 1
+// levels digit 1 for the upper part, as digit 0 ends at level NS - 1).
+template <int NL> struct SgLevels { static constexpr int LO = NL > 4 ? (NL + 1) / 2 : NL / 2; };
 
-template <int NS, bool UPPER>
+template <int NS, int NL, bool UPPER>
 __device__ __forceinline__ void sg_part(uint32_t tmem, uint64_t a0, uint64_t b0, uint32_t acc) {
-  constexpr int L0 = UPPER ? SgLevels<NS>::LO : 0, L1 = UPPER ? NS : SgLevels<NS>::LO;   // levels [L0, L1)
+  constexpr int L0 = UPPER ? SgLevels<NL>::LO : 0, L1 = UPPER ? NL : SgLevels<NL>::LO;   // levels [L0, L1)
+  constexpr int FIRST = UPPER && NL > NS ? 1 : 0;
 #pragma unroll
-  for (int i = 0; i < L1; ++i) {
-    const int j0 = L0 > i ? L0 - i : 0, nj = L1 - i - j0;   // at most four digits: N <= 256
+  for (int q = 0; q < (L1 < NS ? L1 : NS); ++q) {
+    const int i = q <= FIRST ? FIRST - q : q;
+    const int j0 = L0 > i ? L0 - i : 0, j1 = L1 - i < NS ? L1 - i : NS, nj = j1 - j0;   // at most four digits: N <= 256
     sg_mma(tmem + (i + j0) * SG_N, a0 + (uint64_t)(i * (2 * SG_DIG >> 4)), b0 + (uint64_t)(j0 * (SG_DIG >> 4)),
-           sg_idesc(nj * SG_N), i == 0 ? acc : 1u);
+           sg_idesc(nj * SG_N), q == 0 ? acc : 1u);
   }
 }
 
@@ -193,7 +198,7 @@ __device__ __forceinline__ double sg_value(long long hi, long long lo, int E, ui
 }
 
 // MMA issue of one part's levels (one thread).
-template <int NS, bool UPPER>
+template <int NS, int NL, bool UPPER>
 __device__ __forceinline__ void sg_issue(const SliceGemmArgs &g, uint8_t *smem, SgBars &bars, uint32_t tmem,
                                          int64_t n_units, int lane) {
   constexpr int ST = sg_stages(NS);
@@ -206,7 +211,7 @@ __device__ __forceinline__ void sg_issue(const SliceGemmArgs &g, uint8_t *smem, 
     for (int64_t u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
       const SgUnit w = sg_unit(g, u);
       if (!w.valid) continue;
-      const int kb0 = w.sp * g.kb_per_split, kb1 = min(g.nkb, kb0 + g.kb_per_split);
+      const int kb0 = g.kb_first + w.sp * g.kb_per_split, kb1 = min(g.nkb, kb0 + g.kb_per_split);
       for (int kb = kb0; kb < kb1 && ok; kb += g.drain_kb) {
         const int ke = min(kb1, kb + g.drain_kb);
         ok = mbar_wait(&bars.acc_empty[UPPER], pe, &bars.abort, g.err);
@@ -217,7 +222,7 @@ __device__ __forceinline__ void sg_issue(const SliceGemmArgs &g, uint8_t *smem, 
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;");
           const uint64_t a0 = d0 + (uint64_t)((js * STAGE) >> 4);
-          sg_part<NS, UPPER>(tmem, a0, a0 + (uint64_t)(A_BYTES >> 4), k == kb ? 0u : 1u);
+          sg_part<NS, NL, UPPER>(tmem, a0, a0 + (uint64_t)(A_BYTES >> 4), k == kb ? 0u : 1u);
           mma_commit(&bars.empty[js]);
           if (++js == ST) { js = 0; ps ^= 1; }
         }
@@ -231,7 +236,7 @@ __device__ __forceinline__ void sg_issue(const SliceGemmArgs &g, uint8_t *smem, 
   __syncwarp();
 }
 
-template <int NS, int BITS>
+template <int NS, int BITS, int NL>
 __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(SliceGemmArgs g) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -240,7 +245,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(SliceGemmArgs
   constexpr uint32_t STAGE = 3u * NS * SG_DIG;   // A digits (128 rows each), then B digits
   constexpr uint32_t A_BYTES = 2u * NS * SG_DIG;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int LO = SgLevels<NS>::LO;
+  constexpr int LO = SgLevels<NL>::LO;
   const int64_t n_units = (int64_t)g.batch * g.splits * g.n_tiles;
 
   if (threadIdx.x == 0) {
@@ -277,7 +282,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(SliceGemmArgs
     for (int64_t u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
       const SgUnit w = sg_unit(g, u);
       if (!w.valid) continue;
-      const int kb0 = w.sp * g.kb_per_split, kb1 = min(g.nkb, kb0 + g.kb_per_split);
+      const int kb0 = g.kb_first + w.sp * g.kb_per_split, kb1 = min(g.nkb, kb0 + g.kb_per_split);
       const uint8_t *src = lane == 0 ? Bsel + (int64_t)w.b * g.b_batch + (int64_t)w.J * g.nkb * (NS * SG_DIG)
                                      : g.A + (int64_t)w.b * g.a_batch +
                                            (int64_t)(2 * w.I + ah) * g.nkb * (NS * SG_DIG) + dig * SG_DIG;
@@ -296,24 +301,24 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(SliceGemmArgs
         mbar_wait(&bars.full[q % ST], (uint32_t)(q / ST) & 1, &bars.abort, g.err, false);
     __syncwarp();
   } else if (warp == 1) {
-    sg_issue<NS, false>(g, smem, bars, tmem, n_units, lane);
+    sg_issue<NS, NL, false>(g, smem, bars, tmem, n_units, lane);
   } else if (warp == 2) {
-    sg_issue<NS, true>(g, smem, bars, tmem, n_units, lane);
+    sg_issue<NS, NL, true>(g, smem, bars, tmem, n_units, lane);
   } else {
     // ---------------------------------------------------------------- epilogue
     const int ew = warp & 3;              // TMEM lane quarter this warp may read
     const int cq = (warp - SG_EPI0) >> 2;       // columns cq * 16 .. + 15 of every level
     const uint32_t tbase = tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)(cq * SG_CW);
-    constexpr int HS = NS > 4 ? 4 * BITS : 0;   // weight of the upper sum
+    constexpr int HS = NL > 4 ? 4 * BITS : 0;   // weight of the upper sum
     uint32_t pf = 0;
     bool ok = true;
     for (int64_t u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
       const SgUnit w = sg_unit(g, u);
       if (!w.valid) continue;
-      const int kb0 = w.sp * g.kb_per_split, kb1 = min(g.nkb, kb0 + g.kb_per_split);
-      long long lo[SG_CW], hi[NS > 4 ? SG_CW : 1];
+      const int kb0 = g.kb_first + w.sp * g.kb_per_split, kb1 = min(g.nkb, kb0 + g.kb_per_split);
+      long long lo[SG_CW], hi[NL > 4 ? SG_CW : 1];
 #pragma unroll
-      for (int q = 0; q < SG_CW; ++q) { lo[q] = 0; if (NS > 4) hi[NS > 4 ? q : 0] = 0; }
+      for (int q = 0; q < SG_CW; ++q) { lo[q] = 0; if (NL > 4) hi[NL > 4 ? q : 0] = 0; }
       if (g.C && g.beta != 0.0 && !g.partial && (lane & 15) == 0) {
         // the output's lines, read after the contraction: on their way to L2 meanwhile
         const int m0 = w.I * SG_M + ew * 32 + lane, nn = w.J * SG_N + cq * SG_CW;
@@ -328,16 +333,16 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(SliceGemmArgs
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
-          for (int l = part ? LO : 0; l < (part ? NS : LO); ++l) {
-            const bool up = l < NS - 4;
-            const int wgt = 1 << (BITS * ((up ? NS - 5 : NS - 1) - l));
+          for (int l = part ? LO : 0; l < (part ? NL : LO); ++l) {
+            const bool up = l < NL - 4;
+            const int wgt = 1 << (BITS * ((up ? NL - 5 : NL - 1) - l));
             uint32_t r[SG_CW];
             tmem_ld16(r, tbase + (uint32_t)(l * SG_N));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
             for (int q = 0; q < SG_CW; ++q) {
               const long long v = (long long)__float2int_rn(__uint_as_float(r[q])) * (long long)wgt;
-              if (up) hi[NS > 4 ? q : 0] += v; else lo[q] += v;
+              if (up) hi[NL > 4 ? q : 0] += v; else lo[q] += v;
             }
           }
           asm volatile("tcgen05.fence::before_thread_sync;");
@@ -350,17 +355,17 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(SliceGemmArgs
       // ---- the tile's values: A row m (contiguous in the output), B rows n0 ..
       const int m = w.I * SG_M + ew * 32 + lane, n0 = w.J * SG_N + cq * SG_CW;
       const int em = g.ea[(int64_t)w.b * g.ea_batch + m];
-      const int e0 = em + g.alpha_exp - BITS * (NS + 1);
+      const int e0 = em + g.alpha_exp - BITS * (NL + 1);
       const uint32_t neg = g.alpha_neg ? 0xffffffffu : 0u;
       const int4 *ebp = reinterpret_cast<const int4 *>(g.eb + (int64_t)w.b * g.eb_batch + n0);   // n0 is a multiple of 16
       double val[SG_CW];
 #pragma unroll
       for (int q = 0; q < SG_CW; q += 4) {
         const int4 en = __ldg(ebp + q / 4);
-        val[q] = sg_value<HS>(NS > 4 ? hi[NS > 4 ? q : 0] : 0ll, lo[q], e0 + en.x, neg);
-        val[q + 1] = sg_value<HS>(NS > 4 ? hi[NS > 4 ? q + 1 : 0] : 0ll, lo[q + 1], e0 + en.y, neg);
-        val[q + 2] = sg_value<HS>(NS > 4 ? hi[NS > 4 ? q + 2 : 0] : 0ll, lo[q + 2], e0 + en.z, neg);
-        val[q + 3] = sg_value<HS>(NS > 4 ? hi[NS > 4 ? q + 3 : 0] : 0ll, lo[q + 3], e0 + en.w, neg);
+        val[q] = sg_value<HS>(NL > 4 ? hi[NL > 4 ? q : 0] : 0ll, lo[q], e0 + en.x, neg);
+        val[q + 1] = sg_value<HS>(NL > 4 ? hi[NL > 4 ? q + 1 : 0] : 0ll, lo[q + 1], e0 + en.y, neg);
+        val[q + 2] = sg_value<HS>(NL > 4 ? hi[NL > 4 ? q + 2 : 0] : 0ll, lo[q + 2], e0 + en.z, neg);
+        val[q + 3] = sg_value<HS>(NL > 4 ? hi[NL > 4 ? q + 3 : 0] : 0ll, lo[q + 3], e0 + en.w, neg);
       }
       if (g.partial) {
         double *o = g.partial + (((int64_t)w.b * g.splits + w.sp) * g.n_tiles + w.tile) * (SG_M * SG_N) +
@@ -768,7 +773,7 @@ __global__ void __launch_bounds__(256) slice_cols_tiles_kernel(SliceSrc a) {
   const double *x = column_source(a, b, r);
   const bool live = r < a.rows;
   const int e = live ? a.exps[(int64_t)b * a.exp_batch + r] : SL_ZERO;
-  for (int kb = blockIdx.y * 4 + (threadIdx.x >> 6); kb < a.nkb; kb += gridDim.y * 4)
+  for (int kb = a.kb_first + blockIdx.y * 4 + (threadIdx.x >> 6); kb < a.nkb; kb += gridDim.y * 4)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       double v[8];
@@ -837,6 +842,11 @@ cudaError_t slice_operand(const SliceSrc &a, int batch, cudaStream_t s) {
       slice_rows_short_kernel<NS, BITS, 4><<<dim3(a.rows_p / 8, 1, batch), 256, 0, s>>>(a, al);
     return cudaGetLastError();
   }
+  if (a.cols && a.fixed_exp) {
+    const int gy = (int)std::min<int64_t>(((int64_t)(a.nkb - a.kb_first) + 3) / 4, 64);
+    slice_cols_tiles_kernel<NS, BITS><<<dim3(a.rows_p / 64, gy, batch), 256, 0, s>>>(a);
+    return cudaGetLastError();
+  }
   const int64_t n_exp = (int64_t)batch * a.exp_batch;
   fill_int_kernel<<<(int)std::min<int64_t>((n_exp + 255) / 256, 152 * 4), 256, 0, s>>>(a.exps, n_exp, SL_ZERO);
   if (NS == 7 && BITS == 8 && a.colscale && a.x_batch == 0) {
@@ -864,23 +874,24 @@ cudaError_t slice_operand(const SliceSrc &a, int batch, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <int NS, int BITS>
+template <int NS, int BITS, int NL = NS>
 cudaError_t launch_ns(const SliceGemmArgs &g, int blocks, cudaStream_t s) {
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
   std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(slice_gemm_kernel<NS, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    attr_err = cudaFuncSetAttribute(slice_gemm_kernel<NS, BITS, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)sg_smem(NS));
   });
   if (attr_err != cudaSuccess) return attr_err;
-  slice_gemm_kernel<NS, BITS><<<blocks, SG_THREADS, sg_smem(NS), s>>>(g);
+  slice_gemm_kernel<NS, BITS, NL><<<blocks, SG_THREADS, sg_smem(NS), s>>>(g);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_slice_operand(const SliceSrc &a, int ns, int bits, int batch, cudaStream_t s) {
-  if (a.rows < 1 || a.K < 1 || batch < 1 || batch > 65535 || a.rows > a.rows_p || a.rows_p % 128 || (int64_t)a.nkb * 16 < a.K || a.exp_batch < a.rows_p || (a.cols && (a.colscale || a.only_if)) || (!a.cols && a.col_group))
+  if (a.rows < 1 || a.K < 1 || batch < 1 || batch > 65535 || a.rows > a.rows_p || a.rows_p % 128 || (int64_t)a.nkb * 16 < a.K || a.exp_batch < a.rows_p || (a.cols && (a.colscale || a.only_if)) || (!a.cols && a.col_group) ||
+      a.kb_first < 0 || a.kb_first >= a.nkb || ((a.kb_first || a.fixed_exp) && !a.cols))
     return cudaErrorInvalidValue;
   if (bits == 8) return ns == 7 ? slice_operand<7, 8>(a, batch, s) : cudaErrorInvalidValue;
   switch (bits == 7 ? ns : 0) {
@@ -893,6 +904,11 @@ cudaError_t launch_slice_operand(const SliceSrc &a, int ns, int bits, int batch,
     case 8: return slice_operand<8, 7>(a, batch, s);
   }
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_fill_int(int *p, int64_t n, int v, cudaStream_t s) {
+  fill_int_kernel<<<(int)std::min<int64_t>((n + 255) / 256, 152 * 4), 256, 0, s>>>(p, n, v);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_slice_pair(const SlicePairSrc &a, cudaStream_t s) {
@@ -910,30 +926,35 @@ void slice_gemm_tiles(SliceGemmArgs *g) {
   // (two of a level's products, or the leading level's one of 2^14)
   const int per_k = g->bits == 8 ? g->ns << 14 : std::max(1 << 14, (g->ns + 2) << 12);
   g->drain_kb = (1 << 24) / per_k / SL_K;
+  // base 256: the products of level 9 (six per k, about 2^-57.6 sqrt(6 K) of the
+  // rows' scales together) stay below an FP64 sum's own rounding, which grows
+  // with K, from a few thousand on; shorter contractions take them too
+  if (!g->levels) g->levels = g->bits == 8 && (g->nkb - g->kb_first) < 256 ? g->ns + 1 : g->ns;
 }
 
 size_t slice_gemm_plan(SliceGemmArgs *g, int n_sm, size_t max_partial) {
   slice_gemm_tiles(g);
+  const int nkb = g->nkb - g->kb_first;
   const int64_t units = (int64_t)g->batch * g->n_tiles;
   int best = 1;
   double cost_best = 1e300;
   const size_t part1 = (size_t)units * SG_M * SG_N * sizeof(double);
   for (int sp = 1; sp <= 64; ++sp) {
-    if (sp > 1 && (g->cd_out || g->nkb / sp < 16 || (size_t)sp * part1 > max_partial)) break;
+    if (sp > 1 && (g->cd_out || nkb / sp < 8 || (size_t)sp * part1 > max_partial)) break;
     const int64_t waves = (units * sp + n_sm - 1) / n_sm;
     // per unit: its blocks, and about five blocks' time for the exposed drain
     // and store; a split also pays the reduction's pass over its partials
-    const double cost = (double)waves * (5.0 + (double)((g->nkb + sp - 1) / sp)) + (sp > 1 ? 6.0 + 2.0 * sp * units / n_sm : 0.0);
+    const double cost = (double)waves * (5.0 + (double)((nkb + sp - 1) / sp)) + (sp > 1 ? 6.0 + 2.0 * sp * units / n_sm : 0.0);
     if (cost < cost_best) { cost_best = cost; best = sp; }
   }
-  g->kb_per_split = (g->nkb + best - 1) / best;
-  g->splits = (g->nkb + g->kb_per_split - 1) / g->kb_per_split;
+  g->kb_per_split = (nkb + best - 1) / best;
+  g->splits = (nkb + g->kb_per_split - 1) / g->kb_per_split;
   return g->splits > 1 ? (size_t)g->splits * part1 : 0;
 }
 
 cudaError_t launch_slice_gemm(const SliceGemmArgs &g, int n_sm, cudaStream_t s) {
   const int64_t units = (int64_t)g.batch * g.splits * g.n_tiles;
-  if (g.M < 1 || g.N < 1 || g.batch < 1 || g.nkb < 1 || g.splits < 1 || g.kb_per_split < 1 || g.drain_kb < 1 ||
+  if (g.M < 1 || g.N < 1 || g.batch < 1 || g.kb_first < 0 || g.nkb <= g.kb_first || g.splits < 1 || g.kb_per_split < 1 || g.drain_kb < 1 ||
       g.n_tiles < 1 || (g.splits > 1 && !g.partial) || (g.splits == 1 && g.partial) || (g.b_sel && !g.B_alt) || (g.sym && g.M != g.N) ||
       !g.A || !g.B || !g.ea || !g.eb || !g.err || (!g.cd_out && !g.C) || (g.cd_out && (g.sym || g.partial)))
     return cudaErrorInvalidValue;
@@ -947,7 +968,7 @@ cudaError_t launch_slice_gemm(const SliceGemmArgs &g, int n_sm, cudaStream_t s) 
     case 6: e = launch_ns<6, 7>(g, blocks, s); break;
     case 7: e = launch_ns<7, 7>(g, blocks, s); break;
     case 8: e = launch_ns<8, 7>(g, blocks, s); break;
-    case 78: e = launch_ns<7, 8>(g, blocks, s); break;
+    case 78: e = g.levels == 8 ? launch_ns<7, 8, 8>(g, blocks, s) : launch_ns<7, 8>(g, blocks, s); break;
   }
   if (e != cudaSuccess) return e;
   if (g.partial) {

@@ -133,10 +133,12 @@ def test_screen_digits_matches_inverse(ctx, N, J):
     assert e.value.status == ltgw.LTGW_ERR_NOT_SPD
 
 
-# the blocked reduction: its smallest size, one panel and several, remainders
-# on both sides of a panel; a metric of rank 70 (reflectors of a zero column)
-@pytest.mark.parametrize("n,pairs", [(1000, 3000), (1001, 2002), (1063, 2126), (1129, 2258), (1003, 70)])
-def test_naf_blocked_reduction(ctx, n, pairs):
+# the vectors' products from digits: their smallest size, five whole blocks of
+# 64 reflectors and one more; the blocked reduction: its smallest size, one
+# panel and several, remainders on both sides of a panel; a metric of rank 70
+# (reflectors of a zero column)
+@pytest.mark.parametrize("n,pairs", [(200, 600), (322, 644), (323, 646), (1000, 3000), (1001, 2002), (1063, 2126), (1129, 2258), (1003, 70)])
+def test_naf_from_digits(ctx, n, pairs):
     """Residual, orthonormality and eigenvalues of the kept pairs: the reduction
     and the vectors are backward stable to n u |K| each (32 n u with the
     constants of two-sided reflectors and the panel's sums)."""
