@@ -191,12 +191,14 @@ constexpr SliceForm emu_digits(int n_slices) { return {n_slices, 7, true}; }
 constexpr size_t kSliceOperandMax = (size_t)4 << 30;   // digits of one operand held at a time
 constexpr size_t kSlicePartialMax = (size_t)1 << 30;   // K-split partial tiles
 
-// Products this small stay on the CUDA-core kernels: a digit product costs two
-// to four launches before its first MMA (about 30 us in all; the 64 x 64 FP64
-// tiles take that long from about 2e7 multiply-adds on.  Measured at n = 264,
-// 560 pairs, 3.9e7: 0.587 ms of FP64 tiles, 0.059 ms from digits).
+// Products this small stay on the CUDA-core kernels.  Digits take two to four
+// launches (about 20 us), which a 64 x 64 FP64 tile passes at a length of a few
+// hundred however few tiles there are: request of 8 occupied orbitals, metric
+// (264^2 x 560) 0.587 -> 0.042 ms, Pi (65^2 x 560 x 8) 0.616 -> 0.071, projection
+// (65 x 560 x 264) 0.58 -> 0.10, W_nm 0.211 -> 0.057; without NAF 48^2 x 64 x 24
+// 0.062 -> 0.042.  A limit of 2e5 changes no case measured.
 bool slices_pay(int64_t m, int64_t n, int64_t k, int64_t batch) {
-  return k >= 128 && (double)m * (double)n * (double)k * (double)batch >= 2e7;
+  return k >= 48 && (double)m * (double)n * (double)k * (double)batch >= 2e6;
 }
 
 struct SliceOperand {

@@ -98,21 +98,31 @@ __device__ void pade_eval(const cplx *a, const cplx *zn, int np, cplx z, cplx &v
   dval = mk(0.0, 0.0) - a[0] * dt * rt * rt;
 }
 
-// One thread per target: Pade coefficients through every pade_stride-th node,
-// then Newton on f(E) = E - e_n - Re C(E - e_F + i eta) - shift_n.
-__global__ void qp_kernel(QpArgs q) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= q.n_tgt) return;
-  cplx g[MAXP], a[MAXP], zn[MAXP];
-  int np = 0;
-  for (int l = 0; l < q.n_omega && np < MAXP; l += q.pade_stride, ++np) {
-    zn[np] = mk(0.0, q.omega[l]);
-    g[np] = mk(q.sigma[((int64_t)t * q.n_omega + l) * 2], q.sigma[((int64_t)t * q.n_omega + l) * 2 + 1]);
+// One warp per target: Pade coefficients through every pade_stride-th node (at
+// level p the lanes share the nodes p ..; one thread's np^2 / 2 complex
+// divisions in sequence took two thirds of the kernel), then Newton on
+// f(E) = E - e_n - Re C(E - e_F + i eta) - shift_n, the same in every lane.
+// Bound: the fraction's chain of reciprocals, np per Newton step (32
+// frequencies, 4 targets: 151 us, one thread per target 265).
+__global__ void __launch_bounds__(32) qp_kernel(QpArgs q) {
+  __shared__ cplx g[MAXP], a[MAXP], zn[MAXP];
+  const int t = blockIdx.x, lane = threadIdx.x;
+  const int np = min(MAXP, (q.n_omega + q.pade_stride - 1) / q.pade_stride);
+  for (int i = lane; i < np; i += 32) {
+    const int l = i * q.pade_stride;
+    zn[i] = mk(0.0, q.omega[l]);
+    g[i] = mk(q.sigma[((int64_t)t * q.n_omega + l) * 2], q.sigma[((int64_t)t * q.n_omega + l) * 2 + 1]);
   }
-  a[0] = g[0];
+  __syncwarp();
+  if (lane == 0) a[0] = g[0];
   for (int p = 1; p < np; ++p) {
-    for (int i = p; i < np; ++i) g[i] = (g[p - 1] - g[i]) / ((zn[i] - zn[p - 1]) * g[i]);
-    a[p] = g[p];
+    const cplx gp = g[p - 1], zp = zn[p - 1];
+    for (int i = p + lane; i < np; i += 32) {
+      const cplx v = (gp - g[i]) / ((zn[i] - zp) * g[i]);
+      g[i] = v;
+      if (i == p) a[p] = v;
+    }
+    __syncwarp();
   }
   const double en = q.eps_n[t], sh = q.shift[t];
   double E = en;
@@ -127,8 +137,10 @@ __global__ void qp_kernel(QpArgs q) {
     if (!isfinite(E)) break;
     if (fabs(dE) < q.tol) { st = 0; break; }
   }
-  q.e_qp[t] = E;
-  q.status[t] = st;
+  if (lane == 0) {
+    q.e_qp[t] = E;
+    q.status[t] = st;
+  }
 }
 
 }  // namespace
@@ -143,7 +155,7 @@ cudaError_t launch_sigma(const SigmaArgs &a, cudaStream_t s) {
 cudaError_t launch_qp(const QpArgs &q, cudaStream_t s) {
   if (q.n_tgt <= 0) return cudaSuccess;
   if ((q.n_omega + q.pade_stride - 1) / q.pade_stride > MAXP) return cudaErrorInvalidValue;
-  qp_kernel<<<(q.n_tgt + 31) / 32, 32, 0, s>>>(q);
+  qp_kernel<<<q.n_tgt, 32, 0, s>>>(q);
   return cudaGetLastError();
 }
 
