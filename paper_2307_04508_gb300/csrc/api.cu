@@ -789,6 +789,7 @@ ltgw_status polarizability_tc(ltgw_ctx *ctx, int N, int64_t n_pairs, const doubl
   __nv_bfloat16 *Bhi = nullptr, *Blo = nullptr;   // the unscaled operand, pre-split for the TMA-fed kernel
   uint8_t *qa = nullptr, *qb = nullptr;           // FP8 codes: scaled operands [n_t][Mp][3 Kq], B [Mp][3 Kq]
   float *ds_a = nullptr, *ds_b = nullptr;         // FP8 per-row de-scales
+  int *maxima = nullptr;                          // FP8 per-row largest magnitudes
   int *d_tindex;
   auto layout = [&](Arena &A) {
     Af = Af_in ? nullptr : A.take<float>((size_t)Mp * Kp);
@@ -798,6 +799,7 @@ ltgw_status polarizability_tc(ltgw_ctx *ctx, int N, int64_t n_pairs, const doubl
       qb = A.take<uint8_t>((size_t)Mp * 3 * Kq);
       ds_a = A.take<float>((size_t)n_t * Mp);
       ds_b = A.take<float>((size_t)Mp);
+      maxima = A.take<int>((size_t)(n_t + 1) * Mp);
     } else {
       Bhi = A.take<__nv_bfloat16>((size_t)Mp * Kp);
       Blo = A.take<__nv_bfloat16>((size_t)Mp * Kp);
@@ -817,7 +819,7 @@ ltgw_status polarizability_tc(ltgw_ctx *ctx, int N, int64_t n_pairs, const doubl
   TcGemmArgs g;
   if (fp8) {
     // two-term E4M3 expansions of both operands (three products over 3 Kq codes)
-    CHECK_LAUNCH(ctx, launch_fp8_quantize(A, Kp, Kq, scale, n_t, Mp, qa, qb, ds_a, ds_b, s, 1), 1);
+    CHECK_LAUNCH(ctx, launch_fp8_quantize(A, Kp, Kq, scale, n_t, Mp, qa, qb, ds_a, ds_b, maxima, s, 1), 2);
     // FP32 sums of exact E4M3 products: a 4096-code drain keeps the accumulation
     // bias (about 4e-6) below the expansion's rounding error
     g.A8 = qa; g.B8 = qb; g.ds_a = ds_a; g.ds_b = ds_b; g.Kp = 3 * Kq; g.nt_group = 2; g.drain_k = 4096;
@@ -1010,6 +1012,7 @@ ltgw_status wnm_tc(ltgw_ctx *ctx, int N, int n_omega, const double *C, int T, in
   const int ncols = T * n_orb_act, nJ = (ncols + 127) / 128, rowsTp = nJ * 128;
   float *Cf, *ones = nullptr, *dsC = nullptr, *dsR = nullptr;
   uint8_t *qC = nullptr, *qR = nullptr;
+  int *maxima = nullptr;
   __nv_bfloat16 *Rh = nullptr, *Rl = nullptr;   // R~_tgt^T pre-split for the TMA-fed kernel
   auto layout = [&](Arena &A) {
     Cf = A.take<float>((size_t)n_omega * MpN * KpN);
@@ -1018,6 +1021,7 @@ ltgw_status wnm_tc(ltgw_ctx *ctx, int N, int n_omega, const double *C, int T, in
       qR = A.take<uint8_t>((size_t)rowsTp * 3 * Kq);
       dsC = A.take<float>((size_t)n_omega * MpN);
       dsR = A.take<float>((size_t)rowsTp);
+      maxima = A.take<int>((size_t)rowsTp);
     } else {
       ones = A.take<float>((size_t)n_omega * KpN);
       Rh = A.take<__nv_bfloat16>((size_t)rowsTp * KpN);
@@ -1035,7 +1039,7 @@ ltgw_status wnm_tc(ltgw_ctx *ctx, int N, int n_omega, const double *C, int T, in
   if (fp8) {
     // two-term E4M3 expansions: C_j's rows as A operands, R~_tgt^T's as B
     CHECK_LAUNCH(ctx, launch_fp8_quantize_a(Cf, KpN, Kq, n_omega * MpN, qC, dsC, s, 1), 1);
-    CHECK_LAUNCH(ctx, launch_fp8_quantize(BtT32, KpN, Kq, nullptr, 0, rowsTp, nullptr, qR, nullptr, dsR, s, 1), 1);
+    CHECK_LAUNCH(ctx, launch_fp8_quantize(BtT32, KpN, Kq, nullptr, 0, rowsTp, nullptr, qR, nullptr, dsR, maxima, s, 1), 2);
     g.A8 = qC; g.B8 = qR; g.ds_a = dsC; g.ds_b = dsR; g.Kp = 3 * Kq; g.rows_a = MpN; g.rows_b = rowsTp;
   } else {
     CHECK_LAUNCH(ctx, launch_scale_table(nullptr, N, KpN, n_omega, nullptr, nullptr, SCALE_NONE, ones, s), 1);

@@ -159,7 +159,8 @@ cudaError_t launch_split_bf16(const float *x, __nv_bfloat16 *hi, __nv_bfloat16 *
 // in segments h | l | h (A operands) and h | h | l (B operands), so that a contraction
 // over the 3 Kq codes sums h_a h_b + l_a h_b + h_a l_b.
 cudaError_t launch_fp8_quantize(const float *X, int64_t Kp, int64_t Kq, const float *S, int n_t, int rows,
-                                uint8_t *qa, uint8_t *qb, float *ds_a, float *ds_b, cudaStream_t s, int split);
+                                uint8_t *qa, uint8_t *qb, float *ds_a, float *ds_b, int *maxima, cudaStream_t s,
+                                int split);   // maxima: scratch of (n_t + 1) rows ints
 // FP64 factors f[t][k] (k < K) of the Pi contraction per frequency (SCALE_DIRECT,
 // p0 = omega), Laplace point (SCALE_LAPLACE, p0 = x, p1 = w) or imaginary-time
 // node (SCALE_EXPTAU, p0 = tau), no fused operations.

@@ -314,91 +314,127 @@ __device__ __forceinline__ float4 e4m3x4_value(uint32_t c) {
   return make_float4(fa.x, fa.y, fb.x, fb.y);
 }
 
-// Codes of x * inv (one term), or (split) of its two-term expansion h + l
-// with h = e4m3(x inv) and l = e4m3(x inv - h) (exact in FP32), both in the
+// Codes of xs = x * inv (one term), or (split) of its two-term expansion h + l
+// with h = e4m3(xs) and l = e4m3(xs - h) (exact in FP32), both in the
 // row's scaled units: the row's three segments of Kq codes are written as
 // pattern[0..2] of {h, l} (A operands h | l | h, B operands h | h | l, so that
 // one accumulator sums h_a h_b + l_a h_b + h_a l_b).
+__device__ __forceinline__ void codes_of(float4 x, float inv, uint32_t *h, uint32_t *l) {
+  *h = e4m3x4(x, inv);
+  const float4 hv = e4m3x4_value(*h);
+  *l = e4m3x4(make_float4(__fsub_rn(__fmul_rn(x.x, inv), hv.x), __fsub_rn(__fmul_rn(x.y, inv), hv.y), __fsub_rn(__fmul_rn(x.z, inv), hv.z), __fsub_rn(__fmul_rn(x.w, inv), hv.w)), 1.0f);
+}
 __device__ __forceinline__ void write_codes(uint32_t *row, int64_t k, int64_t q4, float4 x, float inv, int split,
                                             bool a_pattern) {
-  const uint32_t h = e4m3x4(x, inv);
+  uint32_t h, l;
+  codes_of(x, inv, &h, &l);
   row[k] = h;
   if (!split) return;
-  const float4 hv = e4m3x4_value(h);
-  const float4 r = make_float4(x.x * inv - hv.x, x.y * inv - hv.y, x.z * inv - hv.z, x.w * inv - hv.w);
-  const uint32_t l = e4m3x4(r, 1.0f);
   row[q4 + k] = a_pattern ? l : h;
   row[2 * q4 + k] = a_pattern ? h : l;
 }
-
-// One block per row r of X [rows][Kp] (FP32; Kp a multiple of 4): the row's
-// scale inv = 448 / max_k |X_rk| and codes qb[r][k] = e4m3(X_rk inv); for each
-// of the n_t factor rows S[t] the products p = X_rk S_tk (FP32) get their own
-// scale and codes qa[t][r][k].  De-scales 1 / inv (0 for a zero row) go to
-// ds_b[r] and ds_a[t][r]; code columns Kp..Kq-1 are zero.  split: each code
-// row holds three segments of Kq (the two-term expansion, write_codes).
-template <int MAXT>
-__global__ void __launch_bounds__(Q8_THREADS)
-    fp8_quantize_kernel(const float *__restrict__ X, int64_t Kp, int64_t Kq, const float *__restrict__ S, int n_t,
-                        int rows, uint8_t *__restrict__ qa, uint8_t *__restrict__ qb, float *__restrict__ ds_a,
-                        float *__restrict__ ds_b, int split) {
-  __shared__ float red[Q8_THREADS / 32];
-  __shared__ float inv_s[MAXT + 1];
-  const int r = blockIdx.x;
-  const float4 *xr = reinterpret_cast<const float4 *>(X + (int64_t)r * Kp);
-  const int64_t n4 = Kp / 4, q4 = Kq / 4;
-  float mb = 0.0f, ma[MAXT];
+// The same for 16 consecutive values, 16 bytes per segment.
+__device__ __forceinline__ void write_codes4(uint32_t *row, int64_t k, int64_t q4, const float4 x[4], float inv,
+                                             int split, bool a_pattern) {
+  uint32_t h[4], l[4];
 #pragma unroll
-  for (int t = 0; t < MAXT; ++t) ma[t] = 0.0f;
-  for (int64_t k = threadIdx.x; k < n4; k += Q8_THREADS) {
+  for (int v = 0; v < 4; ++v) codes_of(x[v], inv, &h[v], &l[v]);
+  const uint4 hh = make_uint4(h[0], h[1], h[2], h[3]), ll = make_uint4(l[0], l[1], l[2], l[3]);
+  *reinterpret_cast<uint4 *>(row + k) = hh;
+  if (!split) return;
+  *reinterpret_cast<uint4 *>(row + q4 + k) = a_pattern ? ll : hh;
+  *reinterpret_cast<uint4 *>(row + 2 * q4 + k) = a_pattern ? hh : ll;
+}
+
+// Row r of X [rows][Kp] (FP32; Kp a multiple of 16): the row's scale inv = 448 /
+// max_k |X_rk| and codes qb[r][k] = e4m3(X_rk inv); for each of the n_t factor
+// rows S[t] the products p = X_rk S_tk (FP32) get their own scale and codes
+// qa[t][r][k].  De-scales 1 / inv (0 for a zero row) go to ds_b[r] and
+// ds_a[t][r]; code columns Kp..Kq-1 are zero.  split: each code row holds three
+// segments of Kq (the two-term expansion, write_codes).
+//
+// Two kernels over (8 rows, a chunk of k, 8 factor rows): the maxima, then the
+// codes.  A warp takes one row, so the eight warps of a block share the factor
+// rows' chunk through L1, and the grid fills the SMs whatever the row count.
+// Bound: HBM, n_t times three code bytes per value.  N = 611, 20,001 pairs, 32
+// frequencies (1.2 GB of codes): 0.55 ms with the maxima; one block per row with all 32 factor
+// rows in its registers took 1.09 ms.
+constexpr int Q8_ROWS = Q8_THREADS / 32, Q8_T = 8, Q8_CHUNK = 512;   // Q8_CHUNK: float4 per row and block (more for rows past 1.3e8 values)
+
+// maxima (float bits, zeroed beforehand) [n_t][rows] of |X_rk S_tk|, then [rows] of |X_rk|
+__global__ void __launch_bounds__(Q8_THREADS)
+    fp8_max_kernel(const float *__restrict__ X, int64_t Kp, const float *__restrict__ S, int n_t, int rows,
+                   int64_t chunk, int *__restrict__ maxima) {
+  const int r = blockIdx.x * Q8_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31, t0 = blockIdx.z * Q8_T;
+  if (r >= rows) return;
+  const float4 *xr = reinterpret_cast<const float4 *>(X + (int64_t)r * Kp);
+  const int64_t n4 = Kp / 4, k0 = (int64_t)blockIdx.y * chunk, k1 = min(n4, k0 + chunk);
+  float mb = 0.0f, ma[Q8_T] = {};
+  for (int64_t k = k0 + lane; k < k1; k += 32) {
     const float4 x = xr[k];
     mb = fmaxf(mb, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))));
 #pragma unroll
-    for (int t = 0; t < MAXT; ++t) {
-      if (t < n_t) {
-        const float4 sv = reinterpret_cast<const float4 *>(S + (int64_t)t * Kp)[k];
-        ma[t] = fmaxf(ma[t], fmaxf(fmaxf(fabsf(x.x * sv.x), fabsf(x.y * sv.y)),
-                                   fmaxf(fabsf(x.z * sv.z), fabsf(x.w * sv.w))));
+    for (int u = 0; u < Q8_T; ++u)
+      if (t0 + u < n_t) {
+        const float4 sv = __ldg(reinterpret_cast<const float4 *>(S + (int64_t)(t0 + u) * Kp) + k);
+        ma[u] = fmaxf(ma[u], fmaxf(fmaxf(fabsf(x.x * sv.x), fabsf(x.y * sv.y)), fmaxf(fabsf(x.z * sv.z), fabsf(x.w * sv.w))));
       }
-    }
   }
-  mb = block_max(mb, red);
-  if (threadIdx.x == 0) inv_s[MAXT] = mb > 0.0f ? E4M3_MAX / mb : 0.0f;
 #pragma unroll
-  for (int t = 0; t < MAXT; ++t) {
-    if (t < n_t) {
-      const float m = block_max(ma[t], red);
-      if (threadIdx.x == 0) inv_s[t] = m > 0.0f ? E4M3_MAX / m : 0.0f;
-    }
+  for (int u = 0; u < Q8_T; ++u) {   // magnitudes order as their bits
+    const int m = __reduce_max_sync(0xffffffffu, __float_as_int(ma[u]));
+    if (lane == 0 && t0 + u < n_t && m) atomicMax(maxima + (int64_t)(t0 + u) * rows + r, m);
   }
-  __syncthreads();
-  const float invb = inv_s[MAXT];
-  if (threadIdx.x == 0) {
-    ds_b[r] = invb > 0.0f ? 1.0f / invb : 0.0f;
-    for (int t = 0; t < n_t; ++t) ds_a[(int64_t)t * rows + r] = inv_s[t] > 0.0f ? 1.0f / inv_s[t] : 0.0f;
-  }
+  const int m = __reduce_max_sync(0xffffffffu, __float_as_int(mb));
+  if (lane == 0 && t0 == 0 && m) atomicMax(maxima + (int64_t)n_t * rows + r, m);
+}
+
+__device__ __forceinline__ float e4m3_inv(int max_bits) {
+  const float m = __int_as_float(max_bits);
+  return m > 0.0f ? E4M3_MAX / m : 0.0f;
+}
+
+__global__ void __launch_bounds__(Q8_THREADS)
+    fp8_quantize_kernel(const float *__restrict__ X, int64_t Kp, int64_t Kq, const float *__restrict__ S, int n_t,
+                        int rows, int64_t chunk, const int *__restrict__ maxima, uint8_t *__restrict__ qa, uint8_t *__restrict__ qb,
+                        float *__restrict__ ds_a, float *__restrict__ ds_b, int split) {
+  const int r = blockIdx.x * Q8_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31, t0 = blockIdx.z * Q8_T;
+  if (r >= rows) return;
+  const float4 *xr = reinterpret_cast<const float4 *>(X + (int64_t)r * Kp);
+  const int64_t n4 = Kp / 4, q4 = Kq / 4, k0 = (int64_t)blockIdx.y * chunk, k1 = min(q4, k0 + chunk);
   const int64_t Ks = split ? 3 * Kq : Kq;   // codes per row
-  uint32_t *qbr = qb ? reinterpret_cast<uint32_t *>(qb + (int64_t)r * Ks) : nullptr;
-  for (int64_t k = threadIdx.x; k < q4; k += Q8_THREADS) {
-    if (k >= n4) {
-      for (int seg = 0; seg < (split ? 3 : 1); ++seg) {
-        if (qbr) qbr[seg * q4 + k] = 0u;
-        for (int t = 0; t < n_t; ++t) reinterpret_cast<uint32_t *>(qa + ((int64_t)t * rows + r) * Ks)[seg * q4 + k] = 0u;
-      }
-      continue;
-    }
-    const float4 x = xr[k];
-    if (qbr) write_codes(qbr, k, q4, x, invb, split, false);
+  const float invb = e4m3_inv(maxima[(int64_t)n_t * rows + r]);
+  float inv[Q8_T];
 #pragma unroll
-    for (int t = 0; t < MAXT; ++t) {
-      if (t < n_t) {
-        const float4 sv = reinterpret_cast<const float4 *>(S + (int64_t)t * Kp)[k];
-        const float4 p = make_float4(x.x * sv.x, x.y * sv.y, x.z * sv.z, x.w * sv.w);
-        write_codes(reinterpret_cast<uint32_t *>(qa + ((int64_t)t * rows + r) * Ks), k, q4, p, inv_s[t], split, true);
+  for (int u = 0; u < Q8_T; ++u) inv[u] = t0 + u < n_t ? e4m3_inv(maxima[(int64_t)(t0 + u) * rows + r]) : 0.0f;
+  if (blockIdx.y == 0 && lane == 0) {
+    if (t0 == 0) ds_b[r] = invb > 0.0f ? 1.0f / invb : 0.0f;
+#pragma unroll
+    for (int u = 0; u < Q8_T; ++u)
+      if (t0 + u < n_t) ds_a[(int64_t)(t0 + u) * rows + r] = inv[u] > 0.0f ? 1.0f / inv[u] : 0.0f;
+  }
+  uint32_t *qbr = qb && t0 == 0 ? reinterpret_cast<uint32_t *>(qb + (int64_t)r * Ks) : nullptr;
+  for (int64_t k = k0 + 4 * lane; k < k1; k += 128) {   // 16 values per lane: n4, q4 and the chunks are multiples of 4
+    const bool in = k < n4;   // past the data: zero codes
+    float4 x[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) x[v] = in ? xr[k + v] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (qbr) write_codes4(qbr, k, q4, x, invb, split, false);
+#pragma unroll
+    for (int u = 0; u < Q8_T; ++u)
+      if (t0 + u < n_t) {
+        float4 p[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const float4 sv = in ? __ldg(reinterpret_cast<const float4 *>(S + (int64_t)(t0 + u) * Kp) + k + v)
+                               : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          p[v] = make_float4(x[v].x * sv.x, x[v].y * sv.y, x[v].z * sv.z, x[v].w * sv.w);
+        }
+        write_codes4(reinterpret_cast<uint32_t *>(qa + ((int64_t)(t0 + u) * rows + r) * Ks), k, q4, p, inv[u], split, true);
       }
-    }
   }
 }
+
 // One block per row r of X [rows][Kp]: codes of X itself as an A operand
 // (split: segments h | l | h), de-scale to ds[r].
 __global__ void __launch_bounds__(Q8_THREADS)
@@ -461,13 +497,16 @@ __global__ void pi_root_factor_kernel(const double *__restrict__ delta, int64_t 
 }  // namespace
 
 cudaError_t launch_fp8_quantize(const float *X, int64_t Kp, int64_t Kq, const float *S, int n_t, int rows,
-                                uint8_t *qa, uint8_t *qb, float *ds_a, float *ds_b, cudaStream_t s, int split) {
+                                uint8_t *qa, uint8_t *qb, float *ds_a, float *ds_b, int *maxima, cudaStream_t s,
+                                int split) {
   if (rows <= 0) return cudaSuccess;
-  if (Kp % 4 || Kq % 16 || Kq < Kp || n_t < 0 || n_t > 32) return cudaErrorInvalidValue;
-  if (n_t <= 8)
-    fp8_quantize_kernel<8><<<rows, Q8_THREADS, 0, s>>>(X, Kp, Kq, S, n_t, rows, qa, qb, ds_a, ds_b, split);
-  else
-    fp8_quantize_kernel<32><<<rows, Q8_THREADS, 0, s>>>(X, Kp, Kq, S, n_t, rows, qa, qb, ds_a, ds_b, split);
+  if (Kp % 16 || Kq % 16 || Kq < Kp || n_t < 0 || n_t > 32) return cudaErrorInvalidValue;   // Kp is padded to 64
+  cudaError_t e = cudaMemsetAsync(maxima, 0, (size_t)(n_t + 1) * rows * sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  const int64_t q4 = Kq / 4, chunk = std::max<int64_t>(Q8_CHUNK, ((q4 + 65534) / 65535 + 3) / 4 * 4), chunks = (q4 + chunk - 1) / chunk;
+  const dim3 grid((rows + Q8_ROWS - 1) / Q8_ROWS, (unsigned)chunks, std::max(1, (n_t + Q8_T - 1) / Q8_T));
+  fp8_max_kernel<<<grid, Q8_THREADS, 0, s>>>(X, Kp, S, n_t, rows, chunk, maxima);
+  fp8_quantize_kernel<<<grid, Q8_THREADS, 0, s>>>(X, Kp, Kq, S, n_t, rows, chunk, maxima, qa, qb, ds_a, ds_b, split);
   return cudaGetLastError();
 }
 
