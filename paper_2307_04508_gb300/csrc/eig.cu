@@ -968,49 +968,162 @@ __global__ void __launch_bounds__(RB) tridiag_bounds_kernel(const double *dg, co
   }
 }
 
-// lam[r] = (n-1-r)-th smallest eigenvalue (r-th largest), r < k, by
-// multisection with BIS_L lanes per eigenvalue: each lane counts the
-// eigenvalues below one of BIS_L interior points, so an interval shrinks
-// (BIS_L + 1)-fold per step.  On this part a warp's FP64 instructions run one
-// after another whatever their dependences, so a whole warp per eigenvalue
-// (33-fold per step, about 11 steps to full precision) beats fewer lanes with
-// more steps.  d and e^2 live in shared memory.
-constexpr int BIS_L = 32;
-__global__ void bisect_kernel(const double *d, const double *e2g, const double *scal, int n,
-                              int k, int epw, double *lam) {
-  extern __shared__ double sm[];
-  double *sd = sm, *se2 = sm + n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    sd[i] = d[i];
-    se2[i] = (i < n - 1) ? e2g[i] : 0.0;
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int sub = lane % BIS_L, grp = lane / BIS_L;
-  const unsigned gmask = (BIS_L >= 32) ? 0xffffffffu : (((1u << (BIS_L & 31)) - 1u) << (grp * BIS_L));
-  const int r = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * epw + grp;
-  const bool live = grp < epw && r < k;
-  const int idx = n - 1 - (live ? r : 0);  // ascending index of the wanted eigenvalue
-  double lo = scal[1], hi = scal[2];
-  const double pivmin = scal[3];
-  bool done = !live;
-  for (int it = 0; it < 200; ++it) {
-    if (!done && hi - lo <= 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) + pivmin) done = true;
-    if (__all_sync(0xffffffffu, done)) break;
-    const double x = lo + (hi - lo) * ((double)(sub + 1) * (1.0 / (BIS_L + 1)));
-    const bool above = !done && sturm_count(sd, se2, n, x, pivmin) > idx;  // eigenvalue idx < x
-    const unsigned b = (__ballot_sync(0xffffffffu, above) & gmask) >> (grp * BIS_L);
-    if (!done) {
-      const int j = b ? (__ffs(b) - 1) : BIS_L;
-      // the same expressions as the lanes' points, so the bracket is exactly two of them
-      const double nlo = (j == 0) ? lo : lo + (hi - lo) * ((double)j * (1.0 / (BIS_L + 1)));
-      const double nhi = (j == BIS_L) ? hi : lo + (hi - lo) * ((double)(j + 1) * (1.0 / (BIS_L + 1)));
-      if (!(nlo > lo || nhi < hi)) done = true;  // no progress at this resolution
-      lo = nlo;
-      hi = nhi;
+// lam[r] = (n-1-r)-th smallest eigenvalue (r-th largest), r < k, one warp per
+// eigenvalue: a sweep counts the eigenvalues below 32 points, one per lane,
+// inside a bracket [lo, hi] whose ends the counts have proven, and the bracket
+// becomes the interval between two neighbouring points.  What the sweeps cost
+// is FP64 instructions: three per row, 16 clocks of the SM's FP64 pipe each and
+// about 64 clocks apart within a warp, whatever their dependences.  So few
+// sweeps: their points may lie anywhere, and lie where the eigenvalue is likely:
+//   - FP32 sweeps first (quotient form, T scaled to norm 1), which cost a tenth;
+//     the first FP64 sweep spans their bracket and its error bound;
+//   - with the eigenvalue alone in the bracket, p_n = det(T - x) at both ends
+//     gives a secant point, and the points close in on it geometrically (the
+//     distances to both ends divided by 4, 16, ...);
+//   - evenly spaced otherwise, and after any sweep that did less than an even one.
+// Measured, bisection to transposition with a quarter of the vectors kept,
+// against evenly spaced FP64 sweeps in blocks of four warps: n = 264 1.43 -> 1.11
+// ms, n = 800 3.81 -> 2.95, n = 1800 9.7 -> 8.0, n = 3300 22.7 -> 16.8.
+constexpr int BS_PRE = 4;                      // FP32 sweeps: 2 / 33^4 of ||T||
+constexpr double BS_PRE_ERR = 1.0 / 524288.0;  // 2^-19 ||T||: above the FP32 counts' error
+
+// p_n = det(T - x) as p 2^ex beside the count; t[i] = (d_i, e_{i-1}^2).
+__device__ __forceinline__ int sturm_value(const double2 *t, int n, double x, double pivmin, double *pv, int *ex) {
+  double pm = 1.0, p = t[0].x - x;
+  if (p == 0.0) p = -pivmin;
+  bool neg = __double2hiint(p) < 0;
+  int c = neg, E = 0;
+  for (int i = 1; i < n; i += 8) {
+    double dx[8], ee[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const double2 v = t[min(i + u, n - 1)];
+      dx[u] = v.x - x;
+      ee[u] = v.y;
+    }
+    const int m = n - i;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (u < m) {
+        double pn = fma(dx[u], p, -(ee[u] * pm));
+        if (is_zero_bits(pn))   // -pivmin with the sign opposite to p
+          pn = __longlong_as_double((~__double_as_longlong(p) & (long long)0x8000000000000000ull) |
+                                    __double_as_longlong(pivmin));
+        const bool nn = __double2hiint(pn) < 0;
+        c += (nn != neg);
+        neg = nn;
+        pm = p;
+        p = pn;
+      }
+    }
+    const int em = max((__double2hiint(p) >> 20) & 0x7ff, (__double2hiint(pm) >> 20) & 0x7ff);
+    if (em > 1023 + 400 || em < 1023 - 400) {
+      const double f = __hiloint2double((2046 - em) << 20, 0);   // 2^(1023 - em), exact
+      p *= f;
+      pm *= f;
+      E += em - 1023;
     }
   }
-  if (live && sub == 0) lam[r] = 0.5 * (lo + hi);
+  *pv = p;
+  *ex = E;
+  return c;
+}
+
+// The FP32 count: pivots q_i = (d_i - x) - e_{i-1}^2 / q_{i-1}, kept away from zero.
+__device__ __forceinline__ int sturm_count32(const float2 *t, int n, float x) {
+  float q = 1.0f;
+  int c = 0;
+#pragma unroll 8
+  for (int i = 0; i < n; ++i) {
+    const float2 v = t[i];   // t[0].y = 0
+    q = fmaf(-v.y, __fdividef(1.0f, q), v.x - x);
+    if (fabsf(q) < 1e-20f) q = -1e-20f;
+    c += q < 0.0f;
+  }
+  return c;
+}
+
+// pre: the block's shared memory also holds T in FP32.
+__global__ void bisect_kernel(const double *d, const double *e2g, const double *scal, int n, int k, bool pre,
+                              double *lam) {
+  extern __shared__ __align__(16) unsigned char bis_raw[];
+  double2 *t = reinterpret_cast<double2 *>(bis_raw);
+  float2 *tf = reinterpret_cast<float2 *>(t + n);
+  const double tn = scal[4], pivmin = scal[3];
+  pre = pre && tn > 0.0 && isfinite(tn);
+  const double rt = pre ? 1.0 / tn : 0.0;
+  pre = pre && isfinite(rt);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const double2 v = make_double2(d[i], i > 0 ? e2g[i - 1] : 0.0);
+    t[i] = v;
+    if (pre) tf[i] = make_float2((float)(v.x * rt), (float)(v.y * rt * rt));
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (r >= k) return;
+  const int idx = n - 1 - r;  // ascending index of the wanted eigenvalue
+  constexpr unsigned ALL = 0xffffffffu;
+  double lo = scal[1], hi = scal[2], hl = lo, hh = hi;
+  bool hint = false;
+  if (pre) {
+    float a = (float)(lo * rt), b = (float)(hi * rt);
+    for (int it = 0; it < BS_PRE; ++it) {
+      const float x = a + (b - a) * ((float)(lane + 1) * (1.0f / 33.0f));
+      const unsigned m = __ballot_sync(ALL, sturm_count32(tf, n, x) > idx);
+      const int j = m ? __ffs(m) - 1 : 32;
+      const float xl = __shfl_sync(ALL, x, max(j - 1, 0)), xh = __shfl_sync(ALL, x, min(j, 31));
+      if (j > 0) a = xl;
+      if (j < 32) b = xh;
+    }
+    hl = fmax(lo, ((double)a - BS_PRE_ERR) * tn);
+    hh = fmin(hi, ((double)b + BS_PRE_ERR) * tn);
+    hint = hl < hh;
+  }
+  // p 2^E and the count at the ends (count -1: not known), both from lanes of a sweep
+  double pl = 0.0, ph = 0.0;
+  int El = 0, Eh = 0, cl = -1, ch = -1;
+  bool even = false;   // the next sweep's points are evenly spaced
+  for (int it = 0; it < 200; ++it) {
+    const double w = hi - lo;
+    // the counts are those of a matrix within a few 2^-53 ||T||
+    if (w <= 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) + 0.125 * DBL_EPSILON * tn + pivmin) break;
+    double x = lo + w * ((double)(lane + 1) * (1.0 / 33.0));
+    bool placed = false;
+    if (hint) {
+      x = lane == 31 ? hh : hl + (hh - hl) * ((double)lane * (1.0 / 31.0));
+      placed = true;
+    } else if (!even && cl >= 0 && ch == cl + 1) {
+      const int sh = min(max(Eh - El, -1000), 1000);
+      const double q = scalbn(fabs(ph / pl), sh), c = lo + w / (1.0 + q);
+      if (c > lo && c < hi) {
+        x = lane < 16 ? c - (c - lo) * __hiloint2double((1023 - 2 * (lane + 1)) << 20, 0)
+                      : c + (hi - c) * __hiloint2double((1023 - 2 * (32 - lane)) << 20, 0);
+        placed = true;
+      }
+    }
+    hint = false;
+    double p;
+    int E;
+    const int c = sturm_value(t, n, x, pivmin, &p, &E);
+    const unsigned m = __ballot_sync(ALL, c > idx);   // eigenvalue idx < x
+    const int j = m ? __ffs(m) - 1 : 32, jl = max(j - 1, 0), jh = min(j, 31);
+    const double xl = __shfl_sync(ALL, x, jl), xh = __shfl_sync(ALL, x, jh);
+    const double p0 = __shfl_sync(ALL, p, jl), p1 = __shfl_sync(ALL, p, jh);
+    const int E0 = __shfl_sync(ALL, E, jl), E1 = __shfl_sync(ALL, E, jh);
+    const int c0 = __shfl_sync(ALL, c, jl), c1 = __shfl_sync(ALL, c, jh);
+    bool moved = false;
+    if (j > 0 && xl >= lo) {
+      moved = xl > lo;
+      lo = xl; pl = p0; El = E0; cl = c0;
+    }
+    if (j < 32 && xh <= hi) {
+      moved = moved || xh < hi;
+      hi = xh; ph = p1; Eh = E1; ch = c1;
+    }
+    if (!placed && !moved) break;   // no progress at this resolution
+    even = placed && !(hi - lo <= w * (1.0 / 32.0));
+  }
+  if (lane == 0) lam[r] = 0.5 * (lo + hi);
 }
 
 // Inverse iteration for the eigenvectors of T, one thread per group of
@@ -1672,17 +1785,19 @@ cudaError_t eig_vectors_impl(EigWork &w, int n, int k, double *Ut, int *flags, c
     if (e != cudaSuccess) return e;
   }
   {
-    // at most 32 / BIS_L eigenvalues per warp, spread so that every SM gets
-    // work; four warps per block, one per scheduler of the SM (the warps of
-    // one-warp blocks can share a scheduler, and each FP64 instruction holds
-    // it for the whole warp), with one copy of d and e^2 in shared memory
-    int dev = 0, nsm = 148;
+    // One warp per eigenvalue, four or more per block, one or more per scheduler
+    // of the SM (the warps of one-warp blocks can share a scheduler, and each
+    // FP64 instruction holds it for the whole warp); just enough for one wave of
+    // blocks, up to 16: 825 warps in blocks of four put eight on some SMs.
+    int dev = 0, nsm = 148, optin = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       nsm = 148;
+    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) optin = 0;
     cudaGetLastError();
-    const int epw = std::max(1, std::min(32 / BIS_L, (k + nsm - 1) / nsm));
-    const int nwarps = (k + epw - 1) / epw;
-    bisect_kernel<<<(nwarps + 3) / 4, 128, smem, s>>>(w.d, w.p, w.scal, n, k, epw, w.lam);
+    const int wpb = std::min(16, std::max(4, (k + nsm - 1) / nsm));
+    const size_t b64 = (size_t)n * sizeof(double2), b32 = (size_t)n * sizeof(float2);
+    const bool pre = b64 + b32 + 1024 <= (size_t)optin;
+    bisect_kernel<<<(k + wpb - 1) / wpb, wpb * 32, pre ? b64 + b32 : b64, s>>>(w.d, w.p, w.scal, n, k, pre, w.lam);
   }
   T *X = reinterpret_cast<T *>(w.X), *lu = reinterpret_cast<T *>(w.lu), *V = reinterpret_cast<T *>(w.V);
   {
