@@ -1,5 +1,7 @@
-"""Eigenvalues by bisection where the bracket's points are placed by an FP32
-estimate, by a secant or evenly: spectra with repeated and nearly repeated
+"""Eigenvalues by bisection and eigenvectors by twisted factorisations (inverse
+iteration for the ones these leave).  Bisection: the bracket's points are placed by
+an FP32 estimate, by a secant or evenly.  Vectors: 4 to 16 per block, in shared or
+global memory, alone or in groups.  Spectra with repeated and nearly repeated
 eigenvalues, a diagonal K (a tridiagonal form that decouples), a graded one,
 and warps at the edges of a block.
 
@@ -50,3 +52,18 @@ def test_eigenvalues_and_vectors(ctx, kind, n, diagonal):
     assert np.abs(g - ref[:k]).max() <= 1e-13 * ref[0]
     assert np.linalg.norm(K @ U.T - U.T * g[None, :], axis=0).max() <= 1e-12 * ref[0]
     assert np.abs(U @ U.T - np.eye(k)).max() <= 1e-12
+
+
+@pytest.mark.parametrize("n", [620, 1300])   # 8 vectors per block in shared memory, 16 in global
+def test_all_vectors_kept(ctx, n):
+    w = _spectrum("decay", n)
+    Q = np.linalg.qr(np.random.default_rng(n).standard_normal((n, n)))[0]
+    B = np.ascontiguousarray(Q * np.sqrt(w)[None, :])
+    K = B @ B.T
+    Ut = torch.zeros((n, n), dtype=torch.float64, device="cuda")
+    lam = torch.zeros(n, dtype=torch.float64, device="cuda")
+    assert ctx.naf_basis(torch.from_numpy(B).cuda(), n, n, 1e-4, Ut, lam) == n
+    g, U = lam.cpu().numpy(), Ut.cpu().numpy()
+    assert np.abs(g - np.sort(np.linalg.eigvalsh(K))[::-1]).max() <= 1e-13 * g[0]
+    assert np.linalg.norm(K @ U.T - U.T * g[None, :], axis=0).max() <= 1e-12 * g[0]
+    assert np.abs(U @ U.T - np.eye(n)).max() <= 1e-12
