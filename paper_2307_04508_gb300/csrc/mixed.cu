@@ -47,8 +47,6 @@ __global__ void scale_table_kernel(const double *__restrict__ delta, int64_t K, 
   }
 }
 
-// One thread per lower-triangle element (i >= j) of one matrix t.  Partial
-// tiles are 128 x 128, four scales per group.
 // Sum of FP32 partials as an unevaluated pair hi + lo of FP32 numbers
 // (Knuth's TwoSum per term; about 48 significant bits): the FP32 partials
 // carry errors of 2^-24 of their own, so the pair's sum equals their FP64 sum
@@ -61,42 +59,81 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float x) {
   hi = s;
 }
 
-__global__ void tc_reduce_sym_kernel(const double *__restrict__ partial, const float *__restrict__ partial32,
-                                     int splits, int groups, int n_tiles, const int *__restrict__ tile_index,
-                                     int nJ, int N, int nt_group, int colmajor, double alpha, double beta,
-                                     double *__restrict__ M) {
-  const int t = blockIdx.y;
-  const int grp = t / nt_group, slot = t % nt_group;
-  const int64_t NN = (int64_t)N * N;
-  const int64_t ntri = (int64_t)N * (N + 1) / 2;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ntri;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    // e -> (i, j), i >= j, row-major lower triangle (an FP32 estimate of the
-    // row, corrected by integer tests)
-    int a = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-    while ((int64_t)(a + 1) * (a + 2) / 2 <= e) ++a;
-    while ((int64_t)a * (a + 1) / 2 > e) --a;
-    const int b = (int)(e - (int64_t)a * (a + 1) / 2);
-    // (a, b), a >= b, b fastest; column-major tiles take (i, j) = (N-1-b, N-1-a) so that
-    // consecutive threads read consecutive rows of one column
-    const int i = colmajor ? N - 1 - b : a, j = colmajor ? N - 1 - a : b;
-    const int tile = tile_index[(i / 128) * nJ + (j / 128)];
-    const int64_t in_tile = colmajor ? (int64_t)(j % 128) * 128 + (i % 128) : (int64_t)(i % 128) * 128 + (j % 128);
-    double acc = 0.0;
-    if (partial32) {
-      float hi = 0.0f, lo = 0.0f;
-      for (int s = 0; s < splits; ++s)
-        two_sum_acc(hi, lo, partial32[((((int64_t)s * groups + grp) * nt_group + slot) * n_tiles + tile) * (128 * 128) +
-                                      in_tile]);
-      acc = (double)hi + (double)lo;
-    } else {
-      for (int s = 0; s < splits; ++s)
-        acc += partial[((((int64_t)s * groups + grp) * nt_group + slot) * n_tiles + tile) * (128 * 128) + in_tile];
+// Sums of the partial tiles, scaled, into both triangles of M; one block per
+// 64 x 64 quarter of a 128 x 128 tile (tiles I >= J, elements i >= j) and matrix
+// t = blockIdx.y.  Bound by memory: the partials are read four entries of one
+// column (row, unless colmajor) at a time, and the quarter goes through shared
+// memory so that the stores of both triangles run along M's rows.  One element
+// per thread with the one triangle stored down M's columns took 908 us for ten
+// matrices of N = 2258, 700 now; reading the partials (35 per entry there) alone
+// takes about 580.
+constexpr int RS_T = 64;
+__global__ void __launch_bounds__(256) tc_reduce_sym_kernel(const double *__restrict__ partial,
+                                                            const float *__restrict__ partial32, int splits,
+                                                            int groups, int n_tiles,
+                                                            const int *__restrict__ tile_index, int nJ, int N,
+                                                            int nt_group, int colmajor, double alpha, double beta,
+                                                            double *__restrict__ M) {
+  __shared__ double sm[RS_T][RS_T + 1];   // [slow][fast]: fast runs along the partials
+  const int t = blockIdx.y, grp = t / nt_group, slot = t % nt_group;
+  const int pair = blockIdx.x >> 2, qi = (blockIdx.x >> 1) & 1, qj = blockIdx.x & 1;
+  int I = (int)((sqrtf(8.0f * (float)pair + 1.0f) - 1.0f) * 0.5f);   // corrected by integer tests
+  while ((I + 1) * (I + 2) / 2 <= pair) ++I;
+  while (I * (I + 1) / 2 > pair) --I;
+  const int J = pair - I * (I + 1) / 2;
+  const int i0 = I * 128 + qi * RS_T, j0 = J * 128 + qj * RS_T;
+  if (i0 >= N || j0 >= N || i0 + RS_T <= j0) return;
+  const int tile = tile_index[I * nJ + J], tid = threadIdx.x;
+  const int f0 = (colmajor ? qi : qj) * RS_T, s0 = (colmajor ? qj : qi) * RS_T;
+  const int f = (tid & 15) * 4, sl = tid >> 4;   // slow rows sl, sl + 16, ...
+  const int64_t in_tile = (int64_t)(s0 + sl) * 128 + f0 + f, step = (int64_t)groups * nt_group * n_tiles * (128 * 128);
+  const int64_t base = (((int64_t)grp * nt_group + slot) * n_tiles + tile) * (128 * 128) + in_tile;
+  double acc[4][4];
+  if (partial32) {
+    float hi[4][4] = {}, lo[4][4] = {};
+    for (int s = 0; s < splits; ++s) {
+      float4 x[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) x[q] = __ldcs(reinterpret_cast<const float4 *>(partial32 + base + s * step + q * (16 * 128)));
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        two_sum_acc(hi[q][0], lo[q][0], x[q].x);
+        two_sum_acc(hi[q][1], lo[q][1], x[q].y);
+        two_sum_acc(hi[q][2], lo[q][2], x[q].z);
+        two_sum_acc(hi[q][3], lo[q][3], x[q].w);
+      }
     }
-    acc *= alpha;
-    if (beta != 0.0) acc += beta * M[t * NN + (int64_t)i * N + j];
-    M[t * NN + (int64_t)i * N + j] = acc;
-    M[t * NN + (int64_t)j * N + i] = acc;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) acc[q >> 2][q & 3] = (double)hi[q >> 2][q & 3] + (double)lo[q >> 2][q & 3];
+  } else {
+#pragma unroll
+    for (int q = 0; q < 16; ++q) acc[q >> 2][q & 3] = 0.0;
+    for (int s = 0; s < splits; ++s)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[q][u] += partial[base + s * step + q * (16 * 128) + u];
+  }
+#pragma unroll
+  for (int q = 0; q < 16; ++q) sm[sl + 16 * (q >> 2)][f + (q & 3)] = acc[q >> 2][q & 3] * alpha;
+  __syncthreads();
+  double *Mt = M + (int64_t)t * N * N;
+  const int c = tid & 63, r0 = tid >> 6;
+#pragma unroll 4
+  for (int r = r0; r < RS_T; r += 4) {   // (i, j), j along the threads
+    const int i = i0 + r, j = j0 + c;
+    if (i < N && i >= j) {
+      double &v = colmajor ? sm[c][r] : sm[r][c];
+      double *d = Mt + (int64_t)i * N + j;
+      if (beta != 0.0) v += beta * *d;
+      *d = v;
+    }
+  }
+  if (beta != 0.0) __syncthreads();
+#pragma unroll 4
+  for (int r = r0; r < RS_T; r += 4) {   // (j, i), i along the threads
+    const int i = i0 + c, j = j0 + r;
+    if (i < N && i > j) Mt[(int64_t)j * N + i] = colmajor ? sm[r][c] : sm[c][r];
   }
 }
 
@@ -205,10 +242,8 @@ cudaError_t launch_tc_reduce_sym(const double *partial, const float *partial32, 
                                  int n_tiles, const int *tile_index, int nJ, int n_t, int N, double alpha,
                                  double *M, cudaStream_t s, double beta, int nt_group, int colmajor) {
   if (N <= 0 || n_t <= 0) return cudaSuccess;
-  int64_t ntri = (int64_t)N * (N + 1) / 2;
-  int bx = (int)((ntri + 255) / 256);
-  if (bx > 152 * 4) bx = 152 * 4;
-  dim3 grid(bx, n_t);
+  const int nI = (N + 127) / 128;
+  dim3 grid(nI * (nI + 1) / 2 * 4, n_t);
   if (nt_group < 1 || (n_t + nt_group - 1) / nt_group != groups) return cudaErrorInvalidValue;
   tc_reduce_sym_kernel<<<grid, 256, 0, s>>>(partial, partial32, splits, groups, n_tiles, tile_index, nJ, N,
                                             nt_group, colmajor, alpha, beta, M);
