@@ -229,21 +229,16 @@ DTYPE = {"fp64": "f64", "bf16x3": "bf16x3", "fp8": "fp8e4m3", "fp8pi": "fp8e4m3 
 def pi_roofline(prec, pi_flops, pi_ms, pk, src, traffic=None):
     """Roofline of the Pi-build kernel: algorithmic flops (SYRK as N^2 K) per launch
     over its CUDA-event time; split-BF16 does three tensor products per useful one."""
-    if prec == "fp64":
-        a = pi_flops / (pi_ms / 1e3) / 1e12
-        peak = fp64_alu_peak_tflops(pk.get("sm_max_mhz", 2070.0))
-        return {"bound": "alu", "kernel": "gemm_tile_kernel<double> (Pi(tau_k) moments, FP64 SYRK)", "achieved": a,
-                "peak": peak, "unit": "TFLOP/s", "frac": a / peak,
-                "peak_source": "FP64 FMA: 152 SMs x 2 FMA/clk x max SM clock (recipe unit counts)",
-                "flops_per_launch": pi_flops, "ms_per_launch": pi_ms, "traffic": traffic}
-    if prec == "fp64emu":
-        a = 21 * pi_flops / (pi_ms / 1e3) / 1e12
-        return {"bound": "tensor", "kernel": "tc_tma_ts_kernel (Pi(tau_k) moments from integer slices: 21 digit "
+    if prec in ("fp64", "fp64emu"):
+        pairs = 28 if prec == "fp64" else 21
+        kern = "slice_gemm_kernel<7, 8, 7>" if prec == "fp64" else "slice_gemm_kernel<6, 7, 6>"
+        a = pairs * pi_flops / (pi_ms / 1e3) / 1e12
+        return {"bound": "tensor", "kernel": f"{kern} (Pi(tau_k) moments from integer digits: {pairs} digit "
                                              "pairs, one BF16 product each)",
                 "achieved": a, "peak": pk["bf16_tflops"], "unit": "TFLOP/s", "frac": a / pk["bf16_tflops"],
                 "peak_source": f"bf16_tflops (burst) of {src} MEASURED_PEAKS.json",
-                "flops_per_launch": 21 * pi_flops, "ms_per_launch": pi_ms, "traffic": traffic,
-                "note": "issued tensor flops; the stage time includes the slicing and the FP64 pair sums"}
+                "flops_per_launch": pairs * pi_flops, "ms_per_launch": pi_ms, "traffic": traffic,
+                "note": "issued tensor flops; the stage time includes forming the digits and the pair sums"}
     if prec in ("fp8", "fp8pi"):
         a = 3 * pi_flops / (pi_ms / 1e3) / 1e12
         peak = 2.0 * pk["bf16_tflops"]
@@ -349,24 +344,23 @@ def run_gpu(args):
     pk, src = peaks()
     alu_peak = fp64_alu_peak_tflops(pk.get("sm_max_mhz", 2070.0))
     # DRAM bytes per launch (read + write) from the ncu captures summarised in profiles/
-    # (tc_tma_ts_pi_mid.md, hh_fused_double_mid.md); mid workload only
+    # (tc_tma_ts_pi_mid.md); mid workload only
     traffic_pi = 112.52e6 + 44.94e6 if args.workload == "mid" and args.precision == "bf16x3" else None
-    traffic_tri = 25.98e6 + 0.05e6 if args.workload == "mid" else None
     roof_pi = pi_roofline(args.precision, pi_flops, pi_ms, pk, src, traffic_pi)
     # Householder reduction of the N_aux x N_aux metric: 4/3 N^3 algorithmic flops,
-    # N - 2 steps of one grid barrier each (latency-bound at mid size)
+    # N - 2 steps of one or two grid barriers each (latency-bound at mid size)
     tri_flops = 4.0 / 3.0 * prob.n_aux ** 3
     tri_ach = tri_flops / (tri_ms / 1e3) / 1e12
     # FP64 in both forms (the mixed form lowers only the dense contractions)
-    roof_tri = {"bound": "alu", "kernel": "hh_fused_kernel<double> (NAF Householder tridiagonalisation, FP64)",
+    roof_tri = {"bound": "alu", "kernel": "hh_panel_kernel, hh_fused_kernel<double> (NAF Householder tridiagonalisation, FP64)",
                 "achieved": tri_ach, "peak": alu_peak, "unit": "TFLOP/s", "frac": tri_ach / alu_peak,
                 "peak_source": "FP64 FMA: 152 SMs x 2 FMA/clk x max SM clock (recipe unit counts)",
                 "flops_per_launch": tri_flops, "ms_per_launch": tri_ms,
                 "us_per_step": 1e3 * tri_ms / max(1, prob.n_aux - 2),
-                "note": "full-storage fused form does 2 N^3 FP64 flops (the 4/3 N^3 counted here exploit "
-                        "symmetry); one grid barrier (1.2 us measured alone) and five block barriers per "
-                        "reflector on top",
-                "traffic": traffic_tri}
+                "note": "the panels' matrix-vector products take 2/3 N^3 FP64 flops (full storage), their "
+                        "updates run from integer digits on the tensor cores; two grid barriers (1.2 us "
+                        "each measured alone) per reflector on top",
+                "traffic": None}
     roofline = roof_tri if tri_ms > pi_ms else roof_pi
     clocks = clk.summary()
     line = {"metric": "G0W0 solves/s", "value": value, "unit": "solves/s", "n_gpus": world, "steps": args.steps,
@@ -692,7 +686,7 @@ def run_large(args):
     roof_pi = pi_roofline(args.precision, pi_flops, pi_ms, pk, src_pk, LARGE_TRAFFIC.get(("pi", args.precision)))
     tri_flops = 4.0 / 3.0 * cfg["n_aux"] ** 3
     tri_ach = tri_flops / (tri_ms / 1e3) / 1e12
-    roof_tri = {"bound": "alu", "kernel": "hh_fused_kernel<double> (NAF Householder tridiagonalisation, FP64)",
+    roof_tri = {"bound": "alu", "kernel": "hh_panel_kernel, hh_fused_kernel<double> (NAF Householder tridiagonalisation, FP64)",
                 "achieved": tri_ach, "peak": alu_peak, "unit": "TFLOP/s", "frac": tri_ach / alu_peak,
                 "peak_source": "FP64 FMA: 152 SMs x 2 FMA/clk x max SM clock (recipe unit counts)",
                 "flops_per_launch": tri_flops, "ms_per_launch": tri_ms,
@@ -794,11 +788,9 @@ def run_large(args):
         dist.destroy_process_group()
 
 
-# DRAM bytes (read + write) per launch at the large workload, from the ncu
-# captures summarised in profiles/ (None until captured for the current kernels):
-# the Householder reduction at N_aux = 9000, profiles/hh_fused_double_large.md
-# (dram__bytes_read.sum 1.835 TB + dram__bytes_write.sum 1.881 TB)
-LARGE_TRAFFIC = {("hh", "any"): 1.835e12 + 1.881e12}
+# DRAM bytes (read + write) per launch at the large workload, by (part, form), from
+# ncu captures summarised in profiles/ (empty: none of the current kernels)
+LARGE_TRAFFIC = {}
 
 
 def run_sweep(args):
@@ -914,9 +906,9 @@ def run_emu(args):
     auxiliary functions, the 10-point Laplace form, 32 frequencies) over
     --emu-pairs occupied-virtual pairs (the pair gaps of the large law's
     first active occupied orbitals; R~ rows Gaussian with the decaying norms
-    of NAF-projected rows): the plain FP64 form (ltgw_polarizability, FP64
-    pipe) beside the FP64-accurate slice form (ltgw_polarizability_emulated,
-    tensor cores), each timed with CUDA events on the launching stream after
+    of NAF-projected rows): the FP64 form (ltgw_polarizability, 7 base-256
+    digits) beside the form with the caller's number of base-128 digits
+    (ltgw_polarizability_emulated), both on the tensor cores, each timed with CUDA events on the launching stream after
     warm-up; the slice form's error against the FP64 one."""
     import torch
     from paper_2307_04508_gb300 import ltgw

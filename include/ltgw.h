@@ -111,7 +111,7 @@ typedef struct {
   double ms_naf_metric;      /* NAF stage parts (device time, ltgw_set_timing on): the */
   double ms_eig_vectors;     /* metric K (streamed: with the block arrivals), the      */
   double ms_naf_project;     /* eigenpairs after the tridiagonalisation (bisection,    */
-                             /* inverse iteration, back-transformation), the projections */
+                             /* vectors of T, back-transformation), the projections  */
 } ltgw_stats;
 
 typedef struct ltgw_ctx ltgw_ctx;
@@ -354,7 +354,7 @@ ltgw_status ltgw_screen(ltgw_ctx *ctx, int N, int n_omega, const double *Pi, dou
  * a_1 .. a_s (|a_1| <= 128, |a_i| <= 64 after it); then
  * C = sum over digit pairs with i + j <= s + 1 of 2^(-7(i+j)) a_i b_j^T,
  * times 2^(e_A + e_B).  Every pair's integer products are exact in BF16 and
- * summed exactly (FP32 sums below 2^24 per drain, FP64 after), so the only
+ * summed exactly (FP32 sums below 2^24 per drain, integers after), so the only
  * errors are the dropped digits: about 2^(-7s) of the rows' largest
  * magnitudes (s = 6: about 1e-12 relative Frobenius on products of Gaussian
  * rows).  A [m][lda], B [n][ldb] (k columns used), C [m][ldc]: device, row
