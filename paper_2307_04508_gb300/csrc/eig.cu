@@ -278,6 +278,45 @@ __device__ __forceinline__ T row_pass(T *row, int j0, int j1, const T *vp, const
   return acc0 + acc1;
 }
 
+// 1/q to the last bits: estimate (about 2^-23) and one cubic step.
+__device__ __forceinline__ double recip_cubic(double q) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(q));
+  const double e = fma(-q, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// tau, beta and sc of the reflector that maps (alpha, x') to (beta, 0), |x'|^2 =
+// sigma.  One thread's FP64 instructions follow one another at 64 clocks, comparisons
+// included, so: the reciprocal square root and the reciprocal from the hardware's
+// estimates by one cubic step each (the errors, about 2^-23, to the third power),
+// signs and ranges on the integer pipe; 12 instructions instead of about 28 with
+// Newton steps and FP64 comparisons, and 2700 clocks of the fused kernel's step
+// with the IEEE square root and divisions.  Outside the range where the squares
+// are safe, those.
+__device__ __forceinline__ void reflector_scalars(double alpha, double sigma, double *tau, double *beta, double *sc) {
+  if (((__double2hiint(sigma) & 0x7fffffff) | __double2loint(sigma)) == 0) { *tau = 0.0; *beta = alpha; *sc = 0.0; return; }
+  const double s = fma(alpha, alpha, sigma), aa = fabs(alpha);
+  const int ex = __double2hiint(s) >> 20;   // biased exponent; above 2047: the sign
+  double nrm, rinv, rden;
+  if ((unsigned)(ex - 223) < 1600u) {       // 2^-800 <= s < 2^800
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s));
+    const double e = fma(-s * y, y, 1.0);
+    rinv = fma(y * e, fma(e, 0.375, 0.5), y);
+    nrm = s * rinv;
+    rden = recip_cubic(aa + nrm);
+  } else {
+    nrm = sqrt(s);
+    rinv = 1.0 / nrm;
+    rden = 1.0 / (aa + nrm);
+  }
+  const bool neg = __double2hiint(alpha) < 0;
+  *beta = neg ? nrm : -nrm;
+  *tau = fma(aa, rinv, 1.0);                            // (beta - alpha) / beta
+  *sc = neg ? -rden : rden;                             // 1 / (alpha - beta)
+}
+
 // FP64 instructions are scarce on this part (about 2 per clock per SM), so
 // the per-step bookkeeping keeps them off paths that every thread runs: the
 // scalars are computed by one thread, and in the FP64 form phase 1 runs on
@@ -374,14 +413,8 @@ __global__ void __launch_bounds__(512, 1) hh_fused_kernel(HhFusedArgs<T> g) {
     if (threadIdx.x == 0) {   // the reflector's scalars, once
       T sigma = 0;
       for (int q = 0; q < p1w; ++q) sigma += wbuf[1][q];
-      const T alpha = s_st[1];
-      T t = 0, beta = alpha, sc = 0;
-      if (sigma != (T)0) {
-        const T nrm = sqrt(alpha * alpha + sigma);
-        beta = (alpha >= (T)0) ? -nrm : nrm;
-        t = (beta - alpha) / beta;
-        sc = (T)1 / (alpha - beta);
-      }
+      double t, beta, sc;
+      reflector_scalars(s_st[1], sigma, &t, &beta, &sc);
       s_st[2] = t; s_st[3] = beta; s_st[4] = sc;
       if (b == 0) {
         g.d[k] = s_st[0];
@@ -394,7 +427,9 @@ __global__ void __launch_bounds__(512, 1) hh_fused_kernel(HhFusedArgs<T> g) {
     // ---- phase 2: own rows r > k: update k-1 (k > 0) fused with s_r
     const int lr0 = (k + 1 > b) ? (k + 1 - b + G - 1) / G : 0;
     const int nact = n_own - lr0;
-    const int wpr = nact > 0 ? max(1, nwarp / nact) : 1;   // warps per row when rows are few
+    // warps per row when rows are few: a row's pass is a chain of about 6 L / wpr
+    // clocks, and every warp's sum holds the FP64 pipe for 80
+    const int wpr = nact > 0 ? max(1, min(nwarp / nact, (int)(sqrtf(0.075f * (float)(n - k - 1) / (float)nact) + 0.5f))) : 1;
     T *Pk = g.P + (size_t)(k & 1) * n;
     if (nact > 0) {
       const int L = n - k - 1;
@@ -680,35 +715,6 @@ __device__ __forceinline__ double own_products(const double *own, int i0, int n_
       }
   }
   return warp_sum4(acc[0], acc[1], acc[2], acc[3]);
-}
-
-// tau, beta and sc of the reflector that maps (alpha, x') to (beta, 0), |x'|^2 =
-// sigma.  The square root and the reciprocal by Newton steps from the hardware's
-// estimates (each step squares the relative error; the last of each is a
-// residual correction), about a third of the IEEE routines' chain here; outside
-// the range where the squares are safe, those.
-__device__ __forceinline__ void reflector_scalars(double alpha, double sigma, double *tau, double *beta, double *sc) {
-  const double s = fma(alpha, alpha, sigma), aa = fabs(alpha);
-  if (sigma == 0.0) { *tau = 0.0; *beta = alpha; *sc = 0.0; return; }
-  double nrm, rinv, rden;
-  if (s > 1e-250 && s < 1e250) {
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(rinv) : "d"(s));
-#pragma unroll
-    for (int it = 0; it < 2; ++it) rinv = fma(0.5 * rinv, fma(-s * rinv, rinv, 1.0), rinv);
-    nrm = s * rinv;
-    nrm = fma(0.5 * rinv, fma(-nrm, nrm, s), nrm);
-    rinv = fma(rinv, fma(-nrm, rinv, 1.0), rinv);       // 1 / nrm
-    const double den = aa + nrm;
-    rden = recip_nr<2>(den);
-    rden = fma(rden, fma(-den, rden, 1.0), rden);
-  } else {
-    nrm = sqrt(s);
-    rinv = 1.0 / nrm;
-    rden = 1.0 / (aa + nrm);
-  }
-  *beta = alpha >= 0.0 ? -nrm : nrm;
-  *tau = fma(aa, rinv, 1.0);                            // (beta - alpha) / beta
-  *sc = alpha >= 0.0 ? rden : -rden;                    // 1 / (alpha - beta)
 }
 
 __global__ void __launch_bounds__(HP_THREADS, 1) hh_panel_kernel(HhPanelArgs g) {
@@ -1334,14 +1340,6 @@ __global__ void inverse_iteration_kernel(const double *dg, const double *eg, con
 // 2e-11 (relative 2-norm over all kept) at n = 3300.
 constexpr double TW_TOL = 8.0 * DBL_EPSILON;
 constexpr int TW_THREADS = 256;
-
-// 1/q to the last bits: estimate (about 2^-23) and one cubic step.
-__device__ __forceinline__ double recip_cubic(double q) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(q));
-  const double e = fma(-q, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
 
 template <bool SM>
 __global__ void __launch_bounds__(TW_THREADS) twisted_kernel(const double *dg, const double *eg, const double *lam,
