@@ -1752,7 +1752,8 @@ bool launch_fused(EigWork &w, int n_all, int k0, cudaStream_t s, int *launches, 
 // The panel's arrays and digits live in the inverse-iteration scratch.
 // Sizes: measured at n = 900 both take 8.0 ms, n = 1100 10.3 against 10.8, n = 1800
 // 20.0 against 25.4, n = 3300 58.7 against 107 ms; leaving the last 800 columns to
-// the fused kernel is 0.1 to 0.5 ms better than 500, 0.6 better than 1100.
+// the fused kernel is 0.1 to 0.5 ms better than 500, 0.6 better than 1100 (all
+// before the fused kernel's scalars were shortened: 0.7 ms off its 6.7 at n = 800).
 constexpr int HP_MIN_N = 1000, HP_TAIL = 800;
 
 cudaError_t launch_blocked(EigWork &w, int n, cudaStream_t s, int *launches, int *k0_out) {
