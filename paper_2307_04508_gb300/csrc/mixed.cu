@@ -59,69 +59,103 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float x) {
   hi = s;
 }
 
-// Sums of the partial tiles, scaled, into both triangles of M; one block per
-// 64 x 64 quarter of a 128 x 128 tile (tiles I >= J, elements i >= j) and matrix
-// t = blockIdx.y.  Bound by memory: the partials are read four entries of one
-// column (row, unless colmajor) at a time, and the quarter goes through shared
-// memory so that the stores of both triangles run along M's rows.  One element
-// per thread with the one triangle stored down M's columns took 908 us for ten
-// matrices of N = 2258, 700 now; reading the partials (35 per entry there) alone
-// takes about 580.
-constexpr int RS_T = 64;
+// Sums of the partial tiles, scaled, into both triangles of M, t = blockIdx.y.
+// Small matrices: one thread per element (i >= j) of the lower triangle.  The
+// FP64 conversions bound this step there, and the blocks below convert whole
+// 128 x 128 tiles: 32 matrices of N = 130, 7.8 us against 11.5; N = 100 with 35
+// partials per element, 13 against 19.  From RS_SMALL on the blocks are no slower
+// (whole Pi, 70,000 pairs: N = 200 626 us by elements, 621 by blocks; N = 300 1104
+// and 1098).
+constexpr int RS_SMALL = 160;
+__global__ void tc_reduce_sym_small_kernel(const double *__restrict__ partial, const float *__restrict__ partial32,
+                                           int splits, int groups, int n_tiles, const int *__restrict__ tile_index,
+                                           int nJ, int N, int nt_group, int colmajor, double alpha, double beta,
+                                           double *__restrict__ M) {
+  const int t = blockIdx.y, grp = t / nt_group, slot = t % nt_group;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= N * (N + 1) / 2) return;
+  // e -> (a, b), a >= b, b fastest (an FP32 estimate corrected by integer tests);
+  // column-major tiles take (i, j) = (N-1-b, N-1-a) so that consecutive threads
+  // read consecutive rows of one column
+  int a = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+  while ((a + 1) * (a + 2) / 2 <= e) ++a;
+  while (a * (a + 1) / 2 > e) --a;
+  const int b = e - a * (a + 1) / 2;
+  const int i = colmajor ? N - 1 - b : a, j = colmajor ? N - 1 - a : b;
+  const int64_t step = (int64_t)groups * nt_group * n_tiles * (128 * 128);
+  const int64_t at = (((int64_t)grp * nt_group + slot) * n_tiles + tile_index[(i / 128) * nJ + j / 128]) * (128 * 128) +
+                     (colmajor ? (j % 128) * 128 + i % 128 : (i % 128) * 128 + j % 128);
+  double acc = 0.0;
+  if (partial32) {
+    float hi = 0.0f, lo = 0.0f;
+    for (int s = 0; s < splits; ++s) two_sum_acc(hi, lo, partial32[at + s * step]);
+    acc = (double)hi + (double)lo;
+  } else {
+    for (int s = 0; s < splits; ++s) acc += partial[at + s * step];
+  }
+  acc *= alpha;
+  double *m = M + (int64_t)t * N * N;
+  if (beta != 0.0) acc += beta * m[(int64_t)i * N + j];
+  m[(int64_t)i * N + j] = acc;
+  m[(int64_t)j * N + i] = acc;
+}
+
+// Larger ones: a block takes a strip of 16 x 64 entries of a 128 x 128 tile
+// (tiles I >= J, elements i >= j).  Bound by memory: the partials are read four
+// entries of one column (row, unless colmajor) at a time, and the strip goes
+// through shared memory so that the stores of both triangles run along M's rows.
+// Ten matrices of N = 2258: with 35 partials per entry 908 us by elements, 700
+// here (reading the partials alone takes about 580); with 5 partials 341 and 220.
+// Strips of 64 x 64 are as fast there, but too few blocks for N of a few hundred
+// (N = 400, 20,000 pairs, 10 points: 306 us for the whole Pi against 294).
+template <bool colmajor>
 __global__ void __launch_bounds__(256) tc_reduce_sym_kernel(const double *__restrict__ partial,
                                                             const float *__restrict__ partial32, int splits,
                                                             int groups, int n_tiles,
                                                             const int *__restrict__ tile_index, int nJ, int N,
-                                                            int nt_group, int colmajor, double alpha, double beta,
+                                                            int nt_group, double alpha, double beta,
                                                             double *__restrict__ M) {
-  __shared__ double sm[RS_T][RS_T + 1];   // [slow][fast]: fast runs along the partials
+  constexpr int SLOW = 16, FAST = 64;
+  __shared__ double sm[SLOW][FAST + 1];   // [slow][fast]: fast runs along the partials
   const int t = blockIdx.y, grp = t / nt_group, slot = t % nt_group;
-  const int pair = blockIdx.x >> 2, qi = (blockIdx.x >> 1) & 1, qj = blockIdx.x & 1;
+  const int strip = blockIdx.x & 7, half = (blockIdx.x >> 3) & 1, pair = blockIdx.x >> 4;
   int I = (int)((sqrtf(8.0f * (float)pair + 1.0f) - 1.0f) * 0.5f);   // corrected by integer tests
   while ((I + 1) * (I + 2) / 2 <= pair) ++I;
   while (I * (I + 1) / 2 > pair) --I;
   const int J = pair - I * (I + 1) / 2;
-  const int i0 = I * 128 + qi * RS_T, j0 = J * 128 + qj * RS_T;
-  if (i0 >= N || j0 >= N || i0 + RS_T <= j0) return;
+  constexpr int EI = colmajor ? FAST : SLOW, EJ = colmajor ? SLOW : FAST;   // the block's rows and columns of M
+  const int i0 = I * 128 + (colmajor ? half : strip) * EI, j0 = J * 128 + (colmajor ? strip : half) * EJ;
+  if (i0 >= N || j0 >= N || i0 + EI <= j0) return;
   const int tile = tile_index[I * nJ + J], tid = threadIdx.x;
-  const int f0 = (colmajor ? qi : qj) * RS_T, s0 = (colmajor ? qj : qi) * RS_T;
-  const int f = (tid & 15) * 4, sl = tid >> 4;   // slow rows sl, sl + 16, ...
-  const int64_t in_tile = (int64_t)(s0 + sl) * 128 + f0 + f, step = (int64_t)groups * nt_group * n_tiles * (128 * 128);
-  const int64_t base = (((int64_t)grp * nt_group + slot) * n_tiles + tile) * (128 * 128) + in_tile;
-  double acc[4][4];
+  const int f = (tid & 15) * 4, sl = tid >> 4;
+  const int64_t step = (int64_t)groups * nt_group * n_tiles * (128 * 128);
+  const int64_t base = (((int64_t)grp * nt_group + slot) * n_tiles + tile) * (128 * 128) +
+                       (strip * SLOW + sl) * 128 + half * FAST + f;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
   if (partial32) {
-    float hi[4][4] = {}, lo[4][4] = {};
+    float hi[4] = {}, lo[4] = {};
+#pragma unroll 4
     for (int s = 0; s < splits; ++s) {
-      float4 x[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) x[q] = __ldcs(reinterpret_cast<const float4 *>(partial32 + base + s * step + q * (16 * 128)));
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        two_sum_acc(hi[q][0], lo[q][0], x[q].x);
-        two_sum_acc(hi[q][1], lo[q][1], x[q].y);
-        two_sum_acc(hi[q][2], lo[q][2], x[q].z);
-        two_sum_acc(hi[q][3], lo[q][3], x[q].w);
-      }
+      const float4 x = __ldcs(reinterpret_cast<const float4 *>(partial32 + base + s * step));
+      two_sum_acc(hi[0], lo[0], x.x);
+      two_sum_acc(hi[1], lo[1], x.y);
+      two_sum_acc(hi[2], lo[2], x.z);
+      two_sum_acc(hi[3], lo[3], x.w);
     }
 #pragma unroll
-    for (int q = 0; q < 16; ++q) acc[q >> 2][q & 3] = (double)hi[q >> 2][q & 3] + (double)lo[q >> 2][q & 3];
+    for (int u = 0; u < 4; ++u) acc[u] = (double)hi[u] + (double)lo[u];
   } else {
-#pragma unroll
-    for (int q = 0; q < 16; ++q) acc[q >> 2][q & 3] = 0.0;
     for (int s = 0; s < splits; ++s)
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc[q][u] += partial[base + s * step + q * (16 * 128) + u];
+      for (int u = 0; u < 4; ++u) acc[u] += partial[base + s * step + u];
   }
 #pragma unroll
-  for (int q = 0; q < 16; ++q) sm[sl + 16 * (q >> 2)][f + (q & 3)] = acc[q >> 2][q & 3] * alpha;
+  for (int u = 0; u < 4; ++u) sm[sl][f + u] = acc[u] * alpha;
   __syncthreads();
   double *Mt = M + (int64_t)t * N * N;
-  const int c = tid & 63, r0 = tid >> 6;
-#pragma unroll 4
-  for (int r = r0; r < RS_T; r += 4) {   // (i, j), j along the threads
-    const int i = i0 + r, j = j0 + c;
+#pragma unroll
+  for (int r = tid / EJ; r < EI; r += 256 / EJ) {   // (i, j), j along the threads
+    const int c = tid % EJ, i = i0 + r, j = j0 + c;
     if (i < N && i >= j) {
       double &v = colmajor ? sm[c][r] : sm[r][c];
       double *d = Mt + (int64_t)i * N + j;
@@ -130,9 +164,9 @@ __global__ void __launch_bounds__(256) tc_reduce_sym_kernel(const double *__rest
     }
   }
   if (beta != 0.0) __syncthreads();
-#pragma unroll 4
-  for (int r = r0; r < RS_T; r += 4) {   // (j, i), i along the threads
-    const int i = i0 + c, j = j0 + r;
+#pragma unroll
+  for (int r = tid / EI; r < EJ; r += 256 / EI) {   // (j, i), i along the threads
+    const int c = tid % EI, i = i0 + c, j = j0 + r;
     if (i < N && i > j) Mt[(int64_t)j * N + i] = colmajor ? sm[r][c] : sm[c][r];
   }
 }
@@ -243,10 +277,15 @@ cudaError_t launch_tc_reduce_sym(const double *partial, const float *partial32, 
                                  double *M, cudaStream_t s, double beta, int nt_group, int colmajor) {
   if (N <= 0 || n_t <= 0) return cudaSuccess;
   const int nI = (N + 127) / 128;
-  dim3 grid(nI * (nI + 1) / 2 * 4, n_t);
   if (nt_group < 1 || (n_t + nt_group - 1) / nt_group != groups) return cudaErrorInvalidValue;
-  tc_reduce_sym_kernel<<<grid, 256, 0, s>>>(partial, partial32, splits, groups, n_tiles, tile_index, nJ, N,
-                                            nt_group, colmajor, alpha, beta, M);
+  if (N < RS_SMALL) {
+    tc_reduce_sym_small_kernel<<<dim3((N * (N + 1) / 2 + 255) / 256, n_t), 256, 0, s>>>(
+        partial, partial32, splits, groups, n_tiles, tile_index, nJ, N, nt_group, colmajor, alpha, beta, M);
+  } else {
+    const auto kernel = colmajor ? tc_reduce_sym_kernel<true> : tc_reduce_sym_kernel<false>;
+    kernel<<<dim3(nI * (nI + 1) / 2 * 16, n_t), 256, 0, s>>>(partial, partial32, splits, groups, n_tiles, tile_index,
+                                                             nJ, N, nt_group, alpha, beta, M);
+  }
   return cudaGetLastError();
 }
 

@@ -29,3 +29,25 @@ def test_both_triangles(N):
     assert np.array_equal(got, np.swapaxes(got, 1, 2))
     for j in range(3):
         assert np.abs(got[j] - ref[j]).max() <= 1e-4 * np.abs(ref[j]).max()
+
+
+@pytest.mark.parametrize("N", [159, 160, 321])
+def test_both_kernels_many_splits(N):
+    """The last size of one thread per element and the first ones of the strips,
+    with several K splits per entry (20,000 pairs) and Laplace moments."""
+    from paper_2307_04508_gb300 import ltgw
+    rng = np.random.default_rng(N)
+    Bt = rng.standard_normal((N, 20000)) * 0.01
+    delta = rng.uniform(0.3, 4.0, 20000)
+    om, _ = O.gl_grid(3, 0.5)
+    x, w = np.array([0.1, 1.0, 3.0]), np.array([0.3, 0.7, 1.1])
+    Pi = torch.full((3, N, N), float("nan"), dtype=torch.float64, device="cuda")
+    ctx = ltgw.Context(0)
+    ctx.polarizability_mixed(torch.from_numpy(Bt).cuda(), torch.from_numpy(delta).cuda(), om, Pi, x=x, w=w, spin=2)
+    got = Pi.cpu().numpy()
+    ctx.close()
+    M = [(Bt * (w[k] * delta * np.exp(-delta * delta * x[k]))[None, :]) @ Bt.T for k in range(3)]
+    assert np.array_equal(got, np.swapaxes(got, 1, 2))
+    for j in range(3):
+        ref = -4.0 * sum(np.exp(-om[j] ** 2 * x[k]) * M[k] for k in range(3))
+        assert np.abs(got[j] - ref).max() <= 1e-4 * np.abs(ref).max()
