@@ -139,6 +139,14 @@ size_t ltgw_workspace_bytes(const ltgw_ctx *ctx);
 /* Free that workspace (no call of this context may be in flight); the next
  * call allocates again. */
 ltgw_status ltgw_trim(ltgw_ctx *ctx);
+/* Most device memory that a context's FP64 and emulated products hold at a time
+ * for their integer digits and partial sums (6 GiB by default); larger products
+ * run in pieces (matrices of a batch, columns, frequencies), which changes no
+ * bit of the result.  A product whose smallest piece exceeds `bytes`, or cannot
+ * be allocated, runs on the FP64 units in the FP64 form (slower, rounded
+ * differently); the emulated forms take their smallest piece all the same and
+ * return LTGW_ERR_NOMEM when it cannot be allocated. */
+ltgw_status ltgw_set_digit_memory(ltgw_ctx *ctx, size_t bytes);
 ltgw_status ltgw_get_stats(const ltgw_ctx *ctx, ltgw_stats *out);
 
 /*

@@ -72,6 +72,8 @@ enum Stage { EV_START = 0, EV_NAF, EV_PI0, EV_PI1, EV_PI, EV_SCREEN, EV_WNM, EV_
 
 }  // namespace
 
+constexpr size_t kSliceHold = (size_t)6 << 30;   // default of ltgw_set_digit_memory
+
 struct ltgw_ctx {
   int device = 0;
   ltgw_status st = LTGW_OK;
@@ -97,6 +99,7 @@ struct ltgw_ctx {
   int n_sm = 148;
   Arena a4;  // tensor-core scratch: tile lists and partial tiles
   Arena a5;  // tensor-core operand copies consumed by the next contraction
+  size_t digit_max = kSliceHold;   // digits and partials held at a time (ltgw_set_digit_memory)
   // Autotuner of the tensor-core contractions (off by default): per shape, the
   // (scales per CTA, K-splits) configuration that timed fastest on this GPU.
   struct TcKey {
@@ -188,8 +191,16 @@ struct SliceForm {
 constexpr SliceForm kFp64Digits{7, 8, false};
 constexpr int kEmuSlices = 6;   // slices per operand row in the LTGW_FP64_EMU solve
 constexpr SliceForm emu_digits(int n_slices) { return {n_slices, 7, true}; }
-constexpr size_t kSliceOperandMax = (size_t)4 << 30;   // digits of one operand held at a time
-constexpr size_t kSlicePartialMax = (size_t)1 << 30;   // K-split partial tiles
+// A product's digits and K-split partials are held in pieces (matrices of a batch,
+// columns, frequencies): as many at a time as the context's limit
+// (ltgw_set_digit_memory) and half of what is free on the device allow.  The
+// lengths of the sums (pair chunks, K splits) follow from the product's sizes
+// alone (the splits from those of a piece of kSliceHold bytes), so a result has
+// the same bits whatever piece fits.  A pair chunk costs another pass over the
+// output: 1 % at N = 2258, whose chunks have 12,000 pairs.
+constexpr size_t kSliceTermMax = (size_t)768 << 20;    // digits of one matrix's operands (sets its pair chunk)
+constexpr size_t kSlicePartialMax = (size_t)1 << 30;   // K-split partial tiles of a piece
+constexpr int64_t kSliceMinCols = 1024;                // columns of a projection's smallest piece
 
 // Products this small stay on the CUDA-core kernels.  Digits take two to four
 // launches (about 20 us), which a 64 x 64 FP64 tile passes at a length of a few
@@ -221,44 +232,92 @@ struct SliceOperand {
   }
 };
 
-// Reserve `layout` in `ar`; false when the memory is not there.  Where the form
-// has CUDA-core kernels to fall back to, also when growing would take more
-// than half of what is free on the device (other contexts' solves size their
-// own workspace from it); no error is recorded then.
-template <class Layout>
-bool slice_reserve(ltgw_ctx *ctx, Arena &ar, bool required, Layout &&layout) {
-  ar.begin_sizing();
-  layout(ar);
-  if (!required && ar.need > ar.cap) {
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
-    else if (ar.need > (free_b + ar.cap) / 2) { ar.sizing = false; return false; }
-  }
-  if (ar.commit() != cudaSuccess) {
+// Memory for the digits (arena a5, `layout`) and the K-split partials (a4,
+// `partial()` bytes, into *part) of the largest piece that fits; `shrink` takes
+// the next smaller piece and is false at the smallest.  False when that one does
+// not fit either: an error in the forms that need the digits, else the product is
+// left to the CUDA-core kernels.  Other contexts' solves size their own workspace
+// from what is free, so more than half of it is taken for the smallest piece only.
+template <class Layout, class Partial, class Shrink>
+bool slice_fit(ltgw_ctx *ctx, bool required, Layout &&layout, Partial &&partial, Shrink &&shrink, double **part) {
+  for (;;) {
+    const size_t pb = partial();
+    auto layout4 = [&](Arena &A) { *part = pb ? A.take<double>(pb / sizeof(double)) : nullptr; };
+    ctx->a5.begin_sizing();
+    layout(ctx->a5);
+    ctx->a4.begin_sizing();
+    layout4(ctx->a4);
+    const size_t n5 = ctx->a5.need, n4 = pb ? ctx->a4.need : 0;
+    ctx->a5.sizing = ctx->a4.sizing = false;
+    bool ok = n5 + n4 <= ctx->digit_max, tried = false;
+    const size_t grow = (n5 > ctx->a5.cap ? n5 : 0) + (n4 > ctx->a4.cap ? n4 : 0);
+    if (ok && grow) {
+      size_t free_b = 0, total_b = 0;
+      if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
+      else ok = grow <= (free_b + (n5 > ctx->a5.cap ? ctx->a5.cap : 0) + (n4 > ctx->a4.cap ? ctx->a4.cap : 0)) / 2;
+      tried = true;
+    }
+    if (!ok && shrink()) continue;
+    if (ok || required || (tried && n5 + n4 <= ctx->digit_max)) {
+      ctx->a5.need = n5;
+      ctx->a4.need = n4;
+      if (ctx->a5.commit() == cudaSuccess && ctx->a4.commit() == cudaSuccess) {
+        layout(ctx->a5);
+        layout4(ctx->a4);
+        return true;
+      }
+      if (ok && shrink()) continue;
+    }
     if (required) ctx->fail(LTGW_ERR_NOMEM, "slice operand allocation failed");
     return false;
   }
-  layout(ar);
+}
+
+// The next smaller equal pieces of n items; false when they are single already.
+bool next_piece(int n, int *blk) {
+  if (*blk == 1) return false;
+  int pieces = (n + *blk - 1) / *blk, b = *blk;
+  while (b >= *blk) b = (n + pieces) / (pieces + 1), ++pieces;
+  *blk = b;
   return true;
 }
 
-// One digit contraction: plan, K-split partials (arena a4), launch.
-ltgw_status slice_run(ltgw_ctx *ctx, SliceGemmArgs &g, SliceForm f, cudaStream_t s) {
-  g.ns = f.ns; g.bits = f.bits; g.err = ctx->flags;
-  size_t part = slice_gemm_plan(&g, ctx->n_sm, kSlicePartialMax);
-  if (part && !slice_reserve(ctx, ctx->a4, false, [&](Arena &A) { g.partial = A.take<double>(part / sizeof(double)); })) {
-    g.splits = 1; g.kb_per_split = g.nkb; g.partial = nullptr;   // no room for partials: one split
-  }
+// One piece of a digit contraction planned by slice_plan.
+ltgw_status slice_run(ltgw_ctx *ctx, SliceGemmArgs &g, double *part, cudaStream_t s) {
+  g.err = ctx->flags;
+  g.partial = slice_gemm_piece(&g) ? part : nullptr;
   CHECK_LAUNCH(ctx, launch_slice_gemm(g, ctx->n_sm, s), g.partial || (g.sym && g.mirror) ? 2 : 1);
   return LTGW_OK;
 }
 
+// Matrices in a piece of kSliceHold bytes, `each` per matrix.
+int planned_piece(int n, size_t each, size_t shared) {
+  int blk = n;
+  while (shared + blk * each > kSliceHold && next_piece(n, &blk)) {}
+  return blk;
+}
+
+// The plan of a product (M, N, nkb, sym, matrices of a piece): its K splits hold
+// for every piece.
+SliceGemmArgs slice_plan(const ltgw_ctx *ctx, int M, int N, int nkb, int sym, int batch, SliceForm f) {
+  SliceGemmArgs g;
+  g.ns = f.ns; g.bits = f.bits;
+  g.M = M; g.N = N; g.nkb = nkb; g.sym = sym; g.batch = batch;
+  slice_gemm_plan(&g, ctx->n_sm, kSlicePartialMax);
+  return g;
+}
+// Bytes of its partials for a piece of `batch` matrices and M columns.
+size_t slice_partial(SliceGemmArgs g, int batch, int M) {
+  g.batch = batch; g.M = M;
+  return slice_gemm_piece(&g);
+}
+
 // Chunk of the contraction length so that `rows` operand rows stay within
-// kSliceOperandMax (the emulated forms' exponents belong to whole rows: one chunk).
-int64_t slice_k_chunk(int64_t rows, int64_t K, int batch, SliceForm f) {
+// kSliceTermMax (the emulated forms' exponents belong to whole rows: one chunk).
+int64_t slice_k_chunk(int64_t rows, int64_t K, SliceForm f) {
   if (f.required) return K;
-  const int64_t per_k = slice_rows_padded(rows) * 2 * f.ns * batch;
-  const int64_t most = std::max<int64_t>(2048, (int64_t)kSliceOperandMax / per_k);
+  const int64_t per_k = slice_rows_padded(rows) * 2 * f.ns;
+  const int64_t most = std::max<int64_t>(2048, (int64_t)kSliceTermMax / per_k);
   const int64_t n = (K + most - 1) / most;
   return std::min(K, ((K + n - 1) / n + 63) / 64 * 64);
 }
@@ -268,16 +327,18 @@ int64_t slice_k_chunk(int64_t rows, int64_t K, int batch, SliceForm f) {
 ltgw_status slice_syrk(ltgw_ctx *ctx, int n, int64_t K, const double *X, int64_t ld, double *C, double beta,
                        SliceForm f, cudaStream_t s, bool *done) {
   SliceOperand o;
-  const int64_t chunk = slice_k_chunk(n, K, 1, f);
-  *done = slice_reserve(ctx, ctx->a5, f.required, [&](Arena &A) { o.layout(A, n, chunk, 1, f); });
+  double *part = nullptr;
+  const int64_t chunk = slice_k_chunk(n, K, f);
+  const SliceGemmArgs plan = slice_plan(ctx, n, n, (int)((chunk + SL_K - 1) / SL_K), 1, 1, f);
+  *done = slice_fit(ctx, f.required, [&](Arena &A) { o.layout(A, n, chunk, 1, f); },
+                    [&] { return slice_partial(plan, 1, n); }, [] { return false; }, &part);
   if (!*done) return ctx->status();
   for (int64_t k0 = 0; k0 < K; k0 += chunk) {
     const int64_t kc = std::min(chunk, K - k0);
     CHECK_LAUNCH(ctx, launch_slice_operand(o.source(X + k0, ld, 0, n, kc, false), f.ns, f.bits, 1, s), 3);
-    SliceGemmArgs g;
-    g.A = g.B = o.dig; g.ea = g.eb = o.exps; g.nkb = o.nkb;
-    g.M = g.N = n; g.sym = 1; g.C = C; g.ldc = n; g.beta = k0 ? 1.0 : beta;
-    if (slice_run(ctx, g, f, s) != LTGW_OK) return ctx->status();
+    SliceGemmArgs g = plan;
+    g.A = g.B = o.dig; g.ea = g.eb = o.exps; g.C = C; g.ldc = n; g.beta = k0 ? 1.0 : beta;
+    if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
   }
   return LTGW_OK;
 }
@@ -287,24 +348,31 @@ ltgw_status slice_project(ltgw_ctx *ctx, int N, int n_aux, const double *Ut, con
                           int64_t x_batch, int64_t cols, int batch, double *out, int64_t ld_out, int64_t out_batch,
                           SliceForm f, cudaStream_t s, bool *done) {
   SliceOperand u, x;
-  const int64_t per_col = (int64_t)((n_aux + SL_K - 1) / SL_K) * SL_K * 2 * f.ns * batch;
-  const int64_t most = std::max<int64_t>(4096, (int64_t)kSliceOperandMax / per_col / 128 * 128);
-  const int64_t n_chunks = (cols + most - 1) / most;
-  const int64_t chunk = std::min(cols, ((cols + n_chunks - 1) / n_chunks + 127) / 128 * 128);
-  *done = slice_reserve(ctx, ctx->a5, f.required, [&](Arena &A) {
-    u.layout(A, N, n_aux, 1, f);
-    x.layout(A, chunk, n_aux, batch, f);
-  });
+  double *part = nullptr;
+  int64_t chunk = cols;
+  const SliceGemmArgs plan = slice_plan(ctx, (int)cols, N, (n_aux + SL_K - 1) / SL_K, 0, batch, f);
+  *done = slice_fit(
+      ctx, f.required,
+      [&](Arena &A) {
+        u.layout(A, N, n_aux, 1, f);
+        x.layout(A, chunk, n_aux, batch, f);
+      },
+      [&] { return slice_partial(plan, batch, (int)chunk); },
+      [&] {
+        if (chunk <= kSliceMinCols) return false;
+        chunk = (chunk / 2 + 127) / 128 * 128;
+        return true;
+      },
+      &part);
   if (!*done) return ctx->status();
   CHECK_LAUNCH(ctx, launch_slice_operand(u.source(Ut, n_aux, 0, N, n_aux, false), f.ns, f.bits, 1, s), 3);
   for (int64_t c0 = 0; c0 < cols; c0 += chunk) {
     const int cc = (int)std::min(chunk, cols - c0);
     CHECK_LAUNCH(ctx, launch_slice_operand(x.source(X + c0, ld, x_batch, cc, n_aux, true), f.ns, f.bits, batch, s), 3);
-    SliceGemmArgs g;
+    SliceGemmArgs g = plan;
     g.A = x.dig; g.a_batch = x.dig_batch; g.ea = x.exps; g.ea_batch = x.rows_p;
-    g.B = u.dig; g.eb = u.exps; g.nkb = u.nkb; g.batch = batch;
-    g.M = cc; g.N = N; g.C = out + c0; g.ldc = ld_out; g.c_batch = out_batch;
-    if (slice_run(ctx, g, f, s) != LTGW_OK) return ctx->status();
+    g.B = u.dig; g.eb = u.exps; g.M = cc; g.C = out + c0; g.ldc = ld_out; g.c_batch = out_batch;
+    if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
   }
   return LTGW_OK;
 }
@@ -316,15 +384,19 @@ ltgw_status slice_wnm(ltgw_ctx *ctx, int N, int n_omega, const double *C, int T,
   const int cols = T * n_orb_act;
   SliceOperand r, c;
   double *cd = nullptr;
-  const int64_t nkb = (N + SL_K - 1) / SL_K;
-  const int blk = (int)std::min<int64_t>(
-      n_omega, std::max<int64_t>(1, (int64_t)kSliceOperandMax / slice_digit_bytes(N, nkb, f.ns)));
+  double *part = nullptr;   // the column dot takes no K splits
   const int tiles_n = (N + 63) / 64;
-  *done = slice_reserve(ctx, ctx->a5, f.required, [&](Arena &A) {
-    r.layout(A, cols, N, 1, f);
-    c.layout(A, N, N, blk, f);
-    cd = A.take<double>((size_t)blk * 4 * tiles_n * cols);
-  });
+  int blk = n_omega;
+  *done = slice_fit(
+      ctx, f.required,
+      [&](Arena &A) {
+        r.layout(A, cols, N, 1, f);
+        c.layout(A, N, N, blk, f);
+        cd = A.take<double>((size_t)blk * 4 * tiles_n * cols);
+      },
+      [] { return (size_t)0; },
+      [&] { return next_piece(n_omega, &blk); },
+      &part);
   if (!*done) return ctx->status();
   SliceSrc rs = r.source(Btt, ld_btt, 0, cols, N, true);
   rs.col_group = n_orb_act; rs.col_stride = stride_btt;
@@ -336,9 +408,10 @@ ltgw_status slice_wnm(ltgw_ctx *ctx, int N, int n_omega, const double *C, int T,
     SliceGemmArgs g;
     g.A = r.dig; g.ea = r.exps;
     g.B = c.dig; g.b_batch = c.dig_batch; g.eb = c.exps; g.eb_batch = c.rows_p;
-    g.nkb = r.nkb; g.batch = nb; g.M = cols; g.N = N;
+    g.ns = f.ns; g.bits = f.bits; g.nkb = r.nkb; g.batch = nb; g.M = cols; g.N = N;
     g.cd_B = Btt; g.cd_ld = ld_btt; g.cd_stride = stride_btt; g.cd_cols = n_orb_act; g.cd_out = cd; g.cd_ldo = cols;
-    if (slice_run(ctx, g, f, s) != LTGW_OK) return ctx->status();
+    slice_gemm_plan(&g, ctx->n_sm, 0);
+    if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
     CHECK_LAUNCH(ctx, launch_slice_coldot_reduce(g, W + (int64_t)j0 * cols, cols, s), 1);
   }
   return LTGW_OK;
@@ -355,16 +428,23 @@ ltgw_status slice_pi(ltgw_ctx *ctx, int N, int64_t n_pairs, const double *Bt, in
   SliceOperand o, o2;   // o2: the unsigned operand, written and read only where some factor is negative
   double *fac = nullptr;
   int *neg = nullptr;
-  const int64_t per_t = 2 * slice_rows_padded(N) * 2 * f.ns;
-  // the pair range first (each chunk is another pass over M), then the points at a time
-  const int64_t chunk = slice_k_chunk(2 * N, n_pairs, 1, f);
-  const int blk = (int)std::min<int64_t>(n_t, std::max<int64_t>(1, (int64_t)kSliceOperandMax / (per_t * chunk)));
-  *done = slice_reserve(ctx, ctx->a5, f.required, [&](Arena &A) {
-    o.layout(A, N, chunk, blk, f);
-    o2.layout(A, N, chunk, blk, f);
-    fac = A.take<double>((size_t)n_t * 2 * chunk);
-    neg = A.take<int>(1);
-  });
+  double *part = nullptr;
+  const int64_t chunk = slice_k_chunk(2 * slice_rows_padded(N), n_pairs, f);
+  const int nkb = (int)((chunk + SL_K - 1) / SL_K);
+  const SliceGemmArgs plan =
+      slice_plan(ctx, N, N, nkb, 1, planned_piece(n_t, 2 * slice_digit_bytes(N, nkb, f.ns), 0), f);
+  int blk = n_t;
+  *done = slice_fit(
+      ctx, f.required,
+      [&](Arena &A) {
+        o.layout(A, N, chunk, blk, f);
+        o2.layout(A, N, chunk, blk, f);
+        fac = A.take<double>((size_t)n_t * 2 * chunk);
+        neg = A.take<int>(1);
+      },
+      [&] { return slice_partial(plan, blk, N); },
+      [&] { return next_piece(n_t, &blk); },
+      &part);
   if (!*done) return ctx->status();
   for (int64_t k0 = 0; k0 < n_pairs; k0 += chunk) {
     const int64_t kc = std::min(chunk, n_pairs - k0);
@@ -378,13 +458,13 @@ ltgw_status slice_pi(ltgw_ctx *ctx, int N, int64_t n_pairs, const double *Bt, in
       SliceSrc b = o2.source(Bt + k0, ldb, 0, N, kc, false);
       b.colscale = fac + (int64_t)(n_t + t0) * kc; b.cs_batch = kc; b.only_if = neg;
       CHECK_LAUNCH(ctx, launch_slice_operand(b, f.ns, f.bits, nb, s), 3);
-      SliceGemmArgs g;
+      SliceGemmArgs g = plan;
       g.A = g.B = o.dig; g.a_batch = g.b_batch = o.dig_batch; g.ea = g.eb = o.exps; g.ea_batch = g.eb_batch = o.rows_p;
       g.B_alt = o2.dig; g.b_sel = neg;   // |sqrt| rows have the same exponents
-      g.nkb = o.nkb; g.batch = nb; g.M = g.N = N; g.sym = 1;
+      g.batch = nb;
       g.C = M + (int64_t)t0 * N * N; g.ldc = N; g.c_batch = (int64_t)N * N;
       g.beta = k0 ? 1.0 : 0.0; g.alpha_exp = alpha_exp; g.alpha_neg = alpha_neg;
-      if (slice_run(ctx, g, f, s) != LTGW_OK) return ctx->status();
+      if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
     }
   }
   return LTGW_OK;
@@ -396,17 +476,20 @@ ltgw_status emu_gemm(ltgw_ctx *ctx, int m, int n, int64_t K, const double *A, in
   bool done = false;
   if (sym) return slice_syrk(ctx, m, K, A, lda, C, 0.0, f, s, &done);
   SliceOperand a, b;
-  if (!slice_reserve(ctx, ctx->a5, f.required, [&](Arena &Ar) {
-        a.layout(Ar, m, K, 1, f);
-        b.layout(Ar, n, K, 1, f);
-      }))
+  double *part = nullptr;
+  const SliceGemmArgs plan = slice_plan(ctx, n, m, (int)((K + SL_K - 1) / SL_K), 0, 1, f);
+  if (!slice_fit(ctx, f.required,
+                 [&](Arena &Ar) {
+                   a.layout(Ar, m, K, 1, f);
+                   b.layout(Ar, n, K, 1, f);
+                 },
+                 [&] { return slice_partial(plan, 1, n); }, [] { return false; }, &part))
     return ctx->status();
   CHECK_LAUNCH(ctx, launch_slice_operand(a.source(A, lda, 0, m, K, false), f.ns, f.bits, 1, s), 3);
   CHECK_LAUNCH(ctx, launch_slice_operand(b.source(B, ldb, 0, n, K, false), f.ns, f.bits, 1, s), 3);
-  SliceGemmArgs g;   // the contiguous dimension of C is B's rows
-  g.A = b.dig; g.ea = b.exps; g.B = a.dig; g.eb = a.exps; g.nkb = a.nkb;
-  g.M = n; g.N = m; g.C = C; g.ldc = ldc;
-  return slice_run(ctx, g, f, s);
+  SliceGemmArgs g = plan;   // the contiguous dimension of C is B's rows
+  g.A = b.dig; g.ea = b.exps; g.B = a.dig; g.eb = a.exps; g.C = C; g.ldc = ldc;
+  return slice_run(ctx, g, part, s);
 }
 
 // Pi from slices (the emulated FP64 form): per frequency (n_tau == 0, Pi_j =
@@ -422,15 +505,22 @@ ltgw_status polarizability_emu(ltgw_ctx *ctx, int N, int64_t n_pairs, const doub
   const int64_t max_chunk = (int64_t)1 << 17;
   const int64_t n_chunks = (n_pairs + max_chunk - 1) / max_chunk;
   const int64_t chunk = std::min(n_pairs, ((n_pairs + n_chunks - 1) / n_chunks + 63) / 64 * 64);   // balanced
-  const int64_t per_t = slice_digit_bytes(N, (chunk + SL_K - 1) / SL_K, f.ns);
-  const int blk = (int)std::min<int64_t>(n_t, std::max<int64_t>(1, (int64_t)kSliceOperandMax / per_t));
   SliceOperand a, b;
-  double *fac = nullptr;
-  if (!slice_reserve(ctx, ctx->a5, true, [&](Arena &A) {
-        a.layout(A, N, chunk, blk, f);
-        b.layout(A, N, chunk, 1, f);
-        fac = A.take<double>((size_t)n_t * chunk);
-      }))
+  double *fac = nullptr, *part = nullptr;
+  const int nkb = (int)((chunk + SL_K - 1) / SL_K);
+  const size_t each = slice_digit_bytes(N, nkb, f.ns);
+  const SliceGemmArgs plan = slice_plan(ctx, N, N, nkb, 1, planned_piece(n_t, each, each), f);
+  int blk = n_t;
+  if (!slice_fit(
+          ctx, f.required,
+          [&](Arena &A) {
+            a.layout(A, N, chunk, blk, f);
+            b.layout(A, N, chunk, 1, f);
+            fac = A.take<double>((size_t)n_t * chunk);
+          },
+          [&] { return slice_partial(plan, blk, N); },
+          [&] { return next_piece(n_t, &blk); },
+          &part))
     return ctx->status();
   ctx->mark(EV_PI0, s);
   const int mode = n_tau ? (lt_form == 2 ? SCALE_EXPTAU : SCALE_LAPLACE) : SCALE_DIRECT;
@@ -445,12 +535,11 @@ ltgw_status polarizability_emu(ltgw_ctx *ctx, int N, int64_t n_pairs, const doub
       SliceSrc sa = a.source(Bt + k0, ldb, 0, N, kc, false);
       sa.colscale = fac + (int64_t)t0 * kc; sa.cs_batch = kc;
       CHECK_LAUNCH(ctx, launch_slice_operand(sa, f.ns, f.bits, nb, s), 3);
-      SliceGemmArgs g;
+      SliceGemmArgs g = plan;
       g.A = a.dig; g.a_batch = a.dig_batch; g.ea = a.exps; g.ea_batch = a.rows_p;
-      g.B = b.dig; g.eb = b.exps; g.nkb = a.nkb; g.batch = nb;
-      g.M = g.N = N; g.sym = 1; g.C = out + (int64_t)t0 * N * N; g.ldc = N; g.c_batch = (int64_t)N * N;
+      g.B = b.dig; g.eb = b.exps; g.batch = nb; g.C = out + (int64_t)t0 * N * N; g.ldc = N; g.c_batch = (int64_t)N * N;
       g.beta = k0 ? 1.0 : 0.0; g.alpha_exp = n_tau ? 0 : spin; g.alpha_neg = n_tau ? 0 : 1;   // -2 s: -2 or -4
-      if (slice_run(ctx, g, f, s) != LTGW_OK) return ctx->status();
+      if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
     }
   }
   ctx->mark(EV_PI1, s);
@@ -889,17 +978,27 @@ ltgw_status naf_metric_tc(ltgw_ctx *ctx, int n, int64_t n_pairs, const double *B
 // C_j = [1 - Pi_j]^-1 - 1 (Eq. ScreenedCoulombOrbital): the blocked sweep with
 // its updates from digits where N is past one pivot block of 128 by more than a
 // sliver (N = 130: 0.76 ms, FP64 tiles 0.56; N = 160: 0.59 against 0.85) and the
-// digits' memory is there, else on the FP64 tiles.
+// digits of one frequency fit, else on the FP64 tiles.
 constexpr int kScreenDigitsMinN = 144;
 
 ltgw_status screen_step(ltgw_ctx *ctx, int N, int n_omega, const double *Pi, double *work, double *C, cudaStream_t s) {
-  int nl = 0;
+  int nl = 0, blk = n_omega;
   void *digits = nullptr;
-  const size_t bytes = screen_digit_bytes(N, n_omega);
+  double *part = nullptr;
   const bool use = N >= kScreenDigitsMinN && N <= 65535 && n_omega <= 65535 &&
-                   slice_reserve(ctx, ctx->a5, false, [&](Arena &A) { digits = A.take<uint8_t>(bytes); });
-  const cudaError_t e = use ? launch_screen_digits(Pi, N, n_omega, work, digits, C, ctx->flags, ctx->n_sm, s, &nl)
-                            : launch_screen_blocked(Pi, N, n_omega, work, C, ctx->flags, s, &nl);
+                   slice_fit(
+                       ctx, false, [&](Arena &A) { digits = A.take<uint8_t>(screen_digit_bytes(N, blk)); },
+                       [] { return (size_t)0; },
+                       [&] { return next_piece(n_omega, &blk); },
+                       &part);
+  cudaError_t e = cudaSuccess;
+  if (use) {
+    for (int j0 = 0; j0 < n_omega && e == cudaSuccess; j0 += blk)
+      e = launch_screen_digits(Pi + (int64_t)j0 * N * N, N, std::min(blk, n_omega - j0), work, digits,
+                               C + (int64_t)j0 * N * N, ctx->flags, ctx->n_sm, s, &nl);
+  } else {
+    e = launch_screen_blocked(Pi, N, n_omega, work, C, ctx->flags, s, &nl);
+  }
   ctx->launches += nl;
   if (e != cudaSuccess) ctx->fail(LTGW_ERR_DEVICE, std::string("screen: ") + cudaGetErrorString(e));
   return ctx->status();
@@ -1175,6 +1274,12 @@ ltgw_status ltgw_trim(ltgw_ctx *ctx) {
 ltgw_status ltgw_set_autotune(ltgw_ctx *ctx, int on) {
   if (!ctx) return LTGW_ERR_BAD_ARG;
   ctx->autotune = (on != 0);
+  return LTGW_OK;
+}
+
+ltgw_status ltgw_set_digit_memory(ltgw_ctx *ctx, size_t bytes) {
+  if (!ctx) return LTGW_ERR_BAD_ARG;
+  ctx->digit_max = bytes;
   return LTGW_OK;
 }
 

@@ -263,6 +263,9 @@ struct SliceGemmArgs {
 };
 // Tiles and K splits for the shape; returns the bytes `partial` needs (0: none).
 size_t slice_gemm_plan(SliceGemmArgs *g, int n_sm, size_t max_partial);
+// The same for a piece of a planned product (fewer matrices or columns): its
+// tiles with the plan's K splits.
+size_t slice_gemm_piece(SliceGemmArgs *g);
 cudaError_t launch_slice_gemm(const SliceGemmArgs &g, int n_sm, cudaStream_t s);
 cudaError_t launch_slice_coldot_reduce(const SliceGemmArgs &g, double *W, int64_t ldw, cudaStream_t s);
 // C[m][n] = C[n][m] for m > n.

@@ -932,6 +932,11 @@ void slice_gemm_tiles(SliceGemmArgs *g) {
   if (!g->levels) g->levels = g->bits == 8 && (g->nkb - g->kb_first) < 256 ? g->ns + 1 : g->ns;
 }
 
+size_t slice_gemm_piece(SliceGemmArgs *g) {
+  slice_gemm_tiles(g);
+  return g->splits > 1 ? (size_t)g->splits * g->batch * g->n_tiles * SG_M * SG_N * sizeof(double) : 0;
+}
+
 size_t slice_gemm_plan(SliceGemmArgs *g, int n_sm, size_t max_partial) {
   slice_gemm_tiles(g);
   const int nkb = g->nkb - g->kb_first;
@@ -949,7 +954,7 @@ size_t slice_gemm_plan(SliceGemmArgs *g, int n_sm, size_t max_partial) {
   }
   g->kb_per_split = (nkb + best - 1) / best;
   g->splits = (nkb + g->kb_per_split - 1) / g->kb_per_split;
-  return g->splits > 1 ? (size_t)g->splits * part1 : 0;
+  return slice_gemm_piece(g);
 }
 
 cudaError_t launch_slice_gemm(const SliceGemmArgs &g, int n_sm, cudaStream_t s) {

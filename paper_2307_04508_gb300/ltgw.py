@@ -78,6 +78,7 @@ SIGNATURES = {
     "ltgw_set_autotune": (_I, [_P, _I]),
     "ltgw_workspace_bytes": (ctypes.c_size_t, [_P]),
     "ltgw_trim": (_I, [_P]),
+    "ltgw_set_digit_memory": (_I, [_P, ctypes.c_size_t]),
     "ltgw_get_stats": (_I, [_P, ctypes.POINTER(Stats)]),
     "ltgw_solve": (_I, [_P, ctypes.POINTER(Params), _P, _P, _P, _P, _I, _P, _P, _P, _P, _P, _P, _P]),
     "ltgw_solve_ev": (_I, [_P, ctypes.POINTER(Params), _P, _P, _P, _P, _I, _P, _P, _P, _I, _D, _P, _P, _P,
@@ -265,6 +266,9 @@ class Context:
 
     def trim(self):
         self._check(self._lib.ltgw_trim(self.handle))
+
+    def set_digit_memory(self, nbytes: int):
+        self._check(self._lib.ltgw_set_digit_memory(self.handle, int(nbytes)))
 
     def stats(self) -> dict:
         s = Stats()
