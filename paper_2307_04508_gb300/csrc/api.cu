@@ -232,42 +232,37 @@ struct SliceOperand {
   }
 };
 
-// Memory for the digits (arena a5, `layout`) and the K-split partials (a4,
-// `partial()` bytes, into *part) of the largest piece that fits; `shrink` takes
+// Memory (arena a5) for the digits (`layout`) and the K-split partials
+// (`partial()` bytes, into *part) of the largest piece that fits; `shrink` takes
 // the next smaller piece and is false at the smallest.  False when that one does
 // not fit either: an error in the forms that need the digits, else the product is
 // left to the CUDA-core kernels.  Other contexts' solves size their own workspace
 // from what is free, so more than half of it is taken for the smallest piece only.
 template <class Layout, class Partial, class Shrink>
 bool slice_fit(ltgw_ctx *ctx, bool required, Layout &&layout, Partial &&partial, Shrink &&shrink, double **part) {
+  Arena &ar = ctx->a5;
   for (;;) {
     const size_t pb = partial();
-    auto layout4 = [&](Arena &A) { *part = pb ? A.take<double>(pb / sizeof(double)) : nullptr; };
-    ctx->a5.begin_sizing();
-    layout(ctx->a5);
-    ctx->a4.begin_sizing();
-    layout4(ctx->a4);
-    const size_t n5 = ctx->a5.need, n4 = pb ? ctx->a4.need : 0;
-    ctx->a5.sizing = ctx->a4.sizing = false;
-    bool ok = n5 + n4 <= ctx->digit_max, tried = false;
-    const size_t grow = (n5 > ctx->a5.cap ? n5 : 0) + (n4 > ctx->a4.cap ? n4 : 0);
-    if (ok && grow) {
+    auto all = [&] {
+      layout(ar);
+      *part = pb ? ar.take<double>(pb / sizeof(double)) : nullptr;
+    };
+    ar.begin_sizing();
+    all();
+    ar.sizing = false;
+    const bool allowed = required || ar.need <= ctx->digit_max;
+    bool ok = ar.need <= ctx->digit_max;
+    if (ok && ar.need > ar.cap) {
       size_t free_b = 0, total_b = 0;
       if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
-      else ok = grow <= (free_b + (n5 > ctx->a5.cap ? ctx->a5.cap : 0) + (n4 > ctx->a4.cap ? ctx->a4.cap : 0)) / 2;
-      tried = true;
+      else ok = ar.need <= (free_b + ar.cap) / 2;
     }
     if (!ok && shrink()) continue;
-    if (ok || required || (tried && n5 + n4 <= ctx->digit_max)) {
-      ctx->a5.need = n5;
-      ctx->a4.need = n4;
-      if (ctx->a5.commit() == cudaSuccess && ctx->a4.commit() == cudaSuccess) {
-        layout(ctx->a5);
-        layout4(ctx->a4);
-        return true;
-      }
-      if (ok && shrink()) continue;
+    if (allowed && ar.commit() == cudaSuccess) {
+      all();
+      return true;
     }
+    if (ok && shrink()) continue;
     if (required) ctx->fail(LTGW_ERR_NOMEM, "slice operand allocation failed");
     return false;
   }
@@ -279,6 +274,13 @@ bool next_piece(int n, int *blk) {
   int pieces = (n + *blk - 1) / *blk, b = *blk;
   while (b >= *blk) b = (n + pieces) / (pieces + 1), ++pieces;
   *blk = b;
+  return true;
+}
+
+// The next fewer columns of one matrix.
+bool next_columns(int64_t *cols) {
+  if (*cols <= kSliceMinCols) return false;
+  *cols = (*cols / 2 + 127) / 128 * 128;
   return true;
 }
 
@@ -349,71 +351,78 @@ ltgw_status slice_project(ltgw_ctx *ctx, int N, int n_aux, const double *Ut, con
                           SliceForm f, cudaStream_t s, bool *done) {
   SliceOperand u, x;
   double *part = nullptr;
+  const int nkb = (n_aux + SL_K - 1) / SL_K;
+  const SliceGemmArgs plan =
+      slice_plan(ctx, (int)cols, N, nkb, 0, planned_piece(batch, slice_digit_bytes(cols, nkb, f.ns), 0), f);
+  int nb = batch;         // a piece: nb matrices, or some columns of one
   int64_t chunk = cols;
-  const SliceGemmArgs plan = slice_plan(ctx, (int)cols, N, (n_aux + SL_K - 1) / SL_K, 0, batch, f);
   *done = slice_fit(
       ctx, f.required,
       [&](Arena &A) {
         u.layout(A, N, n_aux, 1, f);
-        x.layout(A, chunk, n_aux, batch, f);
+        x.layout(A, chunk, n_aux, nb, f);
       },
-      [&] { return slice_partial(plan, batch, (int)chunk); },
-      [&] {
-        if (chunk <= kSliceMinCols) return false;
-        chunk = (chunk / 2 + 127) / 128 * 128;
-        return true;
-      },
-      &part);
+      [&] { return slice_partial(plan, nb, (int)chunk); },
+      [&] { return next_piece(batch, &nb) || next_columns(&chunk); }, &part);
   if (!*done) return ctx->status();
   CHECK_LAUNCH(ctx, launch_slice_operand(u.source(Ut, n_aux, 0, N, n_aux, false), f.ns, f.bits, 1, s), 3);
-  for (int64_t c0 = 0; c0 < cols; c0 += chunk) {
-    const int cc = (int)std::min(chunk, cols - c0);
-    CHECK_LAUNCH(ctx, launch_slice_operand(x.source(X + c0, ld, x_batch, cc, n_aux, true), f.ns, f.bits, batch, s), 3);
-    SliceGemmArgs g = plan;
-    g.A = x.dig; g.a_batch = x.dig_batch; g.ea = x.exps; g.ea_batch = x.rows_p;
-    g.B = u.dig; g.eb = u.exps; g.M = cc; g.C = out + c0; g.ldc = ld_out; g.c_batch = out_batch;
-    if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
+  for (int t0 = 0; t0 < batch; t0 += nb) {
+    for (int64_t c0 = 0; c0 < cols; c0 += chunk) {
+      const int cc = (int)std::min(chunk, cols - c0), bb = std::min(nb, batch - t0);
+      CHECK_LAUNCH(ctx, launch_slice_operand(x.source(X + t0 * x_batch + c0, ld, x_batch, cc, n_aux, true), f.ns,
+                                             f.bits, bb, s), 3);
+      SliceGemmArgs g = plan;
+      g.A = x.dig; g.a_batch = x.dig_batch; g.ea = x.exps; g.ea_batch = x.rows_p;
+      g.B = u.dig; g.eb = u.exps; g.batch = bb; g.M = cc;
+      g.C = out + t0 * out_batch + c0; g.ldc = ld_out; g.c_batch = out_batch;
+      if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
+    }
   }
   return LTGW_OK;
 }
 
 // W_j[t][c] = sum_PQ Btt[t][P][c] C_j[P][Q] Btt[t][Q][c] (Eq. ScreenedCoulombOrbital)
-// with the column dot in the contraction's epilogue; frequencies in blocks.
+// with the column dot in the contraction's epilogue; pieces of frequencies,
+// then of targets, then of one target's columns.
 ltgw_status slice_wnm(ltgw_ctx *ctx, int N, int n_omega, const double *C, int T, int n_orb_act, const double *Btt,
                       int64_t ld_btt, int64_t stride_btt, double *W, SliceForm f, cudaStream_t s, bool *done) {
   const int cols = T * n_orb_act;
   SliceOperand r, c;
-  double *cd = nullptr;
-  double *part = nullptr;   // the column dot takes no K splits
+  double *cd = nullptr, *part = nullptr;   // the column dot takes no K splits
   const int tiles_n = (N + 63) / 64;
-  int blk = n_omega;
+  int blk = n_omega, tb = T;
+  int64_t cc = n_orb_act;
   *done = slice_fit(
       ctx, f.required,
       [&](Arena &A) {
-        r.layout(A, cols, N, 1, f);
+        r.layout(A, tb * cc, N, 1, f);
         c.layout(A, N, N, blk, f);
-        cd = A.take<double>((size_t)blk * 4 * tiles_n * cols);
+        cd = A.take<double>((size_t)blk * 4 * tiles_n * tb * cc);
       },
       [] { return (size_t)0; },
-      [&] { return next_piece(n_omega, &blk); },
-      &part);
+      [&] { return next_piece(n_omega, &blk) || next_piece(T, &tb) || next_columns(&cc); }, &part);
   if (!*done) return ctx->status();
-  SliceSrc rs = r.source(Btt, ld_btt, 0, cols, N, true);
-  rs.col_group = n_orb_act; rs.col_stride = stride_btt;
-  CHECK_LAUNCH(ctx, launch_slice_operand(rs, f.ns, f.bits, 1, s), 3);
-  for (int j0 = 0; j0 < n_omega; j0 += blk) {
-    const int nb = std::min(blk, n_omega - j0);
-    CHECK_LAUNCH(ctx, launch_slice_operand(c.source(C + (int64_t)j0 * N * N, N, (int64_t)N * N, N, N, false), f.ns,
-                                           f.bits, nb, s), 3);
-    SliceGemmArgs g;
-    g.A = r.dig; g.ea = r.exps;
-    g.B = c.dig; g.b_batch = c.dig_batch; g.eb = c.exps; g.eb_batch = c.rows_p;
-    g.ns = f.ns; g.bits = f.bits; g.nkb = r.nkb; g.batch = nb; g.M = cols; g.N = N;
-    g.cd_B = Btt; g.cd_ld = ld_btt; g.cd_stride = stride_btt; g.cd_cols = n_orb_act; g.cd_out = cd; g.cd_ldo = cols;
-    slice_gemm_plan(&g, ctx->n_sm, 0);
-    if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
-    CHECK_LAUNCH(ctx, launch_slice_coldot_reduce(g, W + (int64_t)j0 * cols, cols, s), 1);
-  }
+  for (int t0 = 0; t0 < T; t0 += tb)
+    for (int64_t c0 = 0; c0 < n_orb_act; c0 += cc) {
+      const int nc = (int)std::min<int64_t>(cc, n_orb_act - c0), m = std::min(tb, T - t0) * nc;
+      const double *B = Btt + t0 * stride_btt + c0;
+      SliceSrc rs = r.source(B, ld_btt, 0, m, N, true);
+      rs.col_group = nc; rs.col_stride = stride_btt;
+      CHECK_LAUNCH(ctx, launch_slice_operand(rs, f.ns, f.bits, 1, s), 3);
+      for (int j0 = 0; j0 < n_omega; j0 += blk) {
+        const int nb = std::min(blk, n_omega - j0);
+        CHECK_LAUNCH(ctx, launch_slice_operand(c.source(C + (int64_t)j0 * N * N, N, (int64_t)N * N, N, N, false), f.ns,
+                                               f.bits, nb, s), 3);
+        SliceGemmArgs g;
+        g.A = r.dig; g.ea = r.exps;
+        g.B = c.dig; g.b_batch = c.dig_batch; g.eb = c.exps; g.eb_batch = c.rows_p;
+        g.ns = f.ns; g.bits = f.bits; g.nkb = r.nkb; g.batch = nb; g.M = m; g.N = N;
+        g.cd_B = B; g.cd_ld = ld_btt; g.cd_stride = stride_btt; g.cd_cols = nc; g.cd_out = cd; g.cd_ldo = m;
+        slice_gemm_plan(&g, ctx->n_sm, 0);
+        if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
+        CHECK_LAUNCH(ctx, launch_slice_coldot_reduce(g, W + (int64_t)j0 * cols + (int64_t)t0 * n_orb_act + c0, cols, s), 1);
+      }
+    }
   return LTGW_OK;
 }
 

@@ -71,14 +71,16 @@ def test_screening_in_pieces_has_the_same_bits():
     assert np.abs(got[2] - got[0]).max() <= 1e-12 * np.abs(got[0]).max()
 
 
-def _solve(prec, limit, n_tgt=3):
+def _solve(prec, limit, sizes=(12, 100, 300), n_tgt=3, naf=1e-2, held=None):
     from paper_2307_04508_gb300 import ltgw
-    p = S.make_problem(12, 100, 300, n_frozen=2, seed=5, n_targets=n_tgt)
-    q = ltgw.make_params(12, 100, 300, 2, 16, 6, 0.5, 1e-2, 2, True, prec)
+    p = S.make_problem(*sizes, n_frozen=2, seed=5, n_targets=n_tgt)
+    q = ltgw.make_params(*sizes, 2, 16, 6, 0.5, naf, 2, True, prec)
     T = len(p.targets)
     sig, e, st = np.zeros((T, 16, 2)), np.zeros(T), np.zeros(T, dtype=np.int32)
     c = _ctx(limit)
     c.solve(q, p.eps, p.B_ov, p.B_tgt, p.targets.astype(np.int32), p.shift, sig, e, st)
+    if held is not None:
+        held.append(c.workspace_bytes())
     c.close()
     return sig
 
@@ -93,6 +95,21 @@ def test_solve_in_pieces_has_the_same_bits(emu):
     assert np.array_equal(_solve(prec, 14 * MB), whole)
     low = _solve(prec, 0)
     assert np.array_equal(low, whole) if emu else np.abs(low - whole).max() <= 1e-9 * np.abs(whole).max()
+
+
+@pytest.mark.parametrize("emu", [False, True])
+@pytest.mark.parametrize("naf", [1e-2, -1.0])
+def test_many_targets_in_pieces_have_the_same_bits(emu, naf):
+    """64 targets of 74 orbitals: 24 MB of digits in the projection, 14 MB in W_nm
+    without NAF (a seventh less emulated), above the limit, which the other
+    products keep to in pieces of one moment; the targets run in pieces too."""
+    from paper_2307_04508_gb300 import ltgw
+    prec = ltgw.LTGW_FP64_EMU if emu else ltgw.LTGW_FP64
+    args, held = ((36, 40, 200), 64, naf), []
+    whole = _solve(prec, None, *args)
+    assert np.array_equal(_solve(prec, 13 * MB, *args, held), whole)
+    _solve(prec, 0, *args, held)
+    assert held[0] <= held[1] + 13 * MB
 
 
 def test_pi_chunks_of_a_long_sum():
