@@ -417,7 +417,8 @@ typedef struct ltgw_server ltgw_server;
  * requests; that retained workspace counts against admission. */
 ltgw_status ltgw_server_create(ltgw_server **out, int device, int n_slots, size_t hbm_budget_bytes);
 /* Queue a request (never blocks on the GPU); LTGW_ERR_NOMEM if its estimated
- * footprint alone exceeds the budget. */
+ * footprint without the digit workspace (which then takes what the budget
+ * leaves, see ltgw_set_digit_memory) alone exceeds the budget. */
 ltgw_status ltgw_server_submit(ltgw_server *srv, const ltgw_request *req, uint64_t *ticket);
 /* Move up to max_out completions (oldest first) into out; returns how many. */
 int ltgw_server_poll(ltgw_server *srv, ltgw_completion *out, int max_out);
@@ -426,7 +427,9 @@ ltgw_status ltgw_server_wait_all(ltgw_server *srv, double timeout_s);
 /* Finish the running requests, drop the queued ones, release everything. */
 void ltgw_server_destroy(ltgw_server *srv);
 /* Estimated device bytes of one solve (inputs staged + workspace, tensor-core
- * partial tiles included; with NAF the post-NAF size is taken as n_aux / 2). */
+ * partial tiles included, and a digit workspace of 640 MiB or what the smallest
+ * pieces need, to which the server's contexts keep; with NAF the post-NAF size
+ * is taken as n_aux / 2). */
 size_t ltgw_request_footprint(const ltgw_params *p, int n_tgt);
 
 /* ---- allocation-free screening ------------------------------------------ */

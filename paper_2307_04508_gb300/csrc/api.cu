@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "digit_memory.h"
 #include "kernels.cuh"
 
 namespace ltgw {
@@ -71,8 +72,6 @@ enum Stage { EV_START = 0, EV_NAF, EV_PI0, EV_PI1, EV_PI, EV_SCREEN, EV_WNM, EV_
              EV_K0, EV_VEC1, EV_COUNT };
 
 }  // namespace
-
-constexpr size_t kSliceHold = (size_t)6 << 30;   // default of ltgw_set_digit_memory
 
 struct ltgw_ctx {
   int device = 0;
@@ -212,6 +211,8 @@ bool slices_pay(int64_t m, int64_t n, int64_t k, int64_t batch) {
   return k >= 48 && (double)m * (double)n * (double)k * (double)batch >= 2e6;
 }
 
+int slice_blocks(int64_t K) { return (int)((K + SL_K - 1) / SL_K); }
+
 struct SliceOperand {
   uint8_t *dig = nullptr;
   int *exps = nullptr;
@@ -219,7 +220,7 @@ struct SliceOperand {
   int64_t dig_batch = 0;
   void layout(Arena &A, int64_t rows, int64_t K, int batch, SliceForm f) {
     rows_p = (int)slice_rows_padded(rows);
-    nkb = (int)((K + SL_K - 1) / SL_K);
+    nkb = slice_blocks(K);
     dig_batch = slice_digit_bytes(rows, nkb, f.ns);
     dig = A.take<uint8_t>((size_t)dig_batch * batch);
     exps = A.take<int>((size_t)rows_p * batch);
@@ -231,42 +232,6 @@ struct SliceOperand {
     return a;
   }
 };
-
-// Memory (arena a5) for the digits (`layout`) and the K-split partials
-// (`partial()` bytes, into *part) of the largest piece that fits; `shrink` takes
-// the next smaller piece and is false at the smallest.  False when that one does
-// not fit either: an error in the forms that need the digits, else the product is
-// left to the CUDA-core kernels.  Other contexts' solves size their own workspace
-// from what is free, so more than half of it is taken for the smallest piece only.
-template <class Layout, class Partial, class Shrink>
-bool slice_fit(ltgw_ctx *ctx, bool required, Layout &&layout, Partial &&partial, Shrink &&shrink, double **part) {
-  Arena &ar = ctx->a5;
-  for (;;) {
-    const size_t pb = partial();
-    auto all = [&] {
-      layout(ar);
-      *part = pb ? ar.take<double>(pb / sizeof(double)) : nullptr;
-    };
-    ar.begin_sizing();
-    all();
-    ar.sizing = false;
-    const bool allowed = required || ar.need <= ctx->digit_max;
-    bool ok = ar.need <= ctx->digit_max;
-    if (ok && ar.need > ar.cap) {
-      size_t free_b = 0, total_b = 0;
-      if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
-      else ok = ar.need <= (free_b + ar.cap) / 2;
-    }
-    if (!ok && shrink()) continue;
-    if (allowed && ar.commit() == cudaSuccess) {
-      all();
-      return true;
-    }
-    if (ok && shrink()) continue;
-    if (required) ctx->fail(LTGW_ERR_NOMEM, "slice operand allocation failed");
-    return false;
-  }
-}
 
 // The next smaller equal pieces of n items; false when they are single already.
 bool next_piece(int n, int *blk) {
@@ -282,6 +247,47 @@ bool next_columns(int64_t *cols) {
   if (*cols <= kSliceMinCols) return false;
   *cols = (*cols / 2 + 127) / 128 * 128;
   return true;
+}
+
+// Each product below has a struct of its piece: layout(arena) takes its digits,
+// partial() is the bytes of its K-split partials (pointer `part`), shrink() takes
+// the next smaller piece and is false at the smallest.
+template <class P>
+size_t piece_bytes(Arena &ar, P &p) {
+  ar.begin_sizing();
+  p.layout(ar);
+  if (const size_t pb = p.partial()) ar.take<double>(pb / sizeof(double));
+  ar.sizing = false;
+  return ar.need;
+}
+
+// Memory (arena a5) for the largest piece that fits.  False when the smallest one
+// does not either: an error in the forms that need the digits, else the product is
+// left to the CUDA-core kernels.  Other contexts' solves size their own workspace
+// from what is free, so more than half of it is taken for the smallest piece only.
+template <class P>
+bool slice_fit(ltgw_ctx *ctx, bool required, P &p) {
+  Arena &ar = ctx->a5;
+  for (;;) {
+    const size_t need = piece_bytes(ar, p);
+    const bool allowed = required || need <= ctx->digit_max;
+    bool ok = need <= ctx->digit_max;
+    if (ok && need > ar.cap) {
+      size_t free_b = 0, total_b = 0;
+      if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
+      else ok = need <= (free_b + ar.cap) / 2;
+    }
+    if (!ok && p.shrink()) continue;
+    if (allowed && ar.commit() == cudaSuccess) {
+      p.layout(ar);
+      const size_t pb = p.partial();
+      p.part = pb ? ar.take<double>(pb / sizeof(double)) : nullptr;
+      return true;
+    }
+    if (ok && p.shrink()) continue;
+    if (required) ctx->fail(LTGW_ERR_NOMEM, "slice operand allocation failed");
+    return false;
+  }
 }
 
 // One piece of a digit contraction planned by slice_plan.
@@ -301,11 +307,11 @@ int planned_piece(int n, size_t each, size_t shared) {
 
 // The plan of a product (M, N, nkb, sym, matrices of a piece): its K splits hold
 // for every piece.
-SliceGemmArgs slice_plan(const ltgw_ctx *ctx, int M, int N, int nkb, int sym, int batch, SliceForm f) {
+SliceGemmArgs slice_plan(int n_sm, int M, int N, int nkb, int sym, int batch, SliceForm f) {
   SliceGemmArgs g;
   g.ns = f.ns; g.bits = f.bits;
   g.M = M; g.N = N; g.nkb = nkb; g.sym = sym; g.batch = batch;
-  slice_gemm_plan(&g, ctx->n_sm, kSlicePartialMax);
+  slice_gemm_plan(&g, n_sm, kSlicePartialMax);
   return g;
 }
 // Bytes of its partials for a piece of `batch` matrices and M columns.
@@ -324,62 +330,98 @@ int64_t slice_k_chunk(int64_t rows, int64_t K, SliceForm f) {
   return std::min(K, ((K + n - 1) / n + 63) / 64 * 64);
 }
 
+struct SyrkPiece {   // C = X X^T: one pair chunk
+  SliceForm f;
+  int n;
+  int64_t chunk;
+  SliceGemmArgs plan;
+  SliceOperand o;
+  double *part = nullptr;
+  SyrkPiece(int n_sm, int n_, int64_t K, SliceForm f_) : f(f_), n(n_), chunk(slice_k_chunk(n_, K, f_)) {
+    plan = slice_plan(n_sm, n, n, slice_blocks(chunk), 1, 1, f);
+  }
+  void layout(Arena &A) { o.layout(A, n, chunk, 1, f); }
+  size_t partial() const { return slice_partial(plan, 1, n); }
+  bool shrink() { return false; }
+};
+
 // C = beta C + X X^T (full, symmetric bit for bit), X [n][ld] with K columns.
 // *done is false when the product was left to the caller (no memory).
 ltgw_status slice_syrk(ltgw_ctx *ctx, int n, int64_t K, const double *X, int64_t ld, double *C, double beta,
                        SliceForm f, cudaStream_t s, bool *done) {
-  SliceOperand o;
-  double *part = nullptr;
-  const int64_t chunk = slice_k_chunk(n, K, f);
-  const SliceGemmArgs plan = slice_plan(ctx, n, n, (int)((chunk + SL_K - 1) / SL_K), 1, 1, f);
-  *done = slice_fit(ctx, f.required, [&](Arena &A) { o.layout(A, n, chunk, 1, f); },
-                    [&] { return slice_partial(plan, 1, n); }, [] { return false; }, &part);
+  SyrkPiece p(ctx->n_sm, n, K, f);
+  *done = slice_fit(ctx, f.required, p);
   if (!*done) return ctx->status();
-  for (int64_t k0 = 0; k0 < K; k0 += chunk) {
-    const int64_t kc = std::min(chunk, K - k0);
-    CHECK_LAUNCH(ctx, launch_slice_operand(o.source(X + k0, ld, 0, n, kc, false), f.ns, f.bits, 1, s), 3);
-    SliceGemmArgs g = plan;
-    g.A = g.B = o.dig; g.ea = g.eb = o.exps; g.C = C; g.ldc = n; g.beta = k0 ? 1.0 : beta;
-    if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
+  for (int64_t k0 = 0; k0 < K; k0 += p.chunk) {
+    const int64_t kc = std::min(p.chunk, K - k0);
+    CHECK_LAUNCH(ctx, launch_slice_operand(p.o.source(X + k0, ld, 0, n, kc, false), f.ns, f.bits, 1, s), 3);
+    SliceGemmArgs g = p.plan;
+    g.A = g.B = p.o.dig; g.ea = g.eb = p.o.exps; g.C = C; g.ldc = n; g.beta = k0 ? 1.0 : beta;
+    if (slice_run(ctx, g, p.part, s) != LTGW_OK) return ctx->status();
   }
   return LTGW_OK;
 }
+
+struct ProjectPiece {   // some of the matrices X_b, or some columns of one
+  SliceForm f;
+  int N, n_aux, batch, nb;
+  int64_t chunk;
+  SliceGemmArgs plan;
+  SliceOperand u, x;
+  double *part = nullptr;
+  ProjectPiece(int n_sm, int N_, int n_aux_, int64_t cols, int batch_, SliceForm f_)
+      : f(f_), N(N_), n_aux(n_aux_), batch(batch_), nb(batch_), chunk(cols) {
+    const int nkb = slice_blocks(n_aux);
+    plan = slice_plan(n_sm, (int)cols, N, nkb, 0, planned_piece(batch, slice_digit_bytes(cols, nkb, f.ns), 0), f);
+  }
+  void layout(Arena &A) {
+    u.layout(A, N, n_aux, 1, f);
+    x.layout(A, chunk, n_aux, nb, f);
+  }
+  size_t partial() const { return slice_partial(plan, nb, (int)chunk); }
+  bool shrink() { return next_piece(batch, &nb) || next_columns(&chunk); }
+};
 
 // out_b [N][ld_out] = Ut X_b for the columns of X_b [n_aux][ld] (Ut rows [N][n_aux]).
 ltgw_status slice_project(ltgw_ctx *ctx, int N, int n_aux, const double *Ut, const double *X, int64_t ld,
                           int64_t x_batch, int64_t cols, int batch, double *out, int64_t ld_out, int64_t out_batch,
                           SliceForm f, cudaStream_t s, bool *done) {
-  SliceOperand u, x;
-  double *part = nullptr;
-  const int nkb = (n_aux + SL_K - 1) / SL_K;
-  const SliceGemmArgs plan =
-      slice_plan(ctx, (int)cols, N, nkb, 0, planned_piece(batch, slice_digit_bytes(cols, nkb, f.ns), 0), f);
-  int nb = batch;         // a piece: nb matrices, or some columns of one
-  int64_t chunk = cols;
-  *done = slice_fit(
-      ctx, f.required,
-      [&](Arena &A) {
-        u.layout(A, N, n_aux, 1, f);
-        x.layout(A, chunk, n_aux, nb, f);
-      },
-      [&] { return slice_partial(plan, nb, (int)chunk); },
-      [&] { return next_piece(batch, &nb) || next_columns(&chunk); }, &part);
+  ProjectPiece p(ctx->n_sm, N, n_aux, cols, batch, f);
+  *done = slice_fit(ctx, f.required, p);
   if (!*done) return ctx->status();
+  const SliceOperand &u = p.u, &x = p.x;
   CHECK_LAUNCH(ctx, launch_slice_operand(u.source(Ut, n_aux, 0, N, n_aux, false), f.ns, f.bits, 1, s), 3);
-  for (int t0 = 0; t0 < batch; t0 += nb) {
-    for (int64_t c0 = 0; c0 < cols; c0 += chunk) {
-      const int cc = (int)std::min(chunk, cols - c0), bb = std::min(nb, batch - t0);
+  for (int t0 = 0; t0 < batch; t0 += p.nb) {
+    for (int64_t c0 = 0; c0 < cols; c0 += p.chunk) {
+      const int cc = (int)std::min(p.chunk, cols - c0), bb = std::min(p.nb, batch - t0);
       CHECK_LAUNCH(ctx, launch_slice_operand(x.source(X + t0 * x_batch + c0, ld, x_batch, cc, n_aux, true), f.ns,
                                              f.bits, bb, s), 3);
-      SliceGemmArgs g = plan;
+      SliceGemmArgs g = p.plan;
       g.A = x.dig; g.a_batch = x.dig_batch; g.ea = x.exps; g.ea_batch = x.rows_p;
       g.B = u.dig; g.eb = u.exps; g.batch = bb; g.M = cc;
       g.C = out + t0 * out_batch + c0; g.ldc = ld_out; g.c_batch = out_batch;
-      if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
+      if (slice_run(ctx, g, p.part, s) != LTGW_OK) return ctx->status();
     }
   }
   return LTGW_OK;
 }
+
+struct WnmPiece {   // some frequencies, then some targets, then some columns of one
+  SliceForm f;
+  int N, n_omega, T, blk, tb;
+  int64_t cc;
+  SliceOperand r, c;
+  double *cd = nullptr, *part = nullptr;   // the column dot takes no K splits
+  WnmPiece(int N_, int n_omega_, int T_, int cols, SliceForm f_)
+      : f(f_), N(N_), n_omega(n_omega_), T(T_), blk(n_omega_), tb(T_), cc(cols) {}
+  void layout(Arena &A) {
+    r.layout(A, tb * cc, N, 1, f);
+    c.layout(A, N, N, blk, f);
+    cd = A.take<double>((size_t)blk * 4 * ((N + 63) / 64) * tb * cc);
+  }
+  size_t partial() const { return 0; }
+  bool shrink() { return next_piece(n_omega, &blk) || next_piece(T, &tb) || next_columns(&cc); }
+};
 
 // W_j[t][c] = sum_PQ Btt[t][P][c] C_j[P][Q] Btt[t][Q][c] (Eq. ScreenedCoulombOrbital)
 // with the column dot in the contraction's epilogue; pieces of frequencies,
@@ -387,21 +429,12 @@ ltgw_status slice_project(ltgw_ctx *ctx, int N, int n_aux, const double *Ut, con
 ltgw_status slice_wnm(ltgw_ctx *ctx, int N, int n_omega, const double *C, int T, int n_orb_act, const double *Btt,
                       int64_t ld_btt, int64_t stride_btt, double *W, SliceForm f, cudaStream_t s, bool *done) {
   const int cols = T * n_orb_act;
-  SliceOperand r, c;
-  double *cd = nullptr, *part = nullptr;   // the column dot takes no K splits
-  const int tiles_n = (N + 63) / 64;
-  int blk = n_omega, tb = T;
-  int64_t cc = n_orb_act;
-  *done = slice_fit(
-      ctx, f.required,
-      [&](Arena &A) {
-        r.layout(A, tb * cc, N, 1, f);
-        c.layout(A, N, N, blk, f);
-        cd = A.take<double>((size_t)blk * 4 * tiles_n * tb * cc);
-      },
-      [] { return (size_t)0; },
-      [&] { return next_piece(n_omega, &blk) || next_piece(T, &tb) || next_columns(&cc); }, &part);
+  WnmPiece p(N, n_omega, T, n_orb_act, f);
+  *done = slice_fit(ctx, f.required, p);
   if (!*done) return ctx->status();
+  const SliceOperand &r = p.r, &c = p.c;
+  const int blk = p.blk, tb = p.tb;
+  const int64_t cc = p.cc;
   for (int t0 = 0; t0 < T; t0 += tb)
     for (int64_t c0 = 0; c0 < n_orb_act; c0 += cc) {
       const int nc = (int)std::min<int64_t>(cc, n_orb_act - c0), m = std::min(tb, T - t0) * nc;
@@ -417,14 +450,37 @@ ltgw_status slice_wnm(ltgw_ctx *ctx, int N, int n_omega, const double *C, int T,
         g.A = r.dig; g.ea = r.exps;
         g.B = c.dig; g.b_batch = c.dig_batch; g.eb = c.exps; g.eb_batch = c.rows_p;
         g.ns = f.ns; g.bits = f.bits; g.nkb = r.nkb; g.batch = nb; g.M = m; g.N = N;
-        g.cd_B = B; g.cd_ld = ld_btt; g.cd_stride = stride_btt; g.cd_cols = nc; g.cd_out = cd; g.cd_ldo = m;
+        g.cd_B = B; g.cd_ld = ld_btt; g.cd_stride = stride_btt; g.cd_cols = nc; g.cd_out = p.cd; g.cd_ldo = m;
         slice_gemm_plan(&g, ctx->n_sm, 0);
-        if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
+        if (slice_run(ctx, g, nullptr, s) != LTGW_OK) return ctx->status();
         CHECK_LAUNCH(ctx, launch_slice_coldot_reduce(g, W + (int64_t)j0 * cols + (int64_t)t0 * n_orb_act + c0, cols, s), 1);
       }
     }
   return LTGW_OK;
 }
+
+struct PiPiece {   // some of the factor rows, one pair chunk
+  SliceForm f;
+  int N, n_t, blk;
+  int64_t chunk;
+  SliceGemmArgs plan;
+  SliceOperand o, o2;   // o2: the unsigned operand, written and read only where some factor is negative
+  double *fac = nullptr, *part = nullptr;
+  int *neg = nullptr;
+  PiPiece(int n_sm, int N_, int64_t n_pairs, int n_t_, SliceForm f_)
+      : f(f_), N(N_), n_t(n_t_), blk(n_t_), chunk(slice_k_chunk(2 * slice_rows_padded(N_), n_pairs, f_)) {
+    const int nkb = slice_blocks(chunk);
+    plan = slice_plan(n_sm, N, N, nkb, 1, planned_piece(n_t, 2 * slice_digit_bytes(N, nkb, f.ns), 0), f);
+  }
+  void layout(Arena &A) {
+    o.layout(A, N, chunk, blk, f);
+    o2.layout(A, N, chunk, blk, f);
+    fac = A.take<double>((size_t)n_t * 2 * chunk);
+    neg = A.take<int>(1);
+  }
+  size_t partial() const { return slice_partial(plan, blk, N); }
+  bool shrink() { return next_piece(n_t, &blk); }
+};
 
 // M_t = alpha (Bt diag(f_t)) Bt^T for t < n_t (full, symmetric).  Both operands
 // are Bt diag(sqrt |f_t|), the sign of f_t with the first one: an entry's error
@@ -434,27 +490,14 @@ ltgw_status slice_wnm(ltgw_ctx *ctx, int N, int n_omega, const double *C, int T,
 ltgw_status slice_pi(ltgw_ctx *ctx, int N, int64_t n_pairs, const double *Bt, int64_t ldb, const double *delta,
                      int n_t, const double *p0, const double *p1, int mode, int alpha_exp, int alpha_neg, double *M,
                      SliceForm f, cudaStream_t s, bool *done) {
-  SliceOperand o, o2;   // o2: the unsigned operand, written and read only where some factor is negative
-  double *fac = nullptr;
-  int *neg = nullptr;
-  double *part = nullptr;
-  const int64_t chunk = slice_k_chunk(2 * slice_rows_padded(N), n_pairs, f);
-  const int nkb = (int)((chunk + SL_K - 1) / SL_K);
-  const SliceGemmArgs plan =
-      slice_plan(ctx, N, N, nkb, 1, planned_piece(n_t, 2 * slice_digit_bytes(N, nkb, f.ns), 0), f);
-  int blk = n_t;
-  *done = slice_fit(
-      ctx, f.required,
-      [&](Arena &A) {
-        o.layout(A, N, chunk, blk, f);
-        o2.layout(A, N, chunk, blk, f);
-        fac = A.take<double>((size_t)n_t * 2 * chunk);
-        neg = A.take<int>(1);
-      },
-      [&] { return slice_partial(plan, blk, N); },
-      [&] { return next_piece(n_t, &blk); },
-      &part);
+  PiPiece p(ctx->n_sm, N, n_pairs, n_t, f);
+  *done = slice_fit(ctx, f.required, p);
   if (!*done) return ctx->status();
+  const SliceOperand &o = p.o, &o2 = p.o2;
+  double *const fac = p.fac;
+  int *const neg = p.neg;
+  const int64_t chunk = p.chunk;
+  const int blk = p.blk;
   for (int64_t k0 = 0; k0 < n_pairs; k0 += chunk) {
     const int64_t kc = std::min(chunk, n_pairs - k0);
     LTGW_CUDA(ctx, cudaMemsetAsync(neg, 0, sizeof(int), s));
@@ -467,39 +510,73 @@ ltgw_status slice_pi(ltgw_ctx *ctx, int N, int64_t n_pairs, const double *Bt, in
       SliceSrc b = o2.source(Bt + k0, ldb, 0, N, kc, false);
       b.colscale = fac + (int64_t)(n_t + t0) * kc; b.cs_batch = kc; b.only_if = neg;
       CHECK_LAUNCH(ctx, launch_slice_operand(b, f.ns, f.bits, nb, s), 3);
-      SliceGemmArgs g = plan;
+      SliceGemmArgs g = p.plan;
       g.A = g.B = o.dig; g.a_batch = g.b_batch = o.dig_batch; g.ea = g.eb = o.exps; g.ea_batch = g.eb_batch = o.rows_p;
       g.B_alt = o2.dig; g.b_sel = neg;   // |sqrt| rows have the same exponents
       g.batch = nb;
       g.C = M + (int64_t)t0 * N * N; g.ldc = N; g.c_batch = (int64_t)N * N;
       g.beta = k0 ? 1.0 : 0.0; g.alpha_exp = alpha_exp; g.alpha_neg = alpha_neg;
-      if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
+      if (slice_run(ctx, g, p.part, s) != LTGW_OK) return ctx->status();
     }
   }
   return LTGW_OK;
 }
+
+struct GemmPiece {   // the whole product
+  SliceForm f;
+  int m, n;
+  int64_t K;
+  SliceGemmArgs plan;
+  SliceOperand a, b;
+  double *part = nullptr;
+  GemmPiece(int n_sm, int m_, int n_, int64_t K_, SliceForm f_) : f(f_), m(m_), n(n_), K(K_) {
+    plan = slice_plan(n_sm, n, m, slice_blocks(K), 0, 1, f);
+  }
+  void layout(Arena &A) {
+    a.layout(A, m, K, 1, f);
+    b.layout(A, n, K, 1, f);
+  }
+  size_t partial() const { return slice_partial(plan, 1, n); }
+  bool shrink() { return false; }
+};
 
 // C [m][ldc] = A B^T from slices (sym: C = A A^T, whole).
 ltgw_status emu_gemm(ltgw_ctx *ctx, int m, int n, int64_t K, const double *A, int64_t lda, const double *B,
                      int64_t ldb, double *C, int64_t ldc, bool sym, SliceForm f, cudaStream_t s) {
   bool done = false;
   if (sym) return slice_syrk(ctx, m, K, A, lda, C, 0.0, f, s, &done);
-  SliceOperand a, b;
-  double *part = nullptr;
-  const SliceGemmArgs plan = slice_plan(ctx, n, m, (int)((K + SL_K - 1) / SL_K), 0, 1, f);
-  if (!slice_fit(ctx, f.required,
-                 [&](Arena &Ar) {
-                   a.layout(Ar, m, K, 1, f);
-                   b.layout(Ar, n, K, 1, f);
-                 },
-                 [&] { return slice_partial(plan, 1, n); }, [] { return false; }, &part))
-    return ctx->status();
+  GemmPiece p(ctx->n_sm, m, n, K, f);
+  if (!slice_fit(ctx, f.required, p)) return ctx->status();
+  const SliceOperand &a = p.a, &b = p.b;
   CHECK_LAUNCH(ctx, launch_slice_operand(a.source(A, lda, 0, m, K, false), f.ns, f.bits, 1, s), 3);
   CHECK_LAUNCH(ctx, launch_slice_operand(b.source(B, ldb, 0, n, K, false), f.ns, f.bits, 1, s), 3);
-  SliceGemmArgs g = plan;   // the contiguous dimension of C is B's rows
+  SliceGemmArgs g = p.plan;   // the contiguous dimension of C is B's rows
   g.A = b.dig; g.ea = b.exps; g.B = a.dig; g.eb = a.exps; g.C = C; g.ldc = ldc;
-  return slice_run(ctx, g, part, s);
+  return slice_run(ctx, g, p.part, s);
 }
+
+struct PiEmuPiece {   // some of the factor rows, one chunk of at most 131072 pairs
+  SliceForm f;
+  int N, n_t, blk;
+  int64_t chunk;
+  SliceGemmArgs plan;
+  SliceOperand a, b;
+  double *fac = nullptr, *part = nullptr;
+  PiEmuPiece(int n_sm, int N_, int64_t n_pairs, int n_t_, SliceForm f_) : f(f_), N(N_), n_t(n_t_), blk(n_t_) {
+    const int64_t max_chunk = (int64_t)1 << 17, n_chunks = (n_pairs + max_chunk - 1) / max_chunk;
+    chunk = std::min(n_pairs, ((n_pairs + n_chunks - 1) / n_chunks + 63) / 64 * 64);   // balanced
+    const int nkb = slice_blocks(chunk);
+    const size_t each = slice_digit_bytes(N, nkb, f.ns);
+    plan = slice_plan(n_sm, N, N, nkb, 1, planned_piece(n_t, each, each), f);
+  }
+  void layout(Arena &A) {
+    a.layout(A, N, chunk, blk, f);
+    b.layout(A, N, chunk, 1, f);
+    fac = A.take<double>((size_t)n_t * chunk);
+  }
+  size_t partial() const { return slice_partial(plan, blk, N); }
+  bool shrink() { return next_piece(n_t, &blk); }
+};
 
 // Pi from slices (the emulated FP64 form): per frequency (n_tau == 0, Pi_j =
 // -2 s M_j written directly) or moment t (lt_form 1: Laplace factors; 2:
@@ -511,26 +588,12 @@ ltgw_status polarizability_emu(ltgw_ctx *ctx, int N, int64_t n_pairs, const doub
                                const double *d_w, const double *d_E, double *d_M, int spin, double *Pi,
                                cudaStream_t s, int lt_form, SliceForm f) {
   const int n_t = n_tau ? n_tau : n_omega;
-  const int64_t max_chunk = (int64_t)1 << 17;
-  const int64_t n_chunks = (n_pairs + max_chunk - 1) / max_chunk;
-  const int64_t chunk = std::min(n_pairs, ((n_pairs + n_chunks - 1) / n_chunks + 63) / 64 * 64);   // balanced
-  SliceOperand a, b;
-  double *fac = nullptr, *part = nullptr;
-  const int nkb = (int)((chunk + SL_K - 1) / SL_K);
-  const size_t each = slice_digit_bytes(N, nkb, f.ns);
-  const SliceGemmArgs plan = slice_plan(ctx, N, N, nkb, 1, planned_piece(n_t, each, each), f);
-  int blk = n_t;
-  if (!slice_fit(
-          ctx, f.required,
-          [&](Arena &A) {
-            a.layout(A, N, chunk, blk, f);
-            b.layout(A, N, chunk, 1, f);
-            fac = A.take<double>((size_t)n_t * chunk);
-          },
-          [&] { return slice_partial(plan, blk, N); },
-          [&] { return next_piece(n_t, &blk); },
-          &part))
-    return ctx->status();
+  PiEmuPiece p(ctx->n_sm, N, n_pairs, n_t, f);
+  if (!slice_fit(ctx, f.required, p)) return ctx->status();
+  const SliceOperand &a = p.a, &b = p.b;
+  double *const fac = p.fac;
+  const int64_t chunk = p.chunk;
+  const int blk = p.blk;
   ctx->mark(EV_PI0, s);
   const int mode = n_tau ? (lt_form == 2 ? SCALE_EXPTAU : SCALE_LAPLACE) : SCALE_DIRECT;
   double *out = n_tau ? d_M : Pi;
@@ -544,11 +607,11 @@ ltgw_status polarizability_emu(ltgw_ctx *ctx, int N, int64_t n_pairs, const doub
       SliceSrc sa = a.source(Bt + k0, ldb, 0, N, kc, false);
       sa.colscale = fac + (int64_t)t0 * kc; sa.cs_batch = kc;
       CHECK_LAUNCH(ctx, launch_slice_operand(sa, f.ns, f.bits, nb, s), 3);
-      SliceGemmArgs g = plan;
+      SliceGemmArgs g = p.plan;
       g.A = a.dig; g.a_batch = a.dig_batch; g.ea = a.exps; g.ea_batch = a.rows_p;
       g.B = b.dig; g.eb = b.exps; g.batch = nb; g.C = out + (int64_t)t0 * N * N; g.ldc = N; g.c_batch = (int64_t)N * N;
       g.beta = k0 ? 1.0 : 0.0; g.alpha_exp = n_tau ? 0 : spin; g.alpha_neg = n_tau ? 0 : 1;   // -2 s: -2 or -4
-      if (slice_run(ctx, g, part, s) != LTGW_OK) return ctx->status();
+      if (slice_run(ctx, g, p.part, s) != LTGW_OK) return ctx->status();
     }
   }
   ctx->mark(EV_PI1, s);
@@ -990,20 +1053,24 @@ ltgw_status naf_metric_tc(ltgw_ctx *ctx, int n, int64_t n_pairs, const double *B
 // digits of one frequency fit, else on the FP64 tiles.
 constexpr int kScreenDigitsMinN = 144;
 
-ltgw_status screen_step(ltgw_ctx *ctx, int N, int n_omega, const double *Pi, double *work, double *C, cudaStream_t s) {
-  int nl = 0, blk = n_omega;
+struct ScreenPiece {   // some of the frequencies
+  int N, n_omega, blk;
   void *digits = nullptr;
   double *part = nullptr;
-  const bool use = N >= kScreenDigitsMinN && N <= 65535 && n_omega <= 65535 &&
-                   slice_fit(
-                       ctx, false, [&](Arena &A) { digits = A.take<uint8_t>(screen_digit_bytes(N, blk)); },
-                       [] { return (size_t)0; },
-                       [&] { return next_piece(n_omega, &blk); },
-                       &part);
+  ScreenPiece(int N_, int n_omega_) : N(N_), n_omega(n_omega_), blk(n_omega_) {}
+  void layout(Arena &A) { digits = A.take<uint8_t>(screen_digit_bytes(N, blk)); }
+  size_t partial() const { return 0; }
+  bool shrink() { return next_piece(n_omega, &blk); }
+};
+
+ltgw_status screen_step(ltgw_ctx *ctx, int N, int n_omega, const double *Pi, double *work, double *C, cudaStream_t s) {
+  int nl = 0;
+  ScreenPiece p(N, n_omega);
+  const bool use = N >= kScreenDigitsMinN && N <= 65535 && n_omega <= 65535 && slice_fit(ctx, false, p);
   cudaError_t e = cudaSuccess;
   if (use) {
-    for (int j0 = 0; j0 < n_omega && e == cudaSuccess; j0 += blk)
-      e = launch_screen_digits(Pi + (int64_t)j0 * N * N, N, std::min(blk, n_omega - j0), work, digits,
+    for (int j0 = 0; j0 < n_omega && e == cudaSuccess; j0 += p.blk)
+      e = launch_screen_digits(Pi + (int64_t)j0 * N * N, N, std::min(p.blk, n_omega - j0), work, p.digits,
                                C + (int64_t)j0 * N * N, ctx->flags, ctx->n_sm, s, &nl);
   } else {
     e = launch_screen_blocked(Pi, N, n_omega, work, C, ctx->flags, s, &nl);
@@ -1181,6 +1248,43 @@ ltgw_status validate(ltgw_ctx *ctx, const ltgw_params *p) {
 }
 
 }  // namespace
+
+size_t ltgw::solve_digit_bytes(const ltgw_params &p, int n_tgt, int N, size_t limit) {
+  const int n_sm = 152, n_act = p.n_occ - p.n_frozen, n_orb_act = n_act + p.n_virt;
+  const int n_t = p.use_laplace && p.n_tau > 0 ? p.n_tau : p.n_omega;
+  if (n_act < 1 || p.n_virt < 1 || p.n_aux < 1 || n_t < 1 || p.n_omega < 1 || N < 1 || n_tgt < 1) return 0;
+  const int64_t n_ov = (int64_t)n_act * p.n_virt;
+  const bool emu = p.precision == LTGW_FP64_EMU;
+  Arena ar;
+  size_t most = 0;
+  auto add = [&](auto piece) {
+    size_t b = piece_bytes(ar, piece);
+    if (b > limit) {
+      while (piece.shrink()) b = piece_bytes(ar, piece);
+      b = std::max(b, limit);
+    }
+    most = std::max(most, b);
+  };
+  if (emu || p.precision == LTGW_FP64) {
+    const SliceForm f = emu ? emu_digits(kEmuSlices) : kFp64Digits;
+    if (p.naf_thresh >= 0.0) {
+      add(SyrkPiece(n_sm, p.n_aux, n_ov, f));
+      add(ProjectPiece(n_sm, N, p.n_aux, std::min<int64_t>(n_ov, INT32_MAX), 1, f));
+      add(ProjectPiece(n_sm, N, p.n_aux, n_orb_act, n_tgt, f));
+    }
+    if (emu) add(PiEmuPiece(n_sm, N, n_ov, n_t, f));
+    else add(PiPiece(n_sm, N, n_ov, n_t, f));
+    add(WnmPiece(N, p.n_omega, n_tgt, n_orb_act, f));
+  }
+  if (N >= kScreenDigitsMinN) add(ScreenPiece(N, p.n_omega));
+  return most;
+}
+
+void ltgw::release_products(ltgw_ctx *ctx) {
+  ctx->a4.release();
+  ctx->a5.release();
+}
+
 
 extern "C" {
 

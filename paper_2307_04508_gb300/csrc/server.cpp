@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "../../include/ltgw.h"
+#include "digit_memory.h"
 
 namespace {
 
@@ -33,6 +34,7 @@ struct Pending {
   uint64_t ticket = 0;
   ltgw_request req{};
   size_t footprint = 0;
+  size_t fixed = 0;   // the part of it that is not digit workspace
   Clock::time_point t_submit;
   int bypassed = 0;   // later requests admitted ahead of this one
   int retries = 0;    // solves that ran out of device memory
@@ -41,6 +43,10 @@ struct Pending {
 };
 
 constexpr int kMaxBypass = 8;
+// Digit workspace of a request, where its smallest pieces do not need more:
+// several run beside each other, so a tenth of what a context takes alone
+// (requests of up to 40 occupied orbitals: the Pi of eight moments in two pieces).
+constexpr size_t kDigitMemory = (size_t)640 << 20;
 // A request that runs out of device memory beside others goes back with its
 // footprint doubled until it runs alone; one that fails alone is re-run once
 // after the idle slots released their workspace.  Doubling from the smallest
@@ -139,6 +145,8 @@ struct ltgw_server {
       ltgw_status rs = LTGW_ERR_DEVICE;
       if (ctx) {
         const ltgw_request &r = job.req;
+        // the digits keep to what the footprint leaves them (the bits do not depend on it)
+        ltgw_set_digit_memory(ctx, job.footprint - std::min(job.footprint, job.fixed));
         rs = ltgw_solve(ctx, &r.p, r.eps, r.B_ov, r.B_tgt, r.targets, r.n_tgt, r.shift, r.tau_x, r.tau_w,
                         r.sigma_iw, r.e_qp, r.qp_status, stream);
       }
@@ -147,7 +155,9 @@ struct ltgw_server {
       // what it keeps counts against admission (see dispatch_locked)
       size_t keep = 0;
       if (ctx) {
-        if (rs == LTGW_ERR_NOMEM || ltgw_workspace_bytes(ctx) > budget / (4 * slots.size())) ltgw_trim(ctx);
+        const size_t share = budget / (4 * slots.size());
+        if (ltgw_workspace_bytes(ctx) > share) ltgw::release_products(ctx);
+        if (rs == LTGW_ERR_NOMEM || ltgw_workspace_bytes(ctx) > share) ltgw_trim(ctx);
         keep = ltgw_workspace_bytes(ctx);
       }
       lock.lock();
@@ -207,10 +217,14 @@ struct ltgw_server {
   }
 };
 
-extern "C" {
+// Device bytes of a request: `fixed` without the digit workspace, `admit` what
+// the budget must hold for the request to be accepted at all (the rest of the
+// digit workspace gives way).
+struct Footprint {
+  size_t fixed = 0, admit = 0, all = 0;
+};
 
-size_t ltgw_request_footprint(const ltgw_params *p, int n_tgt) {
-  if (!p || n_tgt < 1) return 0;
+static Footprint request_footprint(const ltgw_params *p, int n_tgt) {
   const size_t n_aux = (size_t)p->n_aux, n_occ = (size_t)p->n_occ, n_virt = (size_t)p->n_virt;
   const size_t n_orb = n_occ + n_virt, n_act = n_occ - (size_t)p->n_frozen;
   // N: auxiliary functions after the NAF step, not known before the solve;
@@ -236,19 +250,30 @@ size_t ltgw_request_footprint(const ltgw_params *p, int n_tgt) {
   const size_t p_part = nN * cdiv(n_ov, 128) * cdiv(n_aux, 2048) * tile;
   const size_t pi_part = nN * (nN + 1) / 2 * t * std::min<size_t>(64, cdiv(n_ov, 2048)) * tile;
   const size_t partials = std::max(k_part, std::max(p_part, pi_part));
+  size_t emu = 0;   // the digit sets that an emulated request must have room for
   if (p->precision == LTGW_FP64_EMU) {
-    // projected ov block; an upper estimate of the largest slice set (three
-    // operands of 6 slices of 2 bytes per value) and the partials
-    d += N * n_ov + 9 * n_aux * n_ov / 2 + partials;
+    d += N * n_ov;                                              // projected ov block
+    emu = 9 * n_aux * n_ov / 2 + partials;
   } else if (p->precision != LTGW_FP64) {
     d += (2 * n_aux * n_ov + N * n_ov) / 2 + n_om * N * N / 2;  // FP32 copies, BF16 hi / lo of the ov block
     if (p->precision == LTGW_FP8 || p->precision == LTGW_FP8_PI)
-      d += 3 * ((n_tau ? n_tau : n_om) + 1) * N * n_ov / 8;     // FP8 codes (two-term: 3 per value)
+      d += 3 * (t + 1) * nN * 16 * cdiv(n_ov, 128) * 128;       // FP8 codes (two-term: 3 per value), padded
     d += partials;
   } else {
     d += N * n_ov;                                              // projected ov block
   }
-  return d * sizeof(double) + (64u << 20);                     // + fixed slack
+  Footprint f;
+  f.fixed = d * sizeof(double) + (64u << 20);                  // + fixed slack
+  f.admit = f.fixed + emu * sizeof(double);
+  f.all = std::max(f.admit, f.fixed + ltgw::solve_digit_bytes(*p, n_tgt, (int)N, kDigitMemory));
+  return f;
+}
+
+extern "C" {
+
+size_t ltgw_request_footprint(const ltgw_params *p, int n_tgt) {
+  if (!p || n_tgt < 1) return 0;
+  return request_footprint(p, n_tgt).all;
 }
 
 ltgw_status ltgw_server_create(ltgw_server **out, int device, int n_slots, size_t hbm_budget_bytes) {
@@ -286,13 +311,14 @@ ltgw_status ltgw_server_submit(ltgw_server *s, const ltgw_request *req, uint64_t
   if (!req->eps || !req->B_ov || !req->B_tgt || !req->targets || !req->shift || !req->sigma_iw || !req->e_qp ||
       !req->qp_status || req->n_tgt < 1)
     return LTGW_ERR_BAD_ARG;
-  const size_t fp = ltgw_request_footprint(&req->p, req->n_tgt);
-  if (fp > s->budget) return LTGW_ERR_NOMEM;
+  const Footprint fp = request_footprint(&req->p, req->n_tgt);
+  if (fp.admit > s->budget) return LTGW_ERR_NOMEM;
   std::lock_guard<std::mutex> lock(s->mu);
   Pending p;
   p.ticket = s->next_ticket++;
   p.req = *req;
-  p.footprint = fp;
+  p.footprint = std::min(s->budget, fp.all);
+  p.fixed = fp.fixed;
   p.t_submit = Clock::now();
   s->queue.push_back(p);
   *ticket = p.ticket;
