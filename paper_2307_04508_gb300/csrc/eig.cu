@@ -26,11 +26,11 @@
 #include <float.h>
 
 #include <algorithm>
-#include <mutex>
 #include <math.h>
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "per_device.h"
 
 namespace ltgw {
 namespace {
@@ -1684,23 +1684,21 @@ __global__ void transpose_kernel(const T *__restrict__ X, int n, int k, double *
   }
 }
 
-// Raise a kernel's dynamic shared-memory limit once, to the most any call
-// may use; setting it per call races between host threads (one thread could
+// Raise a kernel's dynamic shared-memory limit once per device, to the most any
+// call may use; setting it per call races between host threads (one thread could
 // lower it between another thread's set and launch).
-cudaError_t allow_max_dynamic_smem(const void *kernel, std::once_flag &flag) {
-  cudaError_t result = cudaSuccess;
-  std::call_once(flag, [&] {
+cudaError_t allow_max_dynamic_smem(const void *kernel, OncePerDevice &once) {
+  return once([&] {
     int dev = 0, optin = 0;
     cudaFuncAttributes fa;
-    if ((result = cudaGetDevice(&dev)) != cudaSuccess) return;
-    if ((result = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return;
-    if ((result = cudaFuncGetAttributes(&fa, kernel)) != cudaSuccess) return;
-    result = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  optin - (int)fa.sharedSizeBytes);
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
   });
-  return result;
 }
-std::once_flag g_smem_hh, g_smem_hp, g_smem_bisect, g_smem_invit[2], g_smem_tw[2], g_smem_bounds, g_smem_wy, g_smem_wa;
+OncePerDevice g_smem_hh, g_smem_hp, g_smem_bisect, g_smem_invit[2], g_smem_tw[2], g_smem_bounds, g_smem_wy, g_smem_wa;
 
 // Try the fused reduction of the trailing block from row and column k0 on in
 // arithmetic T; false when it cannot be launched.

@@ -48,10 +48,10 @@
 #include <stdint.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "per_device.h"
 #include "tc_ptx.cuh"
 
 namespace ltgw {
@@ -876,13 +876,12 @@ cudaError_t slice_operand(const SliceSrc &a, int batch, cudaStream_t s) {
 
 template <int NS, int BITS, int NL = NS>
 cudaError_t launch_ns(const SliceGemmArgs &g, int blocks, cudaStream_t s) {
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(slice_gemm_kernel<NS, BITS, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sg_smem(NS));
+  static OncePerDevice smem_limit;
+  const cudaError_t e = smem_limit([] {
+    return cudaFuncSetAttribute(slice_gemm_kernel<NS, BITS, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sg_smem(NS));
   });
-  if (attr_err != cudaSuccess) return attr_err;
+  if (e != cudaSuccess) return e;
   slice_gemm_kernel<NS, BITS, NL><<<blocks, SG_THREADS, sg_smem(NS), s>>>(g);
   return cudaGetLastError();
 }

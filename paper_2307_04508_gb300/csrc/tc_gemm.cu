@@ -36,6 +36,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "per_device.h"
 #include "tc_ptx.cuh"
 
 namespace ltgw {
@@ -617,12 +618,10 @@ cudaError_t launch_tc_fp8_gemm(const TcGemmArgs &g, int n_tiles, cudaStream_t s)
                  CU_TENSOR_MAP_SWIZZLE_128B) ||
       !encode_2d(&tb, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g.B8, g.Kp, g.rows_b, F8_K, TN, CU_TENSOR_MAP_SWIZZLE_128B))
     return cudaErrorNotSupported;
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(tc_fp8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F8_SMEM);
-  });
-  if (attr_err != cudaSuccess) return attr_err;
+  static OncePerDevice smem_limit;
+  const cudaError_t e = smem_limit(
+      [] { return cudaFuncSetAttribute(tc_fp8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F8_SMEM); });
+  if (e != cudaSuccess) return e;
   tc_fp8_kernel<<<dim3(n_tiles, groups, splits), F8_THREADS, F8_SMEM, s>>>(g, ta, tb);
   return cudaGetLastError();
 }
@@ -653,13 +652,11 @@ cudaError_t launch_tc_split_gemm(const TcGemmArgs &g, int n_tiles, cudaStream_t 
         !encode_2d(&tbl, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, g.B_lo, g.Kp, g.rows_b, TK, TN,
                    CU_TENSOR_MAP_SWIZZLE_128B))
       return cudaErrorNotSupported;
-    static std::once_flag once2;
-    static cudaError_t attr_err2 = cudaSuccess;
-    std::call_once(once2, [] {
-      attr_err2 = cudaFuncSetAttribute(tc_tma_ts_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)T3_SMEM);
+    static OncePerDevice smem_limit;
+    const cudaError_t e = smem_limit([] {
+      return cudaFuncSetAttribute(tc_tma_ts_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T3_SMEM);
     });
-    if (attr_err2 != cudaSuccess) return attr_err2;
+    if (e != cudaSuccess) return e;
     TcGemmArgs h = g;
     // groups first when they share A (Pi's scales) and there are many tiles, or
     // when the tiles are very many (W_nm's frequencies share only B); measured:
