@@ -990,6 +990,8 @@ __global__ void __launch_bounds__(RB) tridiag_bounds_kernel(const double *dg, co
 // Measured, bisection to transposition with a quarter of the vectors kept,
 // against evenly spaced FP64 sweeps in blocks of four warps: n = 264 1.43 -> 1.11
 // ms, n = 800 3.81 -> 2.95, n = 1800 9.7 -> 8.0, n = 3300 22.7 -> 16.8.
+// (Ending at eps ||T|| instead of eps |lambda| would save 0.03 to 0.4 ms of these and
+// lose the small eigenvalues' last bits.)
 constexpr int BS_PRE = 4;                      // FP32 sweeps: 2 / 33^4 of ||T||
 constexpr double BS_PRE_ERR = 1.0 / 524288.0;  // 2^-19 ||T||: above the FP32 counts' error
 
@@ -1089,16 +1091,18 @@ __global__ void bisect_kernel(const double *d, const double *e2g, const double *
   double pl = 0.0, ph = 0.0;
   int El = 0, Eh = 0, cl = -1, ch = -1;
   bool even = false;   // the next sweep's points are evenly spaced
+  int misses = 0;      // placed sweeps that did less: below the counts' resolution none are placed any more
   for (int it = 0; it < 200; ++it) {
     const double w = hi - lo;
-    // the counts are those of a matrix within a few 2^-53 ||T||
-    if (w <= 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) + 0.125 * DBL_EPSILON * tn + pivmin) break;
+    // relative to the eigenvalue: the small ones of a graded T are as well
+    // determined by its entries
+    if (w <= 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) + pivmin) break;
     double x = lo + w * ((double)(lane + 1) * (1.0 / 33.0));
     bool placed = false;
     if (hint) {
       x = lane == 31 ? hh : hl + (hh - hl) * ((double)lane * (1.0 / 31.0));
       placed = true;
-    } else if (!even && cl >= 0 && ch == cl + 1) {
+    } else if (!even && misses < 2 && cl >= 0 && ch == cl + 1) {
       const int sh = min(max(Eh - El, -1000), 1000);
       const double q = scalbn(fabs(ph / pl), sh), c = lo + w / (1.0 + q);
       if (c > lo && c < hi) {
@@ -1128,6 +1132,7 @@ __global__ void bisect_kernel(const double *d, const double *e2g, const double *
     }
     if (!placed && !moved) break;   // no progress at this resolution
     even = placed && !(hi - lo <= w * (1.0 / 32.0));
+    misses += even;
   }
   if (lane == 0) lam[r] = 0.5 * (lo + hi);
 }

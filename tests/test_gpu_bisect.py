@@ -67,3 +67,16 @@ def test_all_vectors_kept(ctx, n):
     assert np.abs(g - np.sort(np.linalg.eigvalsh(K))[::-1]).max() <= 1e-13 * g[0]
     assert np.linalg.norm(K @ U.T - U.T * g[None, :], axis=0).max() <= 1e-12 * g[0]
     assert np.abs(U @ U.T - np.eye(n)).max() <= 1e-12
+
+
+@pytest.mark.parametrize("n", [33, 153, 264])
+def test_small_eigenvalues_of_a_graded_matrix(ctx, n):
+    """A diagonal K graded over twelve decades: the tridiagonal form is exact, so each
+    eigenvalue, and not only the largest, is the diagonal entry to the rounding of
+    the metric (2^-54 in digits, 2^-53 in FP64) and half a bracket of 2 eps: 4 eps."""
+    b = np.sqrt(_spectrum("graded", n))
+    Ut = torch.zeros((n, n), dtype=torch.float64, device="cuda")
+    lam = torch.zeros(n, dtype=torch.float64, device="cuda")
+    assert ctx.naf_basis(torch.from_numpy(np.diag(b)).cuda(), n, n, 1e-14, Ut, lam) == n
+    ref = b.astype(np.longdouble) ** 2
+    assert np.abs((lam.cpu().numpy() - ref) / ref).max() <= 4 * 2.0 ** -52
