@@ -349,7 +349,9 @@ ltgw_status ltgw_polarizability_emulated(ltgw_ctx *ctx, int N, int64_t n_pairs, 
                                          int n_slices, double *Pi, void *stream);
 
 /* Screening (Eq. ScreenedCoulombOrbital): C_j = [1 - Pi_j]^-1 - 1 for each of
- * n_omega matrices (device [n_omega][N][N] in and out, may not alias).
+ * n_omega matrices (device [n_omega][N][N] in and out, may not alias).  Pi_j is
+ * symmetric; from N = 144 on a Pi_j that is so to rounding is read from its
+ * upper triangle, any other takes the slower form that reads both.
  * Synchronises; LTGW_ERR_NOT_SPD if a pivot was not positive. */
 ltgw_status ltgw_screen(ltgw_ctx *ctx, int N, int n_omega, const double *Pi, double *C,
                         void *stream);

@@ -1063,18 +1063,28 @@ struct ScreenPiece {   // some of the frequencies
   bool shrink() { return next_piece(n_omega, &blk); }
 };
 
-ltgw_status screen_step(ltgw_ctx *ctx, int N, int n_omega, const double *Pi, double *work, double *C, cudaStream_t s) {
+// check: Pi comes from the caller; one that is not symmetric goes to the FP64 tiles,
+// which read both triangles (the solves' own Pi is symmetric bit for bit).
+ltgw_status screen_step(ltgw_ctx *ctx, int N, int n_omega, const double *Pi, double *work, double *C, cudaStream_t s,
+                        bool check = false) {
   int nl = 0;
   ScreenPiece p(N, n_omega);
   const bool use = N >= kScreenDigitsMinN && N <= 65535 && n_omega <= 65535 && slice_fit(ctx, false, p);
   cudaError_t e = cudaSuccess;
+  bool general = !use;
   if (use) {
     for (int j0 = 0; j0 < n_omega && e == cudaSuccess; j0 += p.blk)
       e = launch_screen_digits(Pi + (int64_t)j0 * N * N, N, std::min(p.blk, n_omega - j0), work, p.digits,
-                               C + (int64_t)j0 * N * N, ctx->flags, ctx->n_sm, s, &nl);
-  } else {
-    e = launch_screen_blocked(Pi, N, n_omega, work, C, ctx->flags, s, &nl);
+                               C + (int64_t)j0 * N * N, ctx->flags, ctx->n_sm,
+                               check ? ctx->flags + FLAG_ASYM : nullptr, s, &nl);
+    int asym = 0;
+    if (check && e == cudaSuccess) {
+      if (read_small(ctx, &asym, ctx->flags + FLAG_ASYM, sizeof(int), s) != LTGW_OK) return ctx->status();
+      if (asym) LTGW_CUDA(ctx, cudaMemsetAsync(ctx->flags, 0, FLAG_COUNT * sizeof(int), s));
+      general = asym != 0;
+    }
   }
+  if (general && e == cudaSuccess) e = launch_screen_blocked(Pi, N, n_omega, work, C, ctx->flags, s, &nl);
   ctx->launches += nl;
   if (e != cudaSuccess) ctx->fail(LTGW_ERR_DEVICE, std::string("screen: ") + cudaGetErrorString(e));
   return ctx->status();
@@ -2221,7 +2231,7 @@ ltgw_status ltgw_screen(ltgw_ctx *ctx, int N, int n_omega, const double *Pi, dou
   if (ctx->a2.commit() != cudaSuccess) { ctx->fail(LTGW_ERR_NOMEM, "workspace allocation failed"); return ctx->status(); }
   layout(ctx->a2);
   LTGW_CUDA(ctx, cudaMemsetAsync(ctx->flags, 0, FLAG_COUNT * sizeof(int), s));
-  if (screen_step(ctx, N, n_omega, Pi, X0, C, s) != LTGW_OK) return ctx->status();
+  if (screen_step(ctx, N, n_omega, Pi, X0, C, s, true) != LTGW_OK) return ctx->status();
   LTGW_CUDA(ctx, cudaStreamSynchronize(s));
   return check_flags(ctx, s);
 }

@@ -80,10 +80,11 @@ cudaError_t launch_screen_blocked(const double *Pi, int N, int n_omega, double *
                                   cudaStream_t s, int *launches);
 
 // Pivot blocks of 128 with the updates from digits; work as above, digits:
-// screen_digit_bytes(N, n_omega) bytes, 256-byte aligned.
+// screen_digit_bytes(N, n_omega) bytes, 256-byte aligned.  Takes Pi's upper
+// triangle; asym (if not null) is set when the lower one is not its mirror image.
 size_t screen_digit_bytes(int N, int n_omega);
 cudaError_t launch_screen_digits(const double *Pi, int N, int n_omega, double *work, void *digits, double *C,
-                                 int *flags, int n_sm, cudaStream_t s, int *launches);
+                                 int *flags, int n_sm, int *asym, cudaStream_t s, int *launches);
 
 // ---- eigensolver (eig.cu) ----
 struct EigWork {

@@ -83,8 +83,8 @@ __global__ void form_a_kernel(const double *__restrict__ Pi, T *__restrict__ X, 
 // into every CTA's shared memory; one cluster barrier; then every other row
 // takes the four rank-1 updates in order.  The arithmetic per entry is that of
 // one pivot at a time.  The buffers alternate with the round's parity, so the
-// writes of one round never meet the reads of the round before.  Only the
-// block's upper triangle is read.
+// writes of one round never meet the reads of the round before.  UPPER: only
+// the block's upper triangle is read (the matrix is known to be symmetric).
 // Bound: the owner warp's chain of division, scaled row and three rank-1 rows
 // per pivot (B = 64: 90 us for 32 blocks, 85 us with one pivot per barrier),
 // and for B = 128 the FP64 pipe beside it (2.1e6 multiply-adds a block, two CTAs
@@ -103,7 +103,7 @@ __device__ __forceinline__ void st_cluster_2f64(uint32_t local_addr, unsigned ra
   asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(remote), "d"(v0), "d"(v1) : "memory");
 }
 
-template <int B>
+template <int B, bool UPPER>
 __global__ void __cluster_dims__(B / SB_RPC, 1, 1) __launch_bounds__(SB_THREADS)
     block_inverse_kernel(const double *__restrict__ X, int N, int p0, int bs, double *__restrict__ Z, int *flags) {
   constexpr int NC = B / 32;          // columns per lane, in pairs
@@ -132,7 +132,8 @@ __global__ void __cluster_dims__(B / SB_RPC, 1, 1) __launch_bounds__(SB_THREADS)
 #pragma unroll
     for (int h = 0; h < NC; ++h) {
       const int i = i0 + r, j = col(h);
-      v[r][h] = (i < bs && j < bs) ? Xb[(int64_t)(p0 + min(i, j)) * N + (p0 + max(i, j))] : 0.0;
+      const int a = UPPER ? min(i, j) : i, c = UPPER ? max(i, j) : j;
+      v[r][h] = (i < bs && j < bs) ? Xb[(int64_t)(p0 + a) * N + (p0 + c)] : 0.0;
     }
   const uint32_t rowk_addr = (uint32_t)__cvta_generic_to_shared(&rowk[0][0][0]);
   const uint32_t rpk_addr = (uint32_t)__cvta_generic_to_shared(&rpk[0][0]);
@@ -261,7 +262,7 @@ cudaError_t screen_blocked_impl(const double *Pi, int N, int n_omega, T *work, d
   ++*launches;
   for (int p0 = 0; p0 < N; p0 += SB_B) {
     const int bs = std::min(SB_B, N - p0);
-    block_inverse_kernel<SB_B><<<dim3(SB_B / SB_RPC, n_omega), SB_THREADS, 0, s>>>(X, N, p0, bs, Z, flags);
+    block_inverse_kernel<SB_B, false><<<dim3(SB_B / SB_RPC, n_omega), SB_THREADS, 0, s>>>(X, N, p0, bs, Z, flags);
     dim3 cg((N + 255) / 256 < 8 ? (N + 255) / 256 : 8, bs, n_omega);
     copy_rows_kernel<T><<<cg, 256, 0, s>>>(X, N, p0, bs, rowsP);
     GemmArgs<T> g;   // R = X[:, P] Z
@@ -311,6 +312,37 @@ __global__ void form_upper_kernel(const double *__restrict__ Pi, double *__restr
   const int64_t o = (int64_t)blockIdx.z * N * N + (int64_t)i * N;
   for (int j = (i & ~31) + blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x)
     X[o + j] = (i == j ? 1.0 : 0.0) - Pi[o + j];
+}
+
+// The same for a Pi that need not be symmetric: *asym is set where two mirrored
+// entries differ by more than the rounding of a product of rows, 4 N u
+// sqrt((1 - Pi_ii) (1 - Pi_jj)), or are not both numbers.  FP64 instructions run
+// only where the bits differ.  Grid: 32 x 32 tiles (column, row, frequency).
+__global__ void __launch_bounds__(256) form_upper_checked_kernel(const double *__restrict__ Pi, double *__restrict__ X,
+                                                                 int N, int *__restrict__ asym) {
+  __shared__ double t[32][33];
+  const int bi = blockIdx.y, bj = blockIdx.x;
+  if (bj < bi) return;
+  const double *P = Pi + (int64_t)blockIdx.z * N * N;
+  double *Xb = X + (int64_t)blockIdx.z * N * N;
+  const int tx = threadIdx.x;
+  for (int q = threadIdx.y; q < 32; q += 8) {   // the mirrored tile
+    const int r = bj * 32 + q, c = bi * 32 + tx;
+    if (r < N && c < N) t[q][tx] = P[(int64_t)r * N + c];
+  }
+  __syncthreads();
+  bool bad = false;
+  for (int q = threadIdx.y; q < 32; q += 8) {
+    const int i = bi * 32 + q, j = bj * 32 + tx;
+    if (i >= N || j >= N) continue;
+    const double a = P[(int64_t)i * N + j], b = t[tx][q];
+    Xb[(int64_t)i * N + j] = (i == j ? 1.0 : 0.0) - a;
+    if (__double_as_longlong(a) != __double_as_longlong(b) || !isfinite(a)) {
+      const double di = 1.0 - P[(int64_t)i * N + i], dj = 1.0 - P[(int64_t)j * N + j];
+      bad |= !(fabs(a - b) <= 4.0 * N * 0x1p-53 * sqrt(di * dj));
+    }
+  }
+  if (bad) *asym = 1;
 }
 
 // P[b][i][c] = X[i][p0 + c] from the upper triangle, i < N, c < bs (ld SD_B).
@@ -424,19 +456,23 @@ size_t screen_digit_bytes(int N, int n_omega) {
 }
 
 cudaError_t launch_screen_digits(const double *Pi, int N, int n_omega, double *work, void *digits, double *C,
-                                 int *flags, int n_sm, cudaStream_t s, int *launches) {
+                                 int *flags, int n_sm, int *asym, cudaStream_t s, int *launches) {
   if (N <= 0 || n_omega <= 0) return cudaSuccess;
   if (n_omega > 65535 || N > 65535) return cudaErrorInvalidValue;
   const int64_t NN = (int64_t)N * N;
   double *X = work, *P = X + NN * n_omega;   // P, then R: [n_omega][N][SD_B]
   SdScratch o;
   sd_layout(N, n_omega, digits, &o);
-  form_upper_kernel<<<dim3(std::min((N + 255) / 256, 8), N, n_omega), 256, 0, s>>>(Pi, X, N);
+  const int nt = (N + 31) / 32;
+  if (asym)
+    form_upper_checked_kernel<<<dim3(nt, nt, n_omega), dim3(32, 8), 0, s>>>(Pi, X, N, asym);
+  else
+    form_upper_kernel<<<dim3(std::min((N + 255) / 256, 8), N, n_omega), 256, 0, s>>>(Pi, X, N);
   ++*launches;
   for (int p0 = 0; p0 < N; p0 += SD_B) {
     const int bs = std::min(SD_B, N - p0), nkb = (bs + SL_K - 1) / SL_K;
     const dim3 pg((N + 31) / 32, (bs + 31) / 32, n_omega), tb(32, 8);
-    block_inverse_kernel<SD_B><<<dim3(SD_B / SB_RPC, n_omega), SB_THREADS, 0, s>>>(X, N, p0, bs, o.Z, flags);
+    block_inverse_kernel<SD_B, true><<<dim3(SD_B / SB_RPC, n_omega), SB_THREADS, 0, s>>>(X, N, p0, bs, o.Z, flags);
     gather_panel_kernel<<<pg, tb, 0, s>>>(X, N, p0, bs, P);
     SliceSrc a;
     a.X = P; a.ld = SD_B; a.x_batch = (int64_t)N * SD_B; a.rows = N; a.rows_p = o.Np; a.K = bs; a.nkb = nkb;
@@ -475,7 +511,6 @@ cudaError_t launch_screen_digits(const double *Pi, int N, int n_omega, double *w
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  const int nt = (N + 31) / 32;
   finish_upper_kernel<<<dim3(nt, nt, n_omega), dim3(32, 8), 0, s>>>(X, C, N);
   ++*launches;
   return cudaGetLastError();
