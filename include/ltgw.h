@@ -30,6 +30,14 @@
  *  - Every call returns an ltgw_status; no exception or abort crosses the ABI.
  *    ltgw_last_error() gives a one-line description of the last failure.
  *  - A context is not thread-safe: one host thread at a time per context.
+ *  - LTGW_FP64 products of K terms are formed on the tensor cores from integer
+ *    digits of whole rows: an entry (i, j) is off by at most about K 2^-53
+ *    max|a_i| max|b_j|, in norm an FP64 sum's error or less.  An entry whose terms
+ *    are all far below its rows' largest ones carries that error too, where an
+ *    FP64 sum (K 2^-53 sum |a||b|) would not: ltgw_polarizability sums these in
+ *    FP64, the products inside the NAF basis, the screening and a solve do not.
+ *    A row with an infinity gives NaN there (in ltgw_polarizability what an FP64
+ *    sum gives).
  *
  * Readings of points the paper leaves open (fixed once, shared with the tests):
  *  - closed-shell spatial orbitals: spin factor s (default 2) multiplies the
@@ -279,7 +287,9 @@ ltgw_status ltgw_naf_basis_mixed(ltgw_ctx *ctx, int n_aux, int64_t n_pairs, cons
 /* Polarisability at the GL frequencies `omegas` (host [n_omega]) from the
  * pair block Bt (device [N][n_pairs]) and gaps delta (device [n_pairs]):
  * n_tau == 0 evaluates Eq. Pi directly, n_tau > 0 the Laplace form with the
- * host grid (x, w).  Pi: device [n_omega][N][N], full symmetric.  Stream-ordered. */
+ * host grid (x, w).  Pi: device [n_omega][N][N], full symmetric, every entry of
+ * Eq. Pi or of a moment to an FP64 sum's accuracy (rows that are large on
+ * different pairs cost the FP64 units' time).  Stream-ordered. */
 ltgw_status ltgw_polarizability(ltgw_ctx *ctx, int N, int64_t n_pairs, const double *Bt,
                                 const double *delta, int n_omega, const double *omegas,
                                 int n_tau, const double *x, const double *w, int spin,

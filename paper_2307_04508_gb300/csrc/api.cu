@@ -178,9 +178,14 @@ ltgw_status naf_metric_tc(ltgw_ctx *ctx, int n, int64_t n_pairs, const double *B
 
 // ---- FP64 contractions on the tensor cores from integer digits (slice_gemm.cu)
 // The FP64 form's products: 7 digits in base 256 hold 55 bits relative to each
-// operand row's largest magnitude, and the products kept (levels i + j <= 8)
-// leave an error of about 2^-52 of the rows' scales per entry, no more than a
-// length-K FP64 sum's own rounding.
+// operand row's largest magnitude (2^e a power of two 2 to 4 times that), and with
+// the products kept (levels i + j <= 8, or 9) an entry is off by at most K 2^-55
+// 2^(e_i + e_j).  In norm that is an FP64 sum's error or less; an entry whose terms are
+// all small beside its rows' largest ones loses what lies below, where an FP64
+// sum (K 2^-53 sum |a||b|) would keep it.  So the polarisability as a result has
+// those entries summed in FP64 (pi_weak.cu); inside a solve, in the NAF metric and
+// in the inverse they are summed over or mixed by factorisations whose own error
+// is one of the norm.
 // The emulated FP64 forms: n_slices digits in base 128, one exponent per whole
 // operand row, and no CUDA-core kernel to fall back to.
 struct SliceForm {
@@ -486,10 +491,12 @@ struct PiPiece {   // some of the factor rows, one pair chunk
 // are Bt diag(sqrt |f_t|), the sign of f_t with the first one: an entry's error
 // then follows the pairs that carry it, also where a factor singles out few of
 // them (a factor on one side only would weigh that side's rounding with every
-// pair of the other).
+// pair of the other).  Entries whose terms are all small beside their rows' largest
+// ones (rows that are large on different pairs) would still lose bits to the
+// rows' common scales: with `entries` these are found and summed in FP64 (pi_weak.cu).
 ltgw_status slice_pi(ltgw_ctx *ctx, int N, int64_t n_pairs, const double *Bt, int64_t ldb, const double *delta,
                      int n_t, const double *p0, const double *p1, int mode, int alpha_exp, int alpha_neg, double *M,
-                     SliceForm f, cudaStream_t s, bool *done) {
+                     bool entries, SliceForm f, cudaStream_t s, bool *done) {
   PiPiece p(ctx->n_sm, N, n_pairs, n_t, f);
   *done = slice_fit(ctx, f.required, p);
   if (!*done) return ctx->status();
@@ -517,6 +524,14 @@ ltgw_status slice_pi(ltgw_ctx *ctx, int N, int64_t n_pairs, const double *Bt, in
       g.C = M + (int64_t)t0 * N * N; g.ldc = N; g.c_batch = (int64_t)N * N;
       g.beta = k0 ? 1.0 : 0.0; g.alpha_exp = alpha_exp; g.alpha_neg = alpha_neg;
       if (slice_run(ctx, g, p.part, s) != LTGW_OK) return ctx->status();
+      if (!entries) continue;
+      PiWeakArgs w;   // a chunk's weak entries: the sum so far
+      w.dig = o.dig; w.dig_batch = o.dig_batch; w.exps = o.exps; w.exp_batch = o.rows_p; w.nkb = o.nkb;
+      w.N = N; w.mode = mode; w.K = k0 + kc; w.X = Bt; w.ld = ldb;
+      w.delta = delta; w.p0 = p0 + t0; w.p1 = p1 ? p1 + t0 : nullptr;
+      if (k0 == 0) { w.sgn = a.colscale; w.mag = b.colscale; w.f_batch = kc; }
+      w.alpha = ldexp(alpha_neg ? -1.0 : 1.0, alpha_exp); w.C = g.C;
+      CHECK_LAUNCH(ctx, launch_pi_weak(w, nb, s), 1);
     }
   }
   return LTGW_OK;
@@ -707,11 +722,12 @@ ltgw_status naf_basis_dev(ltgw_ctx *ctx, Arena &ar, int n, int64_t n_pairs, cons
 // Pi at the GL frequencies, direct (n_tau == 0) or through moments M^k and the
 // recombination d_E [n_omega][n_tau]: lt_form 1 = the M^m form of Eq. LT
 // (factors w_m Delta e^{-Delta^2 x_m}), 2 = imaginary time (factors e^{-Delta tau_k},
-// tau_k in d_x).
+// tau_k in d_x).  entries: Pi itself is the result, each entry to an FP64 sum's
+// accuracy; within a solve it is summed over, and the rows' scales are enough.
 ltgw_status polarizability_dev(ltgw_ctx *ctx, int N, int64_t n_pairs, const double *Bt, int64_t ldb,
                                const double *delta, int n_omega, const double *d_omega,
                                int n_tau, const double *d_x, const double *d_w, const double *d_E,
-                               double *M, int spin, double *Pi, cudaStream_t s, int lt_form) {
+                               double *M, int spin, double *Pi, cudaStream_t s, int lt_form, bool entries) {
   const int mode = n_tau == 0 ? SCALE_DIRECT : (lt_form == 2 ? SCALE_EXPTAU : SCALE_LAPLACE);
   const int n_t = n_tau ? n_tau : n_omega;
   const double *p0 = n_tau ? d_x : d_omega, *p1 = mode == SCALE_LAPLACE ? d_w : nullptr;
@@ -720,8 +736,8 @@ ltgw_status polarizability_dev(ltgw_ctx *ctx, int N, int64_t n_pairs, const doub
   bool done = false;
   // alpha: 1 for the moments, -2 spin = -2 or -4 for Pi itself
   if (slices_pay(N, N, n_pairs, n_t) &&
-      slice_pi(ctx, N, n_pairs, Bt, ldb, delta, n_t, p0, p1, mode, n_tau ? 0 : spin, n_tau ? 0 : 1, out, kFp64Digits,
-               s, &done) != LTGW_OK)
+      slice_pi(ctx, N, n_pairs, Bt, ldb, delta, n_t, p0, p1, mode, n_tau ? 0 : spin, n_tau ? 0 : 1, out, entries,
+               kFp64Digits, s, &done) != LTGW_OK)
     return ctx->status();
   if (!done) {
     GemmF64Args g;
@@ -1839,7 +1855,7 @@ ltgw_status solve_impl(ltgw_ctx *ctx, const ltgw_params *p, const double *eps, c
                              d_Pi, s, p->use_laplace, emu_f) != LTGW_OK)
         return ctx->status();
     } else if (polarizability_dev(ctx, N, n_ov, Bt, ld_bt, d_delta, n_omega, d_om, n_tau, d_x, d_w, d_E, d_M,
-                                  p->spin, d_Pi, s, p->use_laplace) != LTGW_OK) {
+                                  p->spin, d_Pi, s, p->use_laplace, false) != LTGW_OK) {
       return ctx->status();
     }
     ctx->mark(EV_PI, s);
@@ -1980,7 +1996,7 @@ ltgw_status polarizability_dev_api(ltgw_ctx *ctx, int N, int64_t n_pairs, const 
   LTGW_CUDA(ctx, cudaMemsetAsync(ctx->flags, 0, FLAG_COUNT * sizeof(int), s));
   if (ctx->status() != LTGW_OK) return ctx->status();
   if (polarizability_dev(ctx, N, n_pairs, Bt, n_pairs, delta, n_omega, d_om, n_tau, d_x, d_w, d_E, d_M,
-                         spin, Pi, s, lt_form) != LTGW_OK)
+                         spin, Pi, s, lt_form, true) != LTGW_OK)
     return ctx->status();
   return check_flags(ctx, s);   // synchronises: the staged grid lives in the workspace
 }

@@ -15,6 +15,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "pair_scale.cuh"
 
 namespace ltgw {
 
@@ -29,14 +30,6 @@ struct TileSmem {
   T Bs[BK][BN + PAD];
   T sc[BK];
 };
-
-// Scale applied to pair (column) k of the A operand for batch entry b.
-__device__ __forceinline__ double pair_scale(int mode, double d, double p0, double p1) {
-  if (mode == SCALE_DIRECT) return d / (p0 * p0 + d * d);   // D / (w^2 + D^2)
-  if (mode == SCALE_LAPLACE) return p1 * d * exp(-d * d * p0);  // w_m D e^{-D^2 x_m}
-  if (mode == SCALE_EXPTAU) return exp(-d * p0);                // e^{-D tau_k}
-  return 1.0;
-}
 
 // Accumulate one BMxBN output tile over the full K range into acc.
 // A is MxK (K-major: A[m*lda+k]; else A[k*lda+m]); B is KxN (K-major:

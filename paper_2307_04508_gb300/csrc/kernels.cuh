@@ -269,6 +269,28 @@ size_t slice_gemm_plan(SliceGemmArgs *g, int n_sm, size_t max_partial);
 size_t slice_gemm_piece(SliceGemmArgs *g);
 cudaError_t launch_slice_gemm(const SliceGemmArgs &g, int n_sm, cudaStream_t s);
 cudaError_t launch_slice_coldot_reduce(const SliceGemmArgs &g, double *W, int64_t ldw, cudaStream_t s);
+// ---- Pi's weak entries (pi_weak.cu) ----
+// C_b = alpha X diag(f_b) X^T (N x N, full) from base-256 digits of the scaled rows
+// (dig, exps): the entries that these hold with fewer bits than
+// an FP64 sum, overwritten with their FP64 sums over k < K.
+struct PiWeakArgs {
+  const uint8_t *dig = nullptr;
+  int64_t dig_batch = 0;
+  const int *exps = nullptr;
+  int64_t exp_batch = 0;
+  int nkb = 0;                   // the digits' own length, which may be the last chunk of K
+  int N = 0, mode = SCALE_NONE;
+  int64_t K = 0;
+  const double *X = nullptr;
+  int64_t ld = 0;
+  const double *delta = nullptr, *p0 = nullptr, *p1 = nullptr;   // f_b from these (ScaleMode), or
+  const double *sgn = nullptr, *mag = nullptr;                   // its two root factors [b][f_batch]
+  int64_t f_batch = 0;
+  double alpha = 1.0;
+  double *C = nullptr;           // [batch][N][N]
+};
+cudaError_t launch_pi_weak(const PiWeakArgs &a, int batch, cudaStream_t s);
+
 // C[m][n] = C[n][m] for m > n.
 cudaError_t launch_mirror_upper(double *C, int N, int64_t ldc, int64_t batch_stride, int batch, cudaStream_t s);
 

@@ -157,3 +157,49 @@ def test_naf_from_digits(ctx, n, pairs):
     assert np.abs(lg - ref[:k]).max() <= tol
     assert np.linalg.norm(K @ U - U * lg[None, :], axis=0).max() <= tol
     assert np.abs(U.T @ U - np.eye(k)).max() <= 32 * n * U_ROUND
+
+
+def _weak_rows(rng, N, K, odd, tail):
+    """Gaussian rows, large on the first half of the pairs and `tail` times smaller on
+    the second; the rows `odd` the other way round, so that every term of their
+    products with the others is small beside the rows' largest entries."""
+    R = rng.standard_normal((N, K))
+    head = np.arange(K) < K // 2
+    R[:, ~head] *= tail
+    R[odd] = rng.standard_normal((len(odd), K)) * np.where(head, tail, 1.0)
+    return R
+
+
+# few weak entries per tile (one pass of 128 and several), most of a tile, whole
+# tiles; eight and seven levels; a tail that the digits hold in part and not at all
+@pytest.mark.parametrize("N,K,odd,tail", [(150, 3001, [5, 77], 1e-9), (150, 3001, [3, 4, 70, 71, 149], 1e-20),
+                                          (130, 5200, list(range(0, 130, 2)), 1e-9), (70, 5200, [69], 1e-6),
+                                          (64, 700, list(range(20, 64)), 1e-12), (40, 300001, [7, 8], 1e-9)])
+def test_pi_weakly_coupled_rows(ctx, N, K, odd, tail):
+    """Componentwise: an entry is off by no more than an FP64 sum's bound, K u of
+    sum |a||b| (1.04 K u where the leading digits have just passed it) and the 16 u of
+    the module docstring."""
+    rng = np.random.default_rng(N + K)
+    R = _weak_rows(rng, N, K, odd, tail)
+    delta = 0.3 + 3.0 * rng.random(K)
+    om = np.array([0.4])
+    got = _pi(ctx, R, delta, om)[0]
+    f = delta / (om[0] ** 2 + delta * delta)
+    size = 4.0 * ((np.abs(R) * f[None, :]) @ np.abs(R).T)
+    Rl, fl = R.astype(np.longdouble), f.astype(np.longdouble)
+    for i in sorted({0, N // 2, N - 1, odd[0], odd[-1]}):
+        ref = -4.0 * (Rl * (Rl[i] * fl)[None, :]).sum(axis=1)
+        err = np.abs((got[i] - ref).astype(np.float64))
+        assert np.all(err <= (1.04 * K + 16) * U * size[i]), (i, (err / size[i]).max())
+    assert np.array_equal(got, got.T)
+
+
+def test_pi_infinite_entries_as_an_fp64_sum(ctx):
+    rng = np.random.default_rng(8)
+    N, K = 140, 4000
+    R = rng.standard_normal((N, K))
+    R[130, 3999] = np.inf
+    R[2, 3999] = 0.0
+    got = _pi(ctx, R, 0.3 + rng.random(K), np.array([0.1]))[0]
+    want = np.where(R[:, 3999] == 0.0, np.nan, -np.inf * np.sign(R[:, 3999]))
+    assert np.array_equal(got[130], want, equal_nan=True) and np.array_equal(got[:, 130], want, equal_nan=True)
