@@ -165,7 +165,7 @@ ltgw_status read_small(ltgw_ctx *ctx, void *dst, const void *src, size_t bytes, 
 ltgw_status check_flags(ltgw_ctx *ctx, cudaStream_t s) {
   int h[FLAG_COUNT];
   if (read_small(ctx, h, ctx->flags, sizeof(h), s) != LTGW_OK) return ctx->status();
-  if (h[FLAG_EIG]) ctx->fail(LTGW_ERR_EIG, "NAF eigensolver: inverse iteration produced a non-finite vector");
+  if (h[FLAG_EIG]) ctx->fail(LTGW_ERR_EIG, "NAF eigensolver: a vector was not finite, or a wait in the reduction timed out");
   if (h[FLAG_NOT_SPD]) ctx->fail(LTGW_ERR_NOT_SPD, "screening: a pivot of 1 - Pi(iw) was not positive");
   if (h[FLAG_TC_TIMEOUT]) ctx->fail(LTGW_ERR_DEVICE, "tensor-core kernel: a pipeline wait timed out");
   return ctx->status();

@@ -1,22 +1,28 @@
 // Symmetric eigensolver for the natural auxiliary functions (Sec. 2:
 // diagonalise K, keep the eigenvectors whose eigenvalue exceeds eps_NAF).
 //
-//  1. Householder reduction K = Q T Q^T to tridiagonal T (one reflector per
-//     step: reflector, symmetric mat-vec, rank-2 update of the trailing block);
+//  1. Householder reduction K = Q T Q^T to tridiagonal T.  From n = 1000 on in
+//     panels of 64 steps, whose rank-128 update comes from integer digits on the
+//     tensor cores; the last 800 or so columns, and smaller matrices, in one
+//     kernel that applies a rank-2 update per step;
 //  2. Sturm-sequence count of the eigenvalues of T above the threshold;
-//  3. multisection for the kept eigenvalues, with T in shared memory;
-//  4. inverse iteration for their eigenvectors (tridiagonal LU with row
-//     interchanges), with modified Gram-Schmidt inside groups of nearly equal
-//     eigenvalues;
-//  5. symmetric re-orthonormalisation X <- X (3 - X^T X)/2 twice, which removes
-//     the small non-orthogonality inverse iteration leaves between close
-//     eigenvalues without leaving the span of X;
-//  6. back-transformation U = Q X in compact-WY blocks of 64 reflectors
-//     (split-K GEMMs), written transposed as the rows of Ut.
+//  3. multisection for the kept eigenvalues, with T in shared memory, its points
+//     placed by an FP32 estimate and by secants;
+//  4. their eigenvectors from twisted factorisations of T; inverse iteration
+//     (tridiagonal LU with row interchanges, modified Gram-Schmidt inside groups
+//     of nearly equal eigenvalues) for those that these leave, and where T does
+//     not fit in shared memory;
+//  5. one symmetric re-orthonormalisation X <- X (3 - X^T X)/2, which squares the
+//     small non-orthogonality left between close eigenvalues without leaving the
+//     span of X;
+//  6. back-transformation U = Q X in compact-WY blocks of 64 reflectors, written
+//     transposed as the rows of Ut.  Steps 5 and 6 from digits from n = 200 on, as
+//     long as their scratch holds the digits (up to about 70 % of the vectors
+//     kept), else on the FP64 units.
 //
-// FP64 throughout (both the plain and the mixed-precision solve: only the
-// dense contractions around the eigensolver change precision).  Only the kept
-// eigenvectors are formed.  Householder convention: H = 1 - tau v v^T,
+// FP64 accuracy in norm throughout (both the plain and the mixed-precision solve:
+// only the dense contractions around the eigensolver change precision).  Only the
+// kept eigenvectors are formed.  Householder convention: H = 1 - tau v v^T,
 // v_0 = 1, H x = beta e_1.
 //
 // On this part an FP64 FMA has a dependent latency of about 64 cycles and an
@@ -29,6 +35,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "fast_fp64.cuh"
 #include "kernels.cuh"
 #include "per_device.h"
 
@@ -276,45 +283,6 @@ __device__ __forceinline__ T row_pass(T *row, int j0, int j1, const T *vp, const
     acc0 = fma(a, vc[j], acc0);
   }
   return acc0 + acc1;
-}
-
-// 1/q to the last bits: estimate (about 2^-23) and one cubic step.
-__device__ __forceinline__ double recip_cubic(double q) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(q));
-  const double e = fma(-q, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
-
-// tau, beta and sc of the reflector that maps (alpha, x') to (beta, 0), |x'|^2 =
-// sigma.  One thread's FP64 instructions follow one another at 64 clocks, comparisons
-// included, so: the reciprocal square root and the reciprocal from the hardware's
-// estimates by one cubic step each (the errors, about 2^-23, to the third power),
-// signs and ranges on the integer pipe; 12 instructions instead of about 28 with
-// Newton steps and FP64 comparisons, and 2700 clocks of the fused kernel's step
-// with the IEEE square root and divisions.  Outside the range where the squares
-// are safe, those.
-__device__ __forceinline__ void reflector_scalars(double alpha, double sigma, double *tau, double *beta, double *sc) {
-  if (((__double2hiint(sigma) & 0x7fffffff) | __double2loint(sigma)) == 0) { *tau = 0.0; *beta = alpha; *sc = 0.0; return; }
-  const double s = fma(alpha, alpha, sigma), aa = fabs(alpha);
-  const int ex = __double2hiint(s) >> 20;   // biased exponent; above 2047: the sign
-  double nrm, rinv, rden;
-  if ((unsigned)(ex - 223) < 1600u) {       // 2^-800 <= s < 2^800
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s));
-    const double e = fma(-s * y, y, 1.0);
-    rinv = fma(y * e, fma(e, 0.375, 0.5), y);
-    nrm = s * rinv;
-    rden = recip_cubic(aa + nrm);
-  } else {
-    nrm = sqrt(s);
-    rinv = 1.0 / nrm;
-    rden = 1.0 / (aa + nrm);
-  }
-  const bool neg = __double2hiint(alpha) < 0;
-  *beta = neg ? nrm : -nrm;
-  *tau = fma(aa, rinv, 1.0);                            // (beta - alpha) / beta
-  *sc = neg ? -rden : rden;                             // 1 / (alpha - beta)
 }
 
 // FP64 instructions are scarce on this part (about 2 per clock per SM), so
