@@ -259,6 +259,31 @@ def pi_roofline(prec, pi_flops, pi_ms, pk, src, traffic=None):
                     "128 x 128 tiles do more MMA work"}
 
 
+def householder_fp64_flops(n):
+    """FP64 instructions' flops of the reduction: a panel step is one matrix-vector
+    product with the (n - k - 1)^2 trailing entries, its updates run from integer
+    digits on the tensor cores; a step of the fused kernel (n < 1000, and the last 800
+    columns or so) adds the rank-2 update, two multiply-adds per entry."""
+    k0 = 0
+    while n >= 1000 and n - k0 >= 864:
+        k0 += 64
+    return float(sum(2 * (n - k - 1) ** 2 for k in range(k0)) + sum(6 * (n - k - 1) ** 2 for k in range(k0, n - 2)))
+
+
+def tri_roofline(n, tri_ms, alu_peak, traffic=None):
+    """Roofline of the Householder reduction of the N_aux x N_aux metric."""
+    flops = householder_fp64_flops(n)
+    ach = flops / (tri_ms / 1e3) / 1e12
+    return {"bound": "alu", "kernel": "hh_panel_kernel, hh_fused_kernel<double> (NAF Householder tridiagonalisation, FP64)",
+            "achieved": ach, "peak": alu_peak, "unit": "TFLOP/s", "frac": ach / alu_peak,
+            "peak_source": "FP64 FMA: 152 SMs x 2 FMA/clk x max SM clock (recipe unit counts)",
+            "flops_per_launch": flops, "ms_per_launch": tri_ms, "us_per_step": 1e3 * tri_ms / max(1, n - 2),
+            "note": "flops of the FP64 pipe: the matrix-vector products (full storage) and the fused kernel's rank-2 "
+                    "updates; the panels' updates run from integer digits on the tensor cores; two grid barriers "
+                    "(1.2 us each measured alone) per panel step, one per fused step on top",
+            "traffic": traffic}
+
+
 def pi_error_vs_fp64(ctx, prob, N, n_omega, prec, stream):
     """Relative Frobenius error of Pi(i w_j) in the given tensor-core form against
     the FP64 form, both through the library's entry points, on the first N
@@ -347,20 +372,7 @@ def run_gpu(args):
     # (tc_tma_ts_pi_mid.md); mid workload only
     traffic_pi = 112.52e6 + 44.94e6 if args.workload == "mid" and args.precision == "bf16x3" else None
     roof_pi = pi_roofline(args.precision, pi_flops, pi_ms, pk, src, traffic_pi)
-    # Householder reduction of the N_aux x N_aux metric: 4/3 N^3 algorithmic flops,
-    # N - 2 steps of one or two grid barriers each (latency-bound at mid size)
-    tri_flops = 4.0 / 3.0 * prob.n_aux ** 3
-    tri_ach = tri_flops / (tri_ms / 1e3) / 1e12
-    # FP64 in both forms (the mixed form lowers only the dense contractions)
-    roof_tri = {"bound": "alu", "kernel": "hh_panel_kernel, hh_fused_kernel<double> (NAF Householder tridiagonalisation, FP64)",
-                "achieved": tri_ach, "peak": alu_peak, "unit": "TFLOP/s", "frac": tri_ach / alu_peak,
-                "peak_source": "FP64 FMA: 152 SMs x 2 FMA/clk x max SM clock (recipe unit counts)",
-                "flops_per_launch": tri_flops, "ms_per_launch": tri_ms,
-                "us_per_step": 1e3 * tri_ms / max(1, prob.n_aux - 2),
-                "note": "the panels' matrix-vector products take 2/3 N^3 FP64 flops (full storage), their "
-                        "updates run from integer digits on the tensor cores; two grid barriers (1.2 us "
-                        "each measured alone) per reflector on top",
-                "traffic": None}
+    roof_tri = tri_roofline(prob.n_aux, tri_ms, alu_peak)
     roofline = roof_tri if tri_ms > pi_ms else roof_pi
     clocks = clk.summary()
     line = {"metric": "G0W0 solves/s", "value": value, "unit": "solves/s", "n_gpus": world, "steps": args.steps,
@@ -684,14 +696,7 @@ def run_large(args):
     pk, src_pk = peaks()
     alu_peak = fp64_alu_peak_tflops(pk.get("sm_max_mhz", 2070.0))
     roof_pi = pi_roofline(args.precision, pi_flops, pi_ms, pk, src_pk, LARGE_TRAFFIC.get(("pi", args.precision)))
-    tri_flops = 4.0 / 3.0 * cfg["n_aux"] ** 3
-    tri_ach = tri_flops / (tri_ms / 1e3) / 1e12
-    roof_tri = {"bound": "alu", "kernel": "hh_panel_kernel, hh_fused_kernel<double> (NAF Householder tridiagonalisation, FP64)",
-                "achieved": tri_ach, "peak": alu_peak, "unit": "TFLOP/s", "frac": tri_ach / alu_peak,
-                "peak_source": "FP64 FMA: 152 SMs x 2 FMA/clk x max SM clock (recipe unit counts)",
-                "flops_per_launch": tri_flops, "ms_per_launch": tri_ms,
-                "note": "4/3 N^3 algorithmic flops of the reduction (symmetry exploited); N = N_aux = 9000",
-                "traffic": LARGE_TRAFFIC.get(("hh", "any"))}
+    roof_tri = tri_roofline(cfg["n_aux"], tri_ms, alu_peak, LARGE_TRAFFIC.get(("hh", "any")))
     roofline = roof_tri if tri_ms > pi_ms else roof_pi
     gold = golden_large()
     line = {"metric": "G0W0 solves/s", "value": value, "unit": "solves/s", "n_gpus": world, "steps": args.steps,
@@ -896,7 +901,7 @@ def run_eig(args):
     line = {"metric": "NAF eigensolver (profiling workload)", "n": n, "n_naf": k, "steps": args.steps,
             "ms_tridiag": tri, "ms_eig_vectors": float(np.mean([r["ms_eig_vectors"] for r in rows])),
             "ms_naf_metric": float(np.mean([r["ms_naf_metric"] for r in rows])),
-            "tridiag_tflops": 4.0 / 3.0 * n ** 3 / (tri / 1e3) / 1e12, "launches": rows[-1]["kernel_launches"]}
+            "tridiag_tflops": householder_fp64_flops(n) / (tri / 1e3) / 1e12, "launches": rows[-1]["kernel_launches"]}
     print(json.dumps(line), flush=True)
     ctx.close()
 
