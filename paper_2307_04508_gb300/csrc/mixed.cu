@@ -396,7 +396,9 @@ __device__ __forceinline__ float4 e4m3x4_value(uint32_t c) {
 __device__ __forceinline__ void codes_of(float4 x, float inv, uint32_t *h, uint32_t *l) {
   *h = e4m3x4(x, inv);
   const float4 hv = e4m3x4_value(*h);
-  *l = e4m3x4(make_float4(__fsub_rn(__fmul_rn(x.x, inv), hv.x), __fsub_rn(__fmul_rn(x.y, inv), hv.y), __fsub_rn(__fmul_rn(x.z, inv), hv.z), __fsub_rn(__fmul_rn(x.w, inv), hv.w)), 1.0f);
+  *l = e4m3x4(make_float4(__fsub_rn(__fmul_rn(x.x, inv), hv.x), __fsub_rn(__fmul_rn(x.y, inv), hv.y),
+                          __fsub_rn(__fmul_rn(x.z, inv), hv.z), __fsub_rn(__fmul_rn(x.w, inv), hv.w)),
+              1.0f);
 }
 __device__ __forceinline__ void write_codes(uint32_t *row, int64_t k, int64_t q4, float4 x, float inv, int split,
                                             bool a_pattern) {
@@ -433,7 +435,8 @@ __device__ __forceinline__ void write_codes4(uint32_t *row, int64_t k, int64_t q
 // Bound: HBM, n_t times three code bytes per value.  N = 611, 20,001 pairs, 32
 // frequencies (1.2 GB of codes): 0.55 ms with the maxima; one block per row with all 32 factor
 // rows in its registers took 1.09 ms.
-constexpr int Q8_ROWS = Q8_THREADS / 32, Q8_T = 8, Q8_CHUNK = 512;   // Q8_CHUNK: float4 per row and block (more for rows past 1.3e8 values)
+constexpr int Q8_ROWS = Q8_THREADS / 32, Q8_T = 8;
+constexpr int Q8_CHUNK = 512;   // float4 per row and block (more for rows past 1.3e8 values)
 
 // maxima (float bits, zeroed beforehand) [n_t][rows] of |X_rk S_tk|, then [rows] of |X_rk|
 __global__ void __launch_bounds__(Q8_THREADS)
@@ -577,7 +580,8 @@ cudaError_t launch_fp8_quantize(const float *X, int64_t Kp, int64_t Kq, const fl
   if (Kp % 16 || Kq % 16 || Kq < Kp || n_t < 0 || n_t > 32) return cudaErrorInvalidValue;   // Kp is padded to 64
   cudaError_t e = cudaMemsetAsync(maxima, 0, (size_t)(n_t + 1) * rows * sizeof(int), s);
   if (e != cudaSuccess) return e;
-  const int64_t q4 = Kq / 4, chunk = std::max<int64_t>(Q8_CHUNK, ((q4 + 65534) / 65535 + 3) / 4 * 4), chunks = (q4 + chunk - 1) / chunk;
+  const int64_t q4 = Kq / 4, chunk = std::max<int64_t>(Q8_CHUNK, ((q4 + 65534) / 65535 + 3) / 4 * 4);
+  const int64_t chunks = (q4 + chunk - 1) / chunk;
   const dim3 grid((rows + Q8_ROWS - 1) / Q8_ROWS, (unsigned)chunks, std::max(1, (n_t + Q8_T - 1) / Q8_T));
   fp8_max_kernel<<<grid, Q8_THREADS, 0, s>>>(X, Kp, S, n_t, rows, chunk, maxima);
   fp8_quantize_kernel<<<grid, Q8_THREADS, 0, s>>>(X, Kp, Kq, S, n_t, rows, chunk, maxima, qa, qb, ds_a, ds_b, split);

@@ -146,30 +146,30 @@ __global__ void __cluster_dims__(B / SB_RPC, 1, 1) __launch_bounds__(SB_THREADS)
 #pragma unroll
       for (int j = 0; j < SB_PR; ++j) {
         if (j < np) {
-        const int k = k0 + j;
-        const double piv = at(v, j, k);
-        if (lane == 0 && !(piv > 0.0 && isfinite(piv))) atomicExch(&flags[FLAG_NOT_SPD], 1);
-        const double rp = 1.0 / piv;
-        rps[j] = rp;
-        double a[NC], c[SB_PR];
+          const int k = k0 + j;
+          const double piv = at(v, j, k);
+          if (lane == 0 && !(piv > 0.0 && isfinite(piv))) atomicExch(&flags[FLAG_NOT_SPD], 1);
+          const double rp = 1.0 / piv;
+          rps[j] = rp;
+          double a[NC], c[SB_PR];
 #pragma unroll
-        for (int r = 0; r < SB_PR; ++r) c[r] = r == j ? 0.0 : at(v, r, k);
+          for (int r = 0; r < SB_PR; ++r) c[r] = r == j ? 0.0 : at(v, r, k);
 #pragma unroll
-        for (int h = 0; h < NC; ++h) a[h] = v[j][h] * rp;
-        const uint32_t row = rowk_addr + (uint32_t)((par * SB_PR + j) * B + 2 * lane) * sizeof(double);
+          for (int h = 0; h < NC; ++h) a[h] = v[j][h] * rp;
+          const uint32_t row = rowk_addr + (uint32_t)((par * SB_PR + j) * B + 2 * lane) * sizeof(double);
 #pragma unroll
-        for (unsigned cta = 0; cta < B / SB_RPC; ++cta)
+          for (unsigned cta = 0; cta < B / SB_RPC; ++cta)
 #pragma unroll
-          for (int h = 0; h < NC; h += 2) st_cluster_2f64(row + 32 * h * sizeof(double), cta, a[h], a[h + 1]);
+            for (int h = 0; h < NC; h += 2) st_cluster_2f64(row + 32 * h * sizeof(double), cta, a[h], a[h + 1]);
 #pragma unroll
-        for (int h = 0; h < NC; ++h) {
-          const bool at_k = col(h) == k;
+          for (int h = 0; h < NC; ++h) {
+            const bool at_k = col(h) == k;
 #pragma unroll
-          for (int r = 0; r < SB_PR; ++r) {
-            if (r == j) v[r][h] = at_k ? -rp : a[h];
-            else v[r][h] = at_k ? c[r] * rp : fma(-c[r], a[h], v[r][h]);
+            for (int r = 0; r < SB_PR; ++r) {
+              if (r == j) v[r][h] = at_k ? -rp : a[h];
+              else v[r][h] = at_k ? c[r] * rp : fma(-c[r], a[h], v[r][h]);
+            }
           }
-        }
         }
       }
       if (lane < B / SB_RPC) {   // one CTA per lane
@@ -183,19 +183,19 @@ __global__ void __cluster_dims__(B / SB_RPC, 1, 1) __launch_bounds__(SB_THREADS)
       for (int j = 0; j < SB_PR; ++j) {
         const int k = k0 + j;
         if (j < np) {
-        const double rp = rpk[par][j];
-        double c[SB_PR], ck[SB_PR];
+          const double rp = rpk[par][j];
+          double c[SB_PR], ck[SB_PR];
 #pragma unroll
-        for (int r = 0; r < SB_PR; ++r) { c[r] = at(v, r, k); ck[r] = c[r] * rp; }
+          for (int r = 0; r < SB_PR; ++r) { c[r] = at(v, r, k); ck[r] = c[r] * rp; }
 #pragma unroll
-        for (int h = 0; h < NC; h += 2) {
-          const double2 a = *reinterpret_cast<const double2 *>(&rowk[par][j][2 * lane + 32 * h]);
+          for (int h = 0; h < NC; h += 2) {
+            const double2 a = *reinterpret_cast<const double2 *>(&rowk[par][j][2 * lane + 32 * h]);
 #pragma unroll
-          for (int r = 0; r < SB_PR; ++r) {
-            v[r][h] = col(h) == k ? ck[r] : fma(-c[r], a.x, v[r][h]);
-            v[r][h + 1] = col(h + 1) == k ? ck[r] : fma(-c[r], a.y, v[r][h + 1]);
+            for (int r = 0; r < SB_PR; ++r) {
+              v[r][h] = col(h) == k ? ck[r] : fma(-c[r], a.x, v[r][h]);
+              v[r][h + 1] = col(h + 1) == k ? ck[r] : fma(-c[r], a.y, v[r][h + 1]);
+            }
           }
-        }
         }
       }
     }
@@ -304,7 +304,7 @@ cudaError_t screen_blocked_impl(const double *Pi, int N, int n_omega, T *work, d
 // 5.58 ms, N = 160: 0.59 against 0.85 ms, error against 64-bit torch not larger
 // at any size from 130 to 2258.
 constexpr int SD_B = 128;
-constexpr int SD_NS = 7, SD_BITS = 8;   // the FP64 digits; levels up to 8 (the ninth changes the error by 1 %, the time by 16 %)
+constexpr int SD_NS = 7, SD_BITS = 8;   // the FP64 digits; levels up to 8 (the ninth: error 1 % less, time 16 % more)
 
 // X = I - Pi on the upper triangle (and what of the lower its 32-column blocks cover)
 __global__ void form_upper_kernel(const double *__restrict__ Pi, double *__restrict__ X, int N) {

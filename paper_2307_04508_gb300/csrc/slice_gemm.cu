@@ -34,8 +34,8 @@
 // instruction per output.
 //
 // Bound: the tensor pipe (28 BF16 products per useful one).  Measured, Pi's
-// eight moments at N = 453, 27,000 pairs: 1.36 ms of MMAs and drains, 58 % of
-// the tensor pipe's cycles (28 products: 0.9 PFLOP/s; useful 32 TFLOP/s), where the
+// eight moments at N = 453, 27,000 pairs: 1.2 ms of MMAs and drains, 70 % of the
+// tensor pipe's cycles (28 products: 1.0 PFLOP/s; useful 37 TFLOP/s), where the
 // FP64 tiles of gemm_f64.cu took 56 ms at 95 % of the FP64 pipe.  Issuing the
 // upper and the lower levels from two threads: 2.60 -> 2.46 ms for the whole
 // call, one copy per lane of the producer: 2.37 ms.
@@ -64,7 +64,9 @@ constexpr int SG_EPI_WARPS = 16;
 // separate accumulators, so one issuer's MMAs run while the other's levels are
 // drained, and the two share the issue overhead), then the epilogue: sixteen warps
 // of 16 columns each (two 64-bit sums per output: eight warps of 32 columns
-// would need 128 registers for the sums alone and spill).
+// would need 128 registers for the sums alone).  608 threads leave 96 registers;
+// ptxas spills 44 bytes of <7, 8, 7>, 256 of <7, 8, 8>, 172 of <6, 7, 6> and 136 of
+// <7, 7, 7> around the drain.
 constexpr int SG_EPI0 = 3, SG_CW = SG_N * 4 / SG_EPI_WARPS;
 constexpr int SG_THREADS = 32 * (SG_EPI0 + SG_EPI_WARPS);
 static_assert(SG_CW == 16, "one 16-column load per level");
@@ -889,8 +891,9 @@ cudaError_t launch_ns(const SliceGemmArgs &g, int blocks, cudaStream_t s) {
 }  // namespace
 
 cudaError_t launch_slice_operand(const SliceSrc &a, int ns, int bits, int batch, cudaStream_t s) {
-  if (a.rows < 1 || a.K < 1 || batch < 1 || batch > 65535 || a.rows > a.rows_p || a.rows_p % 128 || (int64_t)a.nkb * 16 < a.K || a.exp_batch < a.rows_p || (a.cols && (a.colscale || a.only_if)) || (!a.cols && a.col_group) ||
-      a.kb_first < 0 || a.kb_first >= a.nkb || ((a.kb_first || a.fixed_exp) && !a.cols))
+  if (a.rows < 1 || a.K < 1 || batch < 1 || batch > 65535 || a.rows > a.rows_p || a.rows_p % 128 ||
+      (int64_t)a.nkb * 16 < a.K || a.exp_batch < a.rows_p || (a.cols && (a.colscale || a.only_if)) ||
+      (!a.cols && a.col_group) || a.kb_first < 0 || a.kb_first >= a.nkb || ((a.kb_first || a.fixed_exp) && !a.cols))
     return cudaErrorInvalidValue;
   if (bits == 8) return ns == 7 ? slice_operand<7, 8>(a, batch, s) : cudaErrorInvalidValue;
   switch (bits == 7 ? ns : 0) {
@@ -958,9 +961,9 @@ size_t slice_gemm_plan(SliceGemmArgs *g, int n_sm, size_t max_partial) {
 
 cudaError_t launch_slice_gemm(const SliceGemmArgs &g, int n_sm, cudaStream_t s) {
   const int64_t units = (int64_t)g.batch * g.splits * g.n_tiles;
-  if (g.M < 1 || g.N < 1 || g.batch < 1 || g.kb_first < 0 || g.nkb <= g.kb_first || g.splits < 1 || g.kb_per_split < 1 || g.drain_kb < 1 ||
-      g.n_tiles < 1 || (g.splits > 1 && !g.partial) || (g.splits == 1 && g.partial) || (g.b_sel && !g.B_alt) || (g.sym && g.M != g.N) ||
-      !g.A || !g.B || !g.ea || !g.eb || !g.err || (!g.cd_out && !g.C) || (g.cd_out && (g.sym || g.partial)))
+  if (g.M < 1 || g.N < 1 || g.batch < 1 || g.kb_first < 0 || g.nkb <= g.kb_first || g.splits < 1 ||
+      g.kb_per_split < 1 || g.drain_kb < 1 || g.n_tiles < 1 || (g.splits > 1 && !g.partial) ||
+      (g.splits == 1 && g.partial) || (g.b_sel && !g.B_alt) || (g.sym && g.M != g.N) || !g.A || !g.B || !g.ea || !g.eb || !g.err || (!g.cd_out && !g.C) || (g.cd_out && (g.sym || g.partial)))
     return cudaErrorInvalidValue;
   const int blocks = (int)std::min<int64_t>(units, n_sm);
   cudaError_t e = cudaErrorInvalidValue;
