@@ -200,9 +200,10 @@ constexpr SliceForm emu_digits(int n_slices) { return {n_slices, 7, true}; }
 // (ltgw_set_digit_memory) and half of what is free on the device allow.  The
 // lengths of the sums (pair chunks, K splits) follow from the product's sizes
 // alone (the splits from those of a piece of kSliceHold bytes), so a result has
-// the same bits whatever piece fits.  A pair chunk costs another pass over the
-// output: 1 % at N = 2258, whose chunks have 12,000 pairs.
-constexpr size_t kSliceTermMax = (size_t)768 << 20;    // digits of one matrix's operands (sets its pair chunk)
+// the same bits whatever piece fits.  A pair chunk costs another conversion of the
+// sums and pass over the output, 0.5 ms for ten moments of N = 2258: in chunks of
+// 12,000 pairs (768 MiB) 4 % of the time, of 25,000 2 %.
+constexpr size_t kSliceTermMax = (size_t)1536 << 20;   // digits of one matrix's operands (sets its pair chunk)
 constexpr size_t kSlicePartialMax = (size_t)1 << 30;   // K-split partial tiles of a piece
 constexpr int64_t kSliceMinCols = 1024;                // columns of a projection's smallest piece
 

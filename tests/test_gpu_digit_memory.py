@@ -113,8 +113,8 @@ def test_many_targets_in_pieces_have_the_same_bits(emu, naf):
 
 
 def test_pi_chunks_of_a_long_sum():
-    """512,001 pairs of 100 rows: 2 x 128 x 14 bytes a pair, three chunks of at
-    most 768 MB, the last one ragged."""
+    """512,001 pairs of 100 rows: 2 x 128 x 14 bytes a pair, two chunks of at most
+    1.5 GiB, the last one ragged."""
     rng = np.random.default_rng(6)
     N, K = 100, 512001
     R = rng.standard_normal((N, K))
@@ -137,7 +137,7 @@ def test_pi_chunks_of_a_long_sum():
 
 
 def test_metric_chunks_of_a_long_sum():
-    """1,000,003 pairs of 48 rows (three chunks of 128 x 14 bytes a pair) through the
+    """1,000,003 pairs of 48 rows (two chunks of 128 x 14 bytes a pair) through the
     NAF eigenvalues: K to K u of the rows' scales, the eigensolver to n u |K|."""
     rng = np.random.default_rng(7)
     n, K = 48, 1000003

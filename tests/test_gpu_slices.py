@@ -174,7 +174,7 @@ def _weak_rows(rng, N, K, odd, tail):
 # tiles; eight and seven levels; a tail that the digits hold in part and not at all
 @pytest.mark.parametrize("N,K,odd,tail", [(150, 3001, [5, 77], 1e-9), (150, 3001, [3, 4, 70, 71, 149], 1e-20),
                                           (130, 5200, list(range(0, 130, 2)), 1e-9), (70, 5200, [69], 1e-6),
-                                          (64, 700, list(range(20, 64)), 1e-12), (40, 300001, [7, 8], 1e-9)])
+                                          (64, 700, list(range(20, 64)), 1e-12), (40, 500001, [7, 8], 1e-9)])
 def test_pi_weakly_coupled_rows(ctx, N, K, odd, tail):
     """Componentwise: an entry is off by no more than an FP64 sum's bound, K u of
     sum |a||b| (1.04 K u where the leading digits have just passed it) and the 16 u of
