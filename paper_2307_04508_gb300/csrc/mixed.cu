@@ -429,36 +429,42 @@ __device__ __forceinline__ void write_codes4(uint32_t *row, int64_t k, int64_t q
 // ds_a[t][r]; code columns Kp..Kq-1 are zero.  split: each code row holds three
 // segments of Kq (the two-term expansion, write_codes).
 //
-// Two kernels over (8 rows, a chunk of k, 8 factor rows): the maxima, then the
+// Two kernels over (8 rows, a chunk of k, T factor rows): the maxima, then the
 // codes.  A warp takes one row, so the eight warps of a block share the factor
 // rows' chunk through L1, and the grid fills the SMs whatever the row count.
 // Bound: HBM, n_t times three code bytes per value.  N = 611, 20,001 pairs, 32
 // frequencies (1.2 GB of codes): 0.55 ms with the maxima; one block per row with all 32 factor
-// rows in its registers took 1.09 ms.
-constexpr int Q8_ROWS = Q8_THREADS / 32, Q8_T = 8;
-constexpr int Q8_CHUNK = 512;   // float4 per row and block (more for rows past 1.3e8 values)
+// rows in its registers took 1.09 ms.  Few rows: a block's chain of loads bounds
+// it, so fewer factor rows and a shorter chunk per block where those of eight
+// rows and 512 float4 would not fill the SMs (whole Pi, 32 frequencies: N = 120, 4,000
+// pairs 121 -> 107 us, N = 300, 1,500 pairs 147 -> 133; N = 611, 20,001 pairs would be
+// 1262 instead of 1191).
+constexpr int Q8_ROWS = Q8_THREADS / 32;
+constexpr int Q8_CHUNK = 512, Q8_CHUNK_FEW = 128;   // float4 per row and block (more for rows past 1.3e8 values)
+constexpr int64_t Q8_FEW = 152 * 8;                 // blocks
 
 // maxima (float bits, zeroed beforehand) [n_t][rows] of |X_rk S_tk|, then [rows] of |X_rk|
+template <int T>
 __global__ void __launch_bounds__(Q8_THREADS)
     fp8_max_kernel(const float *__restrict__ X, int64_t Kp, const float *__restrict__ S, int n_t, int rows,
                    int64_t chunk, int *__restrict__ maxima) {
-  const int r = blockIdx.x * Q8_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31, t0 = blockIdx.z * Q8_T;
+  const int r = blockIdx.x * Q8_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31, t0 = blockIdx.z * T;
   if (r >= rows) return;
   const float4 *xr = reinterpret_cast<const float4 *>(X + (int64_t)r * Kp);
   const int64_t n4 = Kp / 4, k0 = (int64_t)blockIdx.y * chunk, k1 = min(n4, k0 + chunk);
-  float mb = 0.0f, ma[Q8_T] = {};
+  float mb = 0.0f, ma[T] = {};
   for (int64_t k = k0 + lane; k < k1; k += 32) {
     const float4 x = xr[k];
     mb = fmaxf(mb, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))));
 #pragma unroll
-    for (int u = 0; u < Q8_T; ++u)
+    for (int u = 0; u < T; ++u)
       if (t0 + u < n_t) {
         const float4 sv = __ldg(reinterpret_cast<const float4 *>(S + (int64_t)(t0 + u) * Kp) + k);
         ma[u] = fmaxf(ma[u], fmaxf(fmaxf(fabsf(x.x * sv.x), fabsf(x.y * sv.y)), fmaxf(fabsf(x.z * sv.z), fabsf(x.w * sv.w))));
       }
   }
 #pragma unroll
-  for (int u = 0; u < Q8_T; ++u) {   // magnitudes order as their bits
+  for (int u = 0; u < T; ++u) {   // magnitudes order as their bits
     const int m = __reduce_max_sync(0xffffffffu, __float_as_int(ma[u]));
     if (lane == 0 && t0 + u < n_t && m) atomicMax(maxima + (int64_t)(t0 + u) * rows + r, m);
   }
@@ -471,23 +477,24 @@ __device__ __forceinline__ float e4m3_inv(int max_bits) {
   return m > 0.0f ? E4M3_MAX / m : 0.0f;
 }
 
+template <int T>
 __global__ void __launch_bounds__(Q8_THREADS)
     fp8_quantize_kernel(const float *__restrict__ X, int64_t Kp, int64_t Kq, const float *__restrict__ S, int n_t,
                         int rows, int64_t chunk, const int *__restrict__ maxima, uint8_t *__restrict__ qa, uint8_t *__restrict__ qb,
                         float *__restrict__ ds_a, float *__restrict__ ds_b, int split) {
-  const int r = blockIdx.x * Q8_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31, t0 = blockIdx.z * Q8_T;
+  const int r = blockIdx.x * Q8_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31, t0 = blockIdx.z * T;
   if (r >= rows) return;
   const float4 *xr = reinterpret_cast<const float4 *>(X + (int64_t)r * Kp);
   const int64_t n4 = Kp / 4, q4 = Kq / 4, k0 = (int64_t)blockIdx.y * chunk, k1 = min(q4, k0 + chunk);
   const int64_t Ks = split ? 3 * Kq : Kq;   // codes per row
   const float invb = e4m3_inv(maxima[(int64_t)n_t * rows + r]);
-  float inv[Q8_T];
+  float inv[T];
 #pragma unroll
-  for (int u = 0; u < Q8_T; ++u) inv[u] = t0 + u < n_t ? e4m3_inv(maxima[(int64_t)(t0 + u) * rows + r]) : 0.0f;
+  for (int u = 0; u < T; ++u) inv[u] = t0 + u < n_t ? e4m3_inv(maxima[(int64_t)(t0 + u) * rows + r]) : 0.0f;
   if (blockIdx.y == 0 && lane == 0) {
     if (t0 == 0) ds_b[r] = invb > 0.0f ? 1.0f / invb : 0.0f;
 #pragma unroll
-    for (int u = 0; u < Q8_T; ++u)
+    for (int u = 0; u < T; ++u)
       if (t0 + u < n_t) ds_a[(int64_t)(t0 + u) * rows + r] = inv[u] > 0.0f ? 1.0f / inv[u] : 0.0f;
   }
   uint32_t *qbr = qb && t0 == 0 ? reinterpret_cast<uint32_t *>(qb + (int64_t)r * Ks) : nullptr;
@@ -498,7 +505,7 @@ __global__ void __launch_bounds__(Q8_THREADS)
     for (int v = 0; v < 4; ++v) x[v] = in ? xr[k + v] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (qbr) write_codes4(qbr, k, q4, x, invb, split, false);
 #pragma unroll
-    for (int u = 0; u < Q8_T; ++u)
+    for (int u = 0; u < T; ++u)
       if (t0 + u < n_t) {
         float4 p[4];
 #pragma unroll
@@ -512,6 +519,75 @@ __global__ void __launch_bounds__(Q8_THREADS)
   }
 }
 
+// The same with one block per row, which keeps the maxima of all factor rows (MAXT at
+// most): one launch, and X and the factor rows stay in L1 between its two passes.
+// For up to 12 factor rows of up to Q8_ROW_K codes; whole Pi with eight points,
+// against the two kernels above: N = 200, 2,000 pairs 97 us (105), 8,000 130 (137),
+// 15,000 181 (176); N = 2000, 8,000 pairs 1114 (1152), 15,000 1738 (1700).
+constexpr int Q8_ROW_T = 12;
+constexpr int64_t Q8_ROW_K = 12288;
+template <int MAXT>
+__global__ void __launch_bounds__(Q8_THREADS)
+    fp8_quantize_rows_kernel(const float *__restrict__ X, int64_t Kp, int64_t Kq, const float *__restrict__ S, int n_t,
+                        int rows, uint8_t *__restrict__ qa, uint8_t *__restrict__ qb, float *__restrict__ ds_a,
+                        float *__restrict__ ds_b, int split) {
+  __shared__ float red[Q8_THREADS / 32];
+  __shared__ float inv_s[MAXT + 1];
+  const int r = blockIdx.x;
+  const float4 *xr = reinterpret_cast<const float4 *>(X + (int64_t)r * Kp);
+  const int64_t n4 = Kp / 4, q4 = Kq / 4;
+  float mb = 0.0f, ma[MAXT];
+#pragma unroll
+  for (int t = 0; t < MAXT; ++t) ma[t] = 0.0f;
+  for (int64_t k = threadIdx.x; k < n4; k += Q8_THREADS) {
+    const float4 x = xr[k];
+    mb = fmaxf(mb, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))));
+#pragma unroll
+    for (int t = 0; t < MAXT; ++t) {
+      if (t < n_t) {
+        const float4 sv = reinterpret_cast<const float4 *>(S + (int64_t)t * Kp)[k];
+        ma[t] = fmaxf(ma[t], fmaxf(fmaxf(fabsf(x.x * sv.x), fabsf(x.y * sv.y)),
+                                   fmaxf(fabsf(x.z * sv.z), fabsf(x.w * sv.w))));
+      }
+    }
+  }
+  mb = block_max(mb, red);
+  if (threadIdx.x == 0) inv_s[MAXT] = mb > 0.0f ? E4M3_MAX / mb : 0.0f;
+#pragma unroll
+  for (int t = 0; t < MAXT; ++t) {
+    if (t < n_t) {
+      const float m = block_max(ma[t], red);
+      if (threadIdx.x == 0) inv_s[t] = m > 0.0f ? E4M3_MAX / m : 0.0f;
+    }
+  }
+  __syncthreads();
+  const float invb = inv_s[MAXT];
+  if (threadIdx.x == 0) {
+    ds_b[r] = invb > 0.0f ? 1.0f / invb : 0.0f;
+    for (int t = 0; t < n_t; ++t) ds_a[(int64_t)t * rows + r] = inv_s[t] > 0.0f ? 1.0f / inv_s[t] : 0.0f;
+  }
+  const int64_t Ks = split ? 3 * Kq : Kq;   // codes per row
+  uint32_t *qbr = qb ? reinterpret_cast<uint32_t *>(qb + (int64_t)r * Ks) : nullptr;
+  for (int64_t k = threadIdx.x; k < q4; k += Q8_THREADS) {
+    if (k >= n4) {
+      for (int seg = 0; seg < (split ? 3 : 1); ++seg) {
+        if (qbr) qbr[seg * q4 + k] = 0u;
+        for (int t = 0; t < n_t; ++t) reinterpret_cast<uint32_t *>(qa + ((int64_t)t * rows + r) * Ks)[seg * q4 + k] = 0u;
+      }
+      continue;
+    }
+    const float4 x = xr[k];
+    if (qbr) write_codes(qbr, k, q4, x, invb, split, false);
+#pragma unroll
+    for (int t = 0; t < MAXT; ++t) {
+      if (t < n_t) {
+        const float4 sv = reinterpret_cast<const float4 *>(S + (int64_t)t * Kp)[k];
+        const float4 p = make_float4(x.x * sv.x, x.y * sv.y, x.z * sv.z, x.w * sv.w);
+        write_codes(reinterpret_cast<uint32_t *>(qa + ((int64_t)t * rows + r) * Ks), k, q4, p, inv_s[t], split, true);
+      }
+    }
+  }
+}
 // One block per row r of X [rows][Kp]: codes of X itself as an A operand
 // (split: segments h | l | h), de-scale to ds[r].
 __global__ void __launch_bounds__(Q8_THREADS)
@@ -578,13 +654,24 @@ cudaError_t launch_fp8_quantize(const float *X, int64_t Kp, int64_t Kq, const fl
                                 int split) {
   if (rows <= 0) return cudaSuccess;
   if (Kp % 16 || Kq % 16 || Kq < Kp || n_t < 0 || n_t > 32) return cudaErrorInvalidValue;   // Kp is padded to 64
+  if (n_t > 0 && n_t <= Q8_ROW_T && Kq <= Q8_ROW_K) {
+    const auto kernel = n_t <= 8 ? fp8_quantize_rows_kernel<8> : fp8_quantize_rows_kernel<Q8_ROW_T>;
+    kernel<<<rows, Q8_THREADS, 0, s>>>(X, Kp, Kq, S, n_t, rows, qa, qb, ds_a, ds_b, split);
+    return cudaGetLastError();
+  }
   cudaError_t e = cudaMemsetAsync(maxima, 0, (size_t)(n_t + 1) * rows * sizeof(int), s);
   if (e != cudaSuccess) return e;
-  const int64_t q4 = Kq / 4, chunk = std::max<int64_t>(Q8_CHUNK, ((q4 + 65534) / 65535 + 3) / 4 * 4);
-  const int64_t chunks = (q4 + chunk - 1) / chunk;
-  const dim3 grid((rows + Q8_ROWS - 1) / Q8_ROWS, (unsigned)chunks, std::max(1, (n_t + Q8_T - 1) / Q8_T));
-  fp8_max_kernel<<<grid, Q8_THREADS, 0, s>>>(X, Kp, S, n_t, rows, chunk, maxima);
-  fp8_quantize_kernel<<<grid, Q8_THREADS, 0, s>>>(X, Kp, Kq, S, n_t, rows, chunk, maxima, qa, qb, ds_a, ds_b, split);
+  const int64_t q4 = Kq / 4, least = ((q4 + 65534) / 65535 + 3) / 4 * 4;
+  const int gx = (rows + Q8_ROWS - 1) / Q8_ROWS;
+  auto run = [&](auto max_kernel, auto code_kernel, int64_t chunk, int t) {
+    const dim3 grid(gx, (unsigned)((q4 + chunk - 1) / chunk), std::max(1, (n_t + t - 1) / t));
+    max_kernel<<<grid, Q8_THREADS, 0, s>>>(X, Kp, S, n_t, rows, chunk, maxima);
+    code_kernel<<<grid, Q8_THREADS, 0, s>>>(X, Kp, Kq, S, n_t, rows, chunk, maxima, qa, qb, ds_a, ds_b, split);
+  };
+  if (gx * ((q4 + Q8_CHUNK - 1) / Q8_CHUNK) * std::max(1, (n_t + 7) / 8) >= Q8_FEW)
+    run(fp8_max_kernel<8>, fp8_quantize_kernel<8>, std::max<int64_t>(Q8_CHUNK, least), 8);
+  else
+    run(fp8_max_kernel<2>, fp8_quantize_kernel<2>, std::max<int64_t>(Q8_CHUNK_FEW, least), 2);
   return cudaGetLastError();
 }
 
