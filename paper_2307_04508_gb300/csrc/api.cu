@@ -1994,12 +1994,16 @@ ltgw_status polarizability_dev_api(ltgw_ctx *ctx, int N, int64_t n_pairs, const 
     if (lt_form != 2) copy_in(ctx, d_w, w, n_tau * sizeof(double), s);
     copy_in(ctx, d_E, h_E.data(), h_E.size() * sizeof(double), s);
   }
-  LTGW_CUDA(ctx, cudaMemsetAsync(ctx->flags, 0, FLAG_COUNT * sizeof(int), s));
+  // only the digit kernels set flags
+  const bool flags = slices_pay(N, N, n_pairs, n_tau ? n_tau : n_omega);
+  if (flags) LTGW_CUDA(ctx, cudaMemsetAsync(ctx->flags, 0, FLAG_COUNT * sizeof(int), s));
   if (ctx->status() != LTGW_OK) return ctx->status();
   if (polarizability_dev(ctx, N, n_pairs, Bt, n_pairs, delta, n_omega, d_om, n_tau, d_x, d_w, d_E, d_M,
                          spin, Pi, s, lt_form, true) != LTGW_OK)
     return ctx->status();
-  return check_flags(ctx, s);   // synchronises: the staged grid lives in the workspace
+  if (flags) return check_flags(ctx, s);   // synchronises: the staged grid lives in the workspace
+  LTGW_CUDA(ctx, cudaStreamSynchronize(s));
+  return LTGW_OK;
 }
 
 // lt_form 1: x, w are the Laplace grid of Eq. LT; 2: x holds tau_k and gamma
