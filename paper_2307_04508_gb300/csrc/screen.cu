@@ -77,7 +77,9 @@ __global__ void form_a_kernel(const double *__restrict__ Pi, T *__restrict__ X, 
 // (one CTA per frequency would leave most SMs idle through the bs pivots).
 // CTA c of the cluster holds rows SB_RPC*c .. SB_RPC*c + SB_RPC - 1 of the
 // block in registers: warp w rows 4w .. 4w + 3 of them, lane l the column pairs
-// 2l, 2l + 64, ...  Four pivots form a round: the warp that holds their rows
+// 2l, 2l + 64, ... (B = 32: column l; the FP64 pipe's time is a warp's whatever its
+// lanes hold, so a matrix of up to 32 rows does not take B = 64: N = 32, 32
+// frequencies 138 us for the screening, 148 so).  Four pivots form a round: the warp that holds their rows
 // sweeps those four rows alone (no other row changes them), writes the four
 // rows, each scaled by its pivot's reciprocal at its turn, and the reciprocals
 // into every CTA's shared memory; one cluster barrier; then every other row
@@ -103,11 +105,18 @@ __device__ __forceinline__ void st_cluster_2f64(uint32_t local_addr, unsigned ra
   asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(remote), "d"(v0), "d"(v1) : "memory");
 }
 
+__device__ __forceinline__ void st_cluster_f64(uint32_t local_addr, unsigned rank, double v) {
+  uint32_t remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local_addr), "r"(rank));
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(v) : "memory");
+}
+
 template <int B, bool UPPER>
 __global__ void __cluster_dims__(B / SB_RPC, 1, 1) __launch_bounds__(SB_THREADS)
     block_inverse_kernel(const double *__restrict__ X, int N, int p0, int bs, double *__restrict__ Z, int *flags) {
-  constexpr int NC = B / 32;          // columns per lane, in pairs
-  static_assert(B == 64 || B == 128, "one or two column pairs per lane");
+  constexpr int NC = B / 32;          // columns per lane, in pairs (B = 32: one)
+  constexpr int LDZ = B == 32 ? 64 : B;
+  static_assert(B == 32 || B == 64 || B == 128, "one column or one or two column pairs per lane");
   __shared__ __align__(16) double rowk[2][SB_PR][B];
   __shared__ __align__(16) double rpk[2][SB_PR];
   unsigned crank;
@@ -116,12 +125,13 @@ __global__ void __cluster_dims__(B / SB_RPC, 1, 1) __launch_bounds__(SB_THREADS)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i0 = (int)crank * SB_RPC + SB_PR * warp;
   const double *Xb = X + (int64_t)b * N * N;
-  auto col = [&](int h) { return 2 * lane + 64 * (h >> 1) + (h & 1); };
+  auto col = [&](int h) { return NC == 1 ? lane : 2 * lane + 64 * (h >> 1) + (h & 1); };
   // entry (row r of the warp, block column c), in every lane
   auto at = [&](const double (&v)[SB_PR][NC], int r, int c) {
-    double x = (c & 1) ? v[r][1] : v[r][0];
+    if (NC == 1) return __shfl_sync(0xffffffffu, v[r][0], c);
+    double x = (c & 1) ? v[r][NC > 1] : v[r][0];
     if (NC > 2) {
-      const double y = (c & 1) ? v[r][NC - 1] : v[r][NC - 2];
+      const double y = (c & 1) ? v[r][NC - 1] : v[r][NC > 1 ? NC - 2 : 0];
       if (c >= 64) x = y;
     }
     return __shfl_sync(0xffffffffu, x, (c & 63) >> 1);
@@ -156,11 +166,16 @@ __global__ void __cluster_dims__(B / SB_RPC, 1, 1) __launch_bounds__(SB_THREADS)
           for (int r = 0; r < SB_PR; ++r) c[r] = r == j ? 0.0 : at(v, r, k);
 #pragma unroll
           for (int h = 0; h < NC; ++h) a[h] = v[j][h] * rp;
-          const uint32_t row = rowk_addr + (uint32_t)((par * SB_PR + j) * B + 2 * lane) * sizeof(double);
+          const uint32_t row = rowk_addr + (uint32_t)((par * SB_PR + j) * B + col(0)) * sizeof(double);
 #pragma unroll
-          for (unsigned cta = 0; cta < B / SB_RPC; ++cta)
+          for (unsigned cta = 0; cta < B / SB_RPC; ++cta) {
+            if constexpr (NC == 1) {
+              st_cluster_f64(row, cta, a[0]);
+            } else {
 #pragma unroll
-            for (int h = 0; h < NC; h += 2) st_cluster_2f64(row + 32 * h * sizeof(double), cta, a[h], a[h + 1]);
+              for (int h = 0; h < NC; h += 2) st_cluster_2f64(row + 32 * h * sizeof(double), cta, a[h], a[h + 1]);
+            }
+          }
 #pragma unroll
           for (int h = 0; h < NC; ++h) {
             const bool at_k = col(h) == k;
@@ -187,13 +202,19 @@ __global__ void __cluster_dims__(B / SB_RPC, 1, 1) __launch_bounds__(SB_THREADS)
           double c[SB_PR], ck[SB_PR];
 #pragma unroll
           for (int r = 0; r < SB_PR; ++r) { c[r] = at(v, r, k); ck[r] = c[r] * rp; }
+          if constexpr (NC == 1) {
+            const double a = rowk[par][j][lane];
 #pragma unroll
-          for (int h = 0; h < NC; h += 2) {
-            const double2 a = *reinterpret_cast<const double2 *>(&rowk[par][j][2 * lane + 32 * h]);
+            for (int r = 0; r < SB_PR; ++r) v[r][0] = lane == k ? ck[r] : fma(-c[r], a, v[r][0]);
+          } else {
 #pragma unroll
-            for (int r = 0; r < SB_PR; ++r) {
-              v[r][h] = col(h) == k ? ck[r] : fma(-c[r], a.x, v[r][h]);
-              v[r][h + 1] = col(h + 1) == k ? ck[r] : fma(-c[r], a.y, v[r][h + 1]);
+            for (int h = 0; h < NC; h += 2) {
+              const double2 a = *reinterpret_cast<const double2 *>(&rowk[par][j][2 * lane + 32 * h]);
+#pragma unroll
+              for (int r = 0; r < SB_PR; ++r) {
+                v[r][h] = col(h) == k ? ck[r] : fma(-c[r], a.x, v[r][h]);
+                v[r][h + 1] = col(h + 1) == k ? ck[r] : fma(-c[r], a.y, v[r][h + 1]);
+              }
             }
           }
         }
@@ -201,13 +222,13 @@ __global__ void __cluster_dims__(B / SB_RPC, 1, 1) __launch_bounds__(SB_THREADS)
     }
   }
   cluster_sync();   // no CTA leaves while another may still write to it
-  double *Zb = Z + (int64_t)b * B * B;
+  double *Zb = Z + (int64_t)b * LDZ * LDZ;
 #pragma unroll
   for (int r = 0; r < SB_PR; ++r)
 #pragma unroll
     for (int h = 0; h < NC; ++h) {
       const int i = i0 + r, j = col(h);
-      if (i < bs && j < bs) Zb[i * B + j] = -v[r][h];
+      if (i < bs && j < bs) Zb[i * LDZ + j] = -v[r][h];
     }
 }
 
@@ -262,7 +283,10 @@ cudaError_t screen_blocked_impl(const double *Pi, int N, int n_omega, T *work, d
   ++*launches;
   for (int p0 = 0; p0 < N; p0 += SB_B) {
     const int bs = std::min(SB_B, N - p0);
-    block_inverse_kernel<SB_B, false><<<dim3(SB_B / SB_RPC, n_omega), SB_THREADS, 0, s>>>(X, N, p0, bs, Z, flags);
+    if (N <= 32)
+      block_inverse_kernel<32, false><<<dim3(32 / SB_RPC, n_omega), SB_THREADS, 0, s>>>(X, N, p0, bs, Z, flags);
+    else
+      block_inverse_kernel<SB_B, false><<<dim3(SB_B / SB_RPC, n_omega), SB_THREADS, 0, s>>>(X, N, p0, bs, Z, flags);
     dim3 cg((N + 255) / 256 < 8 ? (N + 255) / 256 : 8, bs, n_omega);
     copy_rows_kernel<T><<<cg, 256, 0, s>>>(X, N, p0, bs, rowsP);
     GemmArgs<T> g;   // R = X[:, P] Z

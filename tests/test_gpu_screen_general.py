@@ -39,7 +39,7 @@ def test_nan_below_the_diagonal_is_reported(ctx, N, i, j):
     assert e.value.status == ltgw.LTGW_ERR_NOT_SPD
 
 
-@pytest.mark.parametrize("N", [2, 40, 64])
+@pytest.mark.parametrize("N", [1, 2, 31, 32, 33, 40, 64])
 def test_one_block_is_inverted_whole(ctx, N):
     """I - Pi + (a skew part of 0.1): its symmetric part's eigenvalues are >= 1, so
     every pivot is positive and the sweep stable: 64 N u of the two norms."""
