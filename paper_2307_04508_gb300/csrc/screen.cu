@@ -349,19 +349,25 @@ __global__ void __launch_bounds__(256) form_upper_checked_kernel(const double *_
   if (bj < bi) return;
   const double *P = Pi + (int64_t)blockIdx.z * N * N;
   double *Xb = X + (int64_t)blockIdx.z * N * N;
-  const int tx = threadIdx.x;
-  for (int q = threadIdx.y; q < 32; q += 8) {   // the mirrored tile
-    const int r = bj * 32 + q, c = bi * 32 + tx;
-    if (r < N && c < N) t[q][tx] = P[(int64_t)r * N + c];
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  double m[4], v[4];   // the mirrored tile and this one: eight loads at once
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = bj * 32 + ty + 8 * u, c = bi * 32 + tx, i = bi * 32 + ty + 8 * u, j = bj * 32 + tx;
+    m[u] = r < N && c < N ? __ldcs(P + (int64_t)r * N + c) : 0.0;
+    v[u] = i < N && j < N ? __ldcs(P + (int64_t)i * N + j) : 0.0;
   }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) t[ty + 8 * u][tx] = m[u];
   __syncthreads();
   bool bad = false;
-  for (int q = threadIdx.y; q < 32; q += 8) {
-    const int i = bi * 32 + q, j = bj * 32 + tx;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int q = ty + 8 * u, i = bi * 32 + q, j = bj * 32 + tx;
     if (i >= N || j >= N) continue;
-    const double a = P[(int64_t)i * N + j], b = t[tx][q];
+    const double a = v[u], b = t[tx][q];
     Xb[(int64_t)i * N + j] = (i == j ? 1.0 : 0.0) - a;
-    if (__double_as_longlong(a) != __double_as_longlong(b) || !isfinite(a)) {
+    if (__double_as_longlong(a) != __double_as_longlong(b) || (__double2hiint(a) & 0x7ff00000) == 0x7ff00000) {
       const double di = 1.0 - P[(int64_t)i * N + i], dj = 1.0 - P[(int64_t)j * N + j];
       bad |= !(fabs(a - b) <= 4.0 * N * 0x1p-53 * sqrt(di * dj));
     }
