@@ -10,7 +10,7 @@ namespace ltgw {
 constexpr size_t kSliceHold = (size_t)6 << 30;   // default of ltgw_set_digit_memory
 
 // Bytes with which the digits and partial sums of a solve with N auxiliary functions
-// after the NAF step run: `limit`, less where all of them take less, more where
+// after the NAF step (or fewer) run: `limit`, less where all of them take less, more where
 // the smallest piece of a product takes more.
 size_t solve_digit_bytes(const ltgw_params &p, int n_tgt, int N, size_t limit);
 

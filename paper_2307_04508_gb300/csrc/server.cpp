@@ -265,7 +265,8 @@ static Footprint request_footprint(const ltgw_params *p, int n_tgt) {
   Footprint f;
   f.fixed = d * sizeof(double) + (64u << 20);                  // + fixed slack
   f.admit = f.fixed + emu * sizeof(double);
-  f.all = std::max(f.admit, f.fixed + ltgw::solve_digit_bytes(*p, n_tgt, (int)N, kDigitMemory));
+  // with every auxiliary function kept: a piece that did not fit would run on the FP64 tiles
+  f.all = std::max(f.admit, f.fixed + ltgw::solve_digit_bytes(*p, n_tgt, p->n_aux, kDigitMemory));
   return f;
 }
 
