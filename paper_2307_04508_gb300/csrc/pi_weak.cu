@@ -14,14 +14,14 @@
 // entries of rows that are not finite are (their FP64 sums keep the sign of an
 // infinity).
 //
-// One block per 64 x 64 tile of the lower triangle: four groups of 16 rows by KG of
-// every KG-th 16-k block (KG = 8, or 2 up to K = 1024).  The groups' sums are added up at
-// growing intervals and the scan ends when every entry has passed: rows of
-// Gaussian entries take a few hundred k whatever K is, so the scan's latency is
-// its cost and not its products; mma.sync needs no tensor memory and reads the
-// fragments straight from the digits' blocks.  Measured: 0.03 of 2.22 ms for eight
-// moments of N = 453 and 27,000 pairs, 0.025 of 0.31 at N = 200 and 5,000 pairs, 0.011
-// of 0.08 at N = 48 and 64 pairs (32 frequencies).
+// One block per 64 x 64 tile of the lower triangle: four groups of 16 rows by four
+// of every fourth 16-k block.  The groups' sums are added up at growing intervals
+// and the scan ends when every entry has passed: rows of Gaussian entries take a
+// few hundred k whatever K is, so the scan's latency is its cost and not its
+// products; mma.sync needs no tensor memory and reads the fragments straight from
+// the digits' blocks.  Measured: 0.03 of 2.22 ms for eight moments of N = 453 and
+// 27,000 pairs (eight groups, one block per SM: 0.04; two groups 0.11), 0.02 of 0.30
+// at N = 200 and 5,000 pairs, 0.012 of 0.08 at N = 48 and 64 pairs (32 frequencies).
 //
 // Weak entries: up to PW_WHOLE of a tile one per warp at a time (a clock of the
 // FP64 pipe per entry and pair), more by the whole tile (2048 clocks per pair).
@@ -58,9 +58,9 @@ struct PwSmem {
   int exi[64], exj[64], n_list;
 };
 
-template <int KG>
-__global__ void __launch_bounds__(128 * KG) pi_weak_kernel(PiWeakArgs g) {
-  constexpr int THREADS = 128 * KG, WARPS = 4 * KG;
+constexpr int KG = 4, THREADS = 128 * KG, WARPS = 4 * KG;
+
+__global__ void __launch_bounds__(THREADS, 2) pi_weak_kernel(PiWeakArgs g) {
   __shared__ PwSmem sm;
   const int b = blockIdx.y, t = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int I = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
@@ -219,9 +219,7 @@ cudaError_t launch_pi_weak(const PiWeakArgs &a, int batch, cudaStream_t s) {
       !a.X || !a.C || !a.delta || !a.p0 || (!a.sgn != !a.mag))
     return cudaErrorInvalidValue;
   const int t = (a.N + 63) / 64;
-  const dim3 grid(t * (t + 1) / 2, batch);
-  if (a.nkb <= 64) pi_weak_kernel<2><<<grid, 256, 0, s>>>(a);
-  else pi_weak_kernel<8><<<grid, 1024, 0, s>>>(a);
+  pi_weak_kernel<<<dim3(t * (t + 1) / 2, batch), THREADS, 0, s>>>(a);
   return cudaGetLastError();
 }
 
